@@ -8,6 +8,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB = None
+_CALLS = None
 
 FLAG_KEEP_ACTIVATIONS = 1
 FLAG_FORCE_GENERIC = 2
@@ -94,9 +95,27 @@ def library() -> C.CDLL:
     return _LIB
 
 
+def _calls():
+    """The native module behind the hot calls (csrc/torch_calls.cpp); built with the library."""
+    global _CALLS
+    if _CALLS is None:
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        library()
+        from . import _calls as native
+        _CALLS = native
+    return _CALLS
+
+
 def _check(status: int):
     if status != 0:
         raise AccerlError(status, library().accerl_last_error().decode())
+
+
+def _done(r):
+    """The results of a native call, or the error its status code stands for."""
+    if type(r) is int:
+        _check(r)
+    return r
 
 
 def _out_hw(l):
@@ -124,6 +143,9 @@ def _stream_of(t, stream):
 
 def kl(logits_original, logits_smaller, stream=None):
     """accerl_policy_kl on two CUDA fp32 [B, A] tensors; returns (kl [B], mean_max [2]) tensors."""
+    r = (_CALLS or _calls()).kl(logits_original, logits_smaller, stream)
+    if r is not None:
+        return _done(r)
     import torch
     assert logits_original.shape == logits_smaller.shape and logits_original.is_contiguous() and \
         logits_smaller.is_contiguous() and logits_original.dtype == logits_smaller.dtype == torch.float32
@@ -138,6 +160,11 @@ def kl(logits_original, logits_smaller, stream=None):
 def vtrace(logp_smaller, logp_original, rewards, values, bootstrap, gamma, rho_hat=1.0, c_hat=1.0,
            discounts=None, stream=None, out=None, checked=True):
     """accerl_vtrace on CUDA fp32 time-major [n, B] tensors; returns (vs, adv) tensors [n, B]."""
+    if out is None:
+        r = (_CALLS or _calls()).vtrace(logp_smaller, logp_original, rewards, values, bootstrap, discounts, gamma,
+                                        rho_hat, c_hat, stream)
+        if r is not None:
+            return _done(r)
     import torch
     n, b = logp_smaller.shape
     if checked:
@@ -156,6 +183,11 @@ def vtrace(logp_smaller, logp_original, rewards, values, bootstrap, gamma, rho_h
 
 def act_mixed(smaller, original, obs, uniforms, select_uniforms, alpha, stream=None):
     """accerl_policy_act_mixed; returns dict(logits, actions, logp, entropy, use_smaller[, value])."""
+    r = (_CALLS or _calls()).act_mixed(smaller._raw, original._raw, smaller.n_actions, smaller.in_kind == "u8",
+                                       smaller.value_head and original.value_head, obs, uniforms, select_uniforms,
+                                       alpha, stream)
+    if r is not None:
+        return _done(r)
     import torch
     b, dev = int(obs.shape[0]), obs.device
     out = dict(logits=torch.empty((b, smaller.n_actions), dtype=torch.float32, device=dev),
@@ -215,6 +247,7 @@ class Policy:
         _check(lib.accerl_policy_create_fp32(C.byref(self._h), 0 if in_kind == "u8" else 1, shape, descs, n,
                                              calib.ctypes.data, int(calib.shape[0]), int(bool(prune24)),
                                              self.max_batch, int(flags), self.device))
+        self._raw = self._h.value
         self.n_actions = int(layers[-1]["out_c"]) - (1 if self.value_head else 0)
         return self
 
@@ -264,12 +297,17 @@ class Policy:
         _check(lib.accerl_policy_create(C.byref(self._h), 0 if self.in_kind == "u8" else 1, shape,
                                         float(policy["s_input"]), descs, n, self.max_batch,
                                         int(flags), self.device))
+        self._raw = self._h.value
         self.value_head = bool(self.layers[-1].get("value"))
         self.n_actions = int(self.layers[-1]["out_c"]) - (1 if self.value_head else 0)
 
     # -- the hot call ---------------------------------------------------------------------
     def act(self, obs, uniforms, out=None, stream=None):
         """obs, uniforms: CUDA torch tensors.  Returns (logits, actions, logp) CUDA tensors."""
+        r = (_CALLS or _calls()).act(self._raw, self.n_actions, self.in_kind == "u8", obs, uniforms, out, stream)
+        if r is not None:
+            return _done(r)
+        # not what the native call takes: say what is wrong, or go through ctypes
         import torch
         b = int(obs.shape[0])
         if out is None:
@@ -289,6 +327,10 @@ class Policy:
 
     def act_ex(self, obs, uniforms, stream=None) -> dict:
         """accerl_policy_act_ex: dict(logits, actions, logp, entropy[, value]) of CUDA tensors."""
+        r = (_CALLS or _calls()).act_ex(self._raw, self.n_actions, self.in_kind == "u8", self.value_head, obs, uniforms,
+                                        stream)
+        if r is not None:
+            return _done(r)
         import torch
         b, dev = int(obs.shape[0]), obs.device
         out = dict(logits=torch.empty((b, self.n_actions), dtype=torch.float32, device=dev),
@@ -320,8 +362,8 @@ class Policy:
     def act_noalloc_raw(self, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr,
                         stream=0) -> int:
         """accerl_policy_act_noalloc with raw device addresses; returns the status code."""
-        return library().accerl_policy_act_noalloc(self._h, obs_ptr, u_ptr, batch, logits_ptr,
-                                                   actions_ptr, logp_ptr, stream)
+        return (_CALLS or _calls()).act_noalloc(self._raw, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr,
+                                                stream)
 
     def act_raw(self, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr, stream=0) -> int:
         """Unchecked pass-through returning the status code (for ABI tests)."""
@@ -366,6 +408,7 @@ class Policy:
         if self._h:
             library().accerl_policy_destroy(self._h)
             self._h = C.c_void_p()
+            self._raw = 0
 
     def __del__(self):
         try:

@@ -6,6 +6,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
+#include <mutex>
 #include <new>
 
 #include "internal.h"
@@ -30,7 +32,8 @@ struct DeviceGuard {
     explicit DeviceGuard(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        ok = cudaSetDevice(dev) == cudaSuccess;
+        if (prev == dev) prev = -1;  // nothing to set, nothing to restore: the usual call of an Actor
+        else ok = cudaSetDevice(dev) == cudaSuccess;
     }
     ~DeviceGuard()
     {
@@ -204,6 +207,35 @@ void pack_generic(const accerl_layer_desc &d, LayerPlan &L, std::vector<int32_t>
 }
 
 }  // namespace
+
+// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) costs about as much as half a launch, and a step has
+// several launches: remember the largest size each (kernel, device) has been given.  The table is open
+// addressing over atomics; a full table only loses the saving.
+cudaError_t allow_smem(const void *kernel, size_t bytes)
+{
+    struct Slot {
+        std::atomic<uintptr_t> key{0};
+        std::atomic<size_t> bytes{0};
+    };
+    static Slot table[1024];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uintptr_t key = (uintptr_t)kernel * 64 + (uintptr_t)(dev & 63);  // never 0
+    Slot *mine = nullptr;
+    for (unsigned i = 0, h = (unsigned)(key >> 4) * 2654435761u >> 22; i < 1024 && !mine; ++i, h = (h + 1) & 1023) {
+        uintptr_t k = table[h].key.load(std::memory_order_acquire);
+        if (k == 0 && table[h].key.compare_exchange_strong(k, key)) k = key;
+        if (k == key) mine = &table[h];
+    }
+    if (mine && mine->bytes.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    static std::mutex mu;  // the attribute must never go back down
+    std::lock_guard<std::mutex> lock(mu);
+    if (mine && mine->bytes.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && mine) mine->bytes.store(bytes, std::memory_order_release);
+    return e;
+}
 
 accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev)
 {

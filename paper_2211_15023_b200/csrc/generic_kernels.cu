@@ -178,8 +178,7 @@ cudaError_t launch_conv_generic(const LayerPlan &L, const int8_t *in, const int8
     a.relu_out = (L.flags & ACCERL_RELU_OUT) != 0;
     size_t smem = (size_t)L.kh * L.kw * a.C4 * 16 * sizeof(int32_t);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(conv_dp4a_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem((const void *)conv_dp4a_kernel, smem);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)((a.total_px + 127) / 128), L.oc_pad / 16);

@@ -17,6 +17,9 @@ namespace accerl {
 
 void set_error(const char *fmt, ...);
 
+// let a kernel use `bytes` of dynamic shared memory on the current device (api.cu)
+cudaError_t allow_smem(const void *kernel, size_t bytes);
+
 #define ACCERL_CUDA_TRY(expr)                                                              \
     do {                                                                                   \
         cudaError_t e_ = (expr);                                                           \

@@ -23,7 +23,8 @@ struct CurrentDevice {
     explicit CurrentDevice(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        ok = cudaSetDevice(dev) == cudaSuccess;
+        ok = prev == dev || cudaSetDevice(dev) == cudaSuccess;
+        if (prev == dev) prev = -1;
     }
     ~CurrentDevice()
     {

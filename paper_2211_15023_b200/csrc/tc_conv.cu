@@ -370,7 +370,7 @@ cudaError_t conv_rows_launch(const void *map_a, const void *map_b, const ConvRow
     const int grid = q.total_steps < sm_count ? q.total_steps : sm_count;
     const size_t smem = conv_rows_smem_bytes(q0);
     auto go = [&](auto kernel) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem((const void *)kernel, smem);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid);

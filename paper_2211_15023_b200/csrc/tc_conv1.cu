@@ -453,7 +453,7 @@ cudaError_t conv1_launch(const void *map_b, const Conv1Params &q0, int batch, co
     const int grid = q.total_steps < sm_count ? q.total_steps : sm_count;
     const size_t smem = conv1_smem_bytes(q);
     auto go = [&](auto kernel) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem((const void *)kernel, smem);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid);

@@ -979,7 +979,7 @@ cudaError_t tc_launch(const void *map_a, const void *map_b, const TcGemmParams &
     if (!p.shifted && p.sub == 1 && !p.ksplit && tiles <= sm_count) one.n_mma = 1;
     const TcGemmParams &q = one;
     auto go = [&](auto kernel) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem((const void *)kernel, smem);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid);
