@@ -1,12 +1,13 @@
 // The Monitor's indicators and the per-state choice between two policies (Section 2.4).
 //
-// kl_kernel: KL(pi_original || pi_smaller) per state from two logit matrices (Eq. KL), one warp
-// per state, lanes striding over the actions; kl_stats_kernel reduces the per-state values to
-// their mean and maximum (the "KL mean" and "KL max" indicators) in one block, in a fixed order,
-// so that the result does not depend on scheduling.  mix_select_kernel overwrites the original
+// kl_rows_kernel / kl_wide_kernel: KL(pi_original || pi_smaller) per state from two logit matrices
+// (Eq. KL); kl_stats_kernel reduces the per-state values to their mean and maximum (the "KL mean" and
+// "KL max" indicators) in one cluster of CTAs, in a fixed order, so that the result does not depend on
+// scheduling.  mix_select_kernel overwrites the original
 // policy's outputs with the smaller policy's for the states whose selector draw falls below alpha
 // (the linear-alpha strategy of Section 3.2: the Actor follows the small network with
 // probability alpha).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "internal.h"
@@ -29,11 +30,125 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+__device__ __forceinline__ float warp_maxf(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
 // Double arithmetic: where the two policies nearly agree the terms p (log p - log q) cancel, and
-// the indicator runs at the Monitor's interval, not per environment step.
+// the indicator runs at the Monitor's interval, not per environment step.  With e_i = exp(zo_i - mo),
+//   KL = sum_i e_i / so (zo_i - zs_i) - (lse_o - lse_s),
+// two exponentials an action instead of three, and identical rows give exactly 0.
+
+// One row, elements at zo[0], zo[1], ... (any address space), by one thread.
+__device__ __forceinline__ float kl_of_row(const float *zo, const float *zs, int A)
+{
+    float fo = zo[0], fs = zs[0];
+    for (int i = 1; i < A; ++i) {
+        fo = fmaxf(fo, zo[i]);
+        fs = fmaxf(fs, zs[i]);
+    }
+    const double mo = fo, ms = fs;
+    double so = 0.0, ss = 0.0, acc = 0.0;
+    for (int i = 0; i < A; ++i) {
+        const double o = zo[i], s = zs[i], e = exp(o - mo);
+        so += e;
+        ss += exp(s - ms);
+        if (e > 0.0) acc += e * (o - s);
+    }
+    return (float)(acc / so - ((mo + log(so)) - (ms + log(ss))));
+}
+
+constexpr int kKlRows = 128;   // rows (and threads) of a block
+constexpr int kKlCluster = 8;  // CTAs that share the reduction to mean and maximum
+
+// Mean and maximum over all threads of a cluster (every CTA calls with its own partial sum and
+// maximum); always the same order of additions.
+__device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float *stats)
+{
+    __shared__ double s_sum[32];
+    __shared__ float s_max[32];
+    __shared__ double c_sum[kKlCluster];  // used in the first CTA
+    __shared__ float c_max[kKlCluster];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    sum = warp_sum(sum);
+    mx = warp_maxf(mx);
+    if (lane == 0) {
+        s_sum[warp] = sum;
+        s_max[warp] = mx;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        sum = warp_sum(lane < warps ? s_sum[lane] : 0.0);
+        mx = warp_maxf(lane < warps ? s_max[lane] : -INFINITY);
+        if (lane == 0) {
+            const unsigned rank = cooperative_groups::this_cluster().block_rank();
+            *cooperative_groups::this_cluster().map_shared_rank(&c_sum[rank], 0) = sum;
+            *cooperative_groups::this_cluster().map_shared_rank(&c_max[rank], 0) = mx;
+        }
+    }
+    cooperative_groups::this_cluster().sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned n = cooperative_groups::this_cluster().num_blocks();
+        sum = 0.0;
+        mx = -INFINITY;
+        for (unsigned i = 0; i < n; ++i) {
+            sum += c_sum[i];
+            mx = fmaxf(mx, c_max[i]);
+        }
+        stats[0] = (float)(sum / (double)B);
+        stats[1] = mx;
+    }
+}
+
+// A <= 64: one thread per row.  A block's rows are contiguous in memory; they pass through shared
+// memory so that the loads are whole lines and every thread then walks its own row (odd pitch: no
+// bank conflicts).  A warp per row, as for wide rows below, leaves 14 of 32 lanes idle at 18 actions
+// and spends its time in shuffles; with that and a one-block reduction the two launches for 131072
+// rows of 18 took 119 us, now 22.  STATS (one cluster, at most kKlCluster blocks' rows a pass): the mean
+// and the maximum come out of the same launch.
+template <bool STATS>
+__global__ void __launch_bounds__(kKlRows)
+kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B, int A, int pitch,
+               float *__restrict__ kl, float *__restrict__ stats)
+{
+    extern __shared__ float s_rows[];  // [2][kKlRows][pitch]
+    double sum = 0.0;
+    float mx = -INFINITY;
+    for (long long row0 = (long long)blockIdx.x * kKlRows; row0 < B; row0 += (long long)gridDim.x * kKlRows) {
+        const int rows = (int)min((long long)kKlRows, B - row0), n = rows * A;
+        const float *src[2] = {zo + row0 * A, zs + row0 * A};
+        int r = (int)threadIdx.x / A, c = (int)threadIdx.x - r * A;
+        const int dr = kKlRows / A, dc = kKlRows - dr * A;
+        for (int i = threadIdx.x; i < n; i += kKlRows) {
+            s_rows[r * pitch + c] = __ldg(src[0] + i);
+            s_rows[(kKlRows + r) * pitch + c] = __ldg(src[1] + i);
+            r += dr;
+            c += dc;
+            if (c >= A) {
+                c -= A;
+                ++r;
+            }
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < rows) {
+            const float v = kl_of_row(s_rows + threadIdx.x * pitch, s_rows + (kKlRows + threadIdx.x) * pitch, A);
+            kl[row0 + threadIdx.x] = v;
+            sum += (double)v;
+            mx = fmaxf(mx, v);
+        }
+        __syncthreads();
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (STATS) cluster_stats(sum, mx, B, stats);
+}
+
+// any A: one warp per row, lanes striding over the actions
 __global__ void __launch_bounds__(128)
-kl_kernel(const float *__restrict__ zo_all, const float *__restrict__ zs_all, int B, int A,
-          float *__restrict__ kl)
+kl_wide_kernel(const float *__restrict__ zo_all, const float *__restrict__ zs_all, int B, int A,
+               float *__restrict__ kl)
 {
     const int lane = threadIdx.x & 31;
     const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -46,47 +161,38 @@ kl_kernel(const float *__restrict__ zo_all, const float *__restrict__ zs_all, in
     }
     mo = warp_max(mo);
     ms = warp_max(ms);
-    double so = 0.0, ss = 0.0;
+    double so = 0.0, ss = 0.0, acc = 0.0;
     for (int i = lane; i < A; i += 32) {
-        so += exp((double)zo[i] - mo);
-        ss += exp((double)zs[i] - ms);
+        const double o = zo[i], s = zs[i], e = exp(o - mo);
+        so += e;
+        ss += exp(s - ms);
+        if (e > 0.0) acc += e * (o - s);
     }
-    const double lseo = mo + log(warp_sum(so)), lses = ms + log(warp_sum(ss));
-    double acc = 0.0;
-    for (int i = lane; i < A; i += 32) {
-        const double lpo = (double)zo[i] - lseo, lps = (double)zs[i] - lses, p = exp(lpo);
-        if (p > 0.0) acc += p * (lpo - lps);
-    }
+    so = warp_sum(so);
+    ss = warp_sum(ss);
     acc = warp_sum(acc);
-    if (lane == 0) kl[row] = (float)acc;
+    if (lane == 0) kl[row] = (float)(acc / so - ((mo + log(so)) - (ms + log(ss))));
 }
 
-// stats[0] = mean, stats[1] = max of kl[0..B)
+// stats[0] = mean, stats[1] = max of kl[0..B): one cluster, each CTA a contiguous part
 __global__ void __launch_bounds__(1024) kl_stats_kernel(const float *__restrict__ kl, int B, float *stats)
 {
-    __shared__ double s_sum[1024];
-    __shared__ float s_max[1024];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     double sum = 0.0;
     float mx = -INFINITY;
-    for (int i = threadIdx.x; i < B; i += blockDim.x) {
-        const float v = kl[i];
-        sum += (double)v;
-        mx = fmaxf(mx, v);
-    }
-    s_sum[threadIdx.x] = sum;
-    s_max[threadIdx.x] = mx;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) {
-            s_sum[threadIdx.x] += s_sum[threadIdx.x + o];
-            s_max[threadIdx.x] = fmaxf(s_max[threadIdx.x], s_max[threadIdx.x + o]);
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    constexpr int kAhead = 8;  // loads in flight per thread: the kernel is a chain of memory latencies
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < B; i += kAhead * stride) {
+        float v[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) v[j] = i + j * stride < B ? __ldcg(kl + i + j * stride) : -INFINITY;
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            if (i + j * stride < B) sum += (double)v[j];
+            mx = fmaxf(mx, v[j]);
         }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        stats[0] = (float)(s_sum[0] / (double)B);
-        stats[1] = s_max[0];
-    }
+    cluster_stats(sum, mx, B, stats);
 }
 
 struct MixOut {
@@ -135,12 +241,45 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
         return ACCERL_ERR_INVALID_ARG;
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const long long blocks = ((long long)batch * 32 + 127) / 128;
-    kl_kernel<<<(unsigned)blocks, 128, 0, st>>>(logits_original_dev, logits_smaller_dev, batch, n_actions, kl_dev);
+    const bool narrow = n_actions <= 64;  // two blocks' worth of rows fit 48 KB up to 47 actions, 66 KB at 64
+    const int pitch = n_actions | 1;
+    const size_t smem = 2 * sizeof(float) * (size_t)kKlRows * pitch;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    cfg.stream = st;
+    cfg.attrs = attr;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    const long long blocks = narrow ? ((long long)batch + kKlRows - 1) / kKlRows : ((long long)batch * 32 + 127) / 128;
+    if (narrow && kl_mean_max_dev && blocks <= 2 * kKlCluster) {
+        // few rows: one cluster does it all, two passes at most (a second launch costs more)
+        const unsigned n = (unsigned)(blocks < kKlCluster ? blocks : kKlCluster);
+        cfg.gridDim = dim3(n);
+        cfg.blockDim = dim3(kKlRows);
+        cfg.dynamicSmemBytes = smem;
+        attr[0].val.clusterDim.x = n;
+        cfg.numAttrs = 1;
+        ACCERL_CUDA_TRY(allow_smem((const void *)kl_rows_kernel<true>, smem));
+        ACCERL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kl_rows_kernel<true>, logits_original_dev, logits_smaller_dev, batch,
+                                           n_actions, pitch, kl_dev, kl_mean_max_dev));
+        return ACCERL_OK;
+    }
+    if (narrow) {
+        ACCERL_CUDA_TRY(allow_smem((const void *)kl_rows_kernel<false>, smem));
+        kl_rows_kernel<false><<<(unsigned)blocks, kKlRows, smem, st>>>(logits_original_dev, logits_smaller_dev, batch,
+                                                                      n_actions, pitch, kl_dev, nullptr);
+    } else {
+        kl_wide_kernel<<<(unsigned)blocks, 128, 0, st>>>(logits_original_dev, logits_smaller_dev, batch, n_actions, kl_dev);
+    }
     ACCERL_CUDA_TRY(cudaGetLastError());
     if (kl_mean_max_dev) {
-        kl_stats_kernel<<<1, 1024, 0, st>>>(kl_dev, batch, kl_mean_max_dev);
-        ACCERL_CUDA_TRY(cudaGetLastError());
+        cfg.gridDim = dim3(kKlCluster);
+        cfg.blockDim = dim3(1024);
+        attr[0].val.clusterDim.x = kKlCluster;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 2;
+        ACCERL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kl_stats_kernel, (const float *)kl_dev, batch, kl_mean_max_dev));
     }
     return ACCERL_OK;
 }
@@ -188,12 +327,12 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
                                            logp_dev, value_dev, entropy_dev, cuda_stream);
     if (s != ACCERL_OK) return s;
     int prev = -1;
-    cudaGetDevice(&prev);
+    if (cudaGetDevice(&prev) == cudaSuccess && prev == smaller->device) prev = -1;
+    else ACCERL_CUDA_TRY(cudaSetDevice(smaller->device));
     struct Restore {
         int prev;
         ~Restore() { if (prev >= 0) cudaSetDevice(prev); }
     } restore{prev};
-    ACCERL_CUDA_TRY(cudaSetDevice(smaller->device));
     if (!smaller->mix_logits) {
         const size_t mb = (size_t)smaller->max_batch;
         const size_t sz[5] = {4 * mb * (size_t)smaller->n_actions, 4 * mb, 4 * mb, 4 * mb, 4 * mb};
