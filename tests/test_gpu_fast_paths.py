@@ -1,0 +1,91 @@
+"""GPU parity at the sizes where the kernels' tiles, rings and clusters end: vector-observation
+networks, the KL indicators, V-trace and the checks of the native calls -- against the CPU oracle,
+at the tolerances of the other parity tests (logits and codes bit for bit)."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+from parity_util import ATOL, RTOL, compare
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _mlp(dims, seed):
+    rng = np.random.default_rng(seed)
+    layers = W.mlp(dims)
+    calib = rng.standard_normal((64, dims[0])).astype(np.float32)
+    return oracle.calibrate("f32", (dims[0], 1, 1), layers, W.parameters_for(layers, seed), calib)
+
+
+@pytest.mark.parametrize("dims", [[5, 256, 256, 256, 256, 3], [33, 40, 17, 2], [256, 255, 31, 32], [1, 1],
+                                  [3, 128, 64, 7]], ids=lambda d: "-".join(map(str, d)))
+def test_mlp_widths_and_depths(dims):
+    """Widths that are no multiple of an instruction's columns or K step, one layer only, and networks
+    whose weights pass through the two-slot ring; batches around both row tiles, taps included."""
+    import paper_2211_15023_b200 as P
+    pol = _mlp(dims, sum(dims))
+    for b, flags in ((1, 1), (17, 5), (33, 0), (4800, 0)):
+        rng = np.random.default_rng(b)
+        obs = rng.standard_normal((b, dims[0])).astype(np.float32)
+        u = rng.random(b, dtype=np.float32)
+        ref = oracle.forward(pol, obs, u, keep=b < 100)
+        g = P.Policy(pol, b, flags=flags)
+        out = [t.cpu().numpy() for t in g.act(torch.from_numpy(obs).cuda(), torch.from_numpy(u).cuda())]
+        g.check()
+        compare(ref, *out, taps=g.read_activation if flags else None)
+        g.close()
+
+
+@pytest.mark.parametrize("b,a", [(127, 18), (128, 18), (129, 3), (1024, 18), (1025, 2), (2048, 9), (2049, 18), (300, 64),
+                                 (300, 65), (70001, 5)])
+def test_kl_at_the_edges_of_blocks_and_clusters(b, a):
+    import paper_2211_15023_b200 as P
+    rng = np.random.default_rng(b + a)
+    zo = (rng.standard_normal((b, a)) * 3).astype(np.float32)
+    zs = (zo + rng.standard_normal((b, a)) * rng.choice([1e-3, 0.5, 4.0], size=(b, 1))).astype(np.float32)
+    zs[b // 2] = zo[b // 2]
+    want = oracle.kl(zo, zs)
+    kl, stats = (t.cpu().numpy() for t in P.kl(torch.from_numpy(zo).cuda(), torch.from_numpy(zs).cuda()))
+    np.testing.assert_allclose(kl, want, rtol=RTOL, atol=ATOL)
+    assert kl[b // 2] == 0.0
+    np.testing.assert_allclose(stats, [want.mean(), want.max()], rtol=RTOL, atol=ATOL)
+
+
+@pytest.mark.parametrize("n,b", [(15, 31), (16, 32), (17, 33), (33, 65), (64, 1)])
+def test_vtrace_at_the_edges_of_chunks(n, b):
+    import paper_2211_15023_b200 as P
+    r = W.rollouts(n, b, seed=n + b)
+    for disc in (None, r["discounts"]):
+        want = oracle.vtrace(r["logp_smaller"], r["logp_original"], r["rewards"], r["values"], r["bootstrap"],
+                             r["gamma"], 1.0, 1.0, disc)
+        t = {k: torch.from_numpy(r[k]).cuda() for k in ("logp_smaller", "logp_original", "rewards", "values", "bootstrap")}
+        vs, adv = P.vtrace(t["logp_smaller"], t["logp_original"], t["rewards"], t["values"], t["bootstrap"], r["gamma"],
+                           discounts=None if disc is None else torch.from_numpy(disc).cuda())
+        np.testing.assert_allclose(vs.cpu().numpy(), want["vs"], rtol=RTOL, atol=ATOL)
+        np.testing.assert_allclose(adv.cpu().numpy(), want["adv"], rtol=RTOL, atol=ATOL)
+
+
+def test_native_calls_refuse_what_the_python_checks_refused():
+    """Tensors of the wrong type, device or layout raise as before, status codes become AccerlError,
+    and a caller's own result buffers come back as the same object."""
+    import paper_2211_15023_b200 as P
+    g = P.Policy(_mlp([4, 8, 2], 3), 16)
+    obs, u = torch.zeros((16, 4), device="cuda"), torch.zeros(16, device="cuda")
+    out = g.act(obs, u)
+    assert g.act(obs, u, out) is out
+    for bad_obs, bad_u in ((obs.double(), u), (obs.cpu(), u), (obs.t(), u), (obs, u[:5]), (obs, u.double())):
+        with pytest.raises((AssertionError, ValueError)):
+            g.act(bad_obs, bad_u)
+    with pytest.raises(P.AccerlError) as e:
+        g.act(torch.zeros((17, 4), device="cuda"), torch.zeros(17, device="cuda"))
+    assert e.value.status == 3
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        same = g.act(obs, u)
+    side.synchronize()
+    assert torch.equal(same[0], out[0]) and torch.equal(same[1], out[1])
+    g.close()
+    with pytest.raises(P.AccerlError):
+        g.act(obs, u)
