@@ -347,6 +347,29 @@ static accerl_status run_steps(accerl_policy *p, const void *obs_dev, const floa
             ACCERL_CUDA_TRY(conv_rows_launch(cs.map_a, cs.map_b, cs.prm, B, p->sm_count, st));
             break;
         }
+        case Step::RES_FIRST: {
+            if ((uintptr_t)obs_dev & 15) {
+                set_error("act: obs_dev must be 16-byte aligned");
+                return ACCERL_ERR_INVALID_ARG;
+            }
+            ResFirstParams prm = p->res_first;
+            prm.obs = (const uint8_t *)obs_dev;
+            prm.batch = B;
+            ACCERL_CUDA_TRY(res_first_launch(prm, p->sm_count, st));
+            break;
+        }
+        case Step::RES_STACK1: {
+            ResStack1Params prm = p->res_stack1;
+            prm.batch = B;
+            ACCERL_CUDA_TRY(res_stack1_launch(prm, p->sm_count, st));
+            break;
+        }
+        case Step::RES_STACK23: {
+            ResStack23Params prm = p->res_stack23;
+            prm.batch = B;
+            ACCERL_CUDA_TRY(res_stack23_launch(prm, p->sm_count, st));
+            break;
+        }
         case Step::INGEST_NHWC4:
             ACCERL_CUDA_TRY(launch_ingest_u8_nhwc4((const uint8_t *)obs_dev, p->lut,
                                                    p->bufs[p->layers[0].in_buf].ptr, B, p->in_h,

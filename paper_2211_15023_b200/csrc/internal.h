@@ -12,6 +12,7 @@
 #include "tc_conv.h"
 #include "tc_conv1.h"
 #include "tc_gemm.h"
+#include "tc_resnet.h"
 
 namespace accerl {
 
@@ -56,7 +57,8 @@ struct LayerPlan {
 // ("ingest", "layer 3", "layers 3-4", "sample", joined by '+').
 struct Step {
     enum Kind { INGEST, CONV_GENERIC, FC_GENERIC, POOL_GENERIC, SAMPLE, INGEST_S2D, TC_GEMM, MLP_FUSED,
-                INGEST_NHWC4, POOL_DUAL, INGEST_PAD4, FC_SAMPLE, CONV1_FRAMES, CONV_ROWS } kind;
+                INGEST_NHWC4, POOL_DUAL, INGEST_PAD4, FC_SAMPLE, CONV1_FRAMES, CONV_ROWS, RES_FIRST,
+                RES_STACK1, RES_STACK23 } kind;
     int layer = -1;
     int tc = -1;  // index into accerl_policy::tc_steps (TC_GEMM), ::pools (POOL_DUAL) or ::conv_rows (CONV_ROWS)
     std::string kernel, covers;
@@ -139,6 +141,10 @@ struct accerl_policy {
     std::vector<accerl::ConvRowsStep> conv_rows;
     accerl::Conv1Params conv1 = {};       // used by a Step::CONV1_FRAMES launch
     alignas(64) unsigned char conv1_map_b[128] = {};
+    // the image-resident kernels of the residual network (Step::RES_*)
+    accerl::ResFirstParams res_first = {};
+    accerl::ResStack1Params res_stack1 = {};
+    accerl::ResStack23Params res_stack23 = {};
     int8_t *in_pad4 = nullptr;            // frames as [n][H+2][PW][4] with the image at (1, 4)
     int in_pad4_w = 0;
     std::vector<accerl::TapDesc> taps;    // per tensor (index t + 1); empty or null ptr = generic buffer
@@ -208,6 +214,12 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
 // mixed tensor-core / CUDA-core plan for residual 3x3 conv stacks (tc_mixed_plan.cu)
 accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *layers, int n_layers,
                                   bool *used);
+// the same network with its images resident in shared memory (tc_res_plan.cu): fills the three kernels'
+// parameters and their steps, buffers and taps when layers 0 .. 17 are the IMPALA stacks on 84 x 84
+// frames; *used = false when they are not, or a layer has no verified division-free requantiser
+constexpr int kResLayers = 18;
+accerl_status build_res_steps(accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int8_t **x3,
+                              std::vector<Step> *steps, bool *used);
 cudaError_t launch_maxpool_dual(const PoolDualParams &q, int B, cudaStream_t st);
 cudaError_t launch_ingest_u8_nhwc4(const uint8_t *obs, const int8_t *lut, int8_t *out, int B, int H, int W,
                                    int out_hpitch, int out_wpitch, int off_y, int off_x, int arith,

@@ -185,7 +185,7 @@ cudaError_t launch_ingest_u8_nhwc4(const uint8_t *obs, const int8_t *lut, int8_t
 // ---------------------------------------------------------------------------------------
 namespace {
 
-enum Role { GENERIC, POOL, TCCONV, TCPX, TCFC, TCFIRST };
+enum Role { GENERIC, POOL, TCCONV, TCPX, TCFC, TCFIRST, RESIDENT };
 
 struct Forms {  // which stored forms of a tensor its readers need
     bool plain = false, plain_relu = false, pad = false, pad_relu = false, slot = false, slot_relu = false;
@@ -279,6 +279,16 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
         if ((long long)p->max_batch * (p->layers[i].in_h + 2) * (p->layers[i].in_w + 2) + 512 >= (1LL << 31))
             return ACCERL_OK;
 
+    // The IMPALA stacks run image by image in three kernels of their own (tc_resnet.cu), unless every
+    // tensor has to exist; what follows then only places the fully connected layers.
+    std::vector<Step> steps;
+    bool resident = false;
+    int8_t *resident_out = nullptr;
+    accerl_status st;
+    if (!keep && (st = build_res_steps(p, layers, n_layers, &resident_out, &steps, &resident)) != ACCERL_OK) return st;
+    if (resident)
+        for (int i = 0; i < kResLayers; ++i) role[i] = RESIDENT;
+
     // A multi-pixel conv cannot write the pad layout of a 16-channel tensor (its pixels are not
     // contiguous there): such a layer falls back to one position per GEMM row.
     for (int i = 0; i + 1 < n_layers; ++i)
@@ -286,11 +296,12 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
 
     // ---- forms of every tensor (index t + 1; tensor -1 is the quantised input)
     std::vector<Forms> forms(n_layers + 1);
-    forms[0].plain = true;  // the input feeds the generic first conv
-    if (role[0] != GENERIC && role[0] != TCFIRST) return ACCERL_OK;
+    forms[0].plain = !resident;  // the input feeds the generic first conv
+    if (role[0] != GENERIC && role[0] != TCFIRST && !resident) return ACCERL_OK;
     for (int j = 1; j < n_layers; ++j)
         if (layers[j].skip_from == 0 && role[0] == TCFIRST) role[0] = GENERIC;  // tensor 0 must be pool-only
     for (int j = 1; j < n_layers; ++j) {
+        if (role[j] == RESIDENT) continue;
         const accerl_layer_desc &d = layers[j];
         Forms &f = forms[j];  // tensor j - 1
         const bool relu_in = (d.flags & ACCERL_RELU_IN) && !(layers[j - 1].flags & ACCERL_RELU_OUT);
@@ -338,9 +349,12 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
     }
 
     // ---- buffers: plain forms live in the generic plan's buffers, the others are new
-    accerl_status st;
     for (int t = 0; t < n_layers; ++t) {
         Forms &f = forms[t];
+        if (resident && t <= kResLayers) {
+            if (t == kResLayers) f.p_plain_relu = resident_out;
+            continue;
+        }
         const int C = t == 0 ? p->in_cp : p->layers[t - 1].out_cp;
         const int H = t == 0 ? p->in_h : p->layers[t - 1].out_h;
         const int W = t == 0 ? p->in_w : p->layers[t - 1].out_w;
@@ -383,14 +397,14 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
     // ---- steps
     auto bail = [&]() {  // the generic plan stays: forget everything built so far
         p->taps.clear();
+        p->tap_missing.assign(n_layers + 1, 0);
         p->pools.clear();
         p->tc_steps.clear();
         return ACCERL_OK;
     };
-    std::vector<Step> steps;
     bool fused_sample = false;
     p->taps.assign(n_layers + 1, TapDesc());
-    {
+    if (!resident) {
         Step s0;
         const bool fast = p->in_c == 4 && p->in_w % 4 == 0;
         s0.kind = role[0] == TCFIRST ? Step::INGEST_PAD4 : (fast ? Step::INGEST_NHWC4 : Step::INGEST);
@@ -407,7 +421,7 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
         s0.covers = "ingest";
         steps.push_back(s0);
     }
-    for (int i = 0; i < n_layers; ++i) {
+    for (int i = resident ? kResLayers : 0; i < n_layers; ++i) {
         const accerl_layer_desc &d = layers[i];
         const LayerPlan &L = p->layers[i];
         const Forms &fin = forms[i], &fout = forms[i + 1];
@@ -838,7 +852,7 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
     }
     if (tap_fused) {
         // tensors the fused plan stores in no un-ReLU'd form cannot be tapped
-        for (int t = 1; t <= n_layers - 1; ++t) {
+        for (int t = resident ? kResLayers + 1 : 1; t <= n_layers - 1; ++t) {
             const Forms &f = forms[t];
             p->tap_missing[t] = !(f.plain || f.pad || f.slot) ? 1 : 0;
         }

@@ -1,0 +1,808 @@
+// The IMPALA residual network with its images resident in shared memory: three launches from the
+// frames to the fully connected layer's input.
+//
+//   res_first    frames -> quantise -> conv 3x3 (4 -> 16) at 84 x 84 -> max-pool        -> 41 x 41 x 16
+//   res_stack1   two residual blocks at 41 x 41 -> conv 3x3 (16 -> 32) -> max-pool      -> 20 x 20 x 32
+//   res_stack23  two blocks at 20 x 20 -> conv 3x3 -> max-pool -> two blocks at 9 x 9   -> 81 x 32
+//
+// Layer by layer (tc_mixed_plan.cu) every conv reads and writes its tensor, and often a second form
+// of it, through HBM: 15 GB for 16384 states, 20 launches, 4.6 ms.  Here a CTA keeps an image's tensors
+// in shared memory from one layer to the next, the tensor that a residual add needs in spare columns of
+// tensor memory, and all weights of the kernel beside them; only the three tensors between the
+// kernels touch HBM (74 KB a state with the frame).
+//
+// An image's layers depend on one another, so a CTA works on two images at once: two contexts, each
+// with its own issuing warp, warpgroups, buffers and half of tensor memory; while one context
+// requantises, the other's MMAs run.  Inside a context the 128-row tiles of a layer overlap as well:
+// a tile is requantised while the next one is contracted.
+//
+// Convolutions are row-shifted implicit GEMMs as everywhere in this library: a GEMM row is 32 bytes of
+// the stored image (two 16-channel pixels or one of 32 channels), a tap a fixed row offset.  16 channels:
+// a row produces two output pixels (N = 2 * 16, banded weights, six K steps); 32 channels: one (N = 32,
+// nine K steps).  N = 32 instructions cost 40 cycles, bound by reading their 4 KB operand: wider rows
+// (N = 64, four pixels) would save a tenth of the tensor time and quadruple the weights' shared memory.
+//
+// What bounds it: the tensor pipe by instruction count (10 080 cycles an image in res_stack1, 8 640 in
+// res_stack23) and, in res_first, instruction issue of the epilogue.
+//
+// Every wait is bounded.  A role whose wait gives up sets the status word and goes on (all further
+// waits return at once), so that the barriers inside a context always see all their warps.
+#include <cuda.h>
+#include <string.h>
+
+#include "epilogue.cuh"
+#include "internal.h"
+#include "tc_ptx.cuh"
+#include "tc_resnet.h"
+
+namespace accerl {
+
+namespace {
+
+constexpr int kCtx = 2;     // images in flight per CTA
+constexpr int kMaxSlots = 6;
+
+struct __align__(8) ResBars {
+    uint64_t w_ready;
+    uint64_t land[kCtx];                // an image has arrived
+    uint64_t ready[kCtx];               // the operand of the next layer is complete
+    uint64_t acc_full[kCtx][kMaxSlots], acc_empty[kCtx][kMaxSlots];
+    uint32_t tmem_base;
+    int abort_flag;
+};
+
+// byte offset of 16-byte half `c` of 32-byte row `row` under the 32-byte swizzle
+__device__ __forceinline__ uint32_t row_off(int row, int c) { return (uint32_t)(row * 32 + ((c ^ ((row >> 2) & 1)) << 4)); }
+
+__device__ __forceinline__ void sts16(uint32_t addr, uint4 v)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ uint4 lds16(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 relu16(uint4 v)
+{
+    return make_uint4(relu_bytes(v.x), relu_bytes(v.y), relu_bytes(v.z), relu_bytes(v.w));
+}
+
+// all warps of a context's epilogue
+template <int THREADS>
+__device__ __forceinline__ void ctx_sync(int ctx)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + ctx), "n"(THREADS) : "memory");
+}
+
+// byte-wise maximum of signed bytes, two at a time as the high bytes of 16-bit lanes (the low bytes only
+// decide between equal high bytes): `odd` keeps bytes 1 and 3 of the words seen, `even` bytes 0 and 2
+struct ByteMax {
+    uint32_t odd[4], even[4];
+    __device__ __forceinline__ static uint32_t max2(uint32_t a, uint32_t b)
+    {
+        uint32_t r;
+        asm("max.s16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+        return r;
+    }
+    __device__ __forceinline__ void first(uint4 v)
+    {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            odd[i] = w[i];
+            even[i] = w[i] << 8;
+        }
+    }
+    __device__ __forceinline__ void take(uint4 v)
+    {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            odd[i] = max2(odd[i], w[i]);
+            even[i] = max2(even[i], w[i] << 8);
+        }
+    }
+    __device__ __forceinline__ uint4 result() const
+    {
+        return make_uint4(__byte_perm(even[0], odd[0], 0x7351), __byte_perm(even[1], odd[1], 0x7351),
+                          __byte_perm(even[2], odd[2], 0x7351), __byte_perm(even[3], odd[3], 0x7351));
+    }
+};
+
+// sixteen accumulators of channels c0 .. c0 + 15 -> sixteen codes
+__device__ __forceinline__ uint4 requant_res(const int (&acc)[16], const ResLayer &L, int c0)
+{
+    float ks[16], bs[16];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const float4 kv = *reinterpret_cast<const float4 *>(&L.k[c0 + 4 * g]);
+        const float4 bv = *reinterpret_cast<const float4 *>(&L.b[c0 + 4 * g]);
+        ks[4 * g] = kv.x; ks[4 * g + 1] = kv.y; ks[4 * g + 2] = kv.z; ks[4 * g + 3] = kv.w;
+        bs[4 * g] = bv.x; bs[4 * g + 1] = bv.y; bs[4 * g + 2] = bv.z; bs[4 * g + 3] = bv.w;
+    }
+    uint32_t w[4];
+    if (L.affine) requant16_affine<false>(acc, ks, bs, w);
+    else requant16_fastdiv<false>(acc, ks, bs, L.s_out, L.inv_s_out, w);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// acc[i] += skip_mul[c0 + i] * x[i], one dp2a each
+__device__ __forceinline__ void add_skip(int (&acc)[16], uint4 x, const ResLayer &L, int c0)
+{
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const uint4 m = *reinterpret_cast<const uint4 *>(&L.mul[c0 + 4 * g]);
+        acc[4 * g] = __dp2a_lo((int)m.x, (int)w[g], acc[4 * g]);
+        acc[4 * g + 1] = __dp2a_lo((int)m.y, (int)w[g], acc[4 * g + 1]);
+        acc[4 * g + 2] = __dp2a_hi((int)m.z, (int)w[g], acc[4 * g + 2]);
+        acc[4 * g + 3] = __dp2a_hi((int)m.w, (int)w[g], acc[4 * g + 3]);
+    }
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint4 &a, uint4 &b)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "r"(taddr)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, uint4 a, uint4 b)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(a.x), "r"(a.y),
+                 "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// descriptors: constant upper words; the lower word is (address >> 4) | flags
+constexpr uint32_t kDescSw32Hi = (256u >> 4) | (1u << 14) | (6u << 29);   // 32-byte rows, 32-byte swizzle
+constexpr uint32_t kDescSw32Lo = 1u << 16;
+constexpr uint32_t kDescFlatHi = (128u >> 4) | (1u << 14);                // 16-byte rows, no swizzle: 8-row groups 128 bytes apart,
+constexpr uint32_t kDescFlatLo = (16u >> 4) << 16;                        // the second half of a K step is the next row
+__host__ __device__ constexpr uint32_t idesc_for(int n)
+{
+    return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
+}
+__device__ __forceinline__ uint64_t desc(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
+
+// what every kernel of this file does first: barriers, tensor memory, weights; returns the tensor-memory base
+template <int EPI_WARPS>
+__device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, int buffer_bytes, uint8_t *w_smem,
+                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals, int wide_slot)
+{
+    // borders and padding stay zero for the life of the CTA
+    for (int i = threadIdx.x; i < buffer_bytes / 16; i += blockDim.x)
+        reinterpret_cast<uint4 *>(buffers)[i] = make_uint4(0, 0, 0, 0);
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&bars.w_ready), 1);
+        for (int c = 0; c < kCtx; ++c) {
+            mbar_init(smem_u32(&bars.land[c]), 1);
+            mbar_init(smem_u32(&bars.ready[c]), epi_arrivals);
+            for (int s = 0; s < kMaxSlots; ++s) {
+                mbar_init(smem_u32(&bars.acc_full[c][s]), 1);
+                mbar_init(smem_u32(&bars.acc_empty[c][s]), s >= wide_slot ? epi_arrivals : 4);
+            }
+        }
+        bars.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    fence_async();
+    if (warp == EPI_WARPS) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars.tmem_base)), "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (threadIdx.x == 0) {
+        mbar_expect_tx(smem_u32(&bars.w_ready), w_bytes);
+        bulk_load(smem_u32(w_smem), w, w_bytes, smem_u32(&bars.w_ready));
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return bars.tmem_base;
+}
+
+__device__ __forceinline__ void res_teardown(ResBars &bars, int warp, int alloc_warp, uint32_t tmem_base)
+{
+    if (*(volatile int *)&bars.abort_flag)
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);  // let copies in flight land
+    fence_before();
+    __syncthreads();
+    if (warp == alloc_warp) {
+        __syncwarp();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    }
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------------------
+// frames -> first conv -> max-pool
+// ---------------------------------------------------------------------------------------
+// The quantised frame lies in shared memory as lines of 88 four-byte pixels, the image from pixel 4 and
+// line 1 on.  A GEMM row starts every four pixels (16 bytes; unswizzled, so that the 32 bytes of a K
+// step may overlap the next row's) and holds the eight pixels 4X - 4 .. 4X + 3 of a line: enough for
+// the five outputs 4X - 2 .. 4X + 2 and thus for two pooled ones, whose three-pixel maxima are taken on
+// the accumulators (the requantiser is non-decreasing): N = 5 * 16, one K step per tap row.  The
+// maximum over three lines follows on the codes in shared memory.  The MMAs take 2 340 cycles an image;
+// the epilogue's instructions (33 k codes an image, some 14 k warp instructions) bound the kernel.
+namespace {
+constexpr int kFirstWg = 3;                                  // warpgroups per context
+constexpr int kFirstT = kFirstWg * 128, kFirstEpi = kCtx * kFirstWg * 4;
+constexpr int kFirstTiles = 15, kFirstSlots = 3;             // ceil(83 lines * 22 rows / 128)
+constexpr int kFrameBytes = 31 * 1024, kHpBytes = 55 * 1024; // quantised frame (last tile reads past it), pooled lines
+constexpr int kFirstSmem = 1024 + 8192 + kCtx * (kFrameBytes + kHpBytes);
+static_assert((kFirstTiles * 128 + 45) * 16 <= kFrameBytes && 83 * 21 * 32 <= kHpBytes, "buffers");
+}  // namespace
+
+template <bool SHIFT>
+__global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(const __grid_constant__ ResFirstParams p)
+{
+    extern __shared__ __align__(1024) uint8_t res_smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ ResBars bars;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t *bufs = smem + 8192;
+    const uint32_t tmem = res_setup<kFirstEpi>(bars, bufs, kCtx * (kFrameBytes + kHpBytes), smem, p.w, kResFirstWeights,
+                                               warp, kFirstWg * 4, kMaxSlots);
+    volatile int *abort_flag = &bars.abort_flag;
+    const int step = kCtx * (int)gridDim.x;
+
+    if (warp >= kFirstEpi) {
+        // ------------------------------------------------------------------ MMA issuers
+        const int ctx = warp - kFirstEpi;
+        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]);
+        const uint32_t a0 = ((smem_u32(bufs) + (uint32_t)ctx * (kFrameBytes + kHpBytes)) >> 4) | kDescFlatLo;
+        const uint32_t b0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
+        mbar_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        uint32_t slot = 0, phase = 0, it = 0;
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step, ++it) {
+            mbar_wait(ready, it & 1, abort_flag, p.status, 8);
+            fence_after();
+            for (int t = 0; t < kFirstTiles; ++t) {
+                mbar_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                fence_after();
+                if (elect_one()) {
+                    const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 80;
+#pragma unroll
+                    for (int ky = 0; ky < 3; ++ky)
+                        mma_i8(d, desc(kDescFlatHi, a0 + (uint32_t)(t * 128 + ky * 22)), desc(kDescSw32Hi, b0 + (uint32_t)(ky * 160)),
+                               idesc_for(80), (uint32_t)ky);
+                    mma_commit(full0 + 8 * slot);
+                }
+                __syncwarp();
+                if (++slot == kFirstSlots) slot = 0, phase ^= 1;
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ conversion, epilogue, pool
+        const int ctx = warp / (kFirstWg * 4), wg = (warp >> 2) % kFirstWg, q = warp & 3;
+        const int tid = (int)threadIdx.x - ctx * kFirstT;
+        const uint32_t frame = smem_u32(bufs) + (uint32_t)ctx * (kFrameBytes + kHpBytes), hp = frame + kFrameBytes;
+        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]);
+        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
+        auto convert = [&](int n) {
+            constexpr int kGroups = 84 * 21, kIter = (kGroups + kFirstT - 1) / kFirstT;
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(p.obs + (size_t)n * 28224);
+            uint32_t w[kIter][4];
+#pragma unroll
+            for (int j = 0; j < kIter; ++j) {
+                const int i = tid + j * kFirstT;
+                if (i < kGroups)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) w[j][c] = __ldg(src + c * 1764 + i);  // the planes' words in order
+            }
+#pragma unroll
+            for (int j = 0; j < kIter; ++j) {
+                const int i = tid + j * kFirstT;
+                if (i < kGroups) {
+                    const int y = i / 21, g = i - y * 21;
+                    uint4 v;
+                    if (SHIFT) v = ingest_shift_line16(w[j][0], w[j][1], w[j][2], w[j][3]);
+                    else
+                        v = make_uint4(ingest_fixed_line4<true>(w[j][0], w[j][1], w[j][2], w[j][3], 0, p.ingest_mul, p.ingest_add),
+                                       ingest_fixed_line4<true>(w[j][0], w[j][1], w[j][2], w[j][3], 1, p.ingest_mul, p.ingest_add),
+                                       ingest_fixed_line4<true>(w[j][0], w[j][1], w[j][2], w[j][3], 2, p.ingest_mul, p.ingest_add),
+                                       ingest_fixed_line4<true>(w[j][0], w[j][1], w[j][2], w[j][3], 3, p.ingest_mul, p.ingest_add));
+                    sts16(frame + (uint32_t)(((y + 1) * 22 + g + 1) * 16), v);
+                    if (p.tap_in) *reinterpret_cast<uint4 *>(p.tap_in + ((size_t)n * kGroups + i) * 16) = v;
+                }
+            }
+            fence_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(ready);
+            if (tid == 0 && n + step < p.batch)  // the image after this one on its way into L2
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)(n + step) * 28224), "r"(28224)
+                             : "memory");
+        };
+        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
+        if (n < p.batch) convert(n);
+        uint32_t seq0 = 0;  // accumulators handed over before this image
+        for (; n < p.batch; n += step, seq0 += kFirstTiles) {
+            for (int t = wg; t < kFirstTiles; t += kFirstWg) {
+                const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kFirstSlots;
+                mbar_wait(full0 + 8 * slot, (seq / kFirstSlots) & 1, abort_flag, p.status, 16);
+                fence_after();
+                const int m = t * 128 + q * 32 + lane;
+                const int y = m / 22, X = m - y * 22, R = y * 21 + X;
+                const bool valid = X < 21 && y < 83;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    int a[16], b[16], c[16];
+                    const uint32_t ta = tlane + slot * 80 + (uint32_t)(32 * j);
+                    tmem_ld16(ta, a);
+                    tmem_ld16(ta + 16, b);
+                    tmem_ld16(ta + 32, c);
+                    tmem_wait_ld();
+                    if (j == 1) {
+                        fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) a[i] = max(max(a[i], b[i]), c[i]);
+                    uint4 v = requant_res(a, p.layer, 0);
+                    if (p.layer.relu) v = relu16(v);
+                    if (valid) sts16(hp + row_off(R, j), v);
+                }
+            }
+            ctx_sync<kFirstT>(ctx);  // all lines pooled along x; the MMAs have read the frame
+            if (n + step < p.batch) convert(n + step);
+            int8_t *out = p.x1 + (size_t)n * kRes1Bytes;
+            for (int i = tid; i < 41 * 41; i += kFirstT) {
+                const int oy = i / 41, ox = i - oy * 41, s = ox + 1, R = 2 * oy * 21 + (s >> 1), c = s & 1;
+                ByteMax mx;
+                mx.first(lds16(hp + row_off(R, c)));
+                mx.take(lds16(hp + row_off(R + 21, c)));
+                mx.take(lds16(hp + row_off(R + 42, c)));
+                const uint4 v = mx.result();
+                *reinterpret_cast<uint4 *>(out + row_off((oy + 1) * 21 + (s >> 1), c)) = v;
+                if (p.tap_x1) *reinterpret_cast<uint4 *>(p.tap_x1 + ((size_t)n * 1681 + i) * 16) = v;
+            }
+            ctx_sync<kFirstT>(ctx);  // before the next image's lines overwrite these
+        }
+    }
+    res_teardown(bars, warp, kFirstEpi, tmem);
+}
+
+// ---------------------------------------------------------------------------------------
+// two residual blocks at 41 x 41 x 16, conv 16 -> 32, max-pool
+// ---------------------------------------------------------------------------------------
+// Per context: a landing buffer for the next image, the operand of a block's first conv (ReLU'd) and
+// the tensor between its two convs.  The block's input x, which the second conv adds, stays in tensor
+// memory: the thread that adds it is the thread that wrote it.  The 16 -> 32 conv runs as two halves of
+// sixteen output channels, so that the un-pooled half fits the buffer between the convs.
+namespace {
+constexpr int kS1Wg = 2;
+constexpr int kS1T = kS1Wg * 128, kS1Epi = kCtx * kS1Wg * 4;
+constexpr int kS1Tiles = 7, kS1Slots = 6, kS1Ops = 6;       // 41 * 21 GEMM rows; accumulators; layers and half layers
+constexpr int kS1Buf = 30 * 1024;                           // an image's rows and what the last tile reads past them
+constexpr int kS1XCol = kS1Slots * 32;                      // x in tensor memory: 8 columns a tile behind the accumulators
+constexpr int kS1Smem = 1024 + kRes1Weights + kCtx * 3 * kS1Buf;
+static_assert((kS1Tiles * 128 + 2 * 21 + 1) * 32 <= kS1Buf && kS1XCol + 8 * kS1Tiles <= 256, "buffers");
+}  // namespace
+
+__global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(const __grid_constant__ ResStack1Params p)
+{
+    extern __shared__ __align__(1024) uint8_t res_smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ ResBars bars;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t *bufs = smem + kRes1Weights;
+    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kCtx * 3 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, kMaxSlots);
+    volatile int *abort_flag = &bars.abort_flag;
+    const int step = kCtx * (int)gridDim.x;
+
+    if (warp >= kS1Epi) {
+        // ------------------------------------------------------------------ MMA issuers
+        const int ctx = warp - kS1Epi;
+        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]);
+        const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)(ctx * 3 + 1) * kS1Buf) >> 4) | kDescSw32Lo, h0 = r0 + (kS1Buf >> 4);
+        const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
+        mbar_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        uint32_t slot = 0, phase = 0, rdy = 0;
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
+            for (int op = 0; op < kS1Ops; ++op) {
+                if (op < 5) {  // (the second half of the last conv reads what the first half read)
+                    mbar_wait(ready, rdy, abort_flag, p.status, 8);
+                    rdy ^= 1;
+                    fence_after();
+                }
+                const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0, b_op = w0 + (uint32_t)op * (6 * 1024 >> 4);
+                for (int t = 0; t < kS1Tiles; ++t) {
+                    mbar_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                    fence_after();
+                    if (elect_one()) {
+                        const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 32, a = a_op + (uint32_t)t * (128 * 2);
+#pragma unroll
+                        for (int j = 0; j < 6; ++j)
+                            mma_i8(d, desc(kDescSw32Hi, a + (uint32_t)((j >> 1) * 21 + (j & 1)) * 2), desc(kDescSw32Hi, b_op + (uint32_t)j * 64),
+                                   idesc_for(32), (uint32_t)j);
+                        mma_commit(full0 + 8 * slot);
+                    }
+                    __syncwarp();
+                    if (++slot == kS1Slots) slot = 0, phase ^= 1;
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue
+        const int ctx = warp / (kS1Wg * 4), wg = (warp >> 2) % kS1Wg, q = warp & 3;
+        const int tid = (int)threadIdx.x - ctx * kS1T;
+        const uint32_t land = smem_u32(bufs) + (uint32_t)(ctx * 3) * kS1Buf, rbuf = land + kS1Buf, hbuf = rbuf + kS1Buf;
+        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
+        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
+        auto fetch = [&](int n) {  // one thread
+            mbar_expect_tx(land_bar, kRes1Bytes);
+            bulk_load(land, p.x1 + (size_t)n * kRes1Bytes, kRes1Bytes, land_bar);
+        };
+        auto operand_done = [&]() {
+            fence_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(ready);
+        };
+        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
+        if (tid == 0 && n < p.batch) fetch(n);
+        uint32_t seq0 = 0, it = 0;
+        for (; n < p.batch; n += step, ++it) {
+            // the image: x to tensor memory, ReLU(x) to the first conv's operand
+            mbar_wait(land_bar, it & 1, abort_flag, p.status, 1);
+            for (int t = wg; t < kS1Tiles; t += kS1Wg) {
+                const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 21;
+                const bool v0 = Y < 41, v1 = v0 && X < 20;
+                uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0;
+                if (v0) x0 = lds16(land + row_off(r, 1));
+                if (v1) x1 = lds16(land + row_off(r + 1, 0));
+                tmem_st8(tlane + kS1XCol + 8 * t, x0, x1);
+                if (v0) sts16(rbuf + row_off(r, 1), relu16(x0));
+                if (v1) sts16(rbuf + row_off(r + 1, 0), relu16(x1));
+            }
+            tmem_wait_st();
+            operand_done();
+            ctx_sync<kS1T>(ctx);  // the landing buffer has been read
+            if (tid == 0 && n + step < p.batch) {
+                fence_async();
+                fetch(n + step);
+            }
+            for (int op = 0; op < kS1Ops; ++op) {
+                const ResLayer &L = p.layer[op < 4 ? op : 4];
+                const bool skip = op == 1 || op == 3;          // second conv of a block
+                const uint32_t dst = skip ? rbuf : hbuf;
+                int8_t *tap = op < 4 ? p.tap[op] : nullptr;
+                const int c0 = op == 5 ? 16 : 0;
+                for (int t = wg; t < kS1Tiles; t += kS1Wg) {
+                    const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS1Slots;
+                    const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 21;
+                    const bool v0 = Y < 41, v1 = v0 && X < 20;
+                    mbar_wait(full0 + 8 * slot, (seq / kS1Slots) & 1, abort_flag, p.status, 16);
+                    fence_after();
+                    int a0[16], a1[16];
+                    uint4 x0, x1;
+                    tmem_ld16(tlane + slot * 32, a0);
+                    tmem_ld16(tlane + slot * 32 + 16, a1);
+                    if (skip) tmem_ld8(tlane + kS1XCol + 8 * t, x0, x1);
+                    tmem_wait_ld();
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                    if (skip) {
+                        add_skip(a0, x0, L, 0);
+                        add_skip(a1, x1, L, 0);
+                    }
+                    uint4 q0 = requant_res(a0, L, c0), q1 = requant_res(a1, L, c0);
+                    if (L.relu) q0 = relu16(q0), q1 = relu16(q1);
+                    if (tap) {
+                        int8_t *d = tap + (((size_t)n * 41 + Y) * 41 + 2 * X) * 16;
+                        if (v0) *reinterpret_cast<uint4 *>(d) = q0;
+                        if (v1) *reinterpret_cast<uint4 *>(d + 16) = q1;
+                    }
+                    if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
+                        tmem_st8(tlane + kS1XCol + 8 * t, q0, q1);
+                        q0 = relu16(q0), q1 = relu16(q1);
+                    }
+                    if (v0) sts16(dst + row_off(r, 1), q0);
+                    if (v1) sts16(dst + row_off(r + 1, 0), q1);
+                }
+                seq0 += kS1Tiles;
+                if (op == 1) tmem_wait_st();
+                if (op < 4) {
+                    operand_done();
+                    continue;
+                }
+                // a half of the 16 -> 32 conv is complete: 3 x 3 stride-2 max over it
+                ctx_sync<kS1T>(ctx);
+                int8_t *out = p.x2 + (size_t)n * kRes2Bytes;
+                for (int i = tid; i < 400; i += kS1T) {
+                    const int oy = i / 20, ox = i - oy * 20, R = (2 * oy + 1) * 21 + ox;
+                    ByteMax mx;
+#pragma unroll
+                    for (int ky = 0; ky < 3; ++ky) {
+                        const int rr = R + 21 * ky;
+                        const uint4 u0 = lds16(hbuf + row_off(rr, 1)), u1 = lds16(hbuf + row_off(rr + 1, 0)),
+                                    u2 = lds16(hbuf + row_off(rr + 1, 1));
+                        if (ky == 0) mx.first(u0);
+                        else mx.take(u0);
+                        mx.take(u1);
+                        mx.take(u2);
+                    }
+                    const uint4 v = mx.result();
+                    *reinterpret_cast<uint4 *>(out + row_off((oy + 1) * 21 + ox + 1, op - 4)) = v;
+                    if (p.tap_x2) *reinterpret_cast<uint4 *>(p.tap_x2 + ((size_t)n * 400 + i) * 32 + 16 * (op - 4)) = v;
+                }
+                ctx_sync<kS1T>(ctx);
+            }
+        }
+    }
+    res_teardown(bars, warp, kS1Epi, tmem);
+}
+
+// ---------------------------------------------------------------------------------------
+// two residual blocks at 20 x 20 x 32, conv 32 -> 32, max-pool, two blocks at 9 x 9 x 32
+// ---------------------------------------------------------------------------------------
+// As above with one pixel per GEMM row.  The 9 x 9 layers are a single tile: the two warpgroups of a
+// context take half of its channels each, and a thread keeps its part of x in registers.
+namespace {
+constexpr int kS2Wg = 2;
+constexpr int kS2T = kS2Wg * 128, kS2Epi = kCtx * kS2Wg * 4;
+constexpr int kS2Tiles = 4, kS2Ops = 9;                     // 20 * 21 GEMM rows; layers
+constexpr int kS2Land = 15 * 1024, kS2Buf = 18 * 1024, kS3Buf = 5 * 1024;
+constexpr int kS2Ctx = kS2Land + 2 * kS2Buf + 2 * kS3Buf;
+constexpr int kS2WideSlot = 4, kS2XCol = kMaxSlots * 32;
+constexpr int kS2Smem = 1024 + kRes2Weights + kCtx * kS2Ctx;
+static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kRes2Bytes <= kS2Land &&
+              kS2XCol + 8 * kS2Tiles <= 256, "buffers");
+}  // namespace
+
+__global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
+{
+    extern __shared__ __align__(1024) uint8_t res_smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ ResBars bars;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t *bufs = smem + kRes2Weights;
+    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kCtx * kS2Ctx, smem, p.w, kRes2Weights, warp, kS2Wg * 4, kS2WideSlot);
+    volatile int *abort_flag = &bars.abort_flag;
+    const int step = kCtx * (int)gridDim.x;
+
+    if (warp >= kS2Epi) {
+        // ------------------------------------------------------------------ MMA issuers
+        const int ctx = warp - kS2Epi;
+        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]);
+        const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2Ctx + kS2Land) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
+                       r3 = h0 + (kS2Buf >> 4), h3 = r3 + (kS3Buf >> 4);
+        const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
+        mbar_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        uint32_t rdy = 0, k2 = 0, k3 = 0;  // layers done at 20 x 20 and at 9 x 9
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
+            for (int op = 0; op < kS2Ops; ++op) {
+                mbar_wait(ready, rdy, abort_flag, p.status, 8);
+                rdy ^= 1;
+                fence_after();
+                const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
+                if (op < 5) {
+                    const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
+                    for (int t = 0; t < kS2Tiles; ++t) {
+                        mbar_wait(empty0 + 8 * t, (k2 & 1) ^ 1, abort_flag, p.status, 4);
+                        fence_after();
+                        if (elect_one()) {
+                            const uint32_t d = tmem + (uint32_t)ctx * 256 + t * 32, a = a_op + (uint32_t)t * (128 * 2);
+#pragma unroll
+                            for (int j = 0; j < 9; ++j)
+                                mma_i8(d, desc(kDescSw32Hi, a + (uint32_t)((j / 3) * 21 + j % 3) * 2),
+                                       desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
+                            mma_commit(full0 + 8 * t);
+                        }
+                        __syncwarp();
+                    }
+                    ++k2;
+                } else {
+                    const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3, slot = kS2WideSlot + (k3 & 1);
+                    mbar_wait(empty0 + 8 * slot, ((k3 >> 1) & 1) ^ 1, abort_flag, p.status, 4);
+                    fence_after();
+                    if (elect_one()) {
+                        const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 32;
+#pragma unroll
+                        for (int j = 0; j < 9; ++j)
+                            mma_i8(d, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
+                                   desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
+                        mma_commit(full0 + 8 * slot);
+                    }
+                    __syncwarp();
+                    ++k3;
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue
+        const int ctx = warp / (kS2Wg * 4), wg = (warp >> 2) % kS2Wg, q = warp & 3;
+        const int tid = (int)threadIdx.x - ctx * kS2T;
+        const uint32_t land = smem_u32(bufs) + (uint32_t)ctx * kS2Ctx, rbuf = land + kS2Land, hbuf = rbuf + kS2Buf,
+                       r3buf = hbuf + kS2Buf, h3buf = r3buf + kS3Buf;
+        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
+        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
+        auto fetch = [&](int n) {  // one thread
+            mbar_expect_tx(land_bar, kRes2Bytes);
+            bulk_load(land, p.x2 + (size_t)n * kRes2Bytes, kRes2Bytes, land_bar);
+        };
+        auto operand_done = [&]() {
+            fence_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(ready);
+        };
+        // this thread's pixel of the 9 x 9 tile, and its half (wg) of the channels
+        const int m3 = q * 32 + lane, Y3 = m3 / 10, X3 = m3 - Y3 * 10;
+        const bool v3 = Y3 < 9 && X3 < 9;
+        const uint32_t off3 = row_off(m3 + 11, wg);
+        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
+        if (tid == 0 && n < p.batch) fetch(n);
+        uint32_t k2 = 0, k3 = 0, it = 0;
+        for (; n < p.batch; n += step, ++it) {
+            mbar_wait(land_bar, it & 1, abort_flag, p.status, 1);
+            for (int t = wg; t < kS2Tiles; t += kS2Wg) {
+                const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 22;
+                const bool v = Y < 20 && X < 20;
+                uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0;
+                if (v) {
+                    x0 = lds16(land + row_off(r, 0));
+                    x1 = lds16(land + row_off(r, 1));
+                }
+                tmem_st8(tlane + kS2XCol + 8 * t, x0, x1);
+                if (v) {
+                    sts16(rbuf + row_off(r, 0), relu16(x0));
+                    sts16(rbuf + row_off(r, 1), relu16(x1));
+                }
+            }
+            tmem_wait_st();
+            operand_done();
+            ctx_sync<kS2T>(ctx);  // the landing buffer has been read
+            if (tid == 0 && n + step < p.batch) {
+                fence_async();
+                fetch(n + step);
+            }
+            for (int op = 0; op < 5; ++op, ++k2) {
+                const ResLayer &L = p.layer[op];
+                const bool skip = op == 1 || op == 3;
+                const uint32_t dst = skip ? rbuf : hbuf;
+                int8_t *tap = p.tap[op];
+                for (int t = wg; t < kS2Tiles; t += kS2Wg) {
+                    const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 22;
+                    const bool v = Y < 20 && X < 20;
+                    mbar_wait(full0 + 8 * t, k2 & 1, abort_flag, p.status, 16);
+                    fence_after();
+                    int a0[16], a1[16];
+                    uint4 x0, x1;
+                    tmem_ld16(tlane + t * 32, a0);
+                    tmem_ld16(tlane + t * 32 + 16, a1);
+                    if (skip) tmem_ld8(tlane + kS2XCol + 8 * t, x0, x1);
+                    tmem_wait_ld();
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty0 + 8 * t);
+                    if (skip) {
+                        add_skip(a0, x0, L, 0);
+                        add_skip(a1, x1, L, 16);
+                    }
+                    uint4 q0 = requant_res(a0, L, 0), q1 = requant_res(a1, L, 16);
+                    if (L.relu) q0 = relu16(q0), q1 = relu16(q1);
+                    if (tap && v) {
+                        int8_t *d = tap + (((size_t)n * 20 + Y) * 20 + X) * 32;
+                        *reinterpret_cast<uint4 *>(d) = q0;
+                        *reinterpret_cast<uint4 *>(d + 16) = q1;
+                    }
+                    if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
+                        tmem_st8(tlane + kS2XCol + 8 * t, q0, q1);
+                        q0 = relu16(q0), q1 = relu16(q1);
+                    }
+                    if (v) {
+                        sts16(dst + row_off(r, 0), q0);
+                        sts16(dst + row_off(r, 1), q1);
+                    }
+                }
+                if (op == 1) tmem_wait_st();
+                if (op < 4) operand_done();
+            }
+            // 3 x 3 stride-2 max over the last one: every thread its pixel and channels of the 9 x 9 tensor
+            ctx_sync<kS2T>(ctx);
+            uint4 x = make_uint4(0, 0, 0, 0);
+            if (v3) {
+                const int R = (2 * Y3 + 1) * 21 + 2 * X3 + 1;
+                ByteMax mx;
+                mx.first(lds16(hbuf + row_off(R, wg)));
+#pragma unroll
+                for (int j = 1; j < 9; ++j) mx.take(lds16(hbuf + row_off(R + (j / 3) * 21 + j % 3, wg)));
+                x = mx.result();
+                sts16(r3buf + off3, relu16(x));
+                if (p.tap_x3) *reinterpret_cast<uint4 *>(p.tap_x3 + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = x;
+            }
+            operand_done();
+            for (int op = 5; op < kS2Ops; ++op, ++k3) {
+                const ResLayer &L = p.layer[op];
+                const bool skip = op == 6 || op == 8;
+                const uint32_t slot = kS2WideSlot + (k3 & 1);
+                mbar_wait(full0 + 8 * slot, (k3 >> 1) & 1, abort_flag, p.status, 16);
+                fence_after();
+                int a[16];
+                tmem_ld16(tlane + slot * 32 + 16 * wg, a);
+                tmem_wait_ld();
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                if (skip) add_skip(a, x, L, 16 * wg);
+                uint4 v = requant_res(a, L, 16 * wg);
+                if (L.relu) v = relu16(v);
+                if (v3 && p.tap[op]) *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = v;
+                if (skip) {
+                    x = v;
+                    v = relu16(v);
+                }
+                if (op == 8) {
+                    if (v3) *reinterpret_cast<uint4 *>(p.x3 + (size_t)n * kRes3Bytes + (Y3 * 9 + X3) * 32 + 16 * wg) = v;
+                } else {
+                    if (v3) sts16((skip ? r3buf : h3buf) + off3, v);
+                    operand_done();
+                }
+            }
+        }
+    }
+    res_teardown(bars, warp, kS2Epi, tmem);
+}
+
+// ---------------------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------------------
+namespace {
+
+template <typename K, typename P>
+cudaError_t res_launch(K kernel, const P &p, int threads, size_t smem, int sm_count, cudaStream_t st)
+{
+    cudaError_t e = allow_smem((const void *)kernel, smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    // context c of CTA i starts with image i + c * CTAs: the second contexts come into play when every SM has an image
+    cfg.gridDim = dim3((unsigned)(p.batch < sm_count ? p.batch : sm_count));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
+}  // namespace
+
+cudaError_t res_first_launch(const ResFirstParams &p, int sm_count, cudaStream_t st)
+{
+    const int threads = 32 * (kFirstEpi + kCtx);
+    return p.ingest_mode == 2 ? res_launch(res_first_kernel<true>, p, threads, kFirstSmem, sm_count, st)
+                              : res_launch(res_first_kernel<false>, p, threads, kFirstSmem, sm_count, st);
+}
+
+cudaError_t res_stack1_launch(const ResStack1Params &p, int sm_count, cudaStream_t st)
+{
+    return res_launch(res_stack1_kernel, p, 32 * (kS1Epi + kCtx), kS1Smem, sm_count, st);
+}
+
+cudaError_t res_stack23_launch(const ResStack23Params &p, int sm_count, cudaStream_t st)
+{
+    return res_launch(res_stack23_kernel, p, 32 * (kS2Epi + kCtx), kS2Smem, sm_count, st);
+}
+
+}  // namespace accerl
