@@ -42,6 +42,14 @@ namespace {
 constexpr int kCtx = 2;     // images in flight per CTA
 constexpr int kMaxSlots = 6;
 
+
+// the waits of these kernels are short and on the critical path of their context: poll (try_wait itself
+// suspends the warp for a while) before backing off
+__device__ __forceinline__ void res_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status, int code)
+{
+    mbar_wait_limited(bar, parity, abort_flag, status, code, 2048, kWaitLimitPolls);
+}
+
 struct __align__(8) ResBars {
     uint64_t w_ready;
     uint64_t land[kCtx];                // an image has arrived
@@ -111,22 +119,36 @@ struct ByteMax {
     }
 };
 
-// sixteen accumulators of channels c0 .. c0 + 15 -> sixteen codes
-__device__ __forceinline__ uint4 requant_res(const int (&acc)[16], const ResLayer &L, int c0)
-{
-    float ks[16], bs[16];
+// The constants of sixteen channels of a layer, held in registers while a warp works through the tiles of
+// that layer.  They come from a copy in shared memory: read from the constant bank at a layer index
+// that is not known at compile time, they took the indexed-constant path (4 050 requests an image in
+// res_stack23, half of that unit's peak, with the contexts evicting each other's lines).
+struct Requant {
+    float k[16], b[16], s_out, inv_s_out;
+    bool affine, relu;
+    __device__ __forceinline__ void load(const ResLayer &L, int c0)
+    {
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const float4 kv = *reinterpret_cast<const float4 *>(&L.k[c0 + 4 * g]);
-        const float4 bv = *reinterpret_cast<const float4 *>(&L.b[c0 + 4 * g]);
-        ks[4 * g] = kv.x; ks[4 * g + 1] = kv.y; ks[4 * g + 2] = kv.z; ks[4 * g + 3] = kv.w;
-        bs[4 * g] = bv.x; bs[4 * g + 1] = bv.y; bs[4 * g + 2] = bv.z; bs[4 * g + 3] = bv.w;
+        for (int g = 0; g < 4; ++g) {
+            const float4 kv = *reinterpret_cast<const float4 *>(&L.k[c0 + 4 * g]);
+            const float4 bv = *reinterpret_cast<const float4 *>(&L.b[c0 + 4 * g]);
+            k[4 * g] = kv.x; k[4 * g + 1] = kv.y; k[4 * g + 2] = kv.z; k[4 * g + 3] = kv.w;
+            b[4 * g] = bv.x; b[4 * g + 1] = bv.y; b[4 * g + 2] = bv.z; b[4 * g + 3] = bv.w;
+        }
+        s_out = L.s_out;
+        inv_s_out = L.inv_s_out;
+        affine = L.affine != 0;
+        relu = L.relu != 0;
     }
-    uint32_t w[4];
-    if (L.affine) requant16_affine<false>(acc, ks, bs, w);
-    else requant16_fastdiv<false>(acc, ks, bs, L.s_out, L.inv_s_out, w);
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
+    __device__ __forceinline__ uint4 operator()(const int (&acc)[16]) const
+    {
+        uint32_t w[4];
+        if (affine) requant16_affine<false>(acc, k, b, w);
+        else requant16_fastdiv<false>(acc, k, b, s_out, inv_s_out, w);
+        const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+        return relu ? relu16(v) : v;
+    }
+};
 
 // acc[i] += skip_mul[c0 + i] * x[i], one dp2a each
 __device__ __forceinline__ void add_skip(int (&acc)[16], uint4 x, const ResLayer &L, int c0)
@@ -175,8 +197,11 @@ __device__ __forceinline__ uint64_t desc(uint32_t hi, uint32_t lo) { return ((ui
 // what every kernel of this file does first: barriers, tensor memory, weights; returns the tensor-memory base
 template <int EPI_WARPS>
 __device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, int buffer_bytes, uint8_t *w_smem,
-                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals, int wide_slot)
+                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals,
+                                              int slot_arrivals, const ResLayer *layers, ResLayer *s_layers, int n_layers)
 {
+    for (int i = threadIdx.x; i < n_layers * (int)(sizeof(ResLayer) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(s_layers)[i] = reinterpret_cast<const uint32_t *>(layers)[i];
     // borders and padding stay zero for the life of the CTA
     for (int i = threadIdx.x; i < buffer_bytes / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(buffers)[i] = make_uint4(0, 0, 0, 0);
@@ -187,7 +212,7 @@ __device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, i
             mbar_init(smem_u32(&bars.ready[c]), epi_arrivals);
             for (int s = 0; s < kMaxSlots; ++s) {
                 mbar_init(smem_u32(&bars.acc_full[c][s]), 1);
-                mbar_init(smem_u32(&bars.acc_empty[c][s]), s >= wide_slot ? epi_arrivals : 4);
+                mbar_init(smem_u32(&bars.acc_empty[c][s]), slot_arrivals);
             }
         }
         bars.abort_flag = 0;
@@ -236,7 +261,7 @@ __device__ __forceinline__ void res_teardown(ResBars &bars, int warp, int alloc_
 // maximum over three lines follows on the codes in shared memory.  The MMAs take 2 340 cycles an image;
 // the epilogue's instructions (33 k codes an image, some 14 k warp instructions) bound the kernel.
 namespace {
-constexpr int kFirstWg = 3;                                  // warpgroups per context
+constexpr int kFirstWg = 2;                                  // warpgroups per context
 constexpr int kFirstT = kFirstWg * 128, kFirstEpi = kCtx * kFirstWg * 4;
 constexpr int kFirstTiles = 15, kFirstSlots = 3;             // ceil(83 lines * 22 rows / 128)
 constexpr int kFrameBytes = 31 * 1024, kHpBytes = 55 * 1024; // quantised frame (last tile reads past it), pooled lines
@@ -250,10 +275,11 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
+    __shared__ __align__(16) ResLayer s_layer;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + 8192;
     const uint32_t tmem = res_setup<kFirstEpi>(bars, bufs, kCtx * (kFrameBytes + kHpBytes), smem, p.w, kResFirstWeights,
-                                               warp, kFirstWg * 4, kMaxSlots);
+                                               warp, kFirstWg * 4, 4, &p.layer, &s_layer, 1);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kCtx * (int)gridDim.x;
 
@@ -264,13 +290,13 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t a0 = ((smem_u32(bufs) + (uint32_t)ctx * (kFrameBytes + kHpBytes)) >> 4) | kDescFlatLo;
         const uint32_t b0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
-        mbar_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, it = 0;
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step, ++it) {
-            mbar_wait(ready, it & 1, abort_flag, p.status, 8);
+            res_wait(ready, it & 1, abort_flag, p.status, 8);
             fence_after();
             for (int t = 0; t < kFirstTiles; ++t) {
-                mbar_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                 fence_after();
                 if (elect_one()) {
                     const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 80;
@@ -326,13 +352,15 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)(n + step) * 28224), "r"(28224)
                              : "memory");
         };
+        Requant req;
+        req.load(s_layer, 0);
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (n < p.batch) convert(n);
         uint32_t seq0 = 0;  // accumulators handed over before this image
         for (; n < p.batch; n += step, seq0 += kFirstTiles) {
             for (int t = wg; t < kFirstTiles; t += kFirstWg) {
                 const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kFirstSlots;
-                mbar_wait(full0 + 8 * slot, (seq / kFirstSlots) & 1, abort_flag, p.status, 16);
+                res_wait(full0 + 8 * slot, (seq / kFirstSlots) & 1, abort_flag, p.status, 16);
                 fence_after();
                 const int m = t * 128 + q * 32 + lane;
                 const int y = m / 22, X = m - y * 22, R = y * 21 + X;
@@ -351,9 +379,8 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                         if (lane == 0) mbar_arrive(empty0 + 8 * slot);
                     }
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) a[i] = max(max(a[i], b[i]), c[i]);
-                    uint4 v = requant_res(a, p.layer, 0);
-                    if (p.layer.relu) v = relu16(v);
+                    for (int i = 0; i < 16; ++i) a[i] = __vimax3_s32(a[i], b[i], c[i]);
+                    const uint4 v = req(a);
                     if (valid) sts16(hp + row_off(R, j), v);
                 }
             }
@@ -398,9 +425,11 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
+    __shared__ __align__(16) ResLayer s_layer[5];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes1Weights;
-    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kCtx * 3 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, kMaxSlots);
+    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kCtx * 3 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, 4,
+                                            p.layer, s_layer, 5);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kCtx * (int)gridDim.x;
 
@@ -411,18 +440,18 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)(ctx * 3 + 1) * kS1Buf) >> 4) | kDescSw32Lo, h0 = r0 + (kS1Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
-        mbar_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, rdy = 0;
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
             for (int op = 0; op < kS1Ops; ++op) {
                 if (op < 5) {  // (the second half of the last conv reads what the first half read)
-                    mbar_wait(ready, rdy, abort_flag, p.status, 8);
+                    res_wait(ready, rdy, abort_flag, p.status, 8);
                     rdy ^= 1;
                     fence_after();
                 }
                 const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0, b_op = w0 + (uint32_t)op * (6 * 1024 >> 4);
                 for (int t = 0; t < kS1Tiles; ++t) {
-                    mbar_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                    res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
                         const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 32, a = a_op + (uint32_t)t * (128 * 2);
@@ -454,15 +483,20 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
             __syncwarp();
             if (lane == 0) mbar_arrive(ready);
         };
+        // GEMM row m = 128 t + row of this thread: are its two pixels part of the image?
+        const int row = q * 32 + lane;
+        uint32_t second = 0;  // bit t: the second one is
+        for (int t = 0; t < kS1Tiles; ++t)
+            if ((t * 128 + row) % 21 < 20 && t * 128 + row < 861) second |= 1u << t;
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (tid == 0 && n < p.batch) fetch(n);
         uint32_t seq0 = 0, it = 0;
         for (; n < p.batch; n += step, ++it) {
             // the image: x to tensor memory, ReLU(x) to the first conv's operand
-            mbar_wait(land_bar, it & 1, abort_flag, p.status, 1);
+            res_wait(land_bar, it & 1, abort_flag, p.status, 1);
             for (int t = wg; t < kS1Tiles; t += kS1Wg) {
-                const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 21;
-                const bool v0 = Y < 41, v1 = v0 && X < 20;
+                const int m = t * 128 + row, r = m + 21;
+                const bool v0 = m < 861, v1 = (second >> t) & 1;
                 uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0;
                 if (v0) x0 = lds16(land + row_off(r, 1));
                 if (v1) x1 = lds16(land + row_off(r + 1, 0));
@@ -478,16 +512,17 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
                 fetch(n + step);
             }
             for (int op = 0; op < kS1Ops; ++op) {
-                const ResLayer &L = p.layer[op < 4 ? op : 4];
+                const ResLayer &L = s_layer[op < 4 ? op : 4];
+                Requant req;
+                req.load(L, op == 5 ? 16 : 0);
                 const bool skip = op == 1 || op == 3;          // second conv of a block
                 const uint32_t dst = skip ? rbuf : hbuf;
                 int8_t *tap = op < 4 ? p.tap[op] : nullptr;
-                const int c0 = op == 5 ? 16 : 0;
                 for (int t = wg; t < kS1Tiles; t += kS1Wg) {
                     const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS1Slots;
-                    const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 21;
-                    const bool v0 = Y < 41, v1 = v0 && X < 20;
-                    mbar_wait(full0 + 8 * slot, (seq / kS1Slots) & 1, abort_flag, p.status, 16);
+                    const int m = t * 128 + row, r = m + 21;
+                    const bool v0 = m < 861, v1 = (second >> t) & 1;
+                    res_wait(full0 + 8 * slot, (seq / kS1Slots) & 1, abort_flag, p.status, 16);
                     fence_after();
                     int a0[16], a1[16];
                     uint4 x0, x1;
@@ -502,9 +537,9 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
                         add_skip(a0, x0, L, 0);
                         add_skip(a1, x1, L, 0);
                     }
-                    uint4 q0 = requant_res(a0, L, c0), q1 = requant_res(a1, L, c0);
-                    if (L.relu) q0 = relu16(q0), q1 = relu16(q1);
+                    uint4 q0 = req(a0), q1 = req(a1);
                     if (tap) {
+                        const int Y = m / 21, X = m - Y * 21;
                         int8_t *d = tap + (((size_t)n * 41 + Y) * 41 + 2 * X) * 16;
                         if (v0) *reinterpret_cast<uint4 *>(d) = q0;
                         if (v1) *reinterpret_cast<uint4 *>(d + 16) = q1;
@@ -552,18 +587,18 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
 // ---------------------------------------------------------------------------------------
 // two residual blocks at 20 x 20 x 32, conv 32 -> 32, max-pool, two blocks at 9 x 9 x 32
 // ---------------------------------------------------------------------------------------
-// As above with one pixel per GEMM row.  The 9 x 9 layers are a single tile: the two warpgroups of a
-// context take half of its channels each, and a thread keeps its part of x in registers.
+// As above with one pixel per GEMM row.  The two warpgroups of a context take half of the channels of
+// every tile, and a thread keeps its part of x in registers.
 namespace {
 constexpr int kS2Wg = 2;
 constexpr int kS2T = kS2Wg * 128, kS2Epi = kCtx * kS2Wg * 4;
 constexpr int kS2Tiles = 4, kS2Ops = 9;                     // 20 * 21 GEMM rows; layers
 constexpr int kS2Land = 15 * 1024, kS2Buf = 18 * 1024, kS3Buf = 5 * 1024;
 constexpr int kS2Ctx = kS2Land + 2 * kS2Buf + 2 * kS3Buf;
-constexpr int kS2WideSlot = 4, kS2XCol = kMaxSlots * 32;
+constexpr int kS2WideSlot = 4;  // accumulators 0 .. 3: the tiles at 20 x 20, 4 and 5: the layers at 9 x 9
 constexpr int kS2Smem = 1024 + kRes2Weights + kCtx * kS2Ctx;
-static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kRes2Bytes <= kS2Land &&
-              kS2XCol + 8 * kS2Tiles <= 256, "buffers");
+static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kRes2Bytes <= kS2Land,
+              "buffers");
 }  // namespace
 
 __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
@@ -571,9 +606,11 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
+    __shared__ __align__(16) ResLayer s_layer[9];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes2Weights;
-    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kCtx * kS2Ctx, smem, p.w, kRes2Weights, warp, kS2Wg * 4, kS2WideSlot);
+    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kCtx * kS2Ctx, smem, p.w, kRes2Weights, warp, kS2Wg * 4,
+                                            kS2Wg * 4, p.layer, s_layer, 9);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kCtx * (int)gridDim.x;
 
@@ -585,18 +622,18 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2Ctx + kS2Land) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
                        r3 = h0 + (kS2Buf >> 4), h3 = r3 + (kS3Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
-        mbar_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t rdy = 0, k2 = 0, k3 = 0;  // layers done at 20 x 20 and at 9 x 9
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
             for (int op = 0; op < kS2Ops; ++op) {
-                mbar_wait(ready, rdy, abort_flag, p.status, 8);
+                res_wait(ready, rdy, abort_flag, p.status, 8);
                 rdy ^= 1;
                 fence_after();
                 const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
                 if (op < 5) {
                     const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
                     for (int t = 0; t < kS2Tiles; ++t) {
-                        mbar_wait(empty0 + 8 * t, (k2 & 1) ^ 1, abort_flag, p.status, 4);
+                        res_wait(empty0 + 8 * t, (k2 & 1) ^ 1, abort_flag, p.status, 4);
                         fence_after();
                         if (elect_one()) {
                             const uint32_t d = tmem + (uint32_t)ctx * 256 + t * 32, a = a_op + (uint32_t)t * (128 * 2);
@@ -611,7 +648,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
                     ++k2;
                 } else {
                     const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3, slot = kS2WideSlot + (k3 & 1);
-                    mbar_wait(empty0 + 8 * slot, ((k3 >> 1) & 1) ^ 1, abort_flag, p.status, 4);
+                    res_wait(empty0 + 8 * slot, ((k3 >> 1) & 1) ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
                         const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 32;
@@ -644,30 +681,29 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
             __syncwarp();
             if (lane == 0) mbar_arrive(ready);
         };
-        // this thread's pixel of the 9 x 9 tile, and its half (wg) of the channels
-        const int m3 = q * 32 + lane, Y3 = m3 / 10, X3 = m3 - Y3 * 10;
+        // A warpgroup takes sixteen channels (half wg of a row) of every tile; this thread's pixels:
+        const int row = q * 32 + lane;
+        uint32_t inside = 0;  // bit t: row 128 t + row is a pixel of the 20 x 20 image
+        for (int t = 0; t < kS2Tiles; ++t)
+            if ((t * 128 + row) % 21 < 20 && t * 128 + row < 420) inside |= 1u << t;
+        const int Y3 = row / 10, X3 = row - Y3 * 10;
         const bool v3 = Y3 < 9 && X3 < 9;
-        const uint32_t off3 = row_off(m3 + 11, wg);
+        const uint32_t off3 = row_off(row + 11, wg);
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (tid == 0 && n < p.batch) fetch(n);
         uint32_t k2 = 0, k3 = 0, it = 0;
         for (; n < p.batch; n += step, ++it) {
-            mbar_wait(land_bar, it & 1, abort_flag, p.status, 1);
-            for (int t = wg; t < kS2Tiles; t += kS2Wg) {
-                const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 22;
-                const bool v = Y < 20 && X < 20;
-                uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0;
-                if (v) {
-                    x0 = lds16(land + row_off(r, 0));
-                    x1 = lds16(land + row_off(r, 1));
-                }
-                tmem_st8(tlane + kS2XCol + 8 * t, x0, x1);
-                if (v) {
-                    sts16(rbuf + row_off(r, 0), relu16(x0));
-                    sts16(rbuf + row_off(r, 1), relu16(x1));
+            res_wait(land_bar, it & 1, abort_flag, p.status, 1);
+            uint4 xs[kS2Tiles];  // the block's input, this thread's channels of its pixels
+#pragma unroll
+            for (int t = 0; t < kS2Tiles; ++t) {
+                const uint32_t off = row_off(t * 128 + row + 22, wg);
+                xs[t] = make_uint4(0, 0, 0, 0);
+                if ((inside >> t) & 1) {
+                    xs[t] = lds16(land + off);
+                    sts16(rbuf + off, relu16(xs[t]));
                 }
             }
-            tmem_wait_st();
             operand_done();
             ctx_sync<kS2T>(ctx);  // the landing buffer has been read
             if (tid == 0 && n + step < p.batch) {
@@ -675,45 +711,36 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
                 fetch(n + step);
             }
             for (int op = 0; op < 5; ++op, ++k2) {
-                const ResLayer &L = p.layer[op];
+                const ResLayer &L = s_layer[op];
+                Requant req;
+                req.load(L, 16 * wg);
                 const bool skip = op == 1 || op == 3;
                 const uint32_t dst = skip ? rbuf : hbuf;
                 int8_t *tap = p.tap[op];
-                for (int t = wg; t < kS2Tiles; t += kS2Wg) {
-                    const int m = t * 128 + q * 32 + lane, Y = m / 21, X = m - Y * 21, r = m + 22;
-                    const bool v = Y < 20 && X < 20;
-                    mbar_wait(full0 + 8 * t, k2 & 1, abort_flag, p.status, 16);
+#pragma unroll
+                for (int t = 0; t < kS2Tiles; ++t) {
+                    const uint32_t off = row_off(t * 128 + row + 22, wg);
+                    const bool v = (inside >> t) & 1;
+                    res_wait(full0 + 8 * t, k2 & 1, abort_flag, p.status, 16);
                     fence_after();
-                    int a0[16], a1[16];
-                    uint4 x0, x1;
-                    tmem_ld16(tlane + t * 32, a0);
-                    tmem_ld16(tlane + t * 32 + 16, a1);
-                    if (skip) tmem_ld8(tlane + kS2XCol + 8 * t, x0, x1);
+                    int a[16];
+                    tmem_ld16(tlane + t * 32 + 16 * wg, a);
                     tmem_wait_ld();
                     fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(empty0 + 8 * t);
-                    if (skip) {
-                        add_skip(a0, x0, L, 0);
-                        add_skip(a1, x1, L, 16);
-                    }
-                    uint4 q0 = requant_res(a0, L, 0), q1 = requant_res(a1, L, 16);
-                    if (L.relu) q0 = relu16(q0), q1 = relu16(q1);
+                    if (skip) add_skip(a, xs[t], L, 16 * wg);
+                    uint4 c = req(a);
                     if (tap && v) {
-                        int8_t *d = tap + (((size_t)n * 20 + Y) * 20 + X) * 32;
-                        *reinterpret_cast<uint4 *>(d) = q0;
-                        *reinterpret_cast<uint4 *>(d + 16) = q1;
+                        const int m = t * 128 + row, Y = m / 21, X = m - Y * 21;
+                        *reinterpret_cast<uint4 *>(tap + (((size_t)n * 20 + Y) * 20 + X) * 32 + 16 * wg) = c;
                     }
                     if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
-                        tmem_st8(tlane + kS2XCol + 8 * t, q0, q1);
-                        q0 = relu16(q0), q1 = relu16(q1);
+                        xs[t] = c;
+                        c = relu16(c);
                     }
-                    if (v) {
-                        sts16(dst + row_off(r, 0), q0);
-                        sts16(dst + row_off(r, 1), q1);
-                    }
+                    if (v) sts16(dst + off, c);
                 }
-                if (op == 1) tmem_wait_st();
                 if (op < 4) operand_done();
             }
             // 3 x 3 stride-2 max over the last one: every thread its pixel and channels of the 9 x 9 tensor
@@ -731,10 +758,12 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
             }
             operand_done();
             for (int op = 5; op < kS2Ops; ++op, ++k3) {
-                const ResLayer &L = p.layer[op];
+                const ResLayer &L = s_layer[op];
+                Requant req;
+                req.load(L, 16 * wg);
                 const bool skip = op == 6 || op == 8;
                 const uint32_t slot = kS2WideSlot + (k3 & 1);
-                mbar_wait(full0 + 8 * slot, (k3 >> 1) & 1, abort_flag, p.status, 16);
+                res_wait(full0 + 8 * slot, (k3 >> 1) & 1, abort_flag, p.status, 16);
                 fence_after();
                 int a[16];
                 tmem_ld16(tlane + slot * 32 + 16 * wg, a);
@@ -743,8 +772,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty0 + 8 * slot);
                 if (skip) add_skip(a, x, L, 16 * wg);
-                uint4 v = requant_res(a, L, 16 * wg);
-                if (L.relu) v = relu16(v);
+                uint4 v = req(a);
                 if (v3 && p.tap[op]) *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = v;
                 if (skip) {
                     x = v;
