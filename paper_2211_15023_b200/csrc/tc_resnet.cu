@@ -11,9 +11,9 @@
 // tensor memory, and all weights of the kernel beside them; only the three tensors between the
 // kernels touch HBM (74 KB a state with the frame).
 //
-// An image's layers depend on one another, so a CTA works on two images at once: two contexts, each
-// with its own issuing warp, warpgroups, buffers and half of tensor memory; while one context
-// requantises, the other's MMAs run.  Inside a context the 128-row tiles of a layer overlap as well:
+// An image's layers depend on one another, so a CTA works on two or three images at once: contexts, each
+// with its own issuing warp, warpgroups, buffers and part of tensor memory; while one context
+// requantises, another's MMAs run.  Inside a context the 128-row tiles of a layer overlap as well:
 // a tile is requantised while the next one is contracted.
 //
 // Convolutions are row-shifted implicit GEMMs as everywhere in this library: a GEMM row is 32 bytes of
@@ -22,13 +22,18 @@
 // nine K steps).  N = 32 instructions cost 40 cycles, bound by reading their 4 KB operand: wider rows
 // (N = 64, four pixels) would save a tenth of the tensor time and quadruple the weights' shared memory.
 //
-// What bounds it: the tensor pipe by instruction count (10 080 cycles an image in res_stack1, 8 640 in
-// res_stack23) and, in res_first, instruction issue of the epilogue.
+// What bounds it: instruction issue of the epilogues (about half of the 37 000 warp instructions an image
+// takes in res_stack1 convert and pack its 164 000 codes), then the tensor pipe by instruction count
+// (10 080 cycles an image in res_stack1, 8 640 in res_stack23, of 14 700 and 13 800).  Batch 16384, us per
+// launch: two contexts with constants from the constant bank 608 / 1079 / 1103, as it is
+// 483 / 827 / 775.
 //
 // Every wait is bounded.  A role whose wait gives up sets the status word and goes on (all further
 // waits return at once), so that the barriers inside a context always see all their warps.
 #include <cuda.h>
 #include <string.h>
+
+#include <type_traits>
 
 #include "epilogue.cuh"
 #include "internal.h"
@@ -39,8 +44,8 @@ namespace accerl {
 
 namespace {
 
-constexpr int kCtx = 2;     // images in flight per CTA
-constexpr int kMaxSlots = 6;
+constexpr int kMaxCtx = 3;  // images in flight per CTA
+constexpr int kMaxSlots = 5;
 
 
 // the waits of these kernels are short and on the critical path of their context: poll (try_wait itself
@@ -52,9 +57,9 @@ __device__ __forceinline__ void res_wait(uint32_t bar, uint32_t parity, volatile
 
 struct __align__(8) ResBars {
     uint64_t w_ready;
-    uint64_t land[kCtx];                // an image has arrived
-    uint64_t ready[kCtx];               // the operand of the next layer is complete
-    uint64_t acc_full[kCtx][kMaxSlots], acc_empty[kCtx][kMaxSlots];
+    uint64_t land[kMaxCtx];                // an image has arrived
+    uint64_t ready[kMaxCtx];               // the operand of the next layer is complete
+    uint64_t acc_full[kMaxCtx][kMaxSlots], acc_empty[kMaxCtx][kMaxSlots];
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -119,36 +124,29 @@ struct ByteMax {
     }
 };
 
-// The constants of sixteen channels of a layer, held in registers while a warp works through the tiles of
-// that layer.  They come from a copy in shared memory: read from the constant bank at a layer index
-// that is not known at compile time, they took the indexed-constant path (4 050 requests an image in
-// res_stack23, half of that unit's peak, with the contexts evicting each other's lines).
-struct Requant {
-    float k[16], b[16], s_out, inv_s_out;
-    bool affine, relu;
-    __device__ __forceinline__ void load(const ResLayer &L, int c0)
-    {
+// Sixteen accumulators of channels c0 .. c0 + 15 -> sixteen codes.  The constants are kernel parameters
+// at addresses known at compile time (the layer loops are unrolled for that): indexed at run time they
+// took the indexed-constant path (4 050 requests an image in res_stack23, half of that unit's peak, the
+// contexts evicting each other's lines); from shared memory a broadcast 16-byte load costs four
+// wavefronts of the port the MMAs read their operands through (res_stack1: 12 000 of 20 000 cycles an
+// image); and held in registers over a layer they push the kernels into spills, which are deadly
+// beside 220 KB of shared memory, with hardly any L1 left (2.4 ms instead of 1.1).
+__device__ __forceinline__ uint4 requant_res(const int (&acc)[16], const ResLayer &L, int c0)
+{
+    float ks[16], bs[16];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const float4 kv = *reinterpret_cast<const float4 *>(&L.k[c0 + 4 * g]);
-            const float4 bv = *reinterpret_cast<const float4 *>(&L.b[c0 + 4 * g]);
-            k[4 * g] = kv.x; k[4 * g + 1] = kv.y; k[4 * g + 2] = kv.z; k[4 * g + 3] = kv.w;
-            b[4 * g] = bv.x; b[4 * g + 1] = bv.y; b[4 * g + 2] = bv.z; b[4 * g + 3] = bv.w;
-        }
-        s_out = L.s_out;
-        inv_s_out = L.inv_s_out;
-        affine = L.affine != 0;
-        relu = L.relu != 0;
+    for (int g = 0; g < 4; ++g) {
+        const float4 kv = *reinterpret_cast<const float4 *>(&L.k[c0 + 4 * g]);
+        const float4 bv = *reinterpret_cast<const float4 *>(&L.b[c0 + 4 * g]);
+        ks[4 * g] = kv.x; ks[4 * g + 1] = kv.y; ks[4 * g + 2] = kv.z; ks[4 * g + 3] = kv.w;
+        bs[4 * g] = bv.x; bs[4 * g + 1] = bv.y; bs[4 * g + 2] = bv.z; bs[4 * g + 3] = bv.w;
     }
-    __device__ __forceinline__ uint4 operator()(const int (&acc)[16]) const
-    {
-        uint32_t w[4];
-        if (affine) requant16_affine<false>(acc, k, b, w);
-        else requant16_fastdiv<false>(acc, k, b, s_out, inv_s_out, w);
-        const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-        return relu ? relu16(v) : v;
-    }
-};
+    uint32_t w[4];
+    if (L.affine) requant16_affine<false>(acc, ks, bs, w);
+    else requant16_fastdiv<false>(acc, ks, bs, L.s_out, L.inv_s_out, w);
+    const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+    return L.relu ? relu16(v) : v;
+}
 
 // acc[i] += skip_mul[c0 + i] * x[i], one dp2a each
 __device__ __forceinline__ void add_skip(int (&acc)[16], uint4 x, const ResLayer &L, int c0)
@@ -164,24 +162,24 @@ __device__ __forceinline__ void add_skip(int (&acc)[16], uint4 x, const ResLayer
     }
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint4 &a, uint4 &b)
+__device__ __forceinline__ uint4 tmem_ld4(uint32_t taddr)
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                 : "r"(taddr)
-                 : "memory");
+    uint4 v;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(taddr) : "memory");
+    return v;
 }
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, uint4 a, uint4 b)
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 v)
 {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(a.x), "r"(a.y),
-                 "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
-                 : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+template <int I>
+using OpIndex = std::integral_constant<int, I>;
 
 // descriptors: constant upper words; the lower word is (address >> 4) | flags
 constexpr uint32_t kDescSw32Hi = (256u >> 4) | (1u << 14) | (6u << 29);   // 32-byte rows, 32-byte swizzle
@@ -197,22 +195,19 @@ __device__ __forceinline__ uint64_t desc(uint32_t hi, uint32_t lo) { return ((ui
 // what every kernel of this file does first: barriers, tensor memory, weights; returns the tensor-memory base
 template <int EPI_WARPS>
 __device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, int buffer_bytes, uint8_t *w_smem,
-                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals,
-                                              int slot_arrivals, const ResLayer *layers, ResLayer *s_layers, int n_layers)
+                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals, int wide_slot)
 {
-    for (int i = threadIdx.x; i < n_layers * (int)(sizeof(ResLayer) / 4); i += blockDim.x)
-        reinterpret_cast<uint32_t *>(s_layers)[i] = reinterpret_cast<const uint32_t *>(layers)[i];
     // borders and padding stay zero for the life of the CTA
     for (int i = threadIdx.x; i < buffer_bytes / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(buffers)[i] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&bars.w_ready), 1);
-        for (int c = 0; c < kCtx; ++c) {
+        for (int c = 0; c < kMaxCtx; ++c) {
             mbar_init(smem_u32(&bars.land[c]), 1);
             mbar_init(smem_u32(&bars.ready[c]), epi_arrivals);
             for (int s = 0; s < kMaxSlots; ++s) {
                 mbar_init(smem_u32(&bars.acc_full[c][s]), 1);
-                mbar_init(smem_u32(&bars.acc_empty[c][s]), slot_arrivals);
+                mbar_init(smem_u32(&bars.acc_empty[c][s]), s == wide_slot ? epi_arrivals : 4);
             }
         }
         bars.abort_flag = 0;
@@ -261,27 +256,26 @@ __device__ __forceinline__ void res_teardown(ResBars &bars, int warp, int alloc_
 // maximum over three lines follows on the codes in shared memory.  The MMAs take 2 340 cycles an image;
 // the epilogue's instructions (33 k codes an image, some 14 k warp instructions) bound the kernel.
 namespace {
-constexpr int kFirstWg = 2;                                  // warpgroups per context
-constexpr int kFirstT = kFirstWg * 128, kFirstEpi = kCtx * kFirstWg * 4;
+constexpr int kFirstCtx = 2, kFirstWg = 2;                   // images in flight, warpgroups of each
+constexpr int kFirstT = kFirstWg * 128, kFirstEpi = kFirstCtx * kFirstWg * 4;
 constexpr int kFirstTiles = 15, kFirstSlots = 3;             // ceil(83 lines * 22 rows / 128)
 constexpr int kFrameBytes = 31 * 1024, kHpBytes = 55 * 1024; // quantised frame (last tile reads past it), pooled lines
-constexpr int kFirstSmem = 1024 + 8192 + kCtx * (kFrameBytes + kHpBytes);
+constexpr int kFirstSmem = 1024 + 8192 + kFirstCtx * (kFrameBytes + kHpBytes);
 static_assert((kFirstTiles * 128 + 45) * 16 <= kFrameBytes && 83 * 21 * 32 <= kHpBytes, "buffers");
 }  // namespace
 
-template <bool SHIFT>
-__global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(const __grid_constant__ ResFirstParams p)
+template <bool SHIFT, bool TAP>
+__global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_kernel(const __grid_constant__ ResFirstParams p)
 {
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
-    __shared__ __align__(16) ResLayer s_layer;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + 8192;
-    const uint32_t tmem = res_setup<kFirstEpi>(bars, bufs, kCtx * (kFrameBytes + kHpBytes), smem, p.w, kResFirstWeights,
-                                               warp, kFirstWg * 4, 4, &p.layer, &s_layer, 1);
+    const uint32_t tmem = res_setup<kFirstEpi>(bars, bufs, kFirstCtx * (kFrameBytes + kHpBytes), smem, p.w, kResFirstWeights,
+                                               warp, kFirstWg * 4, -1);
     volatile int *abort_flag = &bars.abort_flag;
-    const int step = kCtx * (int)gridDim.x;
+    const int step = kFirstCtx * (int)gridDim.x;
 
     if (warp >= kFirstEpi) {
         // ------------------------------------------------------------------ MMA issuers
@@ -342,7 +336,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                                        ingest_fixed_line4<true>(w[j][0], w[j][1], w[j][2], w[j][3], 2, p.ingest_mul, p.ingest_add),
                                        ingest_fixed_line4<true>(w[j][0], w[j][1], w[j][2], w[j][3], 3, p.ingest_mul, p.ingest_add));
                     sts16(frame + (uint32_t)(((y + 1) * 22 + g + 1) * 16), v);
-                    if (p.tap_in) *reinterpret_cast<uint4 *>(p.tap_in + ((size_t)n * kGroups + i) * 16) = v;
+                    if (TAP) *reinterpret_cast<uint4 *>(p.tap_in + ((size_t)n * kGroups + i) * 16) = v;
                 }
             }
             fence_async();
@@ -352,8 +346,6 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)(n + step) * 28224), "r"(28224)
                              : "memory");
         };
-        Requant req;
-        req.load(s_layer, 0);
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (n < p.batch) convert(n);
         uint32_t seq0 = 0;  // accumulators handed over before this image
@@ -380,7 +372,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                     }
 #pragma unroll
                     for (int i = 0; i < 16; ++i) a[i] = __vimax3_s32(a[i], b[i], c[i]);
-                    const uint4 v = req(a);
+                    const uint4 v = requant_res(a, p.layer, 0);
                     if (valid) sts16(hp + row_off(R, j), v);
                 }
             }
@@ -395,7 +387,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
                 mx.take(lds16(hp + row_off(R + 42, c)));
                 const uint4 v = mx.result();
                 *reinterpret_cast<uint4 *>(out + row_off((oy + 1) * 21 + (s >> 1), c)) = v;
-                if (p.tap_x1) *reinterpret_cast<uint4 *>(p.tap_x1 + ((size_t)n * 1681 + i) * 16) = v;
+                if (TAP) *reinterpret_cast<uint4 *>(p.tap_x1 + ((size_t)n * 1681 + i) * 16) = v;
             }
             ctx_sync<kFirstT>(ctx);  // before the next image's lines overwrite these
         }
@@ -406,39 +398,38 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kCtx), 1) res_first_kernel(c
 // ---------------------------------------------------------------------------------------
 // two residual blocks at 41 x 41 x 16, conv 16 -> 32, max-pool
 // ---------------------------------------------------------------------------------------
-// Per context: a landing buffer for the next image, the operand of a block's first conv (ReLU'd) and
+// Per context two buffers: the operand of a block's first conv (ReLU'd; the image lands there too) and
 // the tensor between its two convs.  The block's input x, which the second conv adds, stays in tensor
 // memory: the thread that adds it is the thread that wrote it.  The 16 -> 32 conv runs as two halves of
 // sixteen output channels, so that the un-pooled half fits the buffer between the convs.
 namespace {
-constexpr int kS1Wg = 2;
-constexpr int kS1T = kS1Wg * 128, kS1Epi = kCtx * kS1Wg * 4;
-constexpr int kS1Tiles = 7, kS1Slots = 6, kS1Ops = 6;       // 41 * 21 GEMM rows; accumulators; layers and half layers
+constexpr int kS1Ctx = 3, kS1Wg = 2;                        // images in flight, warpgroups of each
+constexpr int kS1T = kS1Wg * 128, kS1Epi = kS1Ctx * kS1Wg * 4;
+constexpr int kS1Tiles = 7, kS1Slots = 3, kS1Ops = 6;       // 41 * 21 GEMM rows; accumulators; layers and half layers
 constexpr int kS1Buf = 30 * 1024;                           // an image's rows and what the last tile reads past them
-constexpr int kS1XCol = kS1Slots * 32;                      // x in tensor memory: 8 columns a tile behind the accumulators
-constexpr int kS1Smem = 1024 + kRes1Weights + kCtx * 3 * kS1Buf;
-static_assert((kS1Tiles * 128 + 2 * 21 + 1) * 32 <= kS1Buf && kS1XCol + 8 * kS1Tiles <= 256, "buffers");
+constexpr int kS1XCol = kS1Slots * 32, kS1Cols = 168;       // tensor memory of a context: accumulators, then 8 columns of x per tile
+constexpr int kS1Smem = 1024 + kRes1Weights + kS1Ctx * 2 * kS1Buf;
+static_assert((kS1Tiles * 128 + 2 * 21 + 1) * 32 <= kS1Buf && kS1XCol + 8 * kS1Tiles <= kS1Cols && kS1Ctx * kS1Cols <= 512, "buffers");
 }  // namespace
 
-__global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(const __grid_constant__ ResStack1Params p)
+template <bool TAP>
+__global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(const __grid_constant__ ResStack1Params p)
 {
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
-    __shared__ __align__(16) ResLayer s_layer[5];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes1Weights;
-    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kCtx * 3 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, 4,
-                                            p.layer, s_layer, 5);
+    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kS1Ctx * 2 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, -1);
     volatile int *abort_flag = &bars.abort_flag;
-    const int step = kCtx * (int)gridDim.x;
+    const int step = kS1Ctx * (int)gridDim.x;
 
     if (warp >= kS1Epi) {
         // ------------------------------------------------------------------ MMA issuers
         const int ctx = warp - kS1Epi;
         const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
-        const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)(ctx * 3 + 1) * kS1Buf) >> 4) | kDescSw32Lo, h0 = r0 + (kS1Buf >> 4);
+        const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)(ctx * 2) * kS1Buf) >> 4) | kDescSw32Lo, h0 = r0 + (kS1Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
         res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, rdy = 0;
@@ -454,7 +445,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
                     res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
-                        const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 32, a = a_op + (uint32_t)t * (128 * 2);
+                        const uint32_t d = tmem + (uint32_t)ctx * kS1Cols + slot * 32, a = a_op + (uint32_t)t * (128 * 2);
 #pragma unroll
                         for (int j = 0; j < 6; ++j)
                             mma_i8(d, desc(kDescSw32Hi, a + (uint32_t)((j >> 1) * 21 + (j & 1)) * 2), desc(kDescSw32Hi, b_op + (uint32_t)j * 64),
@@ -470,95 +461,94 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
         // ------------------------------------------------------------------ epilogue
         const int ctx = warp / (kS1Wg * 4), wg = (warp >> 2) % kS1Wg, q = warp & 3;
         const int tid = (int)threadIdx.x - ctx * kS1T;
-        const uint32_t land = smem_u32(bufs) + (uint32_t)(ctx * 3) * kS1Buf, rbuf = land + kS1Buf, hbuf = rbuf + kS1Buf;
+        const uint32_t rbuf = smem_u32(bufs) + (uint32_t)(ctx * 2) * kS1Buf, hbuf = rbuf + kS1Buf;
         const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
-        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
+        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * kS1Cols;
         auto fetch = [&](int n) {  // one thread
             mbar_expect_tx(land_bar, kRes1Bytes);
-            bulk_load(land, p.x1 + (size_t)n * kRes1Bytes, kRes1Bytes, land_bar);
+            bulk_load(rbuf, p.x1 + (size_t)n * kRes1Bytes, kRes1Bytes, land_bar);
         };
         auto operand_done = [&]() {
             fence_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(ready);
         };
-        // GEMM row m = 128 t + row of this thread: are its two pixels part of the image?
+        // GEMM row m = 128 t + row of this thread: is its second pixel part of the image (bit t)?
         const int row = q * 32 + lane;
-        uint32_t second = 0;  // bit t: the second one is
+        uint32_t second = 0;
         for (int t = 0; t < kS1Tiles; ++t)
             if ((t * 128 + row) % 21 < 20 && t * 128 + row < 861) second |= 1u << t;
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (tid == 0 && n < p.batch) fetch(n);
-        uint32_t seq0 = 0, it = 0;
+        uint32_t seq0 = 0, it = 0;  // tiles handed over before this layer, images
         for (; n < p.batch; n += step, ++it) {
-            // the image: x to tensor memory, ReLU(x) to the first conv's operand
+            // the image: x to tensor memory, ReLU(x) in place for the first conv
             res_wait(land_bar, it & 1, abort_flag, p.status, 1);
             for (int t = wg; t < kS1Tiles; t += kS1Wg) {
                 const int m = t * 128 + row, r = m + 21;
-                const bool v0 = m < 861, v1 = (second >> t) & 1;
-                uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0;
-                if (v0) x0 = lds16(land + row_off(r, 1));
-                if (v1) x1 = lds16(land + row_off(r + 1, 0));
-                tmem_st8(tlane + kS1XCol + 8 * t, x0, x1);
-                if (v0) sts16(rbuf + row_off(r, 1), relu16(x0));
-                if (v1) sts16(rbuf + row_off(r + 1, 0), relu16(x1));
+                const bool v[2] = {m < 861, ((second >> t) & 1) != 0};
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t at = rbuf + row_off(r + h, h ^ 1);
+                    uint4 x = make_uint4(0, 0, 0, 0);
+                    if (v[h]) {
+                        x = lds16(at);
+                        sts16(at, relu16(x));
+                    }
+                    tmem_st4(tlane + kS1XCol + 8 * t + 4 * h, x);
+                }
             }
             tmem_wait_st();
             operand_done();
-            ctx_sync<kS1T>(ctx);  // the landing buffer has been read
-            if (tid == 0 && n + step < p.batch) {
-                fence_async();
-                fetch(n + step);
-            }
-            for (int op = 0; op < kS1Ops; ++op) {
-                const ResLayer &L = s_layer[op < 4 ? op : 4];
-                Requant req;
-                req.load(L, op == 5 ? 16 : 0);
-                const bool skip = op == 1 || op == 3;          // second conv of a block
+            auto layer = [&](auto op_c) {
+                constexpr int op = decltype(op_c)::value, c0 = op == 5 ? 16 : 0;
+                constexpr bool skip = op == 1 || op == 3;      // second conv of a block
+                const ResLayer &L = p.layer[op < 4 ? op : 4];
                 const uint32_t dst = skip ? rbuf : hbuf;
-                int8_t *tap = op < 4 ? p.tap[op] : nullptr;
                 for (int t = wg; t < kS1Tiles; t += kS1Wg) {
                     const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS1Slots;
                     const int m = t * 128 + row, r = m + 21;
-                    const bool v0 = m < 861, v1 = (second >> t) & 1;
+                    const bool v[2] = {m < 861, ((second >> t) & 1) != 0};
                     res_wait(full0 + 8 * slot, (seq / kS1Slots) & 1, abort_flag, p.status, 16);
                     fence_after();
-                    int a0[16], a1[16];
-                    uint4 x0, x1;
-                    tmem_ld16(tlane + slot * 32, a0);
-                    tmem_ld16(tlane + slot * 32 + 16, a1);
-                    if (skip) tmem_ld8(tlane + kS1XCol + 8 * t, x0, x1);
-                    tmem_wait_ld();
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(empty0 + 8 * slot);
-                    if (skip) {
-                        add_skip(a0, x0, L, 0);
-                        add_skip(a1, x1, L, 0);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {  // the row's two pixels
+                        int a[16];
+                        tmem_ld16(tlane + slot * 32 + 16 * h, a);
+                        uint4 x = make_uint4(0, 0, 0, 0);
+                        if (skip) x = tmem_ld4(tlane + kS1XCol + 8 * t + 4 * h);
+                        tmem_wait_ld();
+                        if (h == 1) {
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                        }
+                        if (skip) add_skip(a, x, L, 0);
+                        uint4 c = requant_res(a, L, c0);
+                        if (TAP && op < 4 && v[h]) {
+                            const int Y = m / 21, X = m - Y * 21;
+                            *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 41 + Y) * 41 + 2 * X + h) * 16) = c;
+                        }
+                        if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
+                            tmem_st4(tlane + kS1XCol + 8 * t + 4 * h, c);
+                            c = relu16(c);
+                        }
+                        if (v[h]) sts16(dst + row_off(r + h, h ^ 1), c);
                     }
-                    uint4 q0 = req(a0), q1 = req(a1);
-                    if (tap) {
-                        const int Y = m / 21, X = m - Y * 21;
-                        int8_t *d = tap + (((size_t)n * 41 + Y) * 41 + 2 * X) * 16;
-                        if (v0) *reinterpret_cast<uint4 *>(d) = q0;
-                        if (v1) *reinterpret_cast<uint4 *>(d + 16) = q1;
-                    }
-                    if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
-                        tmem_st8(tlane + kS1XCol + 8 * t, q0, q1);
-                        q0 = relu16(q0), q1 = relu16(q1);
-                    }
-                    if (v0) sts16(dst + row_off(r, 1), q0);
-                    if (v1) sts16(dst + row_off(r + 1, 0), q1);
                 }
                 seq0 += kS1Tiles;
                 if (op == 1) tmem_wait_st();
                 if (op < 4) {
                     operand_done();
-                    continue;
+                    return;
                 }
                 // a half of the 16 -> 32 conv is complete: 3 x 3 stride-2 max over it
                 ctx_sync<kS1T>(ctx);
+                if (op == 5 && tid == 0 && n + step < p.batch) {  // the MMAs have read the image: the next one may land
+                    fence_async();
+                    fetch(n + step);
+                }
                 int8_t *out = p.x2 + (size_t)n * kRes2Bytes;
                 for (int i = tid; i < 400; i += kS1T) {
                     const int oy = i / 20, ox = i - oy * 20, R = (2 * oy + 1) * 21 + ox;
@@ -573,12 +563,18 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
                         mx.take(u1);
                         mx.take(u2);
                     }
-                    const uint4 v = mx.result();
-                    *reinterpret_cast<uint4 *>(out + row_off((oy + 1) * 21 + ox + 1, op - 4)) = v;
-                    if (p.tap_x2) *reinterpret_cast<uint4 *>(p.tap_x2 + ((size_t)n * 400 + i) * 32 + 16 * (op - 4)) = v;
+                    const uint4 c = mx.result();
+                    *reinterpret_cast<uint4 *>(out + row_off((oy + 1) * 21 + ox + 1, op - 4)) = c;
+                    if (TAP) *reinterpret_cast<uint4 *>(p.tap_x2 + ((size_t)n * 400 + i) * 32 + 16 * (op - 4)) = c;
                 }
                 ctx_sync<kS1T>(ctx);
-            }
+            };
+            layer(OpIndex<0>());
+            layer(OpIndex<1>());
+            layer(OpIndex<2>());
+            layer(OpIndex<3>());
+            layer(OpIndex<4>());
+            layer(OpIndex<5>());
         }
     }
     res_teardown(bars, warp, kS1Epi, tmem);
@@ -587,43 +583,42 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kCtx), 1) res_stack1_kernel(con
 // ---------------------------------------------------------------------------------------
 // two residual blocks at 20 x 20 x 32, conv 32 -> 32, max-pool, two blocks at 9 x 9 x 32
 // ---------------------------------------------------------------------------------------
-// As above with one pixel per GEMM row.  The two warpgroups of a context take half of the channels of
-// every tile, and a thread keeps its part of x in registers.
+// As above with one pixel per GEMM row.  At 9 x 9, where a layer is one tile, the two warpgroups of a
+// context take half of the channels each and a thread keeps its part of x in registers.
 namespace {
-constexpr int kS2Wg = 2;
-constexpr int kS2T = kS2Wg * 128, kS2Epi = kCtx * kS2Wg * 4;
+constexpr int kS2Ctx = 3, kS2Wg = 2;                        // images in flight, warpgroups of each
+constexpr int kS2T = kS2Wg * 128, kS2Epi = kS2Ctx * kS2Wg * 4;
 constexpr int kS2Tiles = 4, kS2Ops = 9;                     // 20 * 21 GEMM rows; layers
-constexpr int kS2Land = 15 * 1024, kS2Buf = 18 * 1024, kS3Buf = 5 * 1024;
-constexpr int kS2Ctx = kS2Land + 2 * kS2Buf + 2 * kS3Buf;
-constexpr int kS2WideSlot = 4;  // accumulators 0 .. 3: the tiles at 20 x 20, 4 and 5: the layers at 9 x 9
-constexpr int kS2Smem = 1024 + kRes2Weights + kCtx * kS2Ctx;
-static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kRes2Bytes <= kS2Land,
-              "buffers");
+constexpr int kS2Buf = 18 * 1024, kS3Buf = 5 * 1024, kS2CtxBytes = 2 * kS2Buf + 2 * kS3Buf;
+constexpr int kS2Slots = 3, kS2Slot3 = 3;                   // accumulators 0 .. 2: the tiles at 20 x 20, 3: the layers at 9 x 9
+constexpr int kS2XCol = 128, kS2Cols = 160;                 // x: 8 columns a tile behind them
+constexpr int kS2Smem = 1024 + kRes2Weights + kS2Ctx * kS2CtxBytes;
+static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kS2Ctx * kS2Cols <= 512, "buffers");
 }  // namespace
 
-__global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
+template <bool TAP>
+__global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
 {
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
-    __shared__ __align__(16) ResLayer s_layer[9];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes2Weights;
-    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kCtx * kS2Ctx, smem, p.w, kRes2Weights, warp, kS2Wg * 4,
-                                            kS2Wg * 4, p.layer, s_layer, 9);
+    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kS2Ctx * kS2CtxBytes, smem, p.w, kRes2Weights, warp, kS2Wg * 4,
+                                            kS2Slot3);
     volatile int *abort_flag = &bars.abort_flag;
-    const int step = kCtx * (int)gridDim.x;
+    const int step = kS2Ctx * (int)gridDim.x;
 
     if (warp >= kS2Epi) {
         // ------------------------------------------------------------------ MMA issuers
         const int ctx = warp - kS2Epi;
         const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
-        const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2Ctx + kS2Land) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
+        const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
                        r3 = h0 + (kS2Buf >> 4), h3 = r3 + (kS3Buf >> 4);
-        const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
+        const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo, d0 = tmem + (uint32_t)ctx * kS2Cols;
         res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
-        uint32_t rdy = 0, k2 = 0, k3 = 0;  // layers done at 20 x 20 and at 9 x 9
+        uint32_t rdy = 0, slot = 0, phase = 0, k3 = 0;  // k3: layers done at 9 x 9
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
             for (int op = 0; op < kS2Ops; ++op) {
                 res_wait(ready, rdy, abort_flag, p.status, 8);
@@ -633,30 +628,29 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
                 if (op < 5) {
                     const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
                     for (int t = 0; t < kS2Tiles; ++t) {
-                        res_wait(empty0 + 8 * t, (k2 & 1) ^ 1, abort_flag, p.status, 4);
+                        res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                         fence_after();
                         if (elect_one()) {
-                            const uint32_t d = tmem + (uint32_t)ctx * 256 + t * 32, a = a_op + (uint32_t)t * (128 * 2);
+                            const uint32_t a = a_op + (uint32_t)t * (128 * 2);
 #pragma unroll
                             for (int j = 0; j < 9; ++j)
-                                mma_i8(d, desc(kDescSw32Hi, a + (uint32_t)((j / 3) * 21 + j % 3) * 2),
+                                mma_i8(d0 + slot * 32, desc(kDescSw32Hi, a + (uint32_t)((j / 3) * 21 + j % 3) * 2),
                                        desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
-                            mma_commit(full0 + 8 * t);
+                            mma_commit(full0 + 8 * slot);
                         }
                         __syncwarp();
+                        if (++slot == kS2Slots) slot = 0, phase ^= 1;
                     }
-                    ++k2;
                 } else {
-                    const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3, slot = kS2WideSlot + (k3 & 1);
-                    res_wait(empty0 + 8 * slot, ((k3 >> 1) & 1) ^ 1, abort_flag, p.status, 4);
+                    const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3;
+                    res_wait(empty0 + 8 * kS2Slot3, (k3 & 1) ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
-                        const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 32;
 #pragma unroll
                         for (int j = 0; j < 9; ++j)
-                            mma_i8(d, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
+                            mma_i8(d0 + kS2Slot3 * 32, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
                                    desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
-                        mma_commit(full0 + 8 * slot);
+                        mma_commit(full0 + 8 * kS2Slot3);
                     }
                     __syncwarp();
                     ++k3;
@@ -667,84 +661,96 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
         // ------------------------------------------------------------------ epilogue
         const int ctx = warp / (kS2Wg * 4), wg = (warp >> 2) % kS2Wg, q = warp & 3;
         const int tid = (int)threadIdx.x - ctx * kS2T;
-        const uint32_t land = smem_u32(bufs) + (uint32_t)ctx * kS2Ctx, rbuf = land + kS2Land, hbuf = rbuf + kS2Buf,
-                       r3buf = hbuf + kS2Buf, h3buf = r3buf + kS3Buf;
+        const uint32_t rbuf = smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes, hbuf = rbuf + kS2Buf, r3buf = hbuf + kS2Buf,
+                       h3buf = r3buf + kS3Buf;
         const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
-        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
+        const uint32_t tctx = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ctx * kS2Cols);
         auto fetch = [&](int n) {  // one thread
             mbar_expect_tx(land_bar, kRes2Bytes);
-            bulk_load(land, p.x2 + (size_t)n * kRes2Bytes, kRes2Bytes, land_bar);
+            bulk_load(rbuf, p.x2 + (size_t)n * kRes2Bytes, kRes2Bytes, land_bar);
         };
         auto operand_done = [&]() {
             fence_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(ready);
         };
-        // A warpgroup takes sixteen channels (half wg of a row) of every tile; this thread's pixels:
         const int row = q * 32 + lane;
         uint32_t inside = 0;  // bit t: row 128 t + row is a pixel of the 20 x 20 image
         for (int t = 0; t < kS2Tiles; ++t)
             if ((t * 128 + row) % 21 < 20 && t * 128 + row < 420) inside |= 1u << t;
+        const uint32_t off2 = row_off(row + 22, 0);  // first half of the row of tile 0; the other half: ^ 16, tile t: + 4096 t
         const int Y3 = row / 10, X3 = row - Y3 * 10;
         const bool v3 = Y3 < 9 && X3 < 9;
         const uint32_t off3 = row_off(row + 11, wg);
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (tid == 0 && n < p.batch) fetch(n);
-        uint32_t k2 = 0, k3 = 0, it = 0;
+        uint32_t seq0 = 0, k3 = 0, it = 0;
         for (; n < p.batch; n += step, ++it) {
             res_wait(land_bar, it & 1, abort_flag, p.status, 1);
-            uint4 xs[kS2Tiles];  // the block's input, this thread's channels of its pixels
+            for (int t = wg; t < kS2Tiles; t += kS2Wg)
 #pragma unroll
-            for (int t = 0; t < kS2Tiles; ++t) {
-                const uint32_t off = row_off(t * 128 + row + 22, wg);
-                xs[t] = make_uint4(0, 0, 0, 0);
-                if ((inside >> t) & 1) {
-                    xs[t] = lds16(land + off);
-                    sts16(rbuf + off, relu16(xs[t]));
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t at = rbuf + (off2 ^ (16 * h)) + t * 4096;
+                    uint4 x = make_uint4(0, 0, 0, 0);
+                    if ((inside >> t) & 1) {
+                        x = lds16(at);
+                        sts16(at, relu16(x));
+                    }
+                    tmem_st4(tctx + kS2XCol + 8 * t + 4 * h, x);
                 }
-            }
+            tmem_wait_st();
             operand_done();
-            ctx_sync<kS2T>(ctx);  // the landing buffer has been read
-            if (tid == 0 && n + step < p.batch) {
+            auto layer20 = [&](auto op_c) {
+                constexpr int op = decltype(op_c)::value;
+                constexpr bool skip = op == 1 || op == 3;
+                const ResLayer &L = p.layer[op];
+                const uint32_t dst = skip ? rbuf : hbuf;
+                for (int t = wg; t < kS2Tiles; t += kS2Wg) {
+                    const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS2Slots;
+                    const bool v = (inside >> t) & 1;
+                    res_wait(full0 + 8 * slot, (seq / kS2Slots) & 1, abort_flag, p.status, 16);
+                    fence_after();
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        int a[16];
+                        uint4 x = make_uint4(0, 0, 0, 0);
+                        tmem_ld16(tctx + slot * 32 + 16 * h, a);
+                        if (skip) x = tmem_ld4(tctx + kS2XCol + 8 * t + 4 * h);
+                        tmem_wait_ld();
+                        if (h == 1) {
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                        }
+                        if (skip) add_skip(a, x, L, 16 * h);
+                        uint4 c = requant_res(a, L, 16 * h);
+                        if (TAP && v) {
+                            const int m = t * 128 + row, Y = m / 21, X = m - Y * 21;
+                            *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 20 + Y) * 20 + X) * 32 + 16 * h) = c;
+                        }
+                        if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
+                            tmem_st4(tctx + kS2XCol + 8 * t + 4 * h, c);
+                            c = relu16(c);
+                        }
+                        if (v) sts16(dst + (off2 ^ (16 * h)) + t * 4096, c);
+                    }
+                }
+                seq0 += kS2Tiles;
+                if (op == 1) tmem_wait_st();
+                if (op < 4) operand_done();
+            };
+            layer20(OpIndex<0>());
+            layer20(OpIndex<1>());
+            layer20(OpIndex<2>());
+            layer20(OpIndex<3>());
+            layer20(OpIndex<4>());
+            // 3 x 3 stride-2 max over the last one: every thread its pixel and channels of the 9 x 9 tensor
+            ctx_sync<kS2T>(ctx);
+            if (tid == 0 && n + step < p.batch) {  // the MMAs have read the image's buffer: the next one may land
                 fence_async();
                 fetch(n + step);
             }
-            for (int op = 0; op < 5; ++op, ++k2) {
-                const ResLayer &L = s_layer[op];
-                Requant req;
-                req.load(L, 16 * wg);
-                const bool skip = op == 1 || op == 3;
-                const uint32_t dst = skip ? rbuf : hbuf;
-                int8_t *tap = p.tap[op];
-#pragma unroll
-                for (int t = 0; t < kS2Tiles; ++t) {
-                    const uint32_t off = row_off(t * 128 + row + 22, wg);
-                    const bool v = (inside >> t) & 1;
-                    res_wait(full0 + 8 * t, k2 & 1, abort_flag, p.status, 16);
-                    fence_after();
-                    int a[16];
-                    tmem_ld16(tlane + t * 32 + 16 * wg, a);
-                    tmem_wait_ld();
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(empty0 + 8 * t);
-                    if (skip) add_skip(a, xs[t], L, 16 * wg);
-                    uint4 c = req(a);
-                    if (tap && v) {
-                        const int m = t * 128 + row, Y = m / 21, X = m - Y * 21;
-                        *reinterpret_cast<uint4 *>(tap + (((size_t)n * 20 + Y) * 20 + X) * 32 + 16 * wg) = c;
-                    }
-                    if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
-                        xs[t] = c;
-                        c = relu16(c);
-                    }
-                    if (v) sts16(dst + off, c);
-                }
-                if (op < 4) operand_done();
-            }
-            // 3 x 3 stride-2 max over the last one: every thread its pixel and channels of the 9 x 9 tensor
-            ctx_sync<kS2T>(ctx);
             uint4 x = make_uint4(0, 0, 0, 0);
             if (v3) {
                 const int R = (2 * Y3 + 1) * 21 + 2 * X3 + 1;
@@ -754,37 +760,44 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kCtx), 1) res_stack23_kernel(co
                 for (int j = 1; j < 9; ++j) mx.take(lds16(hbuf + row_off(R + (j / 3) * 21 + j % 3, wg)));
                 x = mx.result();
                 sts16(r3buf + off3, relu16(x));
-                if (p.tap_x3) *reinterpret_cast<uint4 *>(p.tap_x3 + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = x;
+                if (TAP) *reinterpret_cast<uint4 *>(p.tap_x3 + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = x;
             }
             operand_done();
-            for (int op = 5; op < kS2Ops; ++op, ++k3) {
-                const ResLayer &L = s_layer[op];
-                Requant req;
-                req.load(L, 16 * wg);
-                const bool skip = op == 6 || op == 8;
-                const uint32_t slot = kS2WideSlot + (k3 & 1);
-                res_wait(full0 + 8 * slot, (k3 >> 1) & 1, abort_flag, p.status, 16);
+            auto layer9 = [&](auto op_c, auto half_c) {
+                constexpr int op = decltype(op_c)::value, half = decltype(half_c)::value;
+                constexpr bool skip = op == 6 || op == 8;
+                const ResLayer &L = p.layer[op];
+                res_wait(full0 + 8 * kS2Slot3, k3 & 1, abort_flag, p.status, 16);
                 fence_after();
                 int a[16];
-                tmem_ld16(tlane + slot * 32 + 16 * wg, a);
+                tmem_ld16(tctx + kS2Slot3 * 32 + 16 * half, a);
                 tmem_wait_ld();
                 fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(empty0 + 8 * slot);
-                if (skip) add_skip(a, x, L, 16 * wg);
-                uint4 v = req(a);
-                if (v3 && p.tap[op]) *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = v;
+                if (lane == 0) mbar_arrive(empty0 + 8 * kS2Slot3);
+                if (skip) add_skip(a, x, L, 16 * half);
+                uint4 c = requant_res(a, L, 16 * half);
+                if (TAP && v3 && op < 8) *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * half) = c;
                 if (skip) {
-                    x = v;
-                    v = relu16(v);
+                    x = c;
+                    c = relu16(c);
                 }
                 if (op == 8) {
-                    if (v3) *reinterpret_cast<uint4 *>(p.x3 + (size_t)n * kRes3Bytes + (Y3 * 9 + X3) * 32 + 16 * wg) = v;
+                    if (v3) *reinterpret_cast<uint4 *>(p.x3 + (size_t)n * kRes3Bytes + (Y3 * 9 + X3) * 32 + 16 * half) = c;
                 } else {
-                    if (v3) sts16((skip ? r3buf : h3buf) + off3, v);
+                    if (v3) sts16((skip ? r3buf : h3buf) + off3, c);
                     operand_done();
                 }
-            }
+                ++k3;
+            };
+            auto layers9 = [&](auto half_c) {
+                layer9(OpIndex<5>(), half_c);
+                layer9(OpIndex<6>(), half_c);
+                layer9(OpIndex<7>(), half_c);
+                layer9(OpIndex<8>(), half_c);
+            };
+            if (wg == 0) layers9(OpIndex<0>());
+            else layers9(OpIndex<1>());
         }
     }
     res_teardown(bars, warp, kS2Epi, tmem);
@@ -818,19 +831,21 @@ cudaError_t res_launch(K kernel, const P &p, int threads, size_t smem, int sm_co
 
 cudaError_t res_first_launch(const ResFirstParams &p, int sm_count, cudaStream_t st)
 {
-    const int threads = 32 * (kFirstEpi + kCtx);
-    return p.ingest_mode == 2 ? res_launch(res_first_kernel<true>, p, threads, kFirstSmem, sm_count, st)
-                              : res_launch(res_first_kernel<false>, p, threads, kFirstSmem, sm_count, st);
+    auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kFirstEpi + kFirstCtx), kFirstSmem, sm_count, st); };
+    if (p.tap_in) return p.ingest_mode == 2 ? go(res_first_kernel<true, true>) : go(res_first_kernel<false, true>);
+    return p.ingest_mode == 2 ? go(res_first_kernel<true, false>) : go(res_first_kernel<false, false>);
 }
 
 cudaError_t res_stack1_launch(const ResStack1Params &p, int sm_count, cudaStream_t st)
 {
-    return res_launch(res_stack1_kernel, p, 32 * (kS1Epi + kCtx), kS1Smem, sm_count, st);
+    auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kS1Epi + kS1Ctx), kS1Smem, sm_count, st); };
+    return p.tap_x2 ? go(res_stack1_kernel<true>) : go(res_stack1_kernel<false>);
 }
 
 cudaError_t res_stack23_launch(const ResStack23Params &p, int sm_count, cudaStream_t st)
 {
-    return res_launch(res_stack23_kernel, p, 32 * (kS2Epi + kCtx), kS2Smem, sm_count, st);
+    auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kS2Epi + kS2Ctx), kS2Smem, sm_count, st); };
+    return p.tap_x3 ? go(res_stack23_kernel<true>) : go(res_stack23_kernel<false>);
 }
 
 }  // namespace accerl
