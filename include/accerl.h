@@ -318,8 +318,9 @@ accerl_status accerl_policy_act_timed(accerl_policy *p, const void *obs_dev,
  * device footprint fixed after start-up.  For such callers a workspace sized by `max_batch` at
  * create time, or the staging buffers accerl_policy_act_host allocates on first use, are not an
  * option.  Create the handle with max_batch = 1 (it then owns little beyond the weights) and step
- * through this call: it computes exactly what accerl_policy_act computes, with the plain
- * CUDA-core kernels, but keeps all int8 activations in a fixed array of
+ * through this call: it computes exactly what accerl_policy_act computes, along the handle's own
+ * plan where that keeps nothing between calls (else with the plain CUDA-core kernels), but keeps all
+ * int8 activations in a fixed array of
  * ACCERL_NOALLOC_SCRATCH_BYTES bytes that is part of the library image.  Every GPU on which the
  * library's kernels get loaded holds that array until the process exits.
  *

@@ -278,9 +278,9 @@ static accerl_status check_act_args(accerl_policy *p, const void *obs_dev,
 }
 
 // Enqueue the plan's launches; with `ev`, record ev[i] before launch i and ev[n] after the last.
-static accerl_status run_steps(accerl_policy *p, const void *obs_dev, const float *uniforms_dev,
-                               int B, float *logits_dev, int32_t *actions_dev, float *logp_dev,
-                               float *value_dev, float *entropy_dev, cudaStream_t st, cudaEvent_t *ev)
+accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const float *uniforms_dev, int B,
+                                float *logits_dev, int32_t *actions_dev, float *logp_dev, float *value_dev,
+                                float *entropy_dev, cudaStream_t st, cudaEvent_t *ev)
 {
     p->last_stream = st;
     // a last layer with a value column and a sampler launch of its own: the layer's floats go to
@@ -421,6 +421,7 @@ void accerl_policy_destroy(accerl_policy *p)
     for (cudaEvent_t ev : p->events) cudaEventDestroy(ev);
     for (cudaEvent_t ev : p->copy_events) cudaEventDestroy(ev);
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
+    delete p->noalloc_twin;  // owns nothing on the device
     delete p;
 }
 

@@ -64,6 +64,13 @@ struct Step {
     std::string kernel, covers;
 };
 
+// How a step's TMA map of its activations was made, so that it can be made again for another workspace
+struct ActivationMap {
+    const void *base = nullptr;
+    long long rows_per_state = 0, pitch = 0;
+    int row_bytes = 0, box_rows = 0, box_bytes = 0;
+};
+
 // One launch of the tensor-core contraction: TMA descriptors (built once, for max_batch rows) and
 // the parameter block; batch-dependent fields are filled in per call.
 struct TcStep {
@@ -71,6 +78,7 @@ struct TcStep {
     alignas(64) unsigned char map_b[128];
     TcGemmParams prm;
     bool resident_b = false;
+    ActivationMap a_map;
 };
 
 // One launch of the strided-conv kernel (tc_conv.cu)
@@ -78,6 +86,7 @@ struct ConvRowsStep {
     alignas(64) unsigned char map_a[128];
     alignas(64) unsigned char map_b[128];
     ConvRowsParams prm;
+    ActivationMap a_map;
 };
 
 struct MlpFusedParams;  // mlp_fused.cu
@@ -162,6 +171,10 @@ struct accerl_policy {
     uint32_t ingest_fa = 0, ingest_fc1 = 0;  // bit patterns of A and c1
     int *status_word = nullptr;           // device, set by kernels whose bounded waits give up
     size_t workspace_bytes = 0;
+    // accerl_policy_act_noalloc: a copy of this policy whose activations lie in the library's fixed array
+    // (made on its first call; owns no device memory), and whether the plan allows one
+    accerl_policy *noalloc_twin = nullptr;
+    bool noalloc_tried = false;
     std::vector<void *> owned;            // every device allocation, for destroy
     cudaStream_t last_stream = nullptr;
     std::vector<cudaEvent_t> events;      // steps.size() + 1 events, created on first timed call
@@ -191,6 +204,11 @@ static inline bool unfuse_for_taps(const accerl_policy *p)
 {
     return (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) && !(p->flags & ACCERL_FLAG_TAP_FUSED);
 }
+
+// one Actor step along the policy's plan (api.cu); with `ev`, an event before each launch and after the last
+accerl_status run_steps(accerl_policy *p, const void *obs_dev, const float *uniforms_dev, int B, float *logits_dev,
+                        int32_t *actions_dev, float *logp_dev, float *value_dev, float *entropy_dev, cudaStream_t st,
+                        cudaEvent_t *ev);
 
 // generic CUDA-core kernels (generic_kernels.cu); every launcher enqueues on `st` and returns
 // the launch status

@@ -2,7 +2,11 @@
 //
 // The activation workspace of this variant is a fixed array inside the library image instead of
 // buffers obtained from cudaMalloc.  See the declaration in accerl.h for who needs it and why.
+#include <algorithm>
 #include <mutex>
+#include <new>
+#include <type_traits>
+#include <vector>
 
 #include "internal.h"
 
@@ -57,9 +61,117 @@ accerl_status scratch_on(int device, unsigned char **out)
     return ACCERL_OK;
 }
 
-}  // namespace
-
 using namespace accerl;
+
+// The policy's own plan on the fixed array: a copy of the handle whose activation pointers and TMA maps
+// lead there.  Weights, scales and the status word are the handle's; nothing is allocated on the device.
+// (Stepping through the CUDA-core kernels instead took 182 us for 160 states of the Nature-CNN.)
+// Null when the plan keeps tensors whose borders must stay zero, or taps.
+accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
+{
+    std::lock_guard<std::mutex> lock(g_mu);
+    if (p->noalloc_tried) return p->noalloc_twin;
+    p->noalloc_tried = true;
+    if (p->flags & (ACCERL_FLAG_KEEP_ACTIVATIONS | ACCERL_FLAG_FORCE_GENERIC)) return nullptr;
+    bool resident = false;
+    for (const Step &s : p->steps) {
+        switch (s.kind) {
+        case Step::RES_FIRST: resident = true; break;
+        case Step::RES_STACK1: case Step::RES_STACK23: case Step::MLP_FUSED: case Step::CONV1_FRAMES: case Step::CONV_ROWS:
+        case Step::FC_SAMPLE: case Step::SAMPLE: break;
+        case Step::TC_GEMM: {
+            const TcGemmParams &g = p->tc_steps[s.tc].prm;  // no padded layouts, no residual or second output
+            if (g.out2 || g.skip || g.px_per_row || g.out_row_off) return nullptr;
+            break;
+        }
+        default: return nullptr;
+        }
+    }
+    // activation regions of the plan, as bytes per state
+    struct Region {
+        const char *old_base;
+        size_t per_state;
+        char *new_base;
+    };
+    std::vector<Region> regions;
+    if (!p->mlp)
+        for (size_t b = 0; b < p->bufs.size(); ++b) {
+            // (the resident kernels leave the conv layers' buffers unused)
+            bool used = !resident;
+            for (size_t i = kResLayers; i < p->layers.size() && !used; ++i) used = p->layers[i].out_buf == (int)b;
+            if (used) regions.push_back(Region{(const char *)p->bufs[b].ptr, p->bufs[b].bytes_per_state, nullptr});
+        }
+    if (p->z_scratch) regions.push_back(Region{(const char *)p->z_scratch, (size_t)p->n_out * sizeof(float), nullptr});
+    if (resident) {
+        regions.push_back(Region{(const char *)p->res_first.x1, kRes1Bytes, nullptr});
+        regions.push_back(Region{(const char *)p->res_stack1.x2, kRes2Bytes, nullptr});
+        regions.push_back(Region{(const char *)p->res_stack23.x3, kRes3Bytes, nullptr});
+    }
+    size_t per_state = 0;
+    for (const Region &r : regions) per_state += r.per_state;
+    // the largest batch the regions fit, each rounded up to 1 KB (TMA boxes may start in the last rows)
+    size_t cap = (size_t)INT32_MAX;  // the single-launch MLP keeps no activations
+    if (per_state) cap = std::min<size_t>(4096, (kScratchBytes - 1024 * regions.size()) / per_state);
+    size_t at = 0;
+    for (Region &r : regions) {
+        r.new_base = (char *)base + at;
+        at += (r.per_state * cap + 1023) / 1024 * 1024;
+    }
+    accerl_policy *q = new (std::nothrow) accerl_policy(*p);
+    if (!q) return nullptr;
+    q->noalloc_twin = nullptr;
+    q->owned.clear();
+    q->events.clear();
+    q->copy_events.clear();
+    q->copy_stream = nullptr;
+    q->ptq.clear();
+    q->max_batch = (int)cap;
+    bool ok = true;
+    auto move = [&](auto *&ptr) {
+        if (!ptr) return;
+        for (const Region &r : regions)
+            if ((const char *)ptr >= r.old_base && (const char *)ptr < r.old_base + r.per_state * (size_t)p->max_batch + 256) {
+                ptr = (std::remove_reference_t<decltype(ptr)>)(r.new_base + ((const char *)ptr - r.old_base));
+                return;
+            }
+        ok = false;
+    };
+    auto remap = [&](void *map, ActivationMap &m) {
+        move(m.base);
+        if (ok && tc_make_map(map, m.base, m.rows_per_state * (long long)cap, m.row_bytes, m.pitch, m.box_rows, m.box_bytes) != ACCERL_OK)
+            ok = false;
+    };
+    for (const Step &s : q->steps) {
+        if (s.kind == Step::TC_GEMM) {
+            TcStep &t = q->tc_steps[s.tc];
+            if (!t.prm.fuse_ingest) remap(t.map_a, t.a_map);  // (that one reads the frames themselves)
+            if (!t.prm.logits_mode) move(t.prm.out);
+        } else if (s.kind == Step::CONV_ROWS) {
+            ConvRowsStep &c = q->conv_rows[s.tc];
+            remap(c.map_a, c.a_map);
+            move(c.prm.out);
+        } else if (s.kind == Step::CONV1_FRAMES) {
+            move(q->conv1.out);
+        } else if (s.kind == Step::FC_SAMPLE) {
+            move(q->fc_sample.x);
+        } else if (s.kind == Step::RES_FIRST) {
+            move(q->res_first.x1);
+            move(q->res_stack1.x1);
+            move(q->res_stack1.x2);
+            move(q->res_stack23.x2);
+            move(q->res_stack23.x3);
+        }
+    }
+    move(q->z_scratch);
+    if (!ok) {
+        delete q;
+        return nullptr;
+    }
+    p->noalloc_twin = q;
+    return q;
+}
+
+}  // namespace
 
 extern "C" accerl_status accerl_policy_act_noalloc(accerl_policy *p, const void *obs_dev,
                                                    const float *uniforms_dev, int32_t batch,
@@ -110,6 +222,12 @@ extern "C" accerl_status accerl_policy_act_noalloc(accerl_policy *p, const void 
     unsigned char *base = nullptr;
     accerl_status s = scratch_on(p->device, &base);
     if (s != ACCERL_OK) return s;
+    if (accerl_policy *twin = twin_of(p, base); twin && batch <= twin->max_batch) {
+        p->last_stream = (cudaStream_t)cuda_stream;  // accerl_policy_check waits for this step
+        return run_steps(twin, obs_dev, uniforms_dev, batch, logits_dev, actions_dev, logp_dev, nullptr, nullptr,
+                         (cudaStream_t)cuda_stream, nullptr);
+    }
+    // a plan that cannot be moved, or a batch beyond its share of the array: the CUDA-core kernels
     auto buf = [&](int b) { return (int8_t *)(base + offset[b]); };
 
     cudaStream_t st = (cudaStream_t)cuda_stream;

@@ -828,6 +828,7 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
         }
         void *w_dev = nullptr;
         if ((st = upload_bytes(p, packed.data(), packed.size(), &w_dev)) != ACCERL_OK) return st;
+        ts.a_map = ActivationMap{a_ptr, a_rows_total / p->max_batch, row_bytes, row_bytes, g.shifted ? g.a_rows : 128, g.chunk_bytes};
         if ((st = tc_make_map(ts.map_a, a_ptr, a_rows_total, row_bytes, row_bytes,
                               g.shifted ? g.a_rows : 128, g.chunk_bytes)) != ACCERL_OK)
             return st;

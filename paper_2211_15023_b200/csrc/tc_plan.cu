@@ -271,6 +271,10 @@ accerl_status choose_fastdiv(float s_out, bool relu, float y_max, bool allow, fl
 
 namespace {
 
+// the strided-conv kernels' index arithmetic is set up for at least this many states, so that a handle
+// made for one state can step through the fixed workspace of accerl_policy_act_noalloc as well
+constexpr int kNoallocStates = 4096;
+
 bool conv_fits(const accerl_layer_desc &d)
 {
     if (d.pad != 0 || d.kh % d.stride || d.in_h % d.stride || d.in_w % d.stride) return false;
@@ -510,7 +514,7 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
         if (fuse && g.fast_div) {
             Conv1Params c1;
             const int mode = p->ingest_shift1 ? 2 : (g.ingest_clamp ? 1 : 0);
-            if (conv1_plan(d, p->in_h, p->in_w, p->max_batch, n_total, mode, &c1) &&
+            if (conv1_plan(d, p->in_h, p->in_w, std::max(p->max_batch, kNoallocStates), n_total, mode, &c1) &&
                 conv1_smem_bytes(c1) <= 200 * 1024) {
                 c1.ingest_mul = p->ingest_mul;
                 c1.ingest_add = p->ingest_add;
@@ -566,7 +570,7 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
             n_total > 32 && n_total <= 64) {
             ConvRowsStep cs;
             if (conv_rows_plan(g.rows_per_image / g.grid_w, g.grid_w, g.chunk_bytes, d.kh / d.stride, n_total,
-                               p->max_batch, &cs.prm)) {
+                               std::max(p->max_batch, kNoallocStates), &cs.prm)) {
                 ConvRowsParams &c2 = cs.prm;
                 c2.out = g.out;
                 c2.out_h = g.out_h;
@@ -588,6 +592,7 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
                 void *w2_dev = nullptr;
                 accerl_status st2 = upload_bytes(p, packed.data(), packed.size(), &w2_dev);
                 if (st2 != ACCERL_OK) return st2;
+                cs.a_map = ActivationMap{p->bufs[L.in_buf].ptr, rows_in_per_image, row_bytes, row_bytes, c2.box_rows, row_bytes};
                 st2 = tc_make_map(cs.map_a, p->bufs[L.in_buf].ptr, (long long)p->max_batch * rows_in_per_image,
                                   row_bytes, row_bytes, c2.box_rows, row_bytes);
                 if (st2 != ACCERL_OK) return st2;
@@ -621,6 +626,8 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
         accerl_status st = upload_bytes(p, packed.data(), packed.size(), &w_dev);
         if (st != ACCERL_OK) return st;
         const long long rows = (long long)p->max_batch * rows_in_per_image;
+        ts.a_map = ActivationMap{p->bufs[L.in_buf].ptr, rows_in_per_image, row_bytes, row_bytes,
+                                 g.shifted ? g.a_rows : 128, g.chunk_bytes};
         st = tc_make_map(ts.map_a, p->bufs[L.in_buf].ptr, rows, row_bytes, row_bytes,
                          g.shifted ? g.a_rows : 128, g.chunk_bytes);
         if (st != ACCERL_OK) return st;

@@ -130,7 +130,7 @@ accerl_status build_res_steps(accerl_policy *p, const accerl_layer_desc *layers,
     if (st == ACCERL_OK) st = upload_bytes(p, w2.data(), w2.size(), &d2);
     if (st != ACCERL_OK) return st;
 
-    // ---- the tensors between the kernels; their borders are zeroed here and never written
+    // ---- the tensors between the kernels
     const size_t mb = (size_t)p->max_batch, bytes[3] = {mb * kRes1Bytes, mb * kRes2Bytes, mb * kRes3Bytes};
     int8_t *x[3];
     for (int i = 0; i < 3; ++i) {
@@ -138,7 +138,6 @@ accerl_status build_res_steps(accerl_policy *p, const accerl_layer_desc *layers,
         ACCERL_CUDA_TRY(cudaMalloc(&d, bytes[i] + 4096));
         p->owned.push_back(d);
         p->workspace_bytes += bytes[i] + 4096;
-        ACCERL_CUDA_TRY(cudaMemsetAsync(d, 0, bytes[i] + 4096, 0));
         x[i] = (int8_t *)d;
     }
     *x3 = x[2];

@@ -379,6 +379,10 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
             ctx_sync<kFirstT>(ctx);  // all lines pooled along x; the MMAs have read the frame
             if (n + step < p.batch) convert(n + step);
             int8_t *out = p.x1 + (size_t)n * kRes1Bytes;
+            if (tid < 125) {  // the zero pixels: lines 0 and 42, the first one of the lines between
+                const int s = tid < 42 ? tid : tid < 84 ? 42 * 42 + tid - 42 : (tid - 83) * 42;
+                *reinterpret_cast<uint4 *>(out + row_off(s >> 1, s & 1)) = make_uint4(0, 0, 0, 0);
+            }
             for (int i = tid; i < 41 * 41; i += kFirstT) {
                 const int oy = i / 41, ox = i - oy * 41, s = ox + 1, R = 2 * oy * 21 + (s >> 1), c = s & 1;
                 ByteMax mx;
@@ -550,6 +554,10 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                     fetch(n + step);
                 }
                 int8_t *out = p.x2 + (size_t)n * kRes2Bytes;
+                if (tid < 62) {  // the zero pixels: lines 0 and 21, the first one of the lines between
+                    const int s = tid < 21 ? tid : tid < 42 ? 21 * 21 + tid - 21 : (tid - 41) * 21;
+                    *reinterpret_cast<uint4 *>(out + row_off(s, op - 4)) = make_uint4(0, 0, 0, 0);
+                }
                 for (int i = tid; i < 400; i += kS1T) {
                     const int oy = i / 20, ox = i - oy * 20, R = (2 * oy + 1) * 21 + ox;
                     ByteMax mx;

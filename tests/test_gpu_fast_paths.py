@@ -89,3 +89,32 @@ def test_native_calls_refuse_what_the_python_checks_refused():
     g.close()
     with pytest.raises(P.AccerlError):
         g.act(obs, u)
+
+
+@pytest.mark.parametrize("name,batches", [("nature_cnn_b160", (1, 129, 1200)), ("student_cnn_b8192", (3, 700)),
+                                          ("impala_resnet_b16384", (2, 149, 264)), ("lunarlander_mlp", (5, 4500))])
+@pytest.mark.parametrize("value", [False, True], ids=["plain", "value_head"])
+def test_noalloc_runs_the_plan_on_the_fixed_array(name, batches, value):
+    """The policy's own plan with its activations in the library's array: batches up to what the array
+    holds, two handles in turn so that each finds the other's bytes in it (the residual network's zero
+    borders among them), against the device call."""
+    import paper_2211_15023_b200 as P
+    pol = W.drawn_int8_policy(name, seed=4)
+    if value:
+        pol["layers"][-1]["value"] = True
+    big, tiny = P.Policy(pol, max(batches)), P.Policy(pol, 1)
+    other = P.Policy(W.drawn_int8_policy("nature_cnn_b160", seed=5), 1)
+    stream = torch.cuda.current_stream().cuda_stream
+    for b in batches:
+        for g, n in ((other, "nature_cnn_b160"), (tiny, name)):
+            obs, u = torch.from_numpy(W.observations(n, b)).cuda(), torch.from_numpy(W.uniforms(n, b)).cuda()
+            got = (torch.full((b, g.n_actions), 7.0, device="cuda"), torch.full((b,), -1, dtype=torch.int32, device="cuda"),
+                   torch.full((b,), 7.0, device="cuda"))
+            status = g.act_noalloc_raw(obs.data_ptr(), u.data_ptr(), b, *(t.data_ptr() for t in got), stream)
+            assert status == (3 if g is other and b > 1636 else 0)
+        want = big.act(obs, u)
+        tiny.check()
+        for x, y in zip(got, want):
+            assert torch.equal(x, y)
+    for g in (big, tiny, other):
+        g.close()
