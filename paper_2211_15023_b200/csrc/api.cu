@@ -44,15 +44,7 @@ struct DeviceGuard {
 template <typename T>
 accerl_status upload(accerl_policy *p, const std::vector<T> &host, T **dev)
 {
-    *dev = nullptr;
-    size_t bytes = std::max<size_t>(host.size() * sizeof(T), 16);
-    void *d = nullptr;
-    ACCERL_CUDA_TRY(cudaMalloc(&d, bytes));
-    p->owned.push_back(d);
-    if (!host.empty())
-        ACCERL_CUDA_TRY(cudaMemcpy(d, host.data(), host.size() * sizeof(T), cudaMemcpyHostToDevice));
-    *dev = (T *)d;
-    return ACCERL_OK;
+    return upload_bytes(p, host.data(), host.size() * sizeof(T), (void **)dev);
 }
 
 struct Shape {
@@ -181,28 +173,24 @@ void pack_generic(const accerl_layer_desc &d, LayerPlan &L, std::vector<int32_t>
     const int C4 = L.in_cp / 4;
     if (d.kind == ACCERL_CONV2D) {
         words.assign((size_t)d.kh * d.kw * C4 * L.oc_pad, 0);
+        int8_t *bytes = reinterpret_cast<int8_t *>(words.data());
+        const int8_t *w = d.w;
         for (int oc = 0; oc < d.out_c; ++oc)
             for (int ic = 0; ic < d.in_c; ++ic)
-                for (int ky = 0; ky < d.kh; ++ky)
-                    for (int kx = 0; kx < d.kw; ++kx) {
-                        int8_t v = d.w[((oc * d.in_c + ic) * d.kh + ky) * d.kw + kx];
-                        size_t wi = ((size_t)(ky * d.kw + kx) * C4 + ic / 4) * L.oc_pad + oc;
-                        words[wi] |= (int32_t)((uint32_t)(uint8_t)v << (8 * (ic % 4)));
-                    }
+                for (int tap = 0; tap < d.kh * d.kw; ++tap)
+                    bytes[(((size_t)tap * C4 + ic / 4) * L.oc_pad + oc) * 4 + ic % 4] = *w++;
     } else {
         // FC input is the previous tensor in (y, x, c) order with c padded to in_cp; the
         // descriptor's columns are in (c, y, x) order
-        const int K_int = L.in_h * L.in_w * L.in_cp;
+        const int HW = L.in_h * L.in_w, K_int = HW * L.in_cp;
         words.assign((size_t)L.oc_pad * (K_int / 4), 0);
+        int8_t *bytes = reinterpret_cast<int8_t *>(words.data());
         for (int oc = 0; oc < d.out_c; ++oc)
-            for (int c = 0; c < L.in_c; ++c)
-                for (int y = 0; y < L.in_h; ++y)
-                    for (int x = 0; x < L.in_w; ++x) {
-                        int8_t v = d.w[(size_t)oc * d.in_c + (c * L.in_h + y) * L.in_w + x];
-                        int ki = (y * L.in_w + x) * L.in_cp + c;
-                        words[(size_t)oc * (K_int / 4) + ki / 4] |=
-                            (int32_t)((uint32_t)(uint8_t)v << (8 * (ki % 4)));
-                    }
+            for (int c = 0; c < L.in_c; ++c) {
+                const int8_t *src = d.w + (size_t)oc * d.in_c + (size_t)c * HW;
+                int8_t *dst = bytes + (size_t)oc * K_int + c;
+                for (int i = 0; i < HW; ++i) dst[(size_t)i * L.in_cp] = src[i];
+            }
     }
 }
 
@@ -237,14 +225,36 @@ cudaError_t allow_smem(const void *kernel, size_t bytes)
     return e;
 }
 
+// Parameters go to the device in a few large blocks, collected on the host and copied when the plan is
+// complete: an allocation and a blocking copy for each of some fifty small arrays took longer than
+// everything else accerl_policy_create does.
 accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev)
 {
     *dev = nullptr;
-    void *d = nullptr;
-    ACCERL_CUDA_TRY(cudaMalloc(&d, bytes < 16 ? 16 : bytes));
-    p->owned.push_back(d);
-    ACCERL_CUDA_TRY(cudaMemcpy(d, host, bytes, cudaMemcpyHostToDevice));
-    *dev = d;
+    const size_t need = (bytes + 255) / 256 * 256 + 256;
+    if (p->uploads.empty() || p->uploads.back().used + need > p->uploads.back().host.size()) {
+        UploadBlock b;
+        const size_t size = std::max<size_t>(need, (size_t)1 << 20);
+        void *d = nullptr;
+        ACCERL_CUDA_TRY(cudaMalloc(&d, size));
+        p->owned.push_back(d);
+        b.dev = (char *)d;
+        b.host.resize(size);
+        p->uploads.push_back(std::move(b));
+    }
+    UploadBlock &b = p->uploads.back();
+    if (bytes) memcpy(b.host.data() + b.used, host, bytes);
+    *dev = b.dev + b.used;
+    b.used += need;
+    return ACCERL_OK;
+}
+
+accerl_status flush_uploads(accerl_policy *p)
+{
+    for (UploadBlock &b : p->uploads)
+        if (b.used) ACCERL_CUDA_TRY(cudaMemcpyAsync(b.dev, b.host.data(), b.used, cudaMemcpyHostToDevice, 0));
+    ACCERL_CUDA_TRY(cudaStreamSynchronize(0));
+    p->uploads.clear();
     return ACCERL_OK;
 }
 
@@ -536,7 +546,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         L.skip_from = d.skip_from;
         L.oc_pad = round_up(L.out_c, 16);
         if (d.kind != ACCERL_MAXPOOL) {
-            std::vector<int32_t> words;
+            std::vector<int32_t> &words = L.host_words;
             pack_generic(d, L, words);
             std::vector<float> ks(L.oc_pad, 0.f), bs(L.oc_pad, 0.f);
             for (int c = 0; c < d.out_c; ++c) {
@@ -556,9 +566,9 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         } else {
             L.how = "maxpool_kernel";
         }
-        p->layers.push_back(L);
+        p->layers.push_back(std::move(L));
         in = shapes[i];
-        in_cp = L.out_cp;
+        in_cp = p->layers.back().out_cp;
     }
 
     // ---- workspace: tensor -1 is the quantised input, tensor i is layer i's int8 output.
@@ -596,19 +606,22 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
             L.out_buf = buf_of[i + 1];
         }
     }
-    for (DeviceBuf &b : p->bufs) {
-        size_t bytes = b.bytes_per_state * (size_t)max_batch + 256;
+    {
+        size_t total = 0;
+        for (DeviceBuf &b : p->bufs) total += (b.bytes_per_state * (size_t)max_batch + 256 + 1023) / 1024 * 1024;
         void *d = nullptr;
-        cudaError_t e = cudaMalloc(&d, bytes);
+        cudaError_t e = cudaMalloc(&d, total);
         if (e != cudaSuccess) {
-            set_error("create: cudaMalloc of %zu workspace bytes failed: %s", bytes,
-                      cudaGetErrorString(e));
+            set_error("create: cudaMalloc of %zu workspace bytes failed: %s", total, cudaGetErrorString(e));
             cudaGetLastError();
             return fail(e == cudaErrorMemoryAllocation ? ACCERL_ERR_OOM : ACCERL_ERR_CUDA);
         }
         p->owned.push_back(d);
-        b.ptr = (int8_t *)d;
-        p->workspace_bytes += bytes;
+        p->workspace_bytes += total;
+        for (DeviceBuf &b : p->bufs) {
+            b.ptr = (int8_t *)d;
+            d = (char *)d + (b.bytes_per_state * (size_t)max_batch + 256 + 1023) / 1024 * 1024;
+        }
     }
 
     // ---- input table: the frame quantiser evaluated for all 256 byte values
@@ -674,16 +687,17 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
     p->tensor_s2d.assign(n_layers + 1, 1);
     p->tap_missing.assign(n_layers + 1, 0);
     {
-        cudaDeviceProp prop;
-        cudaError_t pe = cudaGetDeviceProperties(&prop, device);
+        // (cudaGetDeviceProperties takes milliseconds)
+        int major = 0, minor = 0;
+        cudaError_t pe = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, device);
+        if (pe == cudaSuccess) pe = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
+        if (pe == cudaSuccess) pe = cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
         if (pe != cudaSuccess) {
-            set_error("create: cudaGetDeviceProperties: %s", cudaGetErrorString(pe));
+            set_error("create: cudaDeviceGetAttribute: %s", cudaGetErrorString(pe));
             return fail(ACCERL_ERR_CUDA);
         }
-        p->sm_count = prop.multiProcessorCount;
-        if (prop.major != 10) {
-            set_error("create: this library is built for sm_100a only (device is sm_%d%d)",
-                      prop.major, prop.minor);
+        if (major != 10) {
+            set_error("create: this library is built for sm_100a only (device is sm_%d%d)", major, minor);
             return fail(ACCERL_ERR_UNSUPPORTED);
         }
     }
@@ -696,6 +710,8 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
             (st = build_mlp_plan(p, layers, n_layers, &used)) != ACCERL_OK)
             return fail(st);
     }
+    if ((st = flush_uploads(p)) != ACCERL_OK) return fail(st);
+    for (LayerPlan &L : p->layers) std::vector<int32_t>().swap(L.host_words);
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         set_error("create: %s", cudaGetErrorString(e));

@@ -51,6 +51,7 @@ struct LayerPlan {
     int32_t *skip_mul = nullptr;   // [oc_pad] or null
     int oc_pad = 0;                // out_c rounded up to 16
     std::string how;               // which kernel serves the layer (for accerl_policy_info)
+    std::vector<int32_t> host_words;  // w_generic on the host, while the policy is built
 };
 
 // One kernel launch of the plan: which kernel, and which part of the path it covers
@@ -124,6 +125,21 @@ struct TapDesc {
     int off_y = 0, off_x = 0;    // where pixel (0, 0) sits
 };
 
+// How a layer requantises (requant_fit.cu): per channel the single-fma pair when `affine`, else
+// (s_in * s_w, bias); fast_div: that pair, or the three-step division with inv_s_out, is verified
+struct LayerRequant {
+    std::vector<float> k, b;
+    float inv_s_out = 0.f;
+    int affine = 0, fast_div = 0;
+};
+
+// parameters on their way to the device (see upload_bytes)
+struct UploadBlock {
+    char *dev = nullptr;
+    std::vector<char> host;
+    size_t used = 0;
+};
+
 struct DeviceBuf {
     int8_t *ptr = nullptr;
     size_t bytes_per_state = 0;
@@ -169,12 +185,14 @@ struct accerl_policy {
     bool ingest_shift1 = false;           // the table is exactly u >> 1 (s_input = 1/127)
     bool ingest_float = false;            // the same line in float form: code = low byte of fma(f - c1, A, 1.5 * 2^23)
     uint32_t ingest_fa = 0, ingest_fc1 = 0;  // bit patterns of A and c1
+    std::vector<accerl::LayerRequant> requant;  // per layer, once fit_requants has run
     int *status_word = nullptr;           // device, set by kernels whose bounded waits give up
     size_t workspace_bytes = 0;
     // accerl_policy_act_noalloc: a copy of this policy whose activations lie in the library's fixed array
     // (made on its first call; owns no device memory), and whether the plan allows one
     accerl_policy *noalloc_twin = nullptr;
     bool noalloc_tried = false;
+    std::vector<accerl::UploadBlock> uploads;  // while the policy is built
     std::vector<void *> owned;            // every device allocation, for destroy
     cudaStream_t last_stream = nullptr;
     std::vector<cudaEvent_t> events;      // steps.size() + 1 events, created on first timed call
@@ -220,11 +238,18 @@ cudaError_t launch_conv_generic(const LayerPlan &L, const int8_t *in, const int8
                                 int8_t *out, int B, cudaStream_t st);
 cudaError_t launch_fc_generic(const LayerPlan &L, const int8_t *in, int8_t *out, float *logits,
                               int B, cudaStream_t st);
+// the same contractions for calibration: int32 accumulators [positions][out_cp] (residual added) and the
+// largest |y| of the layer, atomically into *ymax
+cudaError_t launch_conv_acc(const LayerPlan &L, const int8_t *in, const int8_t *skip, int *acc, float *ymax, int B,
+                            cudaStream_t st);
+cudaError_t launch_fc_acc(const LayerPlan &L, const int8_t *in, int *acc, float *ymax, int B, cudaStream_t st);
 cudaError_t launch_maxpool_generic(const LayerPlan &L, const int8_t *in, int8_t *out, int B,
                                    cudaStream_t st);
 cudaError_t launch_sample(const float *z, int pitch, const float *u, int B, int A, float *logits_out,
                           int32_t *actions, float *logp, float *value, float *entropy, cudaStream_t st);
 
+// fills p->requant (requant_fit.cu)
+accerl_status fit_requants(accerl_policy *p, const accerl_layer_desc *layers, int n_layers);
 // tensor-core plan (tc_plan.cu): replaces p->steps when the whole network qualifies; returns
 // ACCERL_OK with *used = false when it does not
 accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, int n_layers,
@@ -248,7 +273,8 @@ accerl_status build_mlp_plan(accerl_policy *p, const accerl_layer_desc *layers, 
 cudaError_t launch_mlp_fused(const accerl_policy *p, const float *obs, const float *u, int B,
                              float *logits, int32_t *actions, float *logp, float *value, float *entropy,
                              cudaStream_t st);
-accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev);
+accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev);  // there once create is done
+accerl_status flush_uploads(accerl_policy *p);
 bool fc_sample_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
 accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int layer, const int8_t *x,
                               int pitch, Step *out);

@@ -6,25 +6,35 @@
 // calibration batch, pushed through the already quantised preceding layers), the integer
 // multipliers of the residual adds -- and then builds the handle with accerl_policy_create.
 //
-// This is create-time work: the kernels are plain (one thread per output element, NCHW int8
-// activations, int32 accumulators kept in memory between the passes of a layer) and every result
-// is order-independent (integer sums, maxima), so the scales and codes are the same bits whatever
-// the launch shape.  The Actor step itself never runs these kernels.
+// The Compressor runs this for every policy it hands over, so it is a path of its own: one block of
+// device memory, the contractions on the dp4a kernels (NHWC words) with the maximum of the epilogue
+// value taken as they go, and no host round trip between the layers -- scales, epilogue constants and
+// residual multipliers are computed where the maxima lie.  Every result is order-independent (integer
+// sums, maxima), so the scales and codes are the same bits whatever the launch shape.  (One thread per
+// output walking NCHW bytes, an atomic maximum per element and ten blocking copies a layer took 44 ms
+// for the residual network with 256 calibration frames, building the handle included; now 9.)  The
+// Actor step itself never runs these kernels.
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
+#include "epilogue.cuh"
 #include "internal.h"
 
 namespace accerl {
 
 namespace {
 
-__device__ __forceinline__ void atomic_max_nonneg(float *addr, float v)
+// the scale max-abs calibration gives (1 where nothing was seen)
+__device__ __forceinline__ float scale_of(float ymax) { return ymax > 0.f ? __fdiv_rn(ymax, 127.0f) : 1.0f; }
+
+__device__ __forceinline__ void warp_max_to(float v, float *out)  // v >= 0: the bit patterns order like the values
 {
-    atomicMax(reinterpret_cast<int *>(addr), __float_as_int(v));  // v >= 0: the bit patterns order like the values
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(reinterpret_cast<unsigned *>(out), m);
 }
 
 // 2:4 pruning along K = (kh, kw, c_in), c_in fastest: of every four consecutive K positions keep
@@ -76,106 +86,99 @@ __global__ void quantise_weights_kernel(const float *w, int K, float *s_w, int8_
     }
 }
 
-// max |x| of the real-valued input: frames are u / 255, vectors are taken as they are
-__global__ void input_absmax_kernel(const void *obs, long long n, int is_u8, float *out)
+// max |x| of the real-valued input: frames are u / 255 (non-decreasing in u), vectors are taken as they are
+__global__ void input_absmax_u8_kernel(const uint8_t *obs, long long n, float *out)
+{
+    const long long words = n / 16, first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+    unsigned m = 0;
+    for (long long i = first; i < words; i += stride) {
+        const uint4 v = reinterpret_cast<const uint4 *>(obs)[i];
+        m = __vmaxu4(m, __vmaxu4(__vmaxu4(v.x, v.y), __vmaxu4(v.z, v.w)));
+    }
+    for (long long i = 16 * words + first; i < n; i += stride) m = __vmaxu4(m, obs[i]);
+    const unsigned u = max(max(m & 0xff, (m >> 8) & 0xff), max((m >> 16) & 0xff, m >> 24));
+    warp_max_to(__fdiv_rn((float)u, 255.0f), out);
+}
+
+__global__ void input_absmax_f32_kernel(const float *obs, long long n, float *out)
 {
     float m = 0.f;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        m = fmaxf(m, is_u8 ? __fdiv_rn((float)((const uint8_t *)obs)[i], 255.0f) : fabsf(((const float *)obs)[i]));
-    if (m > 0.f) atomic_max_nonneg(out, m);
+        m = fmaxf(m, fabsf(obs[i]));
+    warp_max_to(m, out);
 }
 
-__global__ void input_quantise_kernel(const void *obs, long long n, int is_u8, float s_input, int8_t *q)
+__device__ __forceinline__ int8_t quantise_real(float x, float s) { return (int8_t)clamp_round_i8(__fdiv_rn(x, s)); }
+
+// the 256-entry input table of launch_ingest_u8
+__global__ void input_table_kernel(const float *ymax, int8_t *lut)
+{
+    lut[threadIdx.x] = quantise_real(__fdiv_rn((float)threadIdx.x, 255.0f), scale_of(*ymax));
+}
+
+__global__ void input_quantise_f32_kernel(const float *obs, long long rows, int D, int pitch, const float *ymax, int8_t *q)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * pitch) return;
+    const long long r = i / pitch;
+    const int k = (int)(i - r * pitch);
+    q[i] = k < D ? quantise_real(obs[r * D + k], scale_of(*ymax)) : 0;
+}
+
+// int8 OIHW weights -> the word layouts of the dp4a kernels (see pack_generic): one byte per thread
+__global__ void pack_conv_kernel(const int8_t *w, long long n, int ic, int taps, int oc_pad, int8_t *out)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float x = is_u8 ? __fdiv_rn((float)((const uint8_t *)obs)[i], 255.0f) : ((const float *)obs)[i];
-    float t = rintf(__fdiv_rn(x, s_input));
-    t = fminf(fmaxf(t, -128.f), 127.f);
-    q[i] = (int8_t)t;
+    const int tap = (int)(i % taps), c = (int)(i / taps % ic), o = (int)(i / taps / ic), c4 = (ic + 3) / 4;
+    out[(((size_t)tap * c4 + c / 4) * oc_pad + o) * 4 + c % 4] = w[i];
 }
-
-struct CalibLayer {
-    int in_c, in_h, in_w, out_c, out_h, out_w, kh, kw, stride, pad, relu_in, relu_out;
-};
-
-// int32 accumulators of a conv or fc layer (fc: 1 x 1 spatial), NCHW int8 in, residual added
-__global__ void calib_acc_kernel(const int8_t *x, const int8_t *w, const int8_t *skip, const int *skip_mul,
-                                 CalibLayer L, long long total, int *acc)
+__global__ void pack_fc_kernel(const int8_t *w, long long n, int C, int HW, int pitch, int8_t *out)
 {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    const int ox = (int)(idx % L.out_w);
-    long long t = idx / L.out_w;
-    const int oy = (int)(t % L.out_h);
-    t /= L.out_h;
-    const int oc = (int)(t % L.out_c);
-    const long long n = t / L.out_c;
-    int a = 0;
-    for (int c = 0; c < L.in_c; ++c)
-        for (int ky = 0; ky < L.kh; ++ky) {
-            const int iy = oy * L.stride + ky - L.pad;
-            if (iy < 0 || iy >= L.in_h) continue;
-            for (int kx = 0; kx < L.kw; ++kx) {
-                const int ix = ox * L.stride + kx - L.pad;
-                if (ix < 0 || ix >= L.in_w) continue;
-                int xv = x[((n * L.in_c + c) * L.in_h + iy) * L.in_w + ix];
-                if (L.relu_in && xv < 0) xv = 0;
-                a += xv * (int)w[((oc * L.in_c + c) * L.kh + ky) * L.kw + kx];
-            }
-        }
-    if (skip) a += skip_mul[oc] * (int)skip[idx];
-    acc[idx] = a;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int hw = (int)(i % HW), c = (int)(i / HW % C);
+    const long long o = i / HW / C;
+    out[o * (long long)HW * pitch + (size_t)hw * pitch + c] = w[i];
 }
 
-// y = fmaf((float)acc, s_in * s_w[c], b[c]) (+ ReLU); pass 0: max|y| into *ymax, pass 1: requantise
-__global__ void calib_epilogue_kernel(const int *acc, const float *kscale, const float *bias, CalibLayer L,
-                                      long long total, int pass, float s_out, float *ymax, int8_t *q)
+// epilogue constants of a layer: k = s_in * s_w, rounded once, and the integer multiplier that brings
+// the skip tensor (scale s_x) onto the accumulators' grid
+__global__ void layer_scales_kernel(const float *s_w, int oc, const float *ymax_in, const float *ymax_skip, float *k, int *mul)
 {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    const int oc = (int)((idx / ((long long)L.out_h * L.out_w)) % L.out_c);
-    float y = __fmaf_rn(__int2float_rn(acc[idx]), kscale[oc], bias[oc]);
-    if (L.relu_out) y = fmaxf(y, 0.f);
-    if (pass == 0) {
-        const float a = fabsf(y);
-        if (a > 0.f) atomic_max_nonneg(ymax, a);
-    } else {
-        float t = rintf(__fdiv_rn(y, s_out));
-        t = fminf(fmaxf(t, -128.f), 127.f);
-        q[idx] = (int8_t)t;
-    }
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= oc) return;
+    const float kc = __fmul_rn(scale_of(*ymax_in), s_w[c]);
+    k[c] = kc;
+    if (ymax_skip) mul[c] = (int)fminf(fmaxf(rintf(__fdiv_rn(scale_of(*ymax_skip), kc)), 0.f), 32767.f);
 }
 
-__global__ void calib_maxpool_kernel(const int8_t *x, CalibLayer L, long long total, int8_t *q)
+// accumulators -> codes, four channels per thread
+__global__ void calib_requant_kernel(const int4 *acc, const float *k, const float *b, int relu, int c4s, long long words,
+                                     const float *ymax, uint32_t *q)
 {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    const int ox = (int)(idx % L.out_w);
-    long long t = idx / L.out_w;
-    const int oy = (int)(t % L.out_h);
-    t /= L.out_h;  // t = n * C + c
-    int m = -128;
-    for (int ky = 0; ky < L.kh; ++ky)
-        for (int kx = 0; kx < L.kw; ++kx)
-            m = max(m, (int)x[(t * L.in_h + oy * L.stride + ky) * L.in_w + ox * L.stride + kx]);
-    q[idx] = (int8_t)m;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= words) return;
+    const int c = (int)(i % c4s) * 4;
+    const int4 a = acc[i];
+    const float s = scale_of(*ymax);
+    q[i] = (uint32_t)(uint8_t)requant(epilogue_float(a.x, k[c], b[c], relu), s) |
+           (uint32_t)(uint8_t)requant(epilogue_float(a.y, k[c + 1], b[c + 1], relu), s) << 8 |
+           (uint32_t)(uint8_t)requant(epilogue_float(a.z, k[c + 2], b[c + 2], relu), s) << 16 |
+           (uint32_t)(uint8_t)requant(epilogue_float(a.w, k[c + 3], b[c + 3], relu), s) << 24;
 }
 
-struct DevMem {  // frees what it holds
-    std::vector<void *> ptrs;
-    ~DevMem()
-    {
-        for (void *p : ptrs) cudaFree(p);
-    }
+// one block of device memory, handed out piece by piece: sized in a first pass, filled in a second
+struct DeviceArena {
+    char *base = nullptr;
+    size_t at = 0;
+    ~DeviceArena() { cudaFree(base); }
     template <typename T>
-    cudaError_t get(T **out, size_t count)
+    T *take(size_t count)
     {
-        void *d = nullptr;
-        cudaError_t e = cudaMalloc(&d, count * sizeof(T) + 16);
-        if (e == cudaSuccess) ptrs.push_back(d);
-        *out = (T *)d;
-        return e;
+        T *p = (T *)(base + at);  // (meaningless while base is null: the sizing pass)
+        at += (count * sizeof(T) + 255) / 256 * 256;
+        return p;
     }
 };
 
@@ -270,27 +273,150 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
     const long long B = calib_rows;
     const long long in_elems = (long long)in_shape[0] * in_shape[1] * in_shape[2] * B;
     const bool u8 = in_kind == ACCERL_IN_U8_NCHW;
-    DevMem mem;
-    // ---- input scale and quantised calibration batch
+    struct Layer {
+        LayerPlan L;      // the dp4a kernels' view of the layer
+        int8_t *act;      // its int8 output, NHWC
+        float *w;
+        int8_t *wq, *packed;
+        float *s_w, *k, *b;
+        int *mul;
+        size_t nw, packed_bytes;
+        int scale;        // index of the maximum its output scale comes from (a pool passes its input's on)
+    };
+    std::vector<Layer> net;
+    try {
+        net.resize(n_layers);
+    } catch (const std::bad_alloc &) {
+        set_error("create_fp32: out of host memory");
+        return ACCERL_ERR_OOM;
+    }
+    int n_run = n_layers;  // layers up to the one with the logits
+    DeviceArena mem;
     void *obs_dev = nullptr;
-    ACCERL_CUDA_TRY(mem.get((uint8_t **)&obs_dev, (size_t)in_elems * (u8 ? 1 : 4)));
-    ACCERL_CUDA_TRY(cudaMemcpy(obs_dev, calib_obs_host, (size_t)in_elems * (u8 ? 1 : 4), cudaMemcpyHostToDevice));
-    float *scal = nullptr;  // [0]: running maximum
-    ACCERL_CUDA_TRY(mem.get(&scal, 4));
-    ACCERL_CUDA_TRY(cudaMemset(scal, 0, 16));
-    input_absmax_kernel<<<1024, 256>>>(obs_dev, in_elems, u8 ? 1 : 0, scal);
-    float m = 0.f;
-    ACCERL_CUDA_TRY(cudaMemcpy(&m, scal, 4, cudaMemcpyDeviceToHost));
-    volatile float s_input_v = m > 0.f ? m / 127.0f : 1.0f;
-    const float s_input = s_input_v;
-    std::vector<int8_t *> act(n_layers + 1, nullptr);  // act[t + 1]: int8 NCHW tensor t of the calibration batch
-    ACCERL_CUDA_TRY(mem.get(&act[0], (size_t)in_elems));
-    input_quantise_kernel<<<blocks_for(in_elems), 256>>>(obs_dev, in_elems, u8 ? 1 : 0, s_input, act[0]);
-    ACCERL_CUDA_TRY(cudaGetLastError());
+    int8_t *lut = nullptr, *act0 = nullptr;
+    float *ymax = nullptr;
     int *acc = nullptr;
-    ACCERL_CUDA_TRY(mem.get(&acc, max_elems * (size_t)B));
+    char *results = nullptr;  // what goes back to the host, in one piece: wq, s_w and mul of every layer, ymax
+    size_t results_bytes = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        mem.at = 0;
+        results = mem.take<char>(0);
+        ymax = mem.take<float>(n_layers + 1);
+        Shape in{in_shape[0], in_shape[1], in_shape[2]};
+        for (int i = 0; i < n_layers; ++i) {
+            const accerl_layer_fp32 &d = layers[i];
+            Layer &l = net[i];
+            LayerPlan &L = l.L;
+            L.kind = d.kind;
+            L.flags = d.flags;
+            L.in_c = in.c; L.in_h = in.h; L.in_w = in.w; L.in_cp = round_up(in.c, 4);
+            L.out_c = shapes[i].c; L.out_h = shapes[i].h; L.out_w = shapes[i].w; L.out_cp = round_up(shapes[i].c, 4);
+            L.oc_pad = round_up(L.out_c, 16);
+            L.kh = d.kh; L.kw = d.kw; L.stride = d.stride; L.pad = d.pad;
+            L.skip_from = d.skip_from;
+            l.nw = l.packed_bytes = 0;
+            if (d.kind != ACCERL_MAXPOOL) {
+                const int taps = d.kind == ACCERL_FC ? 1 : d.kh * d.kw;
+                l.nw = (size_t)d.out_c * (d.kind == ACCERL_FC ? d.in_c : in.c * taps);
+                l.packed_bytes = d.kind == ACCERL_FC ? (size_t)L.oc_pad * in.h * in.w * L.in_cp : (size_t)taps * L.in_cp * L.oc_pad;
+            }
+            l.wq = mem.take<int8_t>(l.nw);
+            l.s_w = mem.take<float>(l.nw ? d.out_c : 0);
+            l.mul = mem.take<int>(d.skip_from >= 0 ? L.oc_pad : 0);
+            in = shapes[i];
+            if ((d.flags & ACCERL_LOGITS) && n_run > i + 1) n_run = i + 1;
+        }
+        results_bytes = mem.at;
+        // (from here on nothing has to start at zero but the packed weights and the padded constants)
+        const size_t zero_from = mem.at;
+        for (int i = 0; i < n_layers; ++i) {
+            Layer &l = net[i];
+            l.packed = mem.take<int8_t>(l.packed_bytes);
+            l.k = mem.take<float>(l.nw ? l.L.oc_pad : 0);
+            l.b = mem.take<float>(l.nw ? l.L.oc_pad : 0);
+        }
+        const size_t zero_to = mem.at;
+        for (int i = 0; i < n_layers; ++i) net[i].w = mem.take<float>(net[i].nw);
+        obs_dev = mem.take<uint8_t>((size_t)in_elems * (u8 ? 1 : 4));
+        lut = mem.take<int8_t>(256);
+        act0 = mem.take<int8_t>((size_t)B * in_shape[1] * in_shape[2] * round_up(in_shape[0], 4));
+        size_t acc_elems = 0;
+        for (int i = 0; i < n_layers; ++i) {
+            const LayerPlan &L = net[i].L;
+            const size_t elems = (size_t)B * L.out_h * L.out_w * L.out_cp;
+            net[i].act = mem.take<int8_t>(elems);
+            if (net[i].nw) acc_elems = std::max(acc_elems, elems);
+        }
+        acc = mem.take<int>(acc_elems);
+        if (pass == 0) {
+            ACCERL_CUDA_TRY(cudaMalloc(&mem.base, mem.at + 256));
+            continue;
+        }
+        ACCERL_CUDA_TRY(cudaMemsetAsync(ymax, 0, (n_layers + 1) * sizeof(float), 0));
+        for (int i = 0; i < n_layers; ++i)
+            if (layers[i].skip_from >= 0) ACCERL_CUDA_TRY(cudaMemsetAsync(net[i].mul, 0, net[i].L.oc_pad * sizeof(int), 0));
+        ACCERL_CUDA_TRY(cudaMemsetAsync(mem.base + zero_from, 0, zero_to - zero_from, 0));
+    }
+
+    // ---- the calibration batch, quantised (ymax[0]: its maximum), and the weights
+    ACCERL_CUDA_TRY(cudaMemcpyAsync(obs_dev, calib_obs_host, (size_t)in_elems * (u8 ? 1 : 4), cudaMemcpyHostToDevice, 0));
+    if (u8) {
+        input_absmax_u8_kernel<<<592, 256>>>((const uint8_t *)obs_dev, in_elems, ymax);
+        input_table_kernel<<<1, 256>>>(ymax, lut);
+        ACCERL_CUDA_TRY(launch_ingest_u8((const uint8_t *)obs_dev, lut, act0, (int)B, in_shape[0], in_shape[1], in_shape[2],
+                                         round_up(in_shape[0], 4), 0));
+    } else {
+        const int pitch = round_up(in_shape[0], 4);
+        input_absmax_f32_kernel<<<592, 256>>>((const float *)obs_dev, in_elems, ymax);
+        input_quantise_f32_kernel<<<blocks_for(B * pitch), 256>>>((const float *)obs_dev, B, in_shape[0], pitch, ymax, act0);
+    }
+    ACCERL_CUDA_TRY(cudaGetLastError());
+    for (int i = 0; i < n_layers; ++i) {
+        const accerl_layer_fp32 &d = layers[i];
+        Layer &l = net[i];
+        if (!l.nw) continue;
+        ACCERL_CUDA_TRY(cudaMemcpyAsync(l.w, d.w, l.nw * 4, cudaMemcpyHostToDevice, 0));
+        ACCERL_CUDA_TRY(cudaMemcpyAsync(l.b, d.bias, (size_t)d.out_c * 4, cudaMemcpyHostToDevice, 0));
+        const int ic = d.in_c, kh = d.kind == ACCERL_FC ? 1 : d.kh;
+        if (prune_2_4) prune24_kernel<<<blocks_for((long long)l.nw / 4), 256>>>(l.w, d.out_c, ic, kh, kh);
+        quantise_weights_kernel<<<(unsigned)d.out_c, 256>>>(l.w, (int)(l.nw / d.out_c), l.s_w, l.wq);
+        if (d.kind == ACCERL_FC)
+            pack_fc_kernel<<<blocks_for((long long)l.nw), 256>>>(l.wq, (long long)l.nw, l.L.in_c, l.L.in_h * l.L.in_w, l.L.in_cp, l.packed);
+        else
+            pack_conv_kernel<<<blocks_for((long long)l.nw), 256>>>(l.wq, (long long)l.nw, d.in_c, kh * kh, l.L.oc_pad, l.packed);
+        ACCERL_CUDA_TRY(cudaGetLastError());
+        l.L.w_generic = (int32_t *)l.packed;
+        l.L.kscale = l.k;
+        l.L.bias = l.b;
+        l.L.skip_mul = d.skip_from >= 0 ? l.mul : nullptr;
+    }
 
     // ---- layer by layer
+    int s_in = 0;  // index of the input scale's maximum
+    for (int i = 0; i < n_run; ++i) {
+        const accerl_layer_fp32 &d = layers[i];
+        Layer &l = net[i];
+        const int8_t *x = i ? net[i - 1].act : act0;
+        l.scale = i + 1;
+        if (d.kind == ACCERL_MAXPOOL) {
+            l.scale = s_in;
+            ACCERL_CUDA_TRY(launch_maxpool_generic(l.L, x, l.act, (int)B, 0));
+            continue;
+        }
+        layer_scales_kernel<<<(unsigned)((d.out_c + 127) / 128), 128>>>(l.s_w, d.out_c, ymax + s_in,
+                                                                        d.skip_from >= 0 ? ymax + net[d.skip_from].scale : nullptr, l.k, l.mul);
+        ACCERL_CUDA_TRY(cudaGetLastError());
+        if (d.flags & ACCERL_LOGITS) break;  // its output is not quantised
+        if (d.kind == ACCERL_FC) ACCERL_CUDA_TRY(launch_fc_acc(l.L, x, acc, ymax + i + 1, (int)B, 0));
+        else
+            ACCERL_CUDA_TRY(launch_conv_acc(l.L, x, d.skip_from >= 0 ? net[d.skip_from].act : nullptr, acc, ymax + i + 1, (int)B, 0));
+        const long long words = B * l.L.out_h * l.L.out_w * (l.L.out_cp / 4);
+        calib_requant_kernel<<<blocks_for(words), 256>>>((const int4 *)acc, l.k, l.b, (d.flags & ACCERL_RELU_OUT) ? 1 : 0,
+                                                         l.L.out_cp / 4, words, ymax + i + 1, (uint32_t *)l.act);
+        ACCERL_CUDA_TRY(cudaGetLastError());
+        s_in = i + 1;
+    }
+    std::vector<char> back;
     struct Quant {
         std::vector<int8_t> w;
         std::vector<float> s_w, bias;
@@ -299,96 +425,39 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
     };
     std::vector<Quant> Q;
     try {
+        back.resize(results_bytes);
         Q.resize(n_layers);
     } catch (const std::bad_alloc &) {
         set_error("create_fp32: out of host memory");
         return ACCERL_ERR_OOM;
     }
-    std::vector<float> scales(n_layers, 1.f);
+    ACCERL_CUDA_TRY(cudaMemcpy(back.data(), results, results_bytes, cudaMemcpyDeviceToHost));
+    auto host = [&](const void *dev) { return back.data() + ((const char *)dev - results); };
+    auto scale = [&](int at) {
+        const float m = reinterpret_cast<const float *>(host(ymax))[at];
+        volatile float s = m > 0.f ? m / 127.0f : 1.0f;
+        return (float)s;
+    };
+    const float s_input = scale(0);
     float s_prev = s_input;
-    Shape in{in_shape[0], in_shape[1], in_shape[2]};
-    for (int i = 0; i < n_layers; ++i) {
+    for (int i = 0; i < n_run; ++i) {
         const accerl_layer_fp32 &d = layers[i];
-        const Shape o = shapes[i];
-        const long long out_elems = (long long)o.c * o.h * o.w * B;
-        CalibLayer L{in.c, in.h, in.w, o.c, o.h, o.w, d.kh, d.kw, d.stride, d.pad,
-                     (d.flags & ACCERL_RELU_IN) ? 1 : 0, (d.flags & ACCERL_RELU_OUT) ? 1 : 0};
+        const Layer &l = net[i];
         Quant &q = Q[i];
         q.s_in = s_prev;
-        const bool last = (d.flags & ACCERL_LOGITS) != 0;
-        if (d.kind == ACCERL_MAXPOOL) {
-            ACCERL_CUDA_TRY(mem.get(&act[i + 1], (size_t)out_elems));
-            calib_maxpool_kernel<<<blocks_for(out_elems), 256>>>(act[i], L, out_elems, act[i + 1]);
-            ACCERL_CUDA_TRY(cudaGetLastError());
-            q.s_out = s_prev;
-        } else {
-            if (d.kind == ACCERL_FC) {
-                L.in_c = d.in_c;
-                L.in_h = L.in_w = L.kh = L.kw = L.stride = 1;
-                L.pad = 0;
-            }
-            const int K = L.in_c * L.kh * L.kw;
-            const size_t nw = (size_t)o.c * K;
-            float *w_dev = nullptr, *sw_dev = nullptr, *k_dev = nullptr, *b_dev = nullptr;
-            int8_t *wq_dev = nullptr;
-            ACCERL_CUDA_TRY(mem.get(&w_dev, nw));
-            ACCERL_CUDA_TRY(mem.get(&sw_dev, (size_t)o.c));
-            ACCERL_CUDA_TRY(mem.get(&k_dev, (size_t)o.c));
-            ACCERL_CUDA_TRY(mem.get(&b_dev, (size_t)o.c));
-            ACCERL_CUDA_TRY(mem.get(&wq_dev, nw));
-            ACCERL_CUDA_TRY(cudaMemcpy(w_dev, d.w, nw * 4, cudaMemcpyHostToDevice));
-            ACCERL_CUDA_TRY(cudaMemcpy(b_dev, d.bias, (size_t)o.c * 4, cudaMemcpyHostToDevice));
-            if (prune_2_4) prune24_kernel<<<blocks_for((long long)nw / 4), 256>>>(w_dev, o.c, L.in_c, L.kh, L.kw);
-            quantise_weights_kernel<<<(unsigned)o.c, 256>>>(w_dev, K, sw_dev, wq_dev);
-            ACCERL_CUDA_TRY(cudaGetLastError());
-            q.w.resize(nw);
-            q.s_w.resize(o.c);
-            q.bias.assign(d.bias, d.bias + o.c);
-            ACCERL_CUDA_TRY(cudaMemcpy(q.w.data(), wq_dev, nw, cudaMemcpyDeviceToHost));
-            ACCERL_CUDA_TRY(cudaMemcpy(q.s_w.data(), sw_dev, (size_t)o.c * 4, cudaMemcpyDeviceToHost));
-            std::vector<float> ks(o.c);
-            for (int c = 0; c < o.c; ++c) {
-                volatile float k = s_prev * q.s_w[c];  // one fp32 rounding
-                ks[c] = k;
-            }
-            ACCERL_CUDA_TRY(cudaMemcpy(k_dev, ks.data(), (size_t)o.c * 4, cudaMemcpyHostToDevice));
-            int *sm_dev = nullptr;
-            if (d.skip_from >= 0) {
-                // integer multiplier that brings the skip tensor (scale s_x) onto the accumulators' grid
-                q.skip_mul.resize(o.c);
-                const float s_x = scales[d.skip_from];
-                for (int c = 0; c < o.c; ++c) {
-                    volatile float r = s_x / ks[c];
-                    float rr = rintf(r);
-                    rr = rr < 0.f ? 0.f : (rr > 32767.f ? 32767.f : rr);
-                    q.skip_mul[c] = (int32_t)rr;
-                }
-                ACCERL_CUDA_TRY(mem.get(&sm_dev, (size_t)o.c));
-                ACCERL_CUDA_TRY(cudaMemcpy(sm_dev, q.skip_mul.data(), (size_t)o.c * 4, cudaMemcpyHostToDevice));
-            }
-            calib_acc_kernel<<<blocks_for(out_elems), 256>>>(act[i], wq_dev, d.skip_from >= 0 ? act[d.skip_from + 1] : nullptr,
-                                                             sm_dev, L, out_elems, acc);
-            ACCERL_CUDA_TRY(cudaGetLastError());
-            q.s_out = 1.0f;
-            if (!last) {
-                ACCERL_CUDA_TRY(cudaMemset(scal, 0, 4));
-                calib_epilogue_kernel<<<blocks_for(out_elems), 256>>>(acc, k_dev, b_dev, L, out_elems, 0, 1.f, scal, nullptr);
-                float ym = 0.f;
-                ACCERL_CUDA_TRY(cudaMemcpy(&ym, scal, 4, cudaMemcpyDeviceToHost));
-                volatile float so = ym > 0.f ? ym / 127.0f : 1.0f;
-                q.s_out = so;
-                ACCERL_CUDA_TRY(mem.get(&act[i + 1], (size_t)out_elems));
-                calib_epilogue_kernel<<<blocks_for(out_elems), 256>>>(acc, k_dev, b_dev, L, out_elems, 1, q.s_out, scal,
-                                                                      act[i + 1]);
-                ACCERL_CUDA_TRY(cudaGetLastError());
-            }
-        }
-        scales[i] = q.s_out;
+        q.s_out = (d.flags & ACCERL_LOGITS) ? 1.0f : scale(l.scale);
         s_prev = q.s_out;
-        in = o;
-        if (last) break;
+        if (!l.nw) continue;
+        const int8_t *w = (const int8_t *)host(l.wq);
+        const float *s_w = (const float *)host(l.s_w);
+        q.w.assign(w, w + l.nw);
+        q.s_w.assign(s_w, s_w + d.out_c);
+        q.bias.assign(d.bias, d.bias + d.out_c);
+        if (d.skip_from >= 0) {
+            const int *m = (const int *)host(l.mul);
+            q.skip_mul.assign(m, m + d.out_c);
+        }
     }
-    ACCERL_CUDA_TRY(cudaDeviceSynchronize());
 
     // ---- hand the quantised network to the ordinary constructor
     std::vector<accerl_layer_desc> descs(n_layers);

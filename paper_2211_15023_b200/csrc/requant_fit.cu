@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "epilogue.cuh"
@@ -30,6 +31,8 @@ constexpr int kPerThread = 16;  // accumulators a thread compares between two vo
 constexpr int kMaxBad = 16;
 
 struct FitJob {
+    float s_out;
+    int relu;
     float k, b;          // the channel's epilogue constants
     float k0, b0;        // fl(k / s_out), fl(b / s_out)
     long long lo, hi;    // band of accumulators to compare (inside int32)
@@ -43,16 +46,18 @@ struct FitResult {
 
 __device__ __forceinline__ int alternate(int i) { return (i & 1) ? (i + 1) / 2 : -(i / 2); }  // 0, 1, -1, 2, -2, ...
 
-template <bool RELU>
-__global__ void __launch_bounds__(kFitThreads) fit_affine_kernel(const FitJob *jobs, FitResult *results, float s_out)
+__global__ void __launch_bounds__(kFitThreads) fit_affine_kernel(const FitJob *jobs, FitResult *results)
 {
     __shared__ long long bad[kMaxBad];  // accumulators on which an earlier candidate failed: tried first
     __shared__ int n_bad;
     const FitJob job = jobs[blockIdx.x];
+    const bool relu = job.relu != 0;
+    const float s_out = job.s_out;
+    auto affine = [&](int acc, float k2, float b2) { return relu ? affine_code<true>(acc, k2, b2) : affine_code<false>(acc, k2, b2); };
     if (threadIdx.x == 0) n_bad = 0;
     __syncthreads();
     auto agree = [&](long long a, float k2, float b2) {
-        return affine_code<RELU>((int)a, k2, b2) == exact_code(epilogue_float((int)a, job.k, job.b, false), s_out, RELU);
+        return affine((int)a, k2, b2) == exact_code(epilogue_float((int)a, job.k, job.b, false), s_out, relu);
     };
     for (int cand = 0; cand < kKOffsets * kBOffsets; ++cand) {
         const float k2 = __uint_as_float(__float_as_uint(job.k0) + (unsigned)alternate(cand % kKOffsets));
@@ -63,8 +68,8 @@ __global__ void __launch_bounds__(kFitThreads) fit_affine_kernel(const FitJob *j
         const int known = min(n_bad, kMaxBad);
         if ((int)threadIdx.x < known) fail = !agree(bad[threadIdx.x], k2, b2);
         if (threadIdx.x == kFitThreads - 1) {
-            if (job.check_lo && affine_code<RELU>((int)job.lo, k2, b2) != (RELU ? 0 : -128)) fail = true;
-            if (job.check_hi && affine_code<RELU>((int)job.hi, k2, b2) != 127) fail = true;
+            if (job.check_lo && affine((int)job.lo, k2, b2) != (relu ? 0 : -128)) fail = true;
+            if (job.check_hi && affine((int)job.hi, k2, b2) != 127) fail = true;
         }
         if (__syncthreads_or(fail)) continue;
         // the whole band, a slice at a time
@@ -104,6 +109,8 @@ bool make_job(float k, float b, float s_out, bool relu, FitJob *job)
     double lo = std::floor(((relu ? -2.0 : -130.0) * ds - db) / dk), hi = std::ceil((130.0 * ds - db) / dk);
     lo -= 16.0 + std::fabs(lo) * 0x1p-20;  // (float)acc is inexact above 2^24
     hi += 16.0 + std::fabs(hi) * 0x1p-20;
+    job->s_out = s_out;
+    job->relu = relu ? 1 : 0;
     job->k = k;
     job->b = b;
     job->k0 = k0;
@@ -118,56 +125,159 @@ bool make_job(float k, float b, float s_out, bool relu, FitJob *job)
 
 }  // namespace
 
-// For n columns with epilogue constants (k[i], b[i]) -- k[i] == 0 marks a padding column -- find the
-// single-fma constants.  *ok = false (and k2, b2 untouched) when some column has none.
-accerl_status fit_affine_requant(const float *k, const float *b, int n, float s_out, bool relu,
-                                 std::vector<float> *k2, std::vector<float> *b2, bool *ok)
+// ---------------------------------------------------------------------------------------
+// the three-step division: is it exact for this scale?
+// ---------------------------------------------------------------------------------------
+namespace {
+
+struct DivJob {
+    float s, r;
+    unsigned lo, hi;  // bit patterns of the positive y to compare
+};
+
+// Positive y only (every operation of both sides is odd in y, and the clamp is applied to equal
+// integers), and only from 0.4 s to 130 s: below, both quotients are far from 0.5 and round to 0; above,
+// both are beyond 129 and saturate.  Some 70 million values instead of 2^32: 0.1 ms instead of 4.5.
+__global__ void __launch_bounds__(256) verify_fastdiv_kernel(const DivJob *jobs, int *bad)
 {
-    *ok = false;
+    const DivJob job = jobs[blockIdx.y];
+    const unsigned stride = gridDim.x * blockDim.x;
+    bool wrong = false;
+    for (unsigned long long i = job.lo + (unsigned long long)(blockIdx.x * blockDim.x + threadIdx.x); i <= job.hi && !wrong; i += stride) {
+        const float y = __uint_as_float((unsigned)i);
+        wrong = fastdiv_rint(y, job.s, job.r) != __float2int_rn(__fdiv_rn(y, job.s));
+    }
+    if (wrong) bad[blockIdx.y] = 1;
+}
+
+struct DivKnown {
+    float s, r;
+    bool ok;
+};
+std::mutex g_div_mu;
+std::vector<DivKnown> g_div_known;  // scales checked before, at most kDivKnown of them
+constexpr size_t kDivKnown = 4096;
+
+}  // namespace
+
+// ---------------------------------------------------------------------------------------
+// the requantisers of a whole network
+// ---------------------------------------------------------------------------------------
+// For every requantising layer: single-fma constants for all its channels, or a verified reciprocal for
+// the three-step division, or neither.  One launch searches the channels of all layers and at most three
+// more check the divisions of the layers the search left over (layer by layer, with an allocation, two
+// copies and a launch each, this was most of the time a policy took to build).
+accerl_status fit_requants(accerl_policy *p, const accerl_layer_desc *layers, int n_layers)
+{
+    if (!p->requant.empty()) return ACCERL_OK;
+    std::vector<LayerRequant> rq(n_layers);
     std::vector<FitJob> jobs;
-    std::vector<int> job_of(n, -1);
-    for (int i = 0; i < n; ++i) {
-        if (k[i] == 0.f && b[i] == 0.f) continue;  // padding column: the code is 0 either way
-        int j = 0;
-        for (; j < (int)jobs.size(); ++j)  // the columns of a multi-pixel row repeat the channels
-            if (memcmp(&jobs[j].k, &k[i], 4) == 0 && memcmp(&jobs[j].b, &b[i], 4) == 0) break;
-        if (j == (int)jobs.size()) {
-            FitJob job;
-            if (!make_job(k[i], b[i], s_out, relu, &job)) return ACCERL_OK;
-            jobs.push_back(job);
+    std::vector<std::vector<int>> job_of(n_layers);
+    for (int i = 0; i < n_layers; ++i) {
+        const accerl_layer_desc &d = layers[i];
+        if (d.kind == ACCERL_MAXPOOL) continue;
+        LayerRequant &q = rq[i];
+        q.k.resize(d.out_c);
+        q.b.resize(d.out_c);
+        for (int c = 0; c < d.out_c; ++c) {
+            volatile float k = d.s_in * d.s_w[c];  // one fp32 rounding, never contracted
+            q.k[c] = k;
+            q.b[c] = d.bias[c];
         }
-        job_of[i] = j;
+        volatile float inv = 1.0f / d.s_out;  // IEEE reciprocal, rounded once
+        q.inv_s_out = inv;
+        if ((d.flags & ACCERL_LOGITS) || (p->flags & (ACCERL_FLAG_TEST_NO_FASTDIV | ACCERL_FLAG_TEST_NO_AFFINE))) continue;
+        std::vector<FitJob> mine(d.out_c);
+        bool all = true;
+        for (int c = 0; c < d.out_c && all; ++c)
+            all = make_job(q.k[c], q.b[c], d.s_out, (d.flags & ACCERL_RELU_OUT) != 0, &mine[c]);
+        if (!all) continue;
+        for (const FitJob &j : mine) {
+            job_of[i].push_back((int)jobs.size());
+            jobs.push_back(j);
+        }
     }
-    std::vector<FitResult> res(jobs.size());
+    struct Device {  // one block of device memory for both steps
+        char *ptr = nullptr;
+        ~Device() { cudaFree(ptr); }
+    } dev;
+    const size_t job_bytes = (jobs.size() * sizeof(FitJob) + 255) / 256 * 256, res_bytes = (jobs.size() * sizeof(FitResult) + 255) / 256 * 256;
+    const size_t div_bytes = ((size_t)n_layers * sizeof(DivJob) + 255) / 256 * 256;
+    ACCERL_CUDA_TRY(cudaMalloc(&dev.ptr, job_bytes + res_bytes + div_bytes + (size_t)n_layers * sizeof(int) + 256));
     if (!jobs.empty()) {
-        FitJob *d_jobs = nullptr;
-        FitResult *d_res = nullptr;
-        ACCERL_CUDA_TRY(cudaMalloc(&d_jobs, jobs.size() * sizeof(FitJob)));
-        cudaError_t e = cudaMalloc(&d_res, jobs.size() * sizeof(FitResult));
-        if (e == cudaSuccess) e = cudaMemcpy(d_jobs, jobs.data(), jobs.size() * sizeof(FitJob), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) {
-            if (relu) fit_affine_kernel<true><<<(unsigned)jobs.size(), kFitThreads>>>(d_jobs, d_res, s_out);
-            else fit_affine_kernel<false><<<(unsigned)jobs.size(), kFitThreads>>>(d_jobs, d_res, s_out);
-            e = cudaGetLastError();
+        std::vector<FitResult> res(jobs.size());
+        ACCERL_CUDA_TRY(cudaMemcpyAsync(dev.ptr, jobs.data(), jobs.size() * sizeof(FitJob), cudaMemcpyHostToDevice, 0));
+        fit_affine_kernel<<<(unsigned)jobs.size(), kFitThreads>>>((const FitJob *)dev.ptr, (FitResult *)(dev.ptr + job_bytes));
+        ACCERL_CUDA_TRY(cudaGetLastError());
+        ACCERL_CUDA_TRY(cudaMemcpy(res.data(), dev.ptr + job_bytes, res.size() * sizeof(FitResult), cudaMemcpyDeviceToHost));
+        for (int i = 0; i < n_layers; ++i) {
+            bool found = !job_of[i].empty();
+            for (int j : job_of[i]) found = found && res[j].found;
+            if (!found) continue;
+            for (size_t c = 0; c < job_of[i].size(); ++c) {
+                rq[i].k[c] = res[job_of[i][c]].k2;
+                rq[i].b[c] = res[job_of[i][c]].b2;
+            }
+            rq[i].affine = rq[i].fast_div = 1;  // a verified division-free requantiser exists
         }
-        if (e == cudaSuccess) e = cudaMemcpy(res.data(), d_res, jobs.size() * sizeof(FitResult), cudaMemcpyDeviceToHost);
-        cudaFree(d_jobs);
-        cudaFree(d_res);
-        if (e != cudaSuccess) {
-            set_error("fit_affine_requant: %s", cudaGetErrorString(e));
-            return ACCERL_ERR_CUDA;
-        }
-        for (const FitResult &r : res)
-            if (!r.found) return ACCERL_OK;
     }
-    k2->assign(n, 0.f);
-    b2->assign(n, 0.f);
-    for (int i = 0; i < n; ++i)
-        if (job_of[i] >= 0) {
-            (*k2)[i] = res[job_of[i]].k2;
-            (*b2)[i] = res[job_of[i]].b2;
+    // fl(1 / s_out) or, where that one fails, one of its two neighbours (the correction step works with any
+    // reciprocal that close; which rare operand patterns round wrongly differs between them)
+    std::lock_guard<std::mutex> lock(g_div_mu);
+    for (int cand = 0; cand < 3; ++cand) {
+        std::vector<DivJob> div;
+        std::vector<int> of;
+        auto settle = [&](int i, float r, bool ok) {
+            if (ok) {
+                rq[i].fast_div = 1;
+                rq[i].inv_s_out = r;
+            }
+        };
+        for (int i = 0; i < n_layers; ++i) {
+            const accerl_layer_desc &d = layers[i];
+            if (d.kind == ACCERL_MAXPOOL || (d.flags & ACCERL_LOGITS) || rq[i].fast_div || (p->flags & ACCERL_FLAG_TEST_NO_FASTDIV)) continue;
+            // scales for which a quotient of the largest |y| (|acc| < 2^31) or a correction term could leave
+            // the normal range are not considered
+            float kmax = 0.f, bmax = 0.f;
+            for (size_t c = 0; c < rq[i].k.size(); ++c) {
+                kmax = std::max(kmax, rq[i].k[c]);
+                bmax = std::max(bmax, std::fabs(rq[i].b[c]));
+            }
+            const double y_max = 2147483648.0 * kmax + bmax;
+            if (!(d.s_out > 1e-25f && d.s_out < 1e25f && y_max < 1e30 && y_max / d.s_out < 1e30)) continue;
+            const float r0 = rq[i].inv_s_out, r = cand == 0 ? r0 : (cand == 1 ? std::nextafter(r0, 2.f * r0) : std::nextafter(r0, 0.f));
+            bool known = false;
+            for (const DivKnown &k : g_div_known)
+                if (k.s == d.s_out && k.r == r) {
+                    settle(i, r, k.ok);
+                    known = true;
+                }
+            if (known) continue;
+            DivJob j;
+            const float lo = 0.4f * d.s_out, hi = 130.f * d.s_out;
+            j.s = d.s_out;
+            j.r = r;
+            memcpy(&j.lo, &lo, 4);
+            memcpy(&j.hi, &hi, 4);
+            div.push_back(j);
+            of.push_back(i);
         }
-    *ok = true;
+        if (div.empty()) continue;
+        char *d_div = dev.ptr + job_bytes + res_bytes;
+        int *d_bad = (int *)(d_div + div_bytes);
+        std::vector<int> bad(div.size());
+        ACCERL_CUDA_TRY(cudaMemcpyAsync(d_div, div.data(), div.size() * sizeof(DivJob), cudaMemcpyHostToDevice, 0));
+        ACCERL_CUDA_TRY(cudaMemsetAsync(d_bad, 0, div.size() * sizeof(int), 0));
+        verify_fastdiv_kernel<<<dim3(148 * 2, (unsigned)div.size()), 256>>>((const DivJob *)d_div, d_bad);
+        ACCERL_CUDA_TRY(cudaGetLastError());
+        ACCERL_CUDA_TRY(cudaMemcpy(bad.data(), d_bad, bad.size() * sizeof(int), cudaMemcpyDeviceToHost));
+        if (g_div_known.size() + div.size() > kDivKnown) g_div_known.clear();
+        for (size_t j = 0; j < div.size(); ++j) {
+            g_div_known.push_back(DivKnown{div[j].s, div[j].r, bad[j] == 0});
+            settle(of[j], div[j].r, bad[j] == 0);
+        }
+    }
+    p->requant = std::move(rq);
     return ACCERL_OK;
 }
 

@@ -279,12 +279,13 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
         if ((long long)p->max_batch * (p->layers[i].in_h + 2) * (p->layers[i].in_w + 2) + 512 >= (1LL << 31))
             return ACCERL_OK;
 
+    accerl_status st;
+    if ((st = fit_requants(p, layers, n_layers)) != ACCERL_OK) return st;
     // The IMPALA stacks run image by image in three kernels of their own (tc_resnet.cu), unless every
     // tensor has to exist; what follows then only places the fully connected layers.
     std::vector<Step> steps;
     bool resident = false;
     int8_t *resident_out = nullptr;
-    accerl_status st;
     if (!keep && (st = build_res_steps(p, layers, n_layers, &resident_out, &steps, &resident)) != ACCERL_OK) return st;
     if (resident)
         for (int i = 0; i < kResLayers; ++i) role[i] = RESIDENT;
@@ -658,14 +659,11 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
                 g.row_off[j] = 0;
                 g.col_off[j] = 128 * j;
             }
-            for (int oc = 0; oc < d.out_c; ++oc)
-                for (int c = 0; c < L.in_c; ++c)
-                    for (int y = 0; y < L.in_h; ++y)
-                        for (int x = 0; x < L.in_w; ++x) {
-                            const int ki = (y * L.in_w + x) * L.in_cp + c;
-                            packed[((size_t)(ki / 128) * n_total + oc) * 128 + ki % 128] =
-                                d.w[(size_t)oc * d.in_c + (c * L.in_h + y) * L.in_w + x];
-                        }
+            for (int oc = 0; oc < d.out_c; ++oc) {  // (rows of K bytes in (y, x, c) order)
+                const int8_t *row = reinterpret_cast<const int8_t *>(L.host_words.data()) + (size_t)oc * K;
+                for (int j = 0; j < g.n_chunks; ++j)
+                    memcpy(&packed[((size_t)j * n_total + oc) * 128], &row[128 * j], std::min(128, K - 128 * j));
+            }
             const bool relu_in = (d.flags & ACCERL_RELU_IN) && !(layers[i - 1].flags & ACCERL_RELU_OUT);
             a_ptr = relu_in ? fin.p_plain_relu : fin.p_plain;
             a_rows_total = p->max_batch;
@@ -757,44 +755,25 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
         g.bias = bs_dev;
         g.s_out = L.s_out;
         g.relu_out = (d.flags & ACCERL_RELU_OUT) != 0;
-        {
-            volatile float inv = 1.0f / L.s_out;
-            g.inv_s_out = inv;
-        }
-        // the single-fma requantiser where every channel has verified constants (searched first: a layer
-        // that has them needs no check of the three-step division)
-        if (!logits && !(p->flags & ACCERL_FLAG_TEST_NO_FASTDIV) && !(p->flags & ACCERL_FLAG_TEST_NO_AFFINE)) {
+        // the single-fma requantiser where every channel has verified constants, else the division
+        const LayerRequant &rq = p->requant[i];
+        g.inv_s_out = rq.inv_s_out;
+        g.fast_div = rq.fast_div;
+        if (rq.affine) {
             const bool repeated = role[i] == TCFIRST || P;  // columns = (pixel of the row, channel)
-            std::vector<float> kh(n_total, 0.f), bh(n_total, 0.f), k2, b2;
+            std::vector<float> k2(n_total, 0.f), b2(n_total, 0.f);
             for (int j = 0; j < n_total; ++j) {
                 const int oc = repeated ? j % d.out_c : j;
                 if (oc >= d.out_c) continue;
-                volatile float k = d.s_in * d.s_w[oc];
-                kh[j] = k;
-                bh[j] = d.bias[oc];
+                k2[j] = rq.k[oc];
+                b2[j] = rq.b[oc];
             }
-            bool ok = false;
-            st = fit_affine_requant(kh.data(), bh.data(), n_total, g.s_out, g.relu_out != 0, &k2, &b2, &ok);
-            if (st != ACCERL_OK) return st;
-            if (ok) {
-                void *kd = nullptr, *bd = nullptr;
-                if ((st = upload_bytes(p, k2.data(), k2.size() * 4, &kd)) != ACCERL_OK) return st;
-                if ((st = upload_bytes(p, b2.data(), b2.size() * 4, &bd)) != ACCERL_OK) return st;
-                g.kscale = (const float *)kd;
-                g.bias = (const float *)bd;
-                g.affine = 1;
-                g.fast_div = 1;  // a verified division-free requantiser exists
-            }
-        }
-        if (!logits && !g.affine) {
-            float kmax = 0.f, bmax = 0.f;
-            for (int c = 0; c < d.out_c; ++c) {
-                kmax = std::max(kmax, d.s_in * d.s_w[c]);
-                bmax = std::max(bmax, fabsf(d.bias[c]));
-            }
-            st = choose_fastdiv(g.s_out, g.relu_out != 0, 2147483648.0f * kmax + bmax,
-                                !(p->flags & ACCERL_FLAG_TEST_NO_FASTDIV), &g.inv_s_out, &g.fast_div);
-            if (st != ACCERL_OK) return st;
+            void *kd = nullptr, *bd = nullptr;
+            if ((st = upload_bytes(p, k2.data(), k2.size() * 4, &kd)) != ACCERL_OK) return st;
+            if ((st = upload_bytes(p, b2.data(), b2.size() * 4, &bd)) != ACCERL_OK) return st;
+            g.kscale = (const float *)kd;
+            g.bias = (const float *)bd;
+            g.affine = 1;
         }
         g.split_cols = (g.n_tile > 128 || (role[i] == TCFIRST && hpool_first) || hp_out) ? 1 : 0;
         // (a multi-pixel layer whose output scale fails the division check keeps its place in the plan:

@@ -4,7 +4,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "epilogue.cuh"
 #include "internal.h"
@@ -187,85 +186,6 @@ cudaError_t launch_ingest_u8_s2d(const uint8_t *obs, const int8_t *lut, int8_t *
 }
 
 // ---------------------------------------------------------------------------------------
-// exhaustive verification of the fast division for one output scale
-// ---------------------------------------------------------------------------------------
-template <bool RELU>
-__global__ void verify_fastdiv_kernel(float s, float r, float y_max, unsigned long long *bad)
-{
-    const unsigned long long total = 1ULL << 32;
-    unsigned long long mine = 0;
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
-        const float y = __uint_as_float((unsigned)i);
-        if (!(fabsf(y) <= y_max)) continue;  // also skips NaN
-        if (fastdiv_code<RELU>(y, s, r) != exact_code(y, s, RELU)) ++mine;
-    }
-    if (mine) atomicAdd(bad, mine);
-}
-
-// Compares fastdiv_code with the defining expression for every float |y| <= y_max.  Results are
-// remembered per (scale, relu, range) so that a scale is checked once per process.
-accerl_status verify_fastdiv(float s_out, float inv_s_out, bool relu, float y_max, bool *ok)
-{
-    struct Key {
-        float s, r, ymax;
-        bool relu, ok;
-    };
-    static std::vector<Key> cache;
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    for (const Key &k : cache)
-        if (k.s == s_out && k.r == inv_s_out && k.relu == relu && k.ymax >= y_max) {
-            *ok = k.ok;
-            return ACCERL_OK;
-        }
-    *ok = false;
-    unsigned long long *bad = nullptr, host = 1;
-    ACCERL_CUDA_TRY(cudaMalloc(&bad, sizeof(*bad)));
-    cudaError_t e = cudaMemset(bad, 0, sizeof(*bad));
-    if (e == cudaSuccess) {
-        if (relu) verify_fastdiv_kernel<true><<<148 * 8, 256>>>(s_out, inv_s_out, y_max, bad);
-        else verify_fastdiv_kernel<false><<<148 * 8, 256>>>(s_out, inv_s_out, y_max, bad);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpy(&host, bad, sizeof(host), cudaMemcpyDeviceToHost);
-    cudaFree(bad);
-    if (e != cudaSuccess) {
-        set_error("verify_fastdiv: %s", cudaGetErrorString(e));
-        return ACCERL_ERR_CUDA;
-    }
-    *ok = host == 0;
-    cache.push_back(Key{s_out, inv_s_out, y_max, relu, *ok});
-    return ACCERL_OK;
-}
-
-// Reciprocal for the three-step division by s_out: fl(1 / s_out) or, where that one fails the
-// exhaustive comparison, one of its two neighbours (the correction step works with any reciprocal
-// that close; which rare operand patterns round wrongly differs between them).  *fast_div = 0 and
-// *inv_s_out = fl(1 / s_out) when none verifies or `allow` is false: the layer then runs the
-// epilogue with the exact fallback near ties, which assumes the correctly rounded reciprocal.
-accerl_status choose_fastdiv(float s_out, bool relu, float y_max, bool allow, float *inv_s_out, int *fast_div)
-{
-    volatile float inv = 1.0f / s_out;  // IEEE reciprocal, rounded once
-    const float r0 = inv;
-    *inv_s_out = r0;
-    *fast_div = 0;
-    if (!allow) return ACCERL_OK;
-    const float cand[3] = {r0, nextafterf(r0, 2.f * r0), nextafterf(r0, 0.f)};
-    for (float r : cand) {
-        bool ok = false;
-        accerl_status st = verify_fastdiv(s_out, r, relu, y_max, &ok);
-        if (st != ACCERL_OK) return st;
-        if (ok) {
-            *inv_s_out = r;
-            *fast_div = 1;
-            return ACCERL_OK;
-        }
-    }
-    return ACCERL_OK;
-}
-
-// ---------------------------------------------------------------------------------------
 // plan
 // ---------------------------------------------------------------------------------------
 
@@ -321,6 +241,7 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
     for (int i = 0; i < n_layers; ++i)
         if ((long long)p->max_batch * p->layers[i].in_h * p->layers[i].in_w + 256 >= (1LL << 31))
             return ACCERL_OK;  // GEMM row indices are 32-bit
+    if (accerl_status st = fit_requants(p, layers, n_layers); st != ACCERL_OK) return st;
     // ---- layouts: a tensor is stored space-to-depth(s) when its reader is a conv of stride s
     for (int i = 0; i < n_layers; ++i)
         p->tensor_s2d[i] = layers[i].kind == ACCERL_CONV2D ? layers[i].stride : 1;
@@ -403,14 +324,11 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
                 g.row_off[j] = 0;
                 g.col_off[j] = 128 * j;
             }
-            for (int oc = 0; oc < d.out_c; ++oc)
-                for (int c = 0; c < L.in_c; ++c)
-                    for (int y = 0; y < L.in_h; ++y)
-                        for (int x = 0; x < L.in_w; ++x) {
-                            const int ki = (y * L.in_w + x) * L.in_cp + c;
-                            packed[((size_t)(ki / 128) * n_total + oc) * 128 + ki % 128] =
-                                d.w[(size_t)oc * d.in_c + (c * L.in_h + y) * L.in_w + x];
-                        }
+            for (int oc = 0; oc < d.out_c; ++oc) {  // (rows of K bytes in (y, x, c) order)
+                const int8_t *row = reinterpret_cast<const int8_t *>(L.host_words.data()) + (size_t)oc * K;
+                for (int j = 0; j < g.n_chunks; ++j)
+                    memcpy(&packed[((size_t)j * n_total + oc) * 128], &row[128 * j], std::min(128, K - 128 * j));
+            }
         }
         g.out_h = L.out_h;
         g.out_w = L.out_w;
@@ -426,47 +344,21 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
         g.bias = L.bias;
         g.s_out = L.s_out;
         g.relu_out = (d.flags & ACCERL_RELU_OUT) != 0;
-        {
-            volatile float inv = 1.0f / L.s_out;  // IEEE reciprocal, rounded once
-            g.inv_s_out = inv;
-        }
-        const bool allow_fastdiv = !(p->flags & ACCERL_FLAG_TEST_NO_FASTDIV);
-        // The single-fma requantiser where every channel has verified constants (searched first: a
-        // layer that has them needs no check of the three-step division, 4.5 ms per output scale).
+        // the single-fma requantiser where every channel has verified constants, else the division
+        const LayerRequant &rq = p->requant[i];
         std::vector<float> k_use(n_total, 0.f), b_use(n_total, 0.f);
-        for (int c = 0; c < d.out_c; ++c) {
-            volatile float k = d.s_in * d.s_w[c];  // one fp32 rounding, never contracted
-            k_use[c] = k;
-            b_use[c] = d.bias[c];
-        }
-        if (!logits && allow_fastdiv && !(p->flags & ACCERL_FLAG_TEST_NO_AFFINE)) {
-            bool ok = false;
-            std::vector<float> k2, b2;
-            accerl_status vs = fit_affine_requant(k_use.data(), b_use.data(), n_total, g.s_out, g.relu_out != 0,
-                                                  &k2, &b2, &ok);
+        std::copy(rq.k.begin(), rq.k.end(), k_use.begin());
+        std::copy(rq.b.begin(), rq.b.end(), b_use.begin());
+        g.inv_s_out = rq.inv_s_out;
+        g.fast_div = rq.fast_div;
+        if (rq.affine) {
+            void *kd = nullptr, *bd = nullptr;
+            accerl_status vs = upload_bytes(p, k_use.data(), k_use.size() * 4, &kd);
+            if (vs == ACCERL_OK) vs = upload_bytes(p, b_use.data(), b_use.size() * 4, &bd);
             if (vs != ACCERL_OK) return vs;
-            if (ok) {
-                void *kd = nullptr, *bd = nullptr;
-                if ((vs = upload_bytes(p, k2.data(), k2.size() * 4, &kd)) != ACCERL_OK) return vs;
-                if ((vs = upload_bytes(p, b2.data(), b2.size() * 4, &bd)) != ACCERL_OK) return vs;
-                g.kscale = (const float *)kd;
-                g.bias = (const float *)bd;
-                g.affine = 1;
-                g.fast_div = 1;  // a verified division-free requantiser exists
-                k_use = k2;
-                b_use = b2;
-            }
-        }
-        if (!logits && !g.affine) {
-            // largest |y| = |fma(acc, k, b)| the layer can produce: |acc| < 2^31
-            float kmax = 0.f, bmax = 0.f;
-            for (int c = 0; c < d.out_c; ++c) {
-                kmax = std::max(kmax, d.s_in * d.s_w[c]);
-                bmax = std::max(bmax, fabsf(d.bias[c]));
-            }
-            accerl_status vs = choose_fastdiv(g.s_out, g.relu_out != 0, 2147483648.0f * kmax + bmax,
-                                              allow_fastdiv, &g.inv_s_out, &g.fast_div);
-            if (vs != ACCERL_OK) return vs;
+            g.kscale = (const float *)kd;
+            g.bias = (const float *)bd;
+            g.affine = 1;
         }
         const char *requant_note = g.affine ? "[single-fma requantiser verified]" : "[3-step divide verified]";
         g.split_cols = g.n_tile >= 128 ? 1 : 0;  // 128 / 256 columns: 32 / 64 per warpgroup

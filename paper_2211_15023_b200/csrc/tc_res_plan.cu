@@ -44,38 +44,19 @@ bool is_impala(const accerl_layer_desc *layers, int n_layers)
     return (layers[kResLayers].flags & ACCERL_RELU_IN) != 0;  // the last block's output is only kept ReLU'd
 }
 
-// the layer's requantiser: single-fma constants where every channel has them, else the verified division
-accerl_status res_layer(accerl_policy *p, const accerl_layer_desc &d, ResLayer *L, bool *ok)
+// a layer's requantiser in the kernels' form
+void res_layer(const accerl_layer_desc &d, const LayerRequant &rq, ResLayer *L)
 {
     memset(L, 0, sizeof(*L));
-    const bool relu = (d.flags & ACCERL_RELU_OUT) != 0;
-    float kmax = 0.f, bmax = 0.f;
     for (int c = 0; c < d.out_c; ++c) {
-        volatile float k = d.s_in * d.s_w[c];  // one fp32 rounding, never contracted
-        L->k[c] = k;
-        L->b[c] = d.bias[c];
+        L->k[c] = rq.k[c];
+        L->b[c] = rq.b[c];
         if (d.skip_from >= 0) L->mul[c] = (uint32_t)d.skip_mul[c] << (16 * (c & 1));
-        kmax = std::max(kmax, L->k[c]);
-        bmax = std::max(bmax, fabsf(L->b[c]));
     }
     L->s_out = d.s_out;
-    L->relu = relu;
-    if (!(p->flags & ACCERL_FLAG_TEST_NO_AFFINE)) {
-        bool fit = false;
-        std::vector<float> k2, b2;
-        accerl_status st = fit_affine_requant(L->k, L->b, d.out_c, d.s_out, relu, &k2, &b2, &fit);
-        if (st != ACCERL_OK) return st;
-        if (fit) {
-            std::copy(k2.begin(), k2.end(), L->k);
-            std::copy(b2.begin(), b2.end(), L->b);
-            L->affine = 1;
-            return ACCERL_OK;
-        }
-    }
-    int fast = 0;
-    accerl_status st = choose_fastdiv(d.s_out, relu, 2147483648.0f * kmax + bmax, true, &L->inv_s_out, &fast);
-    if (!fast) *ok = false;
-    return st;
+    L->inv_s_out = rq.inv_s_out;
+    L->affine = rq.affine;
+    L->relu = (d.flags & ACCERL_RELU_OUT) != 0;
 }
 
 // byte of K position kk of column n inside a K step's [columns][32 bytes] block, 32-byte swizzle
@@ -96,13 +77,11 @@ accerl_status build_res_steps(accerl_policy *p, const accerl_layer_desc *layers,
         !(p->ingest_shift1 || p->ingest_arith == 1) || !is_impala(layers, n_layers))
         return ACCERL_OK;
     ResLayer L[kResLayers];
-    bool ok = true;
-    for (int i = 0; i < kResLayers && ok; ++i)
+    for (int i = 0; i < kResLayers; ++i)
         if (layers[i].kind == ACCERL_CONV2D) {
-            accerl_status st = res_layer(p, layers[i], &L[i], &ok);
-            if (st != ACCERL_OK) return st;
+            if (!p->requant[i].fast_div) return ACCERL_OK;
+            res_layer(layers[i], p->requant[i], &L[i]);
         }
-    if (!ok) return ACCERL_OK;
 
     // ---- weights
     std::vector<int8_t> w0(kResFirstWeights, 0), w1(kRes1Weights, 0), w2(kRes2Weights, 0);
