@@ -357,6 +357,17 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             ACCERL_CUDA_TRY(conv_rows_launch(cs.map_a, cs.map_b, cs.prm, B, p->sm_count, st));
             break;
         }
+        case Step::ATARI: {
+            if ((uintptr_t)obs_dev & 15) {
+                set_error("act: obs_dev must be 16-byte aligned");
+                return ACCERL_ERR_INVALID_ARG;
+            }
+            AtariParams prm = p->atari;
+            prm.obs = (const uint8_t *)obs_dev;
+            prm.batch = B;
+            ACCERL_CUDA_TRY(atari_launch(prm, p->sm_count, st));
+            break;
+        }
         case Step::RES_FIRST: {
             if ((uintptr_t)obs_dev & 15) {
                 set_error("act: obs_dev must be 16-byte aligned");

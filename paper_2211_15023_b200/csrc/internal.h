@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "accerl.h"
+#include "tc_atari.h"
 #include "tc_conv.h"
 #include "tc_conv1.h"
 #include "tc_gemm.h"
@@ -59,7 +60,7 @@ struct LayerPlan {
 struct Step {
     enum Kind { INGEST, CONV_GENERIC, FC_GENERIC, POOL_GENERIC, SAMPLE, INGEST_S2D, TC_GEMM, MLP_FUSED,
                 INGEST_NHWC4, POOL_DUAL, INGEST_PAD4, FC_SAMPLE, CONV1_FRAMES, CONV_ROWS, RES_FIRST,
-                RES_STACK1, RES_STACK23 } kind;
+                RES_STACK1, RES_STACK23, ATARI } kind;
     int layer = -1;
     int tc = -1;  // index into accerl_policy::tc_steps (TC_GEMM), ::pools (POOL_DUAL) or ::conv_rows (CONV_ROWS)
     std::string kernel, covers;
@@ -166,6 +167,7 @@ struct accerl_policy {
     std::vector<accerl::ConvRowsStep> conv_rows;
     accerl::Conv1Params conv1 = {};       // used by a Step::CONV1_FRAMES launch
     alignas(64) unsigned char conv1_map_b[128] = {};
+    accerl::AtariParams atari = {};        // used by a Step::ATARI launch
     // the image-resident kernels of the residual network (Step::RES_*)
     accerl::ResFirstParams res_first = {};
     accerl::ResStack1Params res_stack1 = {};

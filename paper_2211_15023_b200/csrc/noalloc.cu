@@ -77,7 +77,7 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
     for (const Step &s : p->steps) {
         switch (s.kind) {
         case Step::RES_FIRST: resident = true; break;
-        case Step::RES_STACK1: case Step::RES_STACK23: case Step::MLP_FUSED: case Step::CONV1_FRAMES: case Step::CONV_ROWS:
+        case Step::RES_STACK1: case Step::RES_STACK23: case Step::MLP_FUSED: case Step::CONV1_FRAMES: case Step::CONV_ROWS: case Step::ATARI:
         case Step::FC_SAMPLE: case Step::SAMPLE: break;
         case Step::TC_GEMM: {
             const TcGemmParams &g = p->tc_steps[s.tc].prm;  // no padded layouts, no residual or second output
@@ -152,6 +152,8 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
             move(c.prm.out);
         } else if (s.kind == Step::CONV1_FRAMES) {
             move(q->conv1.out);
+        } else if (s.kind == Step::ATARI) {
+            move(q->atari.out);
         } else if (s.kind == Step::FC_SAMPLE) {
             move(q->fc_sample.x);
         } else if (s.kind == Step::RES_FIRST) {

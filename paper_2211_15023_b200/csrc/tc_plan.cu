@@ -208,6 +208,92 @@ bool conv_fits(const accerl_layer_desc &d)
     return true;
 }
 
+// The Atari conv stack as one launch (tc_atari.cu): handles for up to this many states.  Above, the
+// launches per layer are faster: their tiles span images, a third of that kernel's tensor work is padding
+// rows.  (us per step, per layer / one launch: 32 / 64 / 64 channels 26.4 / 21.4 at 160 states, 34.4 / 32.4 at
+// 700, 43.5 / 46.2 at 1237; 16 / 32 / 32 channels 25.5 / 17.4, 37.1 / 33.1 at 1237, 70.3 / 79.3 at 4096.)
+constexpr int kAtariMaxWide = 800, kAtariMaxNarrow = 2048;
+
+// byte offset of byte kk of row n of an operand with rb-byte rows under the rb-byte swizzle
+size_t swizzled(int n, int kk, int rb)
+{
+    const int c = kk >> 4, x = rb == 128 ? (n & 7) : rb == 64 ? ((n >> 1) & 3) : ((n >> 2) & 1);
+    return (size_t)n * rb + (size_t)((c ^ x) << 4) + (kk & 15);
+}
+
+// Do layers 0 .. 2 have the shape of that kernel?  Then fills its parameters and its step.
+accerl_status build_atari_step(accerl_policy *p, const accerl_layer_desc *layers, int n_layers, Step *step, bool *used)
+{
+    *used = false;
+    if (n_layers < 5 || p->in_c != 4 || p->in_h != 84 || p->in_w != 84 || p->max_batch > (layers[0].out_c == 32 ? kAtariMaxWide : kAtariMaxNarrow) || unfuse_for_taps(p) ||
+        !(p->ingest_shift1 || p->ingest_arith == 1))
+        return ACCERL_OK;
+    const bool wide = layers[0].out_c == 32;
+    const int c[4] = {4, wide ? 32 : 16, wide ? 64 : 32, wide ? 64 : 32}, k[3] = {8, 4, 3}, stride[3] = {4, 2, 1};
+    for (int i = 0; i < 3; ++i) {
+        const accerl_layer_desc &d = layers[i];
+        if (d.kind != ACCERL_CONV2D || d.in_c != c[i] || d.out_c != c[i + 1] || d.kh != k[i] || d.stride != stride[i] || d.pad != 0 ||
+            d.skip_from >= 0 || !p->requant[i].fast_div)
+            return ACCERL_OK;
+    }
+    if (layers[3].kind != ACCERL_FC) return ACCERL_OK;
+    AtariParams &q = p->atari;
+    memset(&q, 0, sizeof(q));
+    std::vector<int8_t> w(wide ? kAtariWeightsWide : kAtariWeightsNarrow, 0);
+    size_t at = 0;
+    for (int i = 0; i < 3; ++i) {
+        const accerl_layer_desc &d = layers[i];
+        const int s = d.stride, t = d.kh / s, rb = s * s * d.in_c;
+        for (int by = 0; by < t; ++by)
+            for (int bx = 0; bx < t; ++bx, at += (size_t)d.out_c * rb)
+                for (int oc = 0; oc < d.out_c; ++oc)
+                    for (int ic = 0; ic < d.in_c; ++ic)
+                        for (int dy = 0; dy < s; ++dy)
+                            for (int dx = 0; dx < s; ++dx) {
+                                // K: (channel, dy, dx) as the bytes lie in a frame, else (dy, dx, channel)
+                                const int kk = i == 0 ? ic * 16 + dy * 4 + dx : (dy * s + dx) * d.in_c + ic;
+                                w[at + swizzled(oc, kk, rb)] = d.w[((oc * d.in_c + ic) * d.kh + s * by + dy) * d.kw + s * bx + dx];
+                            }
+        const LayerRequant &rq = p->requant[i];
+        AtariLayer &L = q.layer[i];
+        std::copy(rq.k.begin(), rq.k.end(), L.k);
+        std::copy(rq.b.begin(), rq.b.end(), L.b);
+        L.s_out = d.s_out;
+        L.inv_s_out = rq.inv_s_out;
+        L.affine = rq.affine;
+        L.relu = (d.flags & ACCERL_RELU_OUT) != 0;
+    }
+    void *w_dev = nullptr;
+    accerl_status st = upload_bytes(p, w.data(), w.size(), &w_dev);
+    if (st != ACCERL_OK) return st;
+    q.w = (const uint8_t *)w_dev;
+    q.out = p->bufs[p->layers[2].out_buf].ptr;
+    if (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) {
+        q.tap1 = p->bufs[p->layers[0].out_buf].ptr;
+        q.tap2 = p->bufs[p->layers[1].out_buf].ptr;
+    }
+    q.wide = wide;
+    q.ingest_mode = 0;
+    for (unsigned u = 0; u < 256; ++u)
+        if (((unsigned long long)u * p->ingest_mul + p->ingest_add) >> 24 > 127) q.ingest_mode = 1;
+    if (p->ingest_shift1) q.ingest_mode = 2;
+    q.ingest_mul = p->ingest_mul;
+    q.ingest_add = p->ingest_add;
+    q.status = p->status_word;
+    step->kind = Step::ATARI;
+    step->kernel = "atari_kernel";
+    bool division = false;
+    for (int i = 0; i < 3; ++i) {
+        if (p->requant[i].affine) step->kernel += "[single-fma requantiser verified]";
+        else division = true;
+    }
+    step->kernel += std::string(division ? "[3-step divide verified]" : "") + "[frames quantised inside]";
+    step->covers = "ingest+layers 0-2";
+    p->tap_missing[0] = 1;  // no quantised input tensor exists
+    *used = true;
+    return ACCERL_OK;
+}
+
 }  // namespace
 
 accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, int n_layers,
@@ -255,8 +341,12 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
                                                         : "ingest_u8_s2d_any_kernel";
     s0.covers = "ingest";
     steps.push_back(s0);
+    bool atari = false;
+    Step convs;
+    if (accerl_status st = build_atari_step(p, layers, n_layers, &convs, &atari); st != ACCERL_OK) return st;
+    if (atari) steps.assign(1, convs);
 
-    for (int i = 0; i < n_layers; ++i) {
+    for (int i = atari ? 3 : 0; i < n_layers; ++i) {
         const accerl_layer_desc &d = layers[i];
         const LayerPlan &L = p->layers[i];
         if (fc_sample_fits(p, layers, n_layers, i)) {  // the last layer runs fused with the sampler

@@ -37,6 +37,7 @@
 
 #include "epilogue.cuh"
 #include "internal.h"
+#include "tc_image.cuh"
 #include "tc_ptx.cuh"
 #include "tc_resnet.h"
 
@@ -47,13 +48,6 @@ namespace {
 constexpr int kMaxCtx = 3;  // images in flight per CTA
 constexpr int kMaxSlots = 5;
 
-
-// the waits of these kernels are short and on the critical path of their context: poll (try_wait itself
-// suspends the warp for a while) before backing off
-__device__ __forceinline__ void res_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status, int code)
-{
-    mbar_wait_limited(bar, parity, abort_flag, status, code, 2048, kWaitLimitPolls);
-}
 
 struct __align__(8) ResBars {
     uint64_t w_ready;
@@ -66,21 +60,6 @@ struct __align__(8) ResBars {
 
 // byte offset of 16-byte half `c` of 32-byte row `row` under the 32-byte swizzle
 __device__ __forceinline__ uint32_t row_off(int row, int c) { return (uint32_t)(row * 32 + ((c ^ ((row >> 2) & 1)) << 4)); }
-
-__device__ __forceinline__ void sts16(uint32_t addr, uint4 v)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-__device__ __forceinline__ uint4 lds16(uint32_t addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint4 relu16(uint4 v)
-{
-    return make_uint4(relu_bytes(v.x), relu_bytes(v.y), relu_bytes(v.z), relu_bytes(v.w));
-}
 
 // all warps of a context's epilogue
 template <int THREADS>
@@ -172,26 +151,11 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 v)
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-template <int I>
-using OpIndex = std::integral_constant<int, I>;
-
 // descriptors: constant upper words; the lower word is (address >> 4) | flags
 constexpr uint32_t kDescSw32Hi = (256u >> 4) | (1u << 14) | (6u << 29);   // 32-byte rows, 32-byte swizzle
 constexpr uint32_t kDescSw32Lo = 1u << 16;
 constexpr uint32_t kDescFlatHi = (128u >> 4) | (1u << 14);                // 16-byte rows, no swizzle: 8-row groups 128 bytes apart,
 constexpr uint32_t kDescFlatLo = (16u >> 4) << 16;                        // the second half of a K step is the next row
-__host__ __device__ constexpr uint32_t idesc_for(int n)
-{
-    return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-__device__ __forceinline__ uint64_t desc(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
-
 // what every kernel of this file does first: barriers, tensor memory, weights; returns the tensor-memory base
 template <int EPI_WARPS>
 __device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, int buffer_bytes, uint8_t *w_smem,
@@ -284,13 +248,13 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t a0 = ((smem_u32(bufs) + (uint32_t)ctx * (kFrameBytes + kHpBytes)) >> 4) | kDescFlatLo;
         const uint32_t b0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
-        res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, it = 0;
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step, ++it) {
-            res_wait(ready, it & 1, abort_flag, p.status, 8);
+            image_wait(ready, it & 1, abort_flag, p.status, 8);
             fence_after();
             for (int t = 0; t < kFirstTiles; ++t) {
-                res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                image_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                 fence_after();
                 if (elect_one()) {
                     const uint32_t d = tmem + (uint32_t)ctx * 256 + slot * 80;
@@ -352,7 +316,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
         for (; n < p.batch; n += step, seq0 += kFirstTiles) {
             for (int t = wg; t < kFirstTiles; t += kFirstWg) {
                 const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kFirstSlots;
-                res_wait(full0 + 8 * slot, (seq / kFirstSlots) & 1, abort_flag, p.status, 16);
+                image_wait(full0 + 8 * slot, (seq / kFirstSlots) & 1, abort_flag, p.status, 16);
                 fence_after();
                 const int m = t * 128 + q * 32 + lane;
                 const int y = m / 22, X = m - y * 22, R = y * 21 + X;
@@ -435,18 +399,18 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)(ctx * 2) * kS1Buf) >> 4) | kDescSw32Lo, h0 = r0 + (kS1Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
-        res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, rdy = 0;
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
             for (int op = 0; op < kS1Ops; ++op) {
                 if (op < 5) {  // (the second half of the last conv reads what the first half read)
-                    res_wait(ready, rdy, abort_flag, p.status, 8);
+                    image_wait(ready, rdy, abort_flag, p.status, 8);
                     rdy ^= 1;
                     fence_after();
                 }
                 const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0, b_op = w0 + (uint32_t)op * (6 * 1024 >> 4);
                 for (int t = 0; t < kS1Tiles; ++t) {
-                    res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                    image_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
                         const uint32_t d = tmem + (uint32_t)ctx * kS1Cols + slot * 32, a = a_op + (uint32_t)t * (128 * 2);
@@ -488,7 +452,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
         uint32_t seq0 = 0, it = 0;  // tiles handed over before this layer, images
         for (; n < p.batch; n += step, ++it) {
             // the image: x to tensor memory, ReLU(x) in place for the first conv
-            res_wait(land_bar, it & 1, abort_flag, p.status, 1);
+            image_wait(land_bar, it & 1, abort_flag, p.status, 1);
             for (int t = wg; t < kS1Tiles; t += kS1Wg) {
                 const int m = t * 128 + row, r = m + 21;
                 const bool v[2] = {m < 861, ((second >> t) & 1) != 0};
@@ -514,7 +478,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                     const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS1Slots;
                     const int m = t * 128 + row, r = m + 21;
                     const bool v[2] = {m < 861, ((second >> t) & 1) != 0};
-                    res_wait(full0 + 8 * slot, (seq / kS1Slots) & 1, abort_flag, p.status, 16);
+                    image_wait(full0 + 8 * slot, (seq / kS1Slots) & 1, abort_flag, p.status, 16);
                     fence_after();
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {  // the row's two pixels
@@ -625,18 +589,18 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
                        r3 = h0 + (kS2Buf >> 4), h3 = r3 + (kS3Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo, d0 = tmem + (uint32_t)ctx * kS2Cols;
-        res_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
+        image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t rdy = 0, slot = 0, phase = 0, k3 = 0;  // k3: layers done at 9 x 9
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
             for (int op = 0; op < kS2Ops; ++op) {
-                res_wait(ready, rdy, abort_flag, p.status, 8);
+                image_wait(ready, rdy, abort_flag, p.status, 8);
                 rdy ^= 1;
                 fence_after();
                 const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
                 if (op < 5) {
                     const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
                     for (int t = 0; t < kS2Tiles; ++t) {
-                        res_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
+                        image_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                         fence_after();
                         if (elect_one()) {
                             const uint32_t a = a_op + (uint32_t)t * (128 * 2);
@@ -651,7 +615,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                     }
                 } else {
                     const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3;
-                    res_wait(empty0 + 8 * kS2Slot3, (k3 & 1) ^ 1, abort_flag, p.status, 4);
+                    image_wait(empty0 + 8 * kS2Slot3, (k3 & 1) ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
 #pragma unroll
@@ -695,7 +659,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
         if (tid == 0 && n < p.batch) fetch(n);
         uint32_t seq0 = 0, k3 = 0, it = 0;
         for (; n < p.batch; n += step, ++it) {
-            res_wait(land_bar, it & 1, abort_flag, p.status, 1);
+            image_wait(land_bar, it & 1, abort_flag, p.status, 1);
             for (int t = wg; t < kS2Tiles; t += kS2Wg)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -717,7 +681,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                 for (int t = wg; t < kS2Tiles; t += kS2Wg) {
                     const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS2Slots;
                     const bool v = (inside >> t) & 1;
-                    res_wait(full0 + 8 * slot, (seq / kS2Slots) & 1, abort_flag, p.status, 16);
+                    image_wait(full0 + 8 * slot, (seq / kS2Slots) & 1, abort_flag, p.status, 16);
                     fence_after();
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -775,7 +739,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                 constexpr int op = decltype(op_c)::value, half = decltype(half_c)::value;
                 constexpr bool skip = op == 6 || op == 8;
                 const ResLayer &L = p.layer[op];
-                res_wait(full0 + 8 * kS2Slot3, k3 & 1, abort_flag, p.status, 16);
+                image_wait(full0 + 8 * kS2Slot3, k3 & 1, abort_flag, p.status, 16);
                 fence_after();
                 int a[16];
                 tmem_ld16(tctx + kS2Slot3 * 32 + 16 * half, a);
