@@ -413,6 +413,10 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             ACCERL_CUDA_TRY(launch_mlp_fused(p, (const float *)obs_dev, uniforms_dev, B, logits_dev,
                                              actions_dev, logp_dev, value_dev, entropy_dev, st));
             break;
+        case Step::FC_HEAD:
+            ACCERL_CUDA_TRY(launch_fc_head(p->fc_head, p->fc_sample, uniforms_dev, B, logits_dev, actions_dev, logp_dev,
+                                           value_dev, entropy_dev, p->sm_count, st));
+            break;
         case Step::FC_SAMPLE:
             ACCERL_CUDA_TRY(launch_fc_sample(p->fc_sample, uniforms_dev, B, logits_dev, actions_dev, logp_dev,
                                              value_dev, entropy_dev, p->sm_count, st));

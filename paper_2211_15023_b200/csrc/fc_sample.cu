@@ -5,6 +5,7 @@
 // accumulates action j with dp4a from weights held in shared memory as [K/4][32] words, and the
 // logits never leave registers before they are sampled (they are still written out: they are an
 // output of the step).
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -157,6 +158,142 @@ fc_sample_kernel(const FcSampleParams q, const float *__restrict__ u, int B,
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// hidden fully connected layer, last layer and sampler in one launch, for small batches
+// ---------------------------------------------------------------------------------------
+// A hidden layer of 256 or 512 outputs on up to a few hundred states is a stream of weights (1.6 MB for
+// the Nature-CNN) against hardly any rows: as 128-row tiles of the big tensor pipe it occupies 32 SMs and
+// took about 10 us, and the last layer with the sampler another launch after it.  Here a cluster of eight
+// CTAs owns 16 or 32 states; CTA c computes columns c * N / 8 .. of the hidden layer on warp-level int8
+// tensor instructions, sixteen warps with a share of K each (operands straight from L2 to registers, in
+// 64-byte pieces of K so that every load instruction moves whole sectors), adds the partial sums through
+// shared memory, requantises, and hands every state's codes to the CTA that finishes it: two or four
+// states each, last layer by dp4a, softmax, draw.  The weights of the last layer are in registers before
+// the previous launch is done.
+constexpr int kHeadWarps = 16, kHeadCluster = 8;
+
+__device__ __forceinline__ void head_mma(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// MT: 16-state tiles of a cluster; NT: 8-column tiles of a CTA (N = 64 * NT hidden outputs)
+template <int MT, int NT>
+__global__ void __launch_bounds__(32 * kHeadWarps, 1)
+fc_hidden_fc_sample_kernel(const __grid_constant__ FcHeadParams h, const __grid_constant__ FcSampleParams q, const float *__restrict__ u, int B,
+                           float *__restrict__ logits, int32_t *__restrict__ actions, float *__restrict__ logp,
+                           float *__restrict__ value, float *__restrict__ entropy)
+{
+    constexpr int kRows = 16 * MT, kCols = 8 * NT, kN = kCols * kHeadCluster;
+    constexpr int kOwn = kRows / kHeadCluster;          // states a CTA finishes
+    constexpr int kSlices = kHeadWarps / kOwn;          // warps that share one of them
+    constexpr int kWords = kN / 4 / kSlices;            // words of its codes each takes
+    extern __shared__ __align__(16) int32_t head_smem[];  // partial sums [warp][kRows][kCols]
+    __shared__ __align__(16) uint32_t codes[kOwn][kN / 4];
+    __shared__ int s_z[kOwn][kSlices][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    const int row0 = (int)(blockIdx.x / kHeadCluster) * kRows;
+
+    // what does not depend on the previous launch
+    const int own = warp / kSlices, slice = warp % kSlices;
+    int w2[kWords];
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) w2[k] = __ldg(q.w + (slice * kWords + k) * 32 + lane);
+    const bool has_col = lane < q.n_out;
+    const float ks2 = has_col ? q.kscale[lane] : 0.f, bs2 = has_col ? q.bias[lane] : 0.f;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // ---- hidden layer: this warp's pieces of K
+    int acc[MT][NT][4] = {};
+    const int8_t *xr[2 * MT];
+#pragma unroll
+    for (int m = 0; m < 2 * MT; ++m) xr[m] = h.x + (long long)min(row0 + 8 * m + g, B - 1) * h.K + 16 * t;
+    const uint4 *wp = h.w + (size_t)rank * NT * 32 + lane;  // [piece][N / 8][lane]
+#pragma unroll 2
+    for (int p = warp; p < h.pieces; p += kHeadWarps) {
+        uint4 a[2 * MT], b[NT];
+        const bool in = 64 * p + 16 * t < h.K;  // (K is a multiple of 16; the weights are padded with zeros)
+#pragma unroll
+        for (int m = 0; m < 2 * MT; ++m) a[m] = in ? __ldcg(reinterpret_cast<const uint4 *>(xr[m] + 64 * p)) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int n = 0; n < NT; ++n) b[n] = __ldg(wp + ((size_t)p * (NT * kHeadCluster) + n) * 32);
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                head_mma(acc[m][n], a[2 * m].x, a[2 * m + 1].x, a[2 * m].y, a[2 * m + 1].y, b[n].x, b[n].y);
+                head_mma(acc[m][n], a[2 * m].z, a[2 * m + 1].z, a[2 * m].w, a[2 * m + 1].w, b[n].z, b[n].w);
+            }
+    }
+    // (no early trigger: the next launch waits for this one as a whole)
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                *reinterpret_cast<int2 *>(head_smem + (warp * kRows + 16 * m + 8 * r + g) * kCols + 8 * n + 2 * t) =
+                    make_int2(acc[m][n][2 * r], acc[m][n][2 * r + 1]);
+    cooperative_groups::this_cluster().sync();  // also: every CTA of the cluster has started, its shared memory may be written
+    for (int i = threadIdx.x; i < kRows * kCols / 2; i += 32 * kHeadWarps) {
+        const int r = i / (kCols / 2), c = 2 * (i - r * (kCols / 2));
+        int2 s = make_int2(0, 0);
+#pragma unroll
+        for (int w = 0; w < kHeadWarps; ++w) {
+            const int2 v = *reinterpret_cast<const int2 *>(head_smem + (w * kRows + r) * kCols + c);
+            s.x += v.x;
+            s.y += v.y;
+        }
+        const int col = rank * kCols + c;
+        const float2 k = __ldg(reinterpret_cast<const float2 *>(h.kscale + col)), b = __ldg(reinterpret_cast<const float2 *>(h.bias + col));
+        uint32_t code = 0;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            code |= (uint32_t)(uint8_t)requant(epilogue_float(j ? s.y : s.x, j ? k.y : k.x, j ? b.y : b.x, h.relu != 0), h.s_out) << (8 * j);
+        uint16_t *mine = reinterpret_cast<uint16_t *>(&codes[r % kOwn][0]) + col / 2;
+        *cooperative_groups::this_cluster().map_shared_rank(mine, (unsigned)(r / kOwn)) = (uint16_t)code;
+        if (h.tap && row0 + r < B) *reinterpret_cast<uint16_t *>(h.tap + (long long)(row0 + r) * kN + col) = (uint16_t)code;
+    }
+    cooperative_groups::this_cluster().sync();
+    // ---- last layer: lane = column, a slice of K per warp
+    {
+        int z = 0;
+        const uint4 *x = reinterpret_cast<const uint4 *>(&codes[own][slice * kWords]);
+#pragma unroll
+        for (int k = 0; k < kWords / 4; ++k) {
+            const uint4 v = x[k];
+            z = __dp4a((int)v.x, w2[4 * k], z);
+            z = __dp4a((int)v.y, w2[4 * k + 1], z);
+            z = __dp4a((int)v.z, w2[4 * k + 2], z);
+            z = __dp4a((int)v.w, w2[4 * k + 3], z);
+        }
+        s_z[own][slice][lane] = z;
+    }
+    __syncthreads();
+    const int row = row0 + rank * kOwn + own;
+    if (slice != 0 || row >= B) return;
+    int zi = 0;
+#pragma unroll
+    for (int s = 0; s < kSlices; ++s) zi += s_z[own][s][lane];
+    const float z = epilogue_float(zi, ks2, bs2, false);
+    const int A = q.n_actions;
+    const bool live = lane < A;
+    if (live) logits[(long long)row * A + lane] = z;
+    if (value && lane == A && A < q.n_out) value[row] = z;
+    int a;
+    float lpa, hh = 0.f;
+    if (entropy) warp_sample<true>(z, live, u[row], A, lane, a, lpa, hh);
+    else warp_sample<false>(z, live, u[row], A, lane, a, lpa, hh);
+    if (lane == 0) {
+        actions[row] = a;
+        logp[row] = lpa;
+        if (entropy) entropy[row] = hh;
+    }
+}
+
 }  // namespace
 
 // Can layer i (the last one) run fused with the sampler?  Its input must be a plain [B][K] int8
@@ -201,6 +338,81 @@ accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int 
     out->kernel = "fc_sample_kernel";
     out->covers = "layer " + std::to_string(layer) + "+sample";
     return ACCERL_OK;
+}
+
+// Do the hidden layer `i` and the last one behind it run as that launch?  Handles for more states stay
+// with the two launches, whose 128-row tiles read the weights less often (us per step, two launches /
+// one: 512 outputs of 3136 inputs 21.4 / 16.0 at 160 states, 27.3 / 26.9 at 450, 32.5 / 42.0 at 700; 256 of
+// 1568 17.1 / 11.2, 20.4 / 16.9, 24.0 / 24.6).
+bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i)
+{
+    if (i != n_layers - 2 || i < 1 || unfuse_for_taps(p) || p->max_batch > (layers[i].out_c == 512 ? kFcHeadMaxWide : kFcHeadMaxNarrow) || !fc_sample_fits(p, layers, n_layers, i + 1))
+        return false;
+    const accerl_layer_desc &d = layers[i];
+    const LayerPlan &L = p->layers[i];
+    return d.kind == ACCERL_FC && (d.out_c == 256 || d.out_c == 512) && L.in_cp == L.in_c && (L.in_h * L.in_w * L.in_cp) % 16 == 0;
+}
+
+// x: the hidden layer's input rows; its weights in (y, x, c) order are L.host_words
+accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out)
+{
+    const accerl_layer_desc &d = layers[i];
+    const LayerPlan &L = p->layers[i];
+    const int K = L.in_h * L.in_w * L.in_cp, N = d.out_c, pieces = (K + 63) / 64;
+    // [piece][column / 8][lane 4 g + t]: bytes 16 t .. 16 t + 15 of the piece, column g
+    std::vector<int8_t> w((size_t)pieces * N * 64, 0);
+    const int8_t *rows = reinterpret_cast<const int8_t *>(L.host_words.data());
+    for (int o = 0; o < N; ++o)
+        for (int k = 0; k < K; k += 16)
+            memcpy(&w[(((size_t)(k / 64) * (N / 8) + o / 8) * 32 + 4 * (o % 8) + (k % 64) / 16) * 16], rows + (size_t)o * K + k, 16);
+    void *dev = nullptr;
+    accerl_status st = upload_bytes(p, w.data(), w.size(), &dev);
+    if (st != ACCERL_OK) return st;
+    FcHeadParams &h = p->fc_head;
+    h.x = x;
+    h.w = (const uint4 *)dev;
+    h.K = K;
+    h.pieces = pieces;
+    h.N = N;
+    h.kscale = L.kscale;
+    h.bias = L.bias;
+    h.s_out = L.s_out;
+    h.relu = (d.flags & ACCERL_RELU_OUT) != 0;
+    h.tap = (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) ? p->bufs[L.out_buf].ptr : nullptr;
+    Step last;
+    if ((st = build_fc_sample(p, layers[i + 1], i + 1, nullptr, N, &last)) != ACCERL_OK) return st;
+    out->kind = Step::FC_HEAD;
+    out->kernel = "fc_hidden_fc_sample_kernel";
+    out->covers = "layers " + std::to_string(i) + "-" + std::to_string(i + 1) + "+sample";
+    return ACCERL_OK;
+}
+
+cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const float *u, int B, float *logits,
+                           int32_t *actions, float *logp, float *value, float *entropy, int sm_count, cudaStream_t st)
+{
+    auto go = [&](auto kernel, int rows) -> cudaError_t {
+        const size_t smem = sizeof(int) * (size_t)kHeadWarps * rows * (h.N / kHeadCluster);
+        cudaError_t e = allow_smem((const void *)kernel, smem);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((B + rows - 1) / rows * kHeadCluster));
+        cfg.blockDim = dim3(32 * kHeadWarps);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = kHeadCluster;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        return cudaLaunchKernelEx(&cfg, kernel, h, q, u, B, logits, actions, logp, value, entropy);
+    };
+    // 16 states per cluster while their clusters fit the chip once
+    const bool two = (B + 15) / 16 * kHeadCluster > sm_count;
+    if (h.N == 512) return two ? go(fc_hidden_fc_sample_kernel<2, 8>, 32) : go(fc_hidden_fc_sample_kernel<1, 8>, 16);
+    return two ? go(fc_hidden_fc_sample_kernel<2, 4>, 32) : go(fc_hidden_fc_sample_kernel<1, 4>, 16);
 }
 
 cudaError_t launch_fc_sample(const FcSampleParams &q, const float *u, int B, float *logits,

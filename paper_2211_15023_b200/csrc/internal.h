@@ -60,7 +60,7 @@ struct LayerPlan {
 struct Step {
     enum Kind { INGEST, CONV_GENERIC, FC_GENERIC, POOL_GENERIC, SAMPLE, INGEST_S2D, TC_GEMM, MLP_FUSED,
                 INGEST_NHWC4, POOL_DUAL, INGEST_PAD4, FC_SAMPLE, CONV1_FRAMES, CONV_ROWS, RES_FIRST,
-                RES_STACK1, RES_STACK23, ATARI } kind;
+                RES_STACK1, RES_STACK23, ATARI, FC_HEAD } kind;
     int layer = -1;
     int tc = -1;  // index into accerl_policy::tc_steps (TC_GEMM), ::pools (POOL_DUAL) or ::conv_rows (CONV_ROWS)
     std::string kernel, covers;
@@ -101,6 +101,17 @@ struct FcSampleParams {
     const int32_t *w;  // [k4][32] words, lane = output column
     const float *kscale, *bias;
 };
+
+// a hidden FC layer of 256 or 512 outputs in the same launch as that (fc_sample.cu)
+struct FcHeadParams {
+    const int8_t *x;  // [B][K] int8 input rows
+    const uint4 *w;   // [pieces][N / 8][32 lanes] operands of 64 K bytes
+    int K, pieces, N, relu;
+    const float *kscale, *bias;
+    float s_out;
+    int8_t *tap;      // parity tap of its output, or null
+};
+constexpr int kFcHeadMaxWide = 448, kFcHeadMaxNarrow = 640;  // states, for 512 and 256 outputs
 
 // max-pool that writes a plain NHWC output and / or a padded-border one (tc_mixed_plan.cu)
 struct PoolOut {  // one stored form of the pooled tensor
@@ -177,7 +188,8 @@ struct accerl_policy {
     std::vector<accerl::TapDesc> taps;    // per tensor (index t + 1); empty or null ptr = generic buffer
     std::vector<char> tap_missing;        // per tensor (index t + 1): the plan never stores it (TAP_FUSED)
     std::shared_ptr<accerl::MlpFusedParams> mlp;  // set when the whole step is one fused launch
-    accerl::FcSampleParams fc_sample = {};         // used by a Step::FC_SAMPLE launch
+    accerl::FcSampleParams fc_sample = {};         // used by a Step::FC_SAMPLE or FC_HEAD launch
+    accerl::FcHeadParams fc_head = {};             // used by a Step::FC_HEAD launch
     std::vector<int> tensor_s2d;          // space-to-depth factor of tensor t at [t + 1]
     int sm_count = 0;
     std::vector<accerl::DeviceBuf> bufs;  // bufs[0] holds the quantised input
@@ -280,6 +292,10 @@ accerl_status flush_uploads(accerl_policy *p);
 bool fc_sample_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
 accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int layer, const int8_t *x,
                               int pitch, Step *out);
+bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
+accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out);
+cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const float *u, int B, float *logits,
+                           int32_t *actions, float *logp, float *value, float *entropy, int sm_count, cudaStream_t st);
 cudaError_t launch_fc_sample(const FcSampleParams &q, const float *u, int B, float *logits,
                              int32_t *actions, float *logp, float *value, float *entropy, int sm_count,
                              cudaStream_t st);

@@ -496,6 +496,14 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
             steps.push_back(s);
             continue;
         }
+        if (role[i] == TCFC && fc_head_fits(p, layers, n_layers, i)) {
+            const bool relu_in = (d.flags & ACCERL_RELU_IN) && !(layers[i - 1].flags & ACCERL_RELU_OUT);
+            if ((st = build_fc_head(p, layers, i, relu_in ? fin.p_plain_relu : fin.p_plain, &s)) != ACCERL_OK) return st;
+            s.layer = -1;
+            steps.push_back(s);
+            fused_sample = true;
+            break;
+        }
         if (role[i] == TCFC && fin.plain && fc_sample_fits(p, layers, n_layers, i)) {
             // the last layer runs fused with the sampler
             if ((st = build_fc_sample(p, d, i, fin.p_plain, L.in_c, &s)) != ACCERL_OK) return st;
