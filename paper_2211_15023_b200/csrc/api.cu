@@ -262,6 +262,24 @@ accerl_status flush_uploads(accerl_policy *p)
 
 using namespace accerl;
 
+// results up to this size are written to pinned host memory by the kernels themselves
+static constexpr size_t kDirectBytes = 64 << 10;
+
+// Can kernels on the current device use this host range at its own address (pinned and mapped, 4-byte aligned)?
+static bool device_reaches(const void *host, size_t bytes)
+{
+    if ((uintptr_t)host & 3) return false;
+    for (const char *at : {(const char *)host, (const char *)host + bytes - 1}) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, at) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (attr.type != cudaMemoryTypeHost || attr.devicePointer != (void *)at) return false;
+    }
+    return true;
+}
+
 // argument checks shared by the act entry points (nothing is launched when they fail)
 static accerl_status check_act_args(accerl_policy *p, const void *obs_dev,
                                     const float *uniforms_dev, int32_t batch, float *logits_dev,
@@ -837,8 +855,10 @@ accerl_status accerl_policy_act_host(accerl_policy *p, const void *obs_host,
     // Large batches go in chunks: the host->device copy of chunk i + 1 runs on a stream of its own
     // while chunk i computes (the copy is PCIe-bound and by far the longer part; the chunks only
     // hide the compute and the copies back behind it).  States are independent, so the results are
-    // those of one call on the whole batch.
-    const int n_chunks = batch >= 4096 ? 8 : 1;
+    // those of one call on the whole batch.  A chunk is at least 14 MB, a quarter of a millisecond of
+    // copying: what it can hide is then well above the dozen calls it costs the host (eight chunks of
+    // 128 KB each, for 32-byte vector observations, took longer than the whole batch at once).
+    const int n_chunks = (int)std::min<size_t>(8, std::max<size_t>(1, obs_per_state * B / (14u << 20)));
     if (n_chunks > 1 && !p->copy_stream) {
         ACCERL_CUDA_TRY(cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking));
         for (int i = 0; i < 9; ++i) {
@@ -849,14 +869,22 @@ accerl_status accerl_policy_act_host(accerl_policy *p, const void *obs_host,
     }
     if (n_chunks == 1) {
         ACCERL_CUDA_TRY(cudaMemcpyAsync(p->st_obs, obs_host, obs_per_state * B, cudaMemcpyHostToDevice, st));
-        ACCERL_CUDA_TRY(cudaMemcpyAsync(p->st_u, uniforms_host, 4 * B, cudaMemcpyHostToDevice, st));
-        accerl_status s = accerl_policy_act(p, p->st_obs, p->st_u, batch, p->st_logits, p->st_actions,
-                                            p->st_logp, cuda_stream);
+        // Small results and the uniforms do not need copies of their own, each of which costs a few
+        // microseconds behind the observations': the kernels reach pinned memory over the bus.
+        const size_t bytes[3] = {4 * B * (size_t)p->n_actions, 4 * B, 4 * B};
+        const bool direct = bytes[0] <= kDirectBytes && device_reaches(logits_host, bytes[0]) &&
+                            device_reaches(actions_host, bytes[1]) && device_reaches(logp_host, bytes[2]);
+        const bool direct_u = direct && device_reaches(uniforms_host, 4 * B);
+        if (!direct_u) ACCERL_CUDA_TRY(cudaMemcpyAsync(p->st_u, uniforms_host, 4 * B, cudaMemcpyHostToDevice, st));
+        accerl_status s = run_steps(p, p->st_obs, direct_u ? uniforms_host : p->st_u, batch, direct ? logits_host : p->st_logits,
+                                    direct ? actions_host : p->st_actions, direct ? logp_host : p->st_logp, nullptr, nullptr,
+                                    st, nullptr);
         if (s != ACCERL_OK) return s;
-        ACCERL_CUDA_TRY(cudaMemcpyAsync(logits_host, p->st_logits, 4 * B * p->n_actions,
-                                        cudaMemcpyDeviceToHost, st));
-        ACCERL_CUDA_TRY(cudaMemcpyAsync(actions_host, p->st_actions, 4 * B, cudaMemcpyDeviceToHost, st));
-        ACCERL_CUDA_TRY(cudaMemcpyAsync(logp_host, p->st_logp, 4 * B, cudaMemcpyDeviceToHost, st));
+        if (!direct) {
+            ACCERL_CUDA_TRY(cudaMemcpyAsync(logits_host, p->st_logits, bytes[0], cudaMemcpyDeviceToHost, st));
+            ACCERL_CUDA_TRY(cudaMemcpyAsync(actions_host, p->st_actions, bytes[1], cudaMemcpyDeviceToHost, st));
+            ACCERL_CUDA_TRY(cudaMemcpyAsync(logp_host, p->st_logp, bytes[2], cudaMemcpyDeviceToHost, st));
+        }
         ACCERL_CUDA_TRY(cudaStreamSynchronize(st));
         return ACCERL_OK;
     }

@@ -118,3 +118,26 @@ def test_noalloc_runs_the_plan_on_the_fixed_array(name, batches, value):
             assert torch.equal(x, y)
     for g in (big, tiny, other):
         g.close()
+
+
+@pytest.mark.parametrize("b,pinned", [(1, True), (200, True), (200, False), (1101, True), (1700, False)])
+def test_act_host_direct_results_and_chunks(b, pinned):
+    """Results written by the kernels into pinned buffers, copied into pageable ones, and batches on both
+    sides of the size from which frames go in chunks; a buffer that is not 4-byte aligned for the device
+    to write goes through the staging copy.  Against the device call."""
+    import paper_2211_15023_b200 as P
+    name = "student_cnn_b8192"
+    g = P.Policy(W.drawn_int8_policy(name, seed=8), b)
+    obs, u = torch.from_numpy(W.observations(name, b, seed=b)), torch.from_numpy(W.uniforms(name, b, seed=b))
+    want = [t.cpu() for t in g.act(obs.cuda(), u.cuda())]
+    pin = (lambda t: t.pin_memory()) if pinned else (lambda t: t)
+    for _ in range(2):
+        out = (pin(torch.zeros((b, g.n_actions))), pin(torch.zeros(b, dtype=torch.int32)), pin(torch.zeros(b)))
+        g.act_host(pin(obs), pin(u), out)
+        for x, y in zip(out, want):
+            assert torch.equal(x, y)
+    raw = torch.zeros(4 * b + 1, dtype=torch.uint8).pin_memory()[1:]  # log-probs at an odd address
+    g.act_host(pin(obs), pin(u), (out[0], out[1], raw))
+    assert raw.numpy().tobytes() == want[2].numpy().tobytes()
+    g.check()
+    g.close()
