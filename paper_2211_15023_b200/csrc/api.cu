@@ -228,6 +228,19 @@ cudaError_t allow_smem(const void *kernel, size_t bytes)
 // Parameters go to the device in a few large blocks, collected on the host and copied when the plan is
 // complete: an allocation and a blocking copy for each of some fifty small arrays took longer than
 // everything else accerl_policy_create does.
+void set_routed_steps(accerl_policy *p, const std::vector<Step> &front)
+{
+    if (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) return;
+    std::vector<Step> r = front;
+    for (const Step &s : p->steps) {
+        const bool fc = s.kind == Step::FC_HEAD || s.kind == Step::FC_SAMPLE ||
+                        (s.kind == Step::TC_GEMM && p->layers[s.layer].kind == ACCERL_FC && !p->tc_steps[s.tc].prm.logits_mode);
+        if (fc) r.push_back(s);
+        else if (s.kind == Step::SAMPLE) return;  // (wide action sets sample from a logits matrix)
+    }
+    p->routed_steps = r;
+}
+
 accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev)
 {
     *dev = nullptr;
@@ -308,14 +321,15 @@ static accerl_status check_act_args(accerl_policy *p, const void *obs_dev,
 // Enqueue the plan's launches; with `ev`, record ev[i] before launch i and ev[n] after the last.
 accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const float *uniforms_dev, int B,
                                 float *logits_dev, int32_t *actions_dev, float *logp_dev, float *value_dev,
-                                float *entropy_dev, cudaStream_t st, cudaEvent_t *ev)
+                                float *entropy_dev, cudaStream_t st, cudaEvent_t *ev, const Route &route)
 {
+    const std::vector<Step> &steps = route.count ? p->routed_steps : p->steps;
     p->last_stream = st;
     // a last layer with a value column and a sampler launch of its own: the layer's floats go to
     // the handle's scratch rows of n_out, the sampler splits them into logits and value
     float *z_dev = p->n_out != p->n_actions ? p->z_scratch : logits_dev;
-    for (size_t i = 0; i < p->steps.size(); ++i) {
-        const Step &s = p->steps[i];
+    for (size_t i = 0; i < steps.size(); ++i) {
+        const Step &s = steps[i];
         if (ev) ACCERL_CUDA_TRY(cudaEventRecord(ev[i], st));
         const LayerPlan *L = s.layer >= 0 ? &p->layers[s.layer] : nullptr;
         const int8_t *in = L ? p->bufs[L->in_buf].ptr : nullptr;
@@ -351,6 +365,7 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             TcStep &t = p->tc_steps[s.tc];
             TcGemmParams prm = t.prm;
             prm.batch = B;
+            prm.batch_dev = route.count;
             prm.m_tiles = (int)(((long long)B * prm.rows_per_image + 127) / 128);
             prm.logits = prm.logits_mode ? z_dev : nullptr;
             if (prm.fuse_ingest) {
@@ -383,6 +398,7 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             AtariParams prm = p->atari;
             prm.obs = (const uint8_t *)obs_dev;
             prm.batch = B;
+            prm.route = route;
             ACCERL_CUDA_TRY(atari_launch(prm, p->sm_count, st));
             break;
         }
@@ -394,18 +410,21 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             ResFirstParams prm = p->res_first;
             prm.obs = (const uint8_t *)obs_dev;
             prm.batch = B;
+            prm.route = route;
             ACCERL_CUDA_TRY(res_first_launch(prm, p->sm_count, st));
             break;
         }
         case Step::RES_STACK1: {
             ResStack1Params prm = p->res_stack1;
             prm.batch = B;
+            prm.route = route;
             ACCERL_CUDA_TRY(res_stack1_launch(prm, p->sm_count, st));
             break;
         }
         case Step::RES_STACK23: {
             ResStack23Params prm = p->res_stack23;
             prm.batch = B;
+            prm.route = route;
             ACCERL_CUDA_TRY(res_stack23_launch(prm, p->sm_count, st));
             break;
         }
@@ -433,11 +452,11 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             break;
         case Step::FC_HEAD:
             ACCERL_CUDA_TRY(launch_fc_head(p->fc_head, p->fc_sample, uniforms_dev, B, logits_dev, actions_dev, logp_dev,
-                                           value_dev, entropy_dev, p->sm_count, st));
+                                           value_dev, entropy_dev, route, p->sm_count, st));
             break;
         case Step::FC_SAMPLE:
             ACCERL_CUDA_TRY(launch_fc_sample(p->fc_sample, uniforms_dev, B, logits_dev, actions_dev, logp_dev,
-                                             value_dev, entropy_dev, p->sm_count, st));
+                                             value_dev, entropy_dev, route, p->sm_count, st));
             break;
         case Step::SAMPLE:
             ACCERL_CUDA_TRY(launch_sample(z_dev, p->n_out, uniforms_dev, B, p->n_actions,
@@ -446,7 +465,7 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             break;
         }
     }
-    if (ev) ACCERL_CUDA_TRY(cudaEventRecord(ev[p->steps.size()], st));
+    if (ev) ACCERL_CUDA_TRY(cudaEventRecord(ev[steps.size()], st));
     return ACCERL_OK;
 }
 
@@ -464,6 +483,9 @@ void accerl_policy_destroy(accerl_policy *p)
     for (cudaEvent_t ev : p->events) cudaEventDestroy(ev);
     for (cudaEvent_t ev : p->copy_events) cudaEventDestroy(ev);
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
+    for (cudaEvent_t ev : p->mix_events)
+        if (ev) cudaEventDestroy(ev);
+    if (p->mix_stream) cudaStreamDestroy(p->mix_stream);
     delete p->noalloc_twin;  // owns nothing on the device
     delete p;
 }

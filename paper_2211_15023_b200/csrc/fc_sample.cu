@@ -53,11 +53,11 @@ __device__ __forceinline__ void warp_sample(float z, bool live, float uu, int A,
     lpa = __shfl_sync(0xffffffffu, lp, a);
 }
 
-// EXTRAS: the layer may have one output column more than actions, the state value V(s) (lane A;
+// EXTRAS: the states may be routed (Route); the layer may have one output column more than actions, the state value V(s) (lane A;
 // no part of the softmax), and the entropy of the action distribution may be asked for.
 template <bool EXTRAS>
 __global__ void __launch_bounds__(32 * kFsWarps)
-fc_sample_kernel(const FcSampleParams q, const float *__restrict__ u, int B,
+fc_sample_kernel(const FcSampleParams q, const float *__restrict__ u, int B_all, const Route route,
                  float *__restrict__ logits, int32_t *__restrict__ actions, float *__restrict__ logp,
                  float *__restrict__ value, float *__restrict__ entropy)
 {
@@ -68,6 +68,7 @@ fc_sample_kernel(const FcSampleParams q, const float *__restrict__ u, int B,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *x0 = s_x + warp * 2 * K4, *x1 = x0 + K4;
     const bool live = lane < A;
+    int B = B_all;
     const bool has_col = EXTRAS ? lane < q.n_out : live;  // a column of the layer (action or value)
     const long long stride = (long long)gridDim.x * kFsWarps;
     long long pair = (long long)blockIdx.x * kFsWarps + warp;
@@ -97,12 +98,15 @@ fc_sample_kernel(const FcSampleParams q, const float *__restrict__ u, int B,
         for (int i = threadIdx.x; i < K4 * 8; i += blockDim.x) sw[i] = __ldg(gw + i);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (EXTRAS) B = routed_batch(route, B_all);
     fetch(pair);
     __syncthreads();
     for (; 2 * pair < B; pair += stride) {
         const long long row0 = 2 * pair, row1 = row0 + 1;
         const bool has1 = row1 < B;
-        const float u0 = u[row0], u1 = has1 ? u[row1] : 2.f;
+        // where the results go, and the states' uniforms
+        const long long out0 = EXTRAS ? routed_row(route, (int)row0) : row0, out1 = EXTRAS && has1 ? routed_row(route, (int)row1) : row1;
+        const float u0 = u[out0], u1 = has1 ? u[out1] : 2.f;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int i = lane + 32 * j;
@@ -132,28 +136,28 @@ fc_sample_kernel(const FcSampleParams q, const float *__restrict__ u, int B,
         __syncwarp();  // the staged rows are overwritten in the next round
         const float z0 = epilogue_float(acc0, ks, bs, false), z1 = epilogue_float(acc1, ks, bs, false);
         if (live) {
-            logits[row0 * A + lane] = z0;
-            if (has1) logits[row1 * A + lane] = z1;
+            logits[out0 * A + lane] = z0;
+            if (has1) logits[out1 * A + lane] = z1;
         }
         if (EXTRAS && value && lane == A && A < q.n_out) {
-            value[row0] = z0;
-            if (has1) value[row1] = z1;
+            value[out0] = z0;
+            if (has1) value[out1] = z1;
         }
         int a;
         float lpa, h = 0.f;
         if (EXTRAS && entropy) warp_sample<true>(z0, live, u0, A, lane, a, lpa, h);
         else warp_sample<false>(z0, live, u0, A, lane, a, lpa, h);
         if (lane == 0) {
-            actions[row0] = a;
-            logp[row0] = lpa;
-            if (EXTRAS && entropy) entropy[row0] = h;
+            actions[out0] = a;
+            logp[out0] = lpa;
+            if (EXTRAS && entropy) entropy[out0] = h;
         }
         if (EXTRAS && entropy) warp_sample<true>(z1, live, u1, A, lane, a, lpa, h);
         else warp_sample<false>(z1, live, u1, A, lane, a, lpa, h);
         if (lane == 0 && has1) {
-            actions[row1] = a;
-            logp[row1] = lpa;
-            if (EXTRAS && entropy) entropy[row1] = h;
+            actions[out1] = a;
+            logp[out1] = lpa;
+            if (EXTRAS && entropy) entropy[out1] = h;
         }
     }
 }
@@ -182,7 +186,8 @@ __device__ __forceinline__ void head_mma(int (&d)[4], uint32_t a0, uint32_t a1, 
 // MT: 16-state tiles of a cluster; NT: 8-column tiles of a CTA (N = 64 * NT hidden outputs)
 template <int MT, int NT>
 __global__ void __launch_bounds__(32 * kHeadWarps, 1)
-fc_hidden_fc_sample_kernel(const __grid_constant__ FcHeadParams h, const __grid_constant__ FcSampleParams q, const float *__restrict__ u, int B,
+fc_hidden_fc_sample_kernel(const __grid_constant__ FcHeadParams h, const __grid_constant__ FcSampleParams q, const float *__restrict__ u, int B_all,
+                           const Route route,
                            float *__restrict__ logits, int32_t *__restrict__ actions, float *__restrict__ logp,
                            float *__restrict__ value, float *__restrict__ entropy)
 {
@@ -205,6 +210,8 @@ fc_hidden_fc_sample_kernel(const __grid_constant__ FcHeadParams h, const __grid_
     const bool has_col = lane < q.n_out;
     const float ks2 = has_col ? q.kscale[lane] : 0.f, bs2 = has_col ? q.bias[lane] : 0.f;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int B = routed_batch(route, B_all);
+    if (row0 >= B) return;  // the whole cluster
 
     // ---- hidden layer: this warp's pieces of K
     int acc[MT][NT][4] = {};
@@ -279,18 +286,18 @@ fc_hidden_fc_sample_kernel(const __grid_constant__ FcHeadParams h, const __grid_
 #pragma unroll
     for (int s = 0; s < kSlices; ++s) zi += s_z[own][s][lane];
     const float z = epilogue_float(zi, ks2, bs2, false);
-    const int A = q.n_actions;
+    const int A = q.n_actions, out = routed_row(route, row);
     const bool live = lane < A;
-    if (live) logits[(long long)row * A + lane] = z;
-    if (value && lane == A && A < q.n_out) value[row] = z;
+    if (live) logits[(long long)out * A + lane] = z;
+    if (value && lane == A && A < q.n_out) value[out] = z;
     int a;
     float lpa, hh = 0.f;
-    if (entropy) warp_sample<true>(z, live, u[row], A, lane, a, lpa, hh);
-    else warp_sample<false>(z, live, u[row], A, lane, a, lpa, hh);
+    if (entropy) warp_sample<true>(z, live, u[out], A, lane, a, lpa, hh);
+    else warp_sample<false>(z, live, u[out], A, lane, a, lpa, hh);
     if (lane == 0) {
-        actions[row] = a;
-        logp[row] = lpa;
-        if (entropy) entropy[row] = hh;
+        actions[out] = a;
+        logp[out] = lpa;
+        if (entropy) entropy[out] = hh;
     }
 }
 
@@ -388,7 +395,8 @@ accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, i
 }
 
 cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const float *u, int B, float *logits,
-                           int32_t *actions, float *logp, float *value, float *entropy, int sm_count, cudaStream_t st)
+                           int32_t *actions, float *logp, float *value, float *entropy, const Route &route, int sm_count,
+                           cudaStream_t st)
 {
     auto go = [&](auto kernel, int rows) -> cudaError_t {
         const size_t smem = sizeof(int) * (size_t)kHeadWarps * rows * (h.N / kHeadCluster);
@@ -407,17 +415,17 @@ cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const
         attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        return cudaLaunchKernelEx(&cfg, kernel, h, q, u, B, logits, actions, logp, value, entropy);
+        return cudaLaunchKernelEx(&cfg, kernel, h, q, u, B, route, logits, actions, logp, value, entropy);
     };
     // 16 states per cluster while their clusters fit the chip once
-    const bool two = (B + 15) / 16 * kHeadCluster > sm_count;
+    const bool two = ((route.count ? route.expect : B) + 15) / 16 * kHeadCluster > sm_count;
     if (h.N == 512) return two ? go(fc_hidden_fc_sample_kernel<2, 8>, 32) : go(fc_hidden_fc_sample_kernel<1, 8>, 16);
     return two ? go(fc_hidden_fc_sample_kernel<2, 4>, 32) : go(fc_hidden_fc_sample_kernel<1, 4>, 16);
 }
 
 cudaError_t launch_fc_sample(const FcSampleParams &q, const float *u, int B, float *logits,
-                             int32_t *actions, float *logp, float *value, float *entropy, int sm_count,
-                             cudaStream_t st)
+                             int32_t *actions, float *logp, float *value, float *entropy, const Route &route,
+                             int sm_count, cudaStream_t st)
 {
     const int per_block = 2 * kFsWarps;
     long long blocks = ((long long)B + per_block - 1) / per_block;
@@ -433,9 +441,9 @@ cudaError_t launch_fc_sample(const FcSampleParams &q, const float *u, int B, flo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool extras = value || entropy || q.n_out != q.n_actions;
-    cudaError_t e = extras ? cudaLaunchKernelEx(&cfg, fc_sample_kernel<true>, q, u, B, logits, actions, logp, value, entropy)
-                           : cudaLaunchKernelEx(&cfg, fc_sample_kernel<false>, q, u, B, logits, actions, logp,
+    const bool extras = value || entropy || q.n_out != q.n_actions || route.count;
+    cudaError_t e = extras ? cudaLaunchKernelEx(&cfg, fc_sample_kernel<true>, q, u, B, route, logits, actions, logp, value, entropy)
+                           : cudaLaunchKernelEx(&cfg, fc_sample_kernel<false>, q, u, B, route, logits, actions, logp,
                                                 (float *)nullptr, (float *)nullptr);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

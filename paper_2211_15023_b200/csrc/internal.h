@@ -172,6 +172,7 @@ struct accerl_policy {
                                           // plan's sampler is a launch of its own and n_out != n_actions
     std::vector<accerl::LayerPlan> layers;
     std::vector<accerl::Step> steps;      // the launch sequence of one act call
+    std::vector<accerl::Step> routed_steps;  // the same for some states of a batch (Route); empty: not possible
     std::string plan_note;                // why a faster plan was not taken (shown by accerl_policy_info)
     std::vector<accerl::TcStep> tc_steps;
     std::vector<accerl::PoolDualParams> pools;
@@ -227,6 +228,9 @@ struct accerl_policy {
     // outputs of this policy inside accerl_policy_act_mixed (allocated on its first call)
     float *mix_logits = nullptr, *mix_logp = nullptr, *mix_value = nullptr, *mix_entropy = nullptr;
     int32_t *mix_actions = nullptr;
+    cudaStream_t mix_stream = nullptr;            // the smaller network's launches
+    cudaEvent_t mix_events[2] = {nullptr, nullptr};
+    int *mix_rows = nullptr;  // [2][max_batch] states of each network, then their counts
 };
 
 namespace accerl {
@@ -237,10 +241,11 @@ static inline bool unfuse_for_taps(const accerl_policy *p)
     return (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) && !(p->flags & ACCERL_FLAG_TAP_FUSED);
 }
 
-// one Actor step along the policy's plan (api.cu); with `ev`, an event before each launch and after the last
+// one Actor step along the policy's plan (api.cu); with `ev`, an event before each launch and after the last;
+// with a route, along p->routed_steps and for those states only
 accerl_status run_steps(accerl_policy *p, const void *obs_dev, const float *uniforms_dev, int B, float *logits_dev,
                         int32_t *actions_dev, float *logp_dev, float *value_dev, float *entropy_dev, cudaStream_t st,
-                        cudaEvent_t *ev);
+                        cudaEvent_t *ev, const Route &route = Route());
 
 // generic CUDA-core kernels (generic_kernels.cu); every launcher enqueues on `st` and returns
 // the launch status
@@ -287,6 +292,8 @@ accerl_status build_mlp_plan(accerl_policy *p, const accerl_layer_desc *layers, 
 cudaError_t launch_mlp_fused(const accerl_policy *p, const float *obs, const float *u, int B,
                              float *logits, int32_t *actions, float *logp, float *value, float *entropy,
                              cudaStream_t st);
+// fills p->routed_steps from the finished plan: `front`, then the plan's fully connected launches
+void set_routed_steps(accerl_policy *p, const std::vector<Step> &front);
 accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev);  // there once create is done
 accerl_status flush_uploads(accerl_policy *p);
 bool fc_sample_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
@@ -295,9 +302,10 @@ accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int 
 bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
 accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out);
 cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const float *u, int B, float *logits,
-                           int32_t *actions, float *logp, float *value, float *entropy, int sm_count, cudaStream_t st);
+                           int32_t *actions, float *logp, float *value, float *entropy, const Route &route, int sm_count,
+                           cudaStream_t st);
 cudaError_t launch_fc_sample(const FcSampleParams &q, const float *u, int B, float *logits,
-                             int32_t *actions, float *logp, float *value, float *entropy, int sm_count,
-                             cudaStream_t st);
+                             int32_t *actions, float *logp, float *value, float *entropy, const Route &route,
+                             int sm_count, cudaStream_t st);
 
 }  // namespace accerl

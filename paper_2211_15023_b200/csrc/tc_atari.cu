@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(32 * (CTX * WG * 4 + CTX), 1) atari_kernel(con
     fence_after();
     const uint32_t tmem = bars.tmem_base;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int step = CTX * (int)gridDim.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int step = CTX * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kEpi) {
         // ------------------------------------------------------------------ MMA issuers, one per context
@@ -174,8 +175,8 @@ __global__ void __launch_bounds__(32 * (CTX * WG * 4 + CTX), 1) atari_kernel(con
         };
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (n < p.batch) conv1();
-        for (; n < p.batch; n += step, par ^= 1) {
+        if (n < batch) conv1();
+        for (; n < batch; n += step, par ^= 1) {
             image_wait(ready0 + 8, par, abort_flag, p.status, 8);
             fence_after();
             if (elect_one()) {
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(32 * (CTX * WG * 4 + CTX), 1) atari_kernel(con
                 mma_commit(smem_u32(&bars.full2[ctx]));
             }
             __syncwarp();
-            if (n + step < p.batch) conv1();
+            if (n + step < batch) conv1();
             image_wait(ready0 + 16, par, abort_flag, p.status, 8);
             fence_after();
             if (elect_one()) {
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(32 * (CTX * WG * 4 + CTX), 1) atari_kernel(con
         };
         auto convert = [&](int n) {
             constexpr int kIter = (441 + kT - 1) / kT;
-            const uint8_t *img = p.obs + (size_t)n * 28224;
+            const uint8_t *img = p.obs + (size_t)routed_row(p.route, n) * 28224;
             uint32_t w[kIter][16];
 #pragma unroll
             for (int j = 0; j < kIter; ++j) {
@@ -240,17 +241,16 @@ __global__ void __launch_bounds__(32 * (CTX * WG * 4 + CTX), 1) atari_kernel(con
                                                                    quantise_frame_word<MODE>(w[j][4 * c + 3], p.ingest_mul, p.ingest_add)));
             }
             operand_done(0);
-            if (tid == 0 && n + step < p.batch)  // the image after this one on its way into L2
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)(n + step) * 28224), "r"(28224)
+            if (tid == 0 && n + step < batch)  // the image after this one on its way into L2
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)routed_row(p.route, n + step) * 28224), "r"(28224)
                              : "memory");
         };
         const int Y2 = row / 10, X2 = row - Y2 * 10, Y3 = row / 9, X3 = row - Y3 * 9;
         const bool v2 = Y2 < 9 && X2 < 9, v3 = Y3 < 7 && X3 < 7;
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (n < p.batch) convert(n);
+        if (n < batch) convert(n);
         uint32_t par = 0;
-        for (; n < p.batch; n += step, par ^= 1) {
+        for (; n < batch; n += step, par ^= 1) {
             // ---- first layer -> space-to-depth(2) rows
             for (int t = wg; t < 4; t += WG) {
                 const int m = t * 128 + row, Y = m / 21, X = m - Y * 21;
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(32 * (CTX * WG * 4 + CTX), 1) atari_kernel(con
                 });
             }
             operand_done(1);
-            if (n + step < p.batch) {
+            if (n + step < batch) {
                 image_wait(full1 + 8 * 3, par, abort_flag, p.status, 16);  // the last tile's MMAs have read the frame
                 convert(n + step);
             }
@@ -321,7 +321,7 @@ template <int C1, int C2, int C3>
 static cudaError_t atari_go(const AtariParams &p, int sm_count, cudaStream_t st)
 {
     using S = AtariSizes<C1, C2, C3>;
-    const bool one = p.batch <= sm_count || p.tap1;  // (the taps are compiled into one form only)
+    const bool one = (p.route.count ? p.route.expect : p.batch) <= sm_count || p.tap1;  // (the taps are compiled into one form only)
     auto go = [&](auto kernel, int ctx, int wg) -> cudaError_t {
         const size_t smem = 1024 + S::weights + (size_t)ctx * S::ctx;
         cudaError_t e = allow_smem((const void *)kernel, smem);

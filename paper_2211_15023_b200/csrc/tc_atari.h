@@ -5,6 +5,19 @@
 
 namespace accerl {
 
+// Which states of a batch a launch works on: all `batch` of them in order, or, with `count`, the *count
+// states listed in `rows` (both written on the device, see accerl_policy_act_mixed; *count <= batch).
+// Intermediate tensors are compact (entry i belongs to state rows[i]).
+struct Route {
+    const int *rows = nullptr, *count = nullptr;
+    int expect = 0;  // the caller's guess of *count, for choosing launch shapes
+};
+#ifdef __CUDACC__
+// (call after griddepcontrol.wait)
+__device__ __forceinline__ int routed_batch(const Route &r, int batch) { return r.count ? __ldcg(r.count) : batch; }
+__device__ __forceinline__ int routed_row(const Route &r, int i) { return r.rows ? __ldcg(r.rows + i) : i; }
+#endif
+
 struct AtariLayer {
     float k[64], b[64];  // per channel: the single-fma pair, or (s_in * s_w, bias) for the division
     float s_out, inv_s_out;
@@ -18,6 +31,7 @@ struct AtariParams {
     int8_t *out;             // [n][49 * C3]: the fc layer's input rows
     int8_t *tap1, *tap2;     // outputs of the first two convs as the launch-per-layer plan stores them, or null
     int batch, wide;         // wide: 32 / 64 / 64 channels
+    Route route;
     int ingest_mode;         // 2: u >> 1, 1: line with the minimum, 0: line without
     uint32_t ingest_mul, ingest_add;
     int *status;

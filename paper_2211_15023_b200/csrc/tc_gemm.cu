@@ -514,7 +514,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // it touches activations (griddepcontrol.wait in the producer and epilogue roles).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    const int total_tiles = ((p.m_tiles + SUB - 1) / SUB) * p.n_tiles;  // pipeline steps
+    int m_tiles = p.m_tiles;
+    if (p.batch_dev) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        m_tiles = (__ldcg(p.batch_dev) + kTileM - 1) / kTileM;
+    }
+    const int total_tiles = ((m_tiles + SUB - 1) / SUB) * p.n_tiles;  // pipeline steps
 #ifdef ACCERL_TC_TRACE
     const long long trace_start = clock64();
 #endif

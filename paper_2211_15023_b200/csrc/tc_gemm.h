@@ -40,6 +40,7 @@ struct TcGemmParams {
     // Y < out_h and X < out_w; stored at row n * out_rows_per_image + (Y/s) * out_grid_w + X/s,
     // byte ((Y%s) * s + X%s) * n_total + channel, rows `out_pitch` bytes apart (s = out_s2d)
     int batch, rows_per_image, grid_w, out_h, out_w;
+    const int *batch_dev;  // fully connected layers: the number of rows, where only the device knows it (<= batch)
     int out_s2d, out_rows_per_image, out_grid_w, out_pitch;
     int out_s2d_log2;
     int out_row_off;  // added to the output row (a one-pixel border of a padded consumer layout)

@@ -847,6 +847,7 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
         if (hpool_first) p->tap_missing[1] = 1;
     }
     p->steps = steps;
+    if (resident) set_routed_steps(p, std::vector<Step>(steps.begin(), steps.begin() + 3));
     *used = true;
     return ACCERL_OK;
 }

@@ -225,7 +225,7 @@ size_t swizzled(int n, int kk, int rb)
 accerl_status build_atari_step(accerl_policy *p, const accerl_layer_desc *layers, int n_layers, Step *step, bool *used)
 {
     *used = false;
-    if (n_layers < 5 || p->in_c != 4 || p->in_h != 84 || p->in_w != 84 || p->max_batch > (layers[0].out_c == 32 ? kAtariMaxWide : kAtariMaxNarrow) || unfuse_for_taps(p) ||
+    if (n_layers < 5 || p->in_c != 4 || p->in_h != 84 || p->in_w != 84 || unfuse_for_taps(p) ||
         !(p->ingest_shift1 || p->ingest_arith == 1))
         return ACCERL_OK;
     const bool wide = layers[0].out_c == 32;
@@ -289,7 +289,6 @@ accerl_status build_atari_step(accerl_policy *p, const accerl_layer_desc *layers
     }
     step->kernel += std::string(division ? "[3-step divide verified]" : "") + "[frames quantised inside]";
     step->covers = "ingest+layers 0-2";
-    p->tap_missing[0] = 1;  // no quantised input tensor exists
     *used = true;
     return ACCERL_OK;
 }
@@ -344,9 +343,13 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
     bool atari = false;
     Step convs;
     if (accerl_status st = build_atari_step(p, layers, n_layers, &convs, &atari); st != ACCERL_OK) return st;
-    if (atari) steps.assign(1, convs);
+    const bool atari_small = atari && p->max_batch <= (layers[0].out_c == 32 ? kAtariMaxWide : kAtariMaxNarrow);
+    if (atari_small) {
+        steps.assign(1, convs);
+        p->tap_missing[0] = 1;  // no quantised input tensor exists
+    }
 
-    for (int i = atari ? 3 : 0; i < n_layers; ++i) {
+    for (int i = atari_small ? 3 : 0; i < n_layers; ++i) {
         const accerl_layer_desc &d = layers[i];
         const LayerPlan &L = p->layers[i];
         if (fc_head_fits(p, layers, n_layers, i)) {  // the last two layers and the sampler
@@ -649,6 +652,7 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
         steps.push_back(ss);
     }
     p->steps = steps;
+    if (atari) set_routed_steps(p, std::vector<Step>(1, convs));
     *used = true;
     return ACCERL_OK;
 }

@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
     const uint32_t tmem = res_setup<kFirstEpi>(bars, bufs, kFirstCtx * (kFrameBytes + kHpBytes), smem, p.w, kResFirstWeights,
                                                warp, kFirstWg * 4, -1);
     volatile int *abort_flag = &bars.abort_flag;
-    const int step = kFirstCtx * (int)gridDim.x;
+    const int step = kFirstCtx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kFirstEpi) {
         // ------------------------------------------------------------------ MMA issuers
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
         const uint32_t b0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, it = 0;
-        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step, ++it) {
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step, ++it) {
             image_wait(ready, it & 1, abort_flag, p.status, 8);
             fence_after();
             for (int t = 0; t < kFirstTiles; ++t) {
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
         const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
         auto convert = [&](int n) {
             constexpr int kGroups = 84 * 21, kIter = (kGroups + kFirstT - 1) / kFirstT;
-            const uint32_t *src = reinterpret_cast<const uint32_t *>(p.obs + (size_t)n * 28224);
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(p.obs + (size_t)routed_row(p.route, n) * 28224);
             uint32_t w[kIter][4];
 #pragma unroll
             for (int j = 0; j < kIter; ++j) {
@@ -306,14 +306,14 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
             fence_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(ready);
-            if (tid == 0 && n + step < p.batch)  // the image after this one on its way into L2
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)(n + step) * 28224), "r"(28224)
+            if (tid == 0 && n + step < batch)  // the image after this one on its way into L2
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + (size_t)routed_row(p.route, n + step) * 28224), "r"(28224)
                              : "memory");
         };
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (n < p.batch) convert(n);
+        if (n < batch) convert(n);
         uint32_t seq0 = 0;  // accumulators handed over before this image
-        for (; n < p.batch; n += step, seq0 += kFirstTiles) {
+        for (; n < batch; n += step, seq0 += kFirstTiles) {
             for (int t = wg; t < kFirstTiles; t += kFirstWg) {
                 const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kFirstSlots;
                 image_wait(full0 + 8 * slot, (seq / kFirstSlots) & 1, abort_flag, p.status, 16);
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
                 }
             }
             ctx_sync<kFirstT>(ctx);  // all lines pooled along x; the MMAs have read the frame
-            if (n + step < p.batch) convert(n + step);
+            if (n + step < batch) convert(n + step);
             int8_t *out = p.x1 + (size_t)n * kRes1Bytes;
             if (tid < 125) {  // the zero pixels: lines 0 and 42, the first one of the lines between
                 const int s = tid < 42 ? tid : tid < 84 ? 42 * 42 + tid - 42 : (tid - 83) * 42;
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
     uint8_t *bufs = smem + kRes1Weights;
     const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kS1Ctx * 2 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, -1);
     volatile int *abort_flag = &bars.abort_flag;
-    const int step = kS1Ctx * (int)gridDim.x;
+    const int step = kS1Ctx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kS1Epi) {
         // ------------------------------------------------------------------ MMA issuers
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, rdy = 0;
-        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step) {
             for (int op = 0; op < kS1Ops; ++op) {
                 if (op < 5) {  // (the second half of the last conv reads what the first half read)
                     image_wait(ready, rdy, abort_flag, p.status, 8);
@@ -448,9 +448,9 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
         for (int t = 0; t < kS1Tiles; ++t)
             if ((t * 128 + row) % 21 < 20 && t * 128 + row < 861) second |= 1u << t;
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (tid == 0 && n < p.batch) fetch(n);
+        if (tid == 0 && n < batch) fetch(n);
         uint32_t seq0 = 0, it = 0;  // tiles handed over before this layer, images
-        for (; n < p.batch; n += step, ++it) {
+        for (; n < batch; n += step, ++it) {
             // the image: x to tensor memory, ReLU(x) in place for the first conv
             image_wait(land_bar, it & 1, abort_flag, p.status, 1);
             for (int t = wg; t < kS1Tiles; t += kS1Wg) {
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                 }
                 // a half of the 16 -> 32 conv is complete: 3 x 3 stride-2 max over it
                 ctx_sync<kS1T>(ctx);
-                if (op == 5 && tid == 0 && n + step < p.batch) {  // the MMAs have read the image: the next one may land
+                if (op == 5 && tid == 0 && n + step < batch) {  // the MMAs have read the image: the next one may land
                     fence_async();
                     fetch(n + step);
                 }
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
     const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kS2Ctx * kS2CtxBytes, smem, p.w, kRes2Weights, warp, kS2Wg * 4,
                                             kS2Slot3);
     volatile int *abort_flag = &bars.abort_flag;
-    const int step = kS2Ctx * (int)gridDim.x;
+    const int step = kS2Ctx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kS2Epi) {
         // ------------------------------------------------------------------ MMA issuers
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo, d0 = tmem + (uint32_t)ctx * kS2Cols;
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t rdy = 0, slot = 0, phase = 0, k3 = 0;  // k3: layers done at 9 x 9
-        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < p.batch; n += step) {
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step) {
             for (int op = 0; op < kS2Ops; ++op) {
                 image_wait(ready, rdy, abort_flag, p.status, 8);
                 rdy ^= 1;
@@ -656,9 +656,9 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
         const bool v3 = Y3 < 9 && X3 < 9;
         const uint32_t off3 = row_off(row + 11, wg);
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (tid == 0 && n < p.batch) fetch(n);
+        if (tid == 0 && n < batch) fetch(n);
         uint32_t seq0 = 0, k3 = 0, it = 0;
-        for (; n < p.batch; n += step, ++it) {
+        for (; n < batch; n += step, ++it) {
             image_wait(land_bar, it & 1, abort_flag, p.status, 1);
             for (int t = wg; t < kS2Tiles; t += kS2Wg)
 #pragma unroll
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
             layer20(OpIndex<4>());
             // 3 x 3 stride-2 max over the last one: every thread its pixel and channels of the 9 x 9 tensor
             ctx_sync<kS2T>(ctx);
-            if (tid == 0 && n + step < p.batch) {  // the MMAs have read the image's buffer: the next one may land
+            if (tid == 0 && n + step < batch) {  // the MMAs have read the image's buffer: the next one may land
                 fence_async();
                 fetch(n + step);
             }

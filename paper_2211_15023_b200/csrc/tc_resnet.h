@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "tc_atari.h"
+
 namespace accerl {
 
 // Requantisation constants of one conv layer, read from the constant bank.
@@ -28,6 +30,7 @@ struct ResFirstParams {  // frames -> first conv -> max-pool
     int8_t *x1;               // [n][kRes1Bytes]
     int8_t *tap_in, *tap_x1;  // plain NHWC copies for the parity taps, or null
     int batch, ingest_mode;   // 2: u >> 1, else the fixed-point line
+    Route route;
     uint32_t ingest_mul, ingest_add;
     int *status;
     ResLayer layer;
@@ -39,6 +42,7 @@ struct ResStack1Params {  // two residual blocks at 41 x 41, conv 16 -> 32, max-
     int8_t *x2;               // [n][kRes2Bytes]
     int8_t *tap[4], *tap_x2;  // outputs of the block convs and of the pool, or null
     int batch;
+    Route route;
     int *status;
     ResLayer layer[5];
 };
@@ -49,6 +53,7 @@ struct ResStack23Params {  // two blocks at 20 x 20, conv, max-pool, two blocks 
     int8_t *x3;               // [n][kRes3Bytes], ReLU'd
     int8_t *tap[9], *tap_x3;  // outputs of the convs (not the last one) and of the pool, or null
     int batch;
+    Route route;
     int *status;
     ResLayer layer[9];
 };

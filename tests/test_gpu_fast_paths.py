@@ -141,3 +141,29 @@ def test_act_host_direct_results_and_chunks(b, pinned):
     assert raw.numpy().tobytes() == want[2].numpy().tobytes()
     g.check()
     g.close()
+
+
+@pytest.mark.parametrize("small,orig,b", [("student_cnn_b8192", "nature_cnn_b160", 1), ("student_cnn_b8192", "nature_cnn_b160", 2300),
+                                          ("student_cnn_b8192", "impala_resnet_b16384", 1100), ("impala_resnet_b16384", "nature_cnn_b160", 460)])
+@pytest.mark.parametrize("alpha", [0.0, 0.07, 0.8, 1.0])
+def test_mixing_routes_every_state_through_its_network(small, orig, b, alpha):
+    """States listed per network on the device, including empty lists, lists longer and shorter than
+    the host expects, and handles whose own plan runs other kernels; every state must get what its
+    network alone gives, twice in a row with different selections."""
+    import paper_2211_15023_b200 as P
+    gs, go = P.Policy(W.drawn_int8_policy(small, seed=1), b), P.Policy(W.drawn_int8_policy(orig, seed=2), b)
+    obs, u = torch.from_numpy(W.observations(small, b)).cuda(), torch.from_numpy(W.uniforms(small, b)).cuda()
+    a, o = gs.act_ex(obs, u), go.act_ex(obs, u)
+    for call in range(2):
+        rng = np.random.default_rng(call)
+        sel = rng.random(b, dtype=np.float32) if call == 0 else np.full(b, 0.06, np.float32)
+        out = P.act_mixed(gs, go, obs, u, torch.from_numpy(sel).cuda(), alpha)
+        gs.check()
+        go.check()
+        pick = torch.from_numpy(sel < np.float32(alpha)).cuda()
+        assert torch.equal(out["use_smaller"].bool(), pick)
+        for k in ("logits", "actions", "logp", "entropy"):
+            m = pick[:, None] if k == "logits" else pick
+            assert torch.equal(out[k], torch.where(m, a[k], o[k])), k
+    gs.close()
+    go.close()
