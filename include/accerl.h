@@ -435,7 +435,12 @@ accerl_status accerl_tc_probe_i8(int32_t device, int32_t n, int32_t issuing_warp
                                  int32_t a_shift_rows, int32_t commit_every, float *ms_out,
                                  float *cycles_per_mma_out);
 
-/* Free the handle and its device memory.  Synchronises the device.  NULL is allowed. */
+/*
+ * Free the handle and its device memory.  Synchronises the device.  NULL is allowed.  Up to 512 MB of such
+ * memory per process stays with the library for the next policy (building one is then free of cudaMalloc
+ * and cudaFree): no block for more than 30 s without use once another policy is built or destroyed, none
+ * when an allocation fails.
+ */
 void accerl_policy_destroy(accerl_policy *p);
 
 /* Message for the calling thread's most recent failing call; never NULL. */

@@ -249,7 +249,7 @@ accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, voi
         UploadBlock b;
         const size_t size = std::max<size_t>(need, (size_t)1 << 20);
         void *d = nullptr;
-        ACCERL_CUDA_TRY(cudaMalloc(&d, size));
+        ACCERL_CUDA_TRY(device_alloc(&d, size));
         p->owned.push_back(d);
         b.dev = (char *)d;
         b.host.resize(size);
@@ -479,7 +479,7 @@ void accerl_policy_destroy(accerl_policy *p)
     if (!p) return;
     DeviceGuard g(p->device);
     cudaDeviceSynchronize();
-    for (void *d : p->owned) cudaFree(d);
+    for (void *d : p->owned) device_free(d);
     for (cudaEvent_t ev : p->events) cudaEventDestroy(ev);
     for (cudaEvent_t ev : p->copy_events) cudaEventDestroy(ev);
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
@@ -665,7 +665,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         size_t total = 0;
         for (DeviceBuf &b : p->bufs) total += (b.bytes_per_state * (size_t)max_batch + 256 + 1023) / 1024 * 1024;
         void *d = nullptr;
-        cudaError_t e = cudaMalloc(&d, total);
+        cudaError_t e = device_alloc(&d, total);
         if (e != cudaSuccess) {
             set_error("create: cudaMalloc of %zu workspace bytes failed: %s", total, cudaGetErrorString(e));
             cudaGetLastError();
@@ -702,7 +702,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
     if (value_head) {
         void *d = nullptr;
         const size_t bytes = (size_t)max_batch * p->n_out * sizeof(float) + 256;
-        cudaError_t e = cudaMalloc(&d, bytes);
+        cudaError_t e = device_alloc(&d, bytes);
         if (e != cudaSuccess) {
             set_error("create: cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
             cudaGetLastError();
@@ -862,7 +862,7 @@ accerl_status accerl_policy_act_host(accerl_policy *p, const void *obs_host,
         void *d[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
         size_t sz[5] = {obs_per_state * mb, 4 * mb, 4 * mb * (size_t)p->n_actions, 4 * mb, 4 * mb};
         for (int i = 0; i < 5; ++i) {
-            ACCERL_CUDA_TRY(cudaMalloc(&d[i], sz[i] + 256));
+            ACCERL_CUDA_TRY(device_alloc(&d[i], sz[i] + 256));
             p->owned.push_back(d[i]);
             p->workspace_bytes += sz[i] + 256;
         }

@@ -1,0 +1,111 @@
+// Device memory of the library.  cudaMalloc and cudaFree map and unmap memory through the kernel driver:
+// a fraction of a millisecond each on a quiet machine, tens to hundreds when other processes of the host
+// do the same, and a Compressor that hands over a new policy every few seconds pays for a dozen of them
+// each time (building and calibrating the residual network: 9 ms at best, 20 to 300 on a busy host).
+// So blocks that policies give back are kept for the next one: at most kKept bytes per process, none for
+// longer than kIdle without use once the library is called again, and all of them are returned to the
+// driver when an allocation fails.  Blocks are handed back only when nothing on the device uses them any
+// more, so any thread and any stream may have them next.
+#include <algorithm>
+#include <chrono>
+#include <list>
+#include <mutex>
+#include <unordered_map>
+
+#include "internal.h"
+
+namespace accerl {
+
+namespace {
+
+constexpr size_t kKept = (size_t)512 << 20;
+constexpr std::chrono::seconds kIdle(30);
+
+struct Block {
+    void *ptr;
+    size_t bytes;
+    int device;
+    std::chrono::steady_clock::time_point since;
+};
+
+struct Memory {
+    std::mutex mu;
+    std::list<Block> kept;  // oldest first
+    size_t kept_bytes = 0;
+    std::unordered_map<void *, std::pair<size_t, int>> live;  // size and device of every block handed out
+
+    void drop_front()
+    {
+        kept_bytes -= kept.front().bytes;
+        cudaFree(kept.front().ptr);
+        kept.pop_front();
+    }
+    void drop_idle()
+    {
+        const auto now = std::chrono::steady_clock::now();
+        while (!kept.empty() && now - kept.front().since > kIdle) drop_front();
+    }
+};
+
+Memory &memory()
+{
+    static Memory *m = new Memory;  // (never destroyed: the driver may be gone before static objects are)
+    return *m;
+}
+
+}  // namespace
+
+cudaError_t device_alloc(void **out, size_t bytes)
+{
+    *out = nullptr;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    bytes = std::max<size_t>(bytes, 1);
+    const size_t grain = bytes < ((size_t)1 << 20) ? (size_t)64 << 10 : (size_t)2 << 20;
+    const size_t want = (bytes + grain - 1) / grain * grain;
+    Memory &m = memory();
+    std::lock_guard<std::mutex> lock(m.mu);
+    m.drop_idle();
+    auto best = m.kept.end();  // the smallest kept block that is not much too large
+    for (auto it = m.kept.begin(); it != m.kept.end(); ++it)
+        if (it->device == device && it->bytes >= want && it->bytes <= want + want / 2 + grain &&
+            (best == m.kept.end() || it->bytes < best->bytes))
+            best = it;
+    if (best != m.kept.end()) {
+        *out = best->ptr;
+        m.live[best->ptr] = {best->bytes, device};
+        m.kept_bytes -= best->bytes;
+        m.kept.erase(best);
+        return cudaSuccess;
+    }
+    e = cudaMalloc(out, want);
+    if (e == cudaErrorMemoryAllocation && !m.kept.empty()) {
+        cudaGetLastError();
+        while (!m.kept.empty()) m.drop_front();
+        e = cudaMalloc(out, want);
+    }
+    if (e == cudaSuccess) m.live[*out] = {want, device};
+    return e;
+}
+
+void device_free(void *ptr)
+{
+    if (!ptr) return;
+    Memory &m = memory();
+    std::lock_guard<std::mutex> lock(m.mu);
+    m.drop_idle();
+    const auto it = m.live.find(ptr);
+    if (it == m.live.end()) return;
+    const auto [bytes, device] = it->second;
+    m.live.erase(it);
+    if (bytes > kKept) {
+        cudaFree(ptr);
+        return;
+    }
+    m.kept.push_back(Block{ptr, bytes, device, std::chrono::steady_clock::now()});
+    m.kept_bytes += bytes;
+    while (m.kept_bytes > kKept) m.drop_front();
+}
+
+}  // namespace accerl

@@ -387,7 +387,7 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
         if (!smaller->mix_rows) {
             void *d = nullptr;
             const size_t bytes = sizeof(int) * (2 * (size_t)mb + 2) + 256;
-            ACCERL_CUDA_TRY(cudaMalloc(&d, bytes));
+            ACCERL_CUDA_TRY(device_alloc(&d, bytes));
             smaller->owned.push_back(d);
             smaller->workspace_bytes += bytes;
             smaller->mix_rows = (int *)d;
@@ -428,7 +428,7 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
         const size_t sz[5] = {4 * mb * (size_t)smaller->n_actions, 4 * mb, 4 * mb, 4 * mb, 4 * mb};
         void *d[5];
         for (int i = 0; i < 5; ++i) {
-            ACCERL_CUDA_TRY(cudaMalloc(&d[i], sz[i] + 256));
+            ACCERL_CUDA_TRY(device_alloc(&d[i], sz[i] + 256));
             smaller->owned.push_back(d[i]);
             smaller->workspace_bytes += sz[i] + 256;
         }

@@ -19,6 +19,10 @@ namespace accerl {
 
 void set_error(const char *fmt, ...);
 
+// device memory (device_memory.cu); device_free only when nothing on the device uses the block any more
+cudaError_t device_alloc(void **out, size_t bytes);
+void device_free(void *ptr);
+
 // let a kernel use `bytes` of dynamic shared memory on the current device (api.cu)
 cudaError_t allow_smem(const void *kernel, size_t bytes);
 

@@ -172,7 +172,11 @@ __global__ void calib_requant_kernel(const int4 *acc, const float *k, const floa
 struct DeviceArena {
     char *base = nullptr;
     size_t at = 0;
-    ~DeviceArena() { cudaFree(base); }
+    ~DeviceArena()
+    {
+        if (base) cudaStreamSynchronize(0);  // (where a call failed, its kernels may still run)
+        device_free(base);
+    }
     template <typename T>
     T *take(size_t count)
     {
@@ -349,7 +353,7 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
         }
         acc = mem.take<int>(acc_elems);
         if (pass == 0) {
-            ACCERL_CUDA_TRY(cudaMalloc(&mem.base, mem.at + 256));
+            ACCERL_CUDA_TRY(device_alloc((void **)&mem.base, mem.at + 256));
             continue;
         }
         ACCERL_CUDA_TRY(cudaMemsetAsync(ymax, 0, (n_layers + 1) * sizeof(float), 0));

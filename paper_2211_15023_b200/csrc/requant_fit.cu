@@ -199,11 +199,15 @@ accerl_status fit_requants(accerl_policy *p, const accerl_layer_desc *layers, in
     }
     struct Device {  // one block of device memory for both steps
         char *ptr = nullptr;
-        ~Device() { cudaFree(ptr); }
+        ~Device()
+        {
+            if (ptr) cudaStreamSynchronize(0);  // (where a call failed, its kernels may still run)
+            device_free(ptr);
+        }
     } dev;
     const size_t job_bytes = (jobs.size() * sizeof(FitJob) + 255) / 256 * 256, res_bytes = (jobs.size() * sizeof(FitResult) + 255) / 256 * 256;
     const size_t div_bytes = ((size_t)n_layers * sizeof(DivJob) + 255) / 256 * 256;
-    ACCERL_CUDA_TRY(cudaMalloc(&dev.ptr, job_bytes + res_bytes + div_bytes + (size_t)n_layers * sizeof(int) + 256));
+    ACCERL_CUDA_TRY(device_alloc((void **)&dev.ptr, job_bytes + res_bytes + div_bytes + (size_t)n_layers * sizeof(int) + 256));
     if (!jobs.empty()) {
         std::vector<FitResult> res(jobs.size());
         ACCERL_CUDA_TRY(cudaMemcpyAsync(dev.ptr, jobs.data(), jobs.size() * sizeof(FitJob), cudaMemcpyHostToDevice, 0));

@@ -225,7 +225,7 @@ int hp_width(int W, int P) { return slot_pw(W) / P * (P / 2); }
 accerl_status alloc_zeroed(accerl_policy *p, size_t bytes, int8_t **out)
 {
     void *d = nullptr;
-    ACCERL_CUDA_TRY(cudaMalloc(&d, bytes + 4096));  // slack: TMA boxes may start before the tail
+    ACCERL_CUDA_TRY(device_alloc(&d, bytes + 4096));  // slack: TMA boxes may start before the tail
     p->owned.push_back(d);
     p->workspace_bytes += bytes + 4096;
     ACCERL_CUDA_TRY(cudaMemset(d, 0, bytes + 4096));

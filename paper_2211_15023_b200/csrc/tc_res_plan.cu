@@ -114,7 +114,7 @@ accerl_status build_res_steps(accerl_policy *p, const accerl_layer_desc *layers,
     int8_t *x[3];
     for (int i = 0; i < 3; ++i) {
         void *d = nullptr;
-        ACCERL_CUDA_TRY(cudaMalloc(&d, bytes[i] + 4096));
+        ACCERL_CUDA_TRY(device_alloc(&d, bytes[i] + 4096));
         p->owned.push_back(d);
         p->workspace_bytes += bytes[i] + 4096;
         x[i] = (int8_t *)d;
