@@ -483,9 +483,7 @@ void accerl_policy_destroy(accerl_policy *p)
     for (cudaEvent_t ev : p->events) cudaEventDestroy(ev);
     for (cudaEvent_t ev : p->copy_events) cudaEventDestroy(ev);
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
-    for (cudaEvent_t ev : p->mix_events)
-        if (ev) cudaEventDestroy(ev);
-    if (p->mix_stream) cudaStreamDestroy(p->mix_stream);
+    give_side_stream(p->mix);
     delete p->noalloc_twin;  // owns nothing on the device
     delete p;
 }

@@ -11,6 +11,7 @@
 #include <list>
 #include <mutex>
 #include <unordered_map>
+#include <vector>
 
 #include "internal.h"
 
@@ -53,7 +54,61 @@ Memory &memory()
     return *m;
 }
 
+// side streams not in use (creating one, with its events, takes a tenth of a millisecond)
+constexpr size_t kKeptStreams = 8;
+std::mutex g_stream_mu;
+std::vector<SideStream> &kept_streams()
+{
+    static std::vector<SideStream> *v = new std::vector<SideStream>;  // (as above)
+    return *v;
+}
+
 }  // namespace
+
+cudaError_t take_side_stream(SideStream *out)
+{
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lock(g_stream_mu);
+        std::vector<SideStream> &kept = kept_streams();
+        for (size_t i = 0; i < kept.size(); ++i)
+            if (kept[i].device == device) {
+                *out = kept[i];
+                kept.erase(kept.begin() + (long)i);
+                return cudaSuccess;
+            }
+    }
+    SideStream s;
+    s.device = device;
+    for (cudaEvent_t &ev : s.events)
+        if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) break;
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+        *out = s;
+        return e;
+    }
+    for (cudaEvent_t ev : s.events)
+        if (ev) cudaEventDestroy(ev);
+    return e;
+}
+
+void give_side_stream(SideStream &s)
+{
+    if (!s.stream) return;
+    {
+        std::lock_guard<std::mutex> lock(g_stream_mu);
+        if (kept_streams().size() < kKeptStreams) {
+            kept_streams().push_back(s);
+            s = SideStream();
+            return;
+        }
+    }
+    for (cudaEvent_t ev : s.events) cudaEventDestroy(ev);
+    cudaStreamDestroy(s.stream);
+    s = SideStream();
+}
 
 cudaError_t device_alloc(void **out, size_t bytes)
 {

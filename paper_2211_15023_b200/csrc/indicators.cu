@@ -397,12 +397,9 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
         ACCERL_CUDA_TRY(cudaGetLastError());
         // The two networks share nothing but the lists: side by side on two streams their small launches
         // fill each other's gaps (one after the other: 88 us for the case above).
-        if (!smaller->mix_stream) {
-            for (cudaEvent_t &ev : smaller->mix_events) ACCERL_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-            ACCERL_CUDA_TRY(cudaStreamCreateWithFlags(&smaller->mix_stream, cudaStreamNonBlocking));
-        }
-        ACCERL_CUDA_TRY(cudaEventRecord(smaller->mix_events[0], st));
-        ACCERL_CUDA_TRY(cudaStreamWaitEvent(smaller->mix_stream, smaller->mix_events[0], 0));
+        if (!smaller->mix.stream) ACCERL_CUDA_TRY(take_side_stream(&smaller->mix));
+        ACCERL_CUDA_TRY(cudaEventRecord(smaller->mix.events[0], st));
+        ACCERL_CUDA_TRY(cudaStreamWaitEvent(smaller->mix.stream, smaller->mix.events[0], 0));
         accerl_status result = ACCERL_OK;
         for (int i = 1; i >= 0; --i) {
             Route r;
@@ -410,12 +407,12 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
             r.count = rows + 2 * (size_t)mb + i;
             r.expect = (int)ceilf((float)batch * (i ? 1.f - alpha : alpha));
             accerl_status s = run_steps(i ? original : smaller, obs_dev, uniforms_dev, batch, logits_dev, actions_dev, logp_dev,
-                                        value_dev, entropy_dev, i ? st : smaller->mix_stream, nullptr, r);
+                                        value_dev, entropy_dev, i ? st : smaller->mix.stream, nullptr, r);
             if (result == ACCERL_OK) result = s;
         }
         smaller->last_stream = st;  // (which waits for the other)
-        ACCERL_CUDA_TRY(cudaEventRecord(smaller->mix_events[1], smaller->mix_stream));
-        ACCERL_CUDA_TRY(cudaStreamWaitEvent(st, smaller->mix_events[1], 0));
+        ACCERL_CUDA_TRY(cudaEventRecord(smaller->mix.events[1], smaller->mix.stream));
+        ACCERL_CUDA_TRY(cudaStreamWaitEvent(st, smaller->mix.events[1], 0));
         if (result != ACCERL_OK) return result;
         return ACCERL_OK;
     }

@@ -23,6 +23,15 @@ void set_error(const char *fmt, ...);
 cudaError_t device_alloc(void **out, size_t bytes);
 void device_free(void *ptr);
 
+// a non-blocking stream of the library's own with two events, on the current device; given back idle
+struct SideStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t events[2] = {nullptr, nullptr};
+    int device = 0;
+};
+cudaError_t take_side_stream(SideStream *out);
+void give_side_stream(SideStream &s);
+
 // let a kernel use `bytes` of dynamic shared memory on the current device (api.cu)
 cudaError_t allow_smem(const void *kernel, size_t bytes);
 
@@ -232,8 +241,7 @@ struct accerl_policy {
     // outputs of this policy inside accerl_policy_act_mixed (allocated on its first call)
     float *mix_logits = nullptr, *mix_logp = nullptr, *mix_value = nullptr, *mix_entropy = nullptr;
     int32_t *mix_actions = nullptr;
-    cudaStream_t mix_stream = nullptr;            // the smaller network's launches
-    cudaEvent_t mix_events[2] = {nullptr, nullptr};
+    accerl::SideStream mix;   // the smaller network's launches
     int *mix_rows = nullptr;  // [2][max_batch] states of each network, then their counts
 };
 

@@ -123,8 +123,8 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
     q->owned.clear();
     q->events.clear();
     q->copy_events.clear();
-    q->copy_stream = q->mix_stream = nullptr;
-    q->mix_events[0] = q->mix_events[1] = nullptr;
+    q->copy_stream = nullptr;
+    q->mix = SideStream();
     q->ptq.clear();
     q->max_batch = (int)cap;
     bool ok = true;
