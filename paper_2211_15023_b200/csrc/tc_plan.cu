@@ -210,9 +210,9 @@ bool conv_fits(const accerl_layer_desc &d)
 
 // The Atari conv stack as one launch (tc_atari.cu): handles for up to this many states.  Above, the
 // launches per layer are faster: their tiles span images, a third of that kernel's tensor work is padding
-// rows.  (us per step, per layer / one launch: 32 / 64 / 64 channels 26.4 / 21.4 at 160 states, 34.4 / 32.4 at
-// 700, 43.5 / 46.2 at 1237; 16 / 32 / 32 channels 25.5 / 17.4, 37.1 / 33.1 at 1237, 70.3 / 79.3 at 4096.)
-constexpr int kAtariMaxWide = 800, kAtariMaxNarrow = 2048;
+// rows.  (us per step, per layer / one launch: 32 / 64 / 64 channels 43.5 / 42.2 at 1237 states, 60.6 / 57.8 at
+// 2048, 143 / 167 at 8192; 16 / 32 / 32 channels 47.2 / 39.2 at 2048, 112 / 111 at 8192.)
+constexpr int kAtariMaxWide = 2560, kAtariMaxNarrow = 6144;
 
 // byte offset of byte kk of row n of an operand with rb-byte rows under the rb-byte swizzle
 size_t swizzled(int n, int kk, int rb)

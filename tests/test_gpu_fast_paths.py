@@ -167,3 +167,21 @@ def test_mixing_routes_every_state_through_its_network(small, orig, b, alpha):
             assert torch.equal(out[k], torch.where(m, a[k], o[k])), k
     gs.close()
     go.close()
+
+
+@pytest.mark.parametrize("name,b", [("nature_cnn_b160", 149), ("nature_cnn_b160", 297), ("nature_cnn_b160", 600),
+                                    ("student_cnn_b8192", 148), ("student_cnn_b8192", 745)])
+def test_atari_kernel_with_one_two_and_three_images_per_context(name, b):
+    """Batches around one, two and three images per SM and beyond, where CTAs have one to three contexts
+    and contexts one to three images, some CTAs one image less than others."""
+    import paper_2211_15023_b200 as P
+    pol = W.drawn_int8_policy(name, seed=11)
+    obs, u = W.observations(name, b, seed=b), W.uniforms(name, b, seed=b)
+    ref = oracle.forward(pol, obs, u, keep=False)
+    g = P.Policy(pol, b)
+    assert "atari_kernel" in g.info()["plan"]
+    for _ in range(2):
+        out = [t.cpu().numpy() for t in g.act(torch.from_numpy(obs).cuda(), torch.from_numpy(u).cuda())]
+        g.check()
+        compare(ref, *out)
+    g.close()
