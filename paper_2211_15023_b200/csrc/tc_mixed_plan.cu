@@ -783,7 +783,7 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
             g.bias = (const float *)bd;
             g.affine = 1;
         }
-        g.split_cols = (g.n_tile > 128 || (role[i] == TCFIRST && hpool_first) || hp_out) ? 1 : 0;
+        g.split_cols = ((g.n_tile > 128 && g.n_tile % 64 == 0) || (role[i] == TCFIRST && hpool_first) || hp_out) ? 1 : 0;
         // (a multi-pixel layer whose output scale fails the division check keeps its place in the plan:
         // its launch runs the epilogue that re-does elements near a rounding tie with the IEEE divide)
         if (hp_out) {

@@ -462,7 +462,9 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
             g.affine = 1;
         }
         const char *requant_note = g.affine ? "[single-fma requantiser verified]" : "[3-step divide verified]";
-        g.split_cols = g.n_tile >= 128 ? 1 : 0;  // 128 / 256 columns: 32 / 64 per warpgroup
+        // wide tiles: a quarter of the columns per warpgroup, where that is whole 16-column pieces (a quarter of
+        // 240 would put 16-byte stores at byte 60)
+        g.split_cols = (g.n_tile >= 128 && g.n_tile % 64 == 0) ? 1 : 0;
         g.out = L.out_buf >= 0 ? p->bufs[L.out_buf].ptr : nullptr;
         g.logits_mode = logits ? 1 : 0;
         g.n_actions = p->n_out;  // columns of the fp32 rows the logits layer writes

@@ -185,3 +185,24 @@ def test_atari_kernel_with_one_two_and_three_images_per_context(name, b):
         g.check()
         compare(ref, *out)
     g.close()
+
+
+@pytest.mark.parametrize("hidden,actions,value,b", [(16, 1, False, 1), (80, 8, False, 17), (512, 7, True, 449), (48, 9, False, 31),
+                                                    (240, 16, False, 100), (64, 24, True, 15), (128, 31, True, 65), (144, 32, False, 16)])
+def test_last_layer_and_sampler_widths(hidden, actions, value, b):
+    """The launch of the last layer and the sampler on widths at the edges of its instructions' K and column
+    tiles, states that are no multiple of the sixteen of a warp, with and without a value column."""
+    name = "student_cnn_b8192"
+    layers = W.nature_cnn(16, 32, 32, hidden, actions=actions)
+    if value:
+        layers = W.with_value_head(layers)
+    pol = oracle.calibrate("u8", (4, 84, 84), layers, W.parameters_for(layers, hidden), W.calibration_batch(name, 16))
+    obs, u = W.observations(name, b, seed=b), W.uniforms(name, b, seed=b)
+    ref = oracle.forward(pol, obs, u, keep=False)
+    import paper_2211_15023_b200 as P
+    g = P.Policy(pol, b)
+    assert "fc_sample_kernel covers layer 4+sample" in g.info()["plan"]
+    out = {k: v.cpu().numpy() for k, v in g.act_ex(torch.from_numpy(obs).cuda(), torch.from_numpy(u).cuda()).items()}
+    g.check()
+    compare(ref, out["logits"], out["actions"], out["logp"], value=out.get("value"), entropy=out["entropy"])
+    g.close()
