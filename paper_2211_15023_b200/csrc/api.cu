@@ -233,7 +233,7 @@ void set_routed_steps(accerl_policy *p, const std::vector<Step> &front)
     if (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) return;
     std::vector<Step> r = front;
     for (const Step &s : p->steps) {
-        const bool fc = s.kind == Step::FC_HEAD || s.kind == Step::FC_SAMPLE ||
+        const bool fc = s.kind == Step::FC_HEAD || s.kind == Step::FC_TILE || s.kind == Step::FC_SAMPLE ||
                         (s.kind == Step::TC_GEMM && p->layers[s.layer].kind == ACCERL_FC && !p->tc_steps[s.tc].prm.logits_mode);
         if (fc) r.push_back(s);
         else if (s.kind == Step::SAMPLE) return;  // (wide action sets sample from a logits matrix)
@@ -452,6 +452,10 @@ accerl_status accerl::run_steps(accerl_policy *p, const void *obs_dev, const flo
             break;
         case Step::FC_HEAD:
             ACCERL_CUDA_TRY(launch_fc_head(p->fc_head, p->fc_sample, uniforms_dev, B, logits_dev, actions_dev, logp_dev,
+                                           value_dev, entropy_dev, route, p->sm_count, st));
+            break;
+        case Step::FC_TILE:
+            ACCERL_CUDA_TRY(launch_fc_tile(p->fc_tile_map, p->fc_tile, p->fc_sample, uniforms_dev, B, logits_dev, actions_dev, logp_dev,
                                            value_dev, entropy_dev, route, p->sm_count, st));
             break;
         case Step::FC_SAMPLE:

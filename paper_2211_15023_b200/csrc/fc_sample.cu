@@ -13,45 +13,13 @@
 
 #include "epilogue.cuh"
 #include "internal.h"
+#include "warp_sample.cuh"
 
 namespace accerl {
 
 namespace {
 
 constexpr int kFsWarps = 8;
-
-// One row per warp, one lane per action: the arithmetic of sample_warp_kernel for a full-warp
-// segment.  Every lane returns the drawn action and its log-prob.
-template <bool ENTROPY>
-__device__ __forceinline__ void warp_sample(float z, bool live, float uu, int A, int lane, int &a,
-                                            float &lpa, float &h)
-{
-    if (!live) z = -INFINITY;
-    float m = z;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    // the first maximal lane contributes exp(0) = 1 exactly: sum the others, take log1p
-    const unsigned ismax = __ballot_sync(0xffffffffu, live && z == m);
-    const int amax = ismax ? __ffs(ismax) - 1 : 0;
-    float s = (live && lane != amax) ? expf(z - m) : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float lp = live ? (z - m) - log1pf(s) : 0.f;
-    float cdf = live ? expf(lp) : 0.f;  // inclusive scan
-    if (ENTROPY) {  // H = -sum p log p
-        h = cdf > 0.f ? -cdf * lp : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
-    }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float v = __shfl_up_sync(0xffffffffu, cdf, o);
-        if (lane >= o) cdf += v;
-    }
-    const unsigned hit = __ballot_sync(0xffffffffu, live && uu < cdf);
-    a = hit ? __ffs(hit) - 1 : A - 1;
-    lpa = __shfl_sync(0xffffffffu, lp, a);
-}
 
 // EXTRAS: the states may be routed (Route); the layer may have one output column more than actions, the state value V(s) (lane A;
 // no part of the softmax), and the entropy of the action distribution may be asked for.
@@ -347,10 +315,11 @@ accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int 
     return ACCERL_OK;
 }
 
-// Do the hidden layer `i` and the last one behind it run as that launch?  Handles for more states stay
-// with the two launches, whose 128-row tiles read the weights less often (us per step, two launches /
-// one: 512 outputs of 3136 inputs 21.4 / 16.0 at 160 states, 27.3 / 26.9 at 450, 32.5 / 42.0 at 700; 256 of
-// 1568 17.1 / 11.2, 20.4 / 16.9, 24.0 / 24.6).
+// Do the hidden layer `i` and the last one behind it run as that launch?  Handles for more states end in
+// tiles of 128 (fc_tile.cu), which read the weights less often, or in two launches.  The line lies where this
+// launch's clusters no longer fit the chip at once, with 16 states each for 512 outputs, 32 for 256 (us per
+// step, this launch / tiles: 512 outputs of 3136 inputs 15.4 / 19.3 at 160 states, 22.1 / 20.3 at 256; 256 of 1568
+// 11.0 / 13.6, 15.9 / 17.4 at 448, 22.3 / 18.7 at 640).
 bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i)
 {
     if (i != n_layers - 2 || i < 1 || unfuse_for_taps(p) || p->max_batch > (layers[i].out_c == 512 ? kFcHeadMaxWide : kFcHeadMaxNarrow) || !fc_sample_fits(p, layers, n_layers, i + 1))
@@ -417,8 +386,9 @@ cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const
         cfg.numAttrs = 2;
         return cudaLaunchKernelEx(&cfg, kernel, h, q, u, B, route, logits, actions, logp, value, entropy);
     };
-    // 16 states per cluster while their clusters fit the chip once
-    const bool two = ((route.count ? route.expect : B) + 15) / 16 * kHeadCluster > sm_count;
+    // 16 states per cluster while their clusters fit the chip once: 15 clusters of eight find their SMs (one less
+    // here, see launch_fc_tile); with 16, at 256 states, a step of the narrow network took 15.4 us, with half as many 12.9
+    const bool two = ((route.count ? route.expect : B) + 15) / 16 > sm_count / 10;
     if (h.N == 512) return two ? go(fc_hidden_fc_sample_kernel<2, 8>, 32) : go(fc_hidden_fc_sample_kernel<1, 8>, 16);
     return two ? go(fc_hidden_fc_sample_kernel<2, 4>, 32) : go(fc_hidden_fc_sample_kernel<1, 4>, 16);
 }

@@ -73,7 +73,7 @@ struct LayerPlan {
 struct Step {
     enum Kind { INGEST, CONV_GENERIC, FC_GENERIC, POOL_GENERIC, SAMPLE, INGEST_S2D, TC_GEMM, MLP_FUSED,
                 INGEST_NHWC4, POOL_DUAL, INGEST_PAD4, FC_SAMPLE, CONV1_FRAMES, CONV_ROWS, RES_FIRST,
-                RES_STACK1, RES_STACK23, ATARI, FC_HEAD } kind;
+                RES_STACK1, RES_STACK23, ATARI, FC_HEAD, FC_TILE } kind;
     int layer = -1;
     int tc = -1;  // index into accerl_policy::tc_steps (TC_GEMM), ::pools (POOL_DUAL) or ::conv_rows (CONV_ROWS)
     std::string kernel, covers;
@@ -124,7 +124,17 @@ struct FcHeadParams {
     float s_out;
     int8_t *tap;      // parity tap of its output, or null
 };
-constexpr int kFcHeadMaxWide = 448, kFcHeadMaxNarrow = 640;  // states, for 512 and 256 outputs
+constexpr int kFcHeadMaxWide = 224, kFcHeadMaxNarrow = 448;  // states, for 512 and 256 outputs
+
+// the same for more states (fc_tile.cu)
+struct FcTileParams {
+    const uint8_t *w;     // [chunks][N][128 bytes of K, swizzled]
+    int chunks, N, relu, affine;
+    const float *k, *b;   // per column: the single-fma pair, or (s_in * s_w, bias) for the division
+    float s_out, inv_s_out;
+    int8_t *tap;          // parity tap of its output, or null
+    int *status;
+};
 
 // max-pool that writes a plain NHWC output and / or a padded-border one (tc_mixed_plan.cu)
 struct PoolOut {  // one stored form of the pooled tensor
@@ -202,8 +212,11 @@ struct accerl_policy {
     std::vector<accerl::TapDesc> taps;    // per tensor (index t + 1); empty or null ptr = generic buffer
     std::vector<char> tap_missing;        // per tensor (index t + 1): the plan never stores it (TAP_FUSED)
     std::shared_ptr<accerl::MlpFusedParams> mlp;  // set when the whole step is one fused launch
-    accerl::FcSampleParams fc_sample = {};         // used by a Step::FC_SAMPLE or FC_HEAD launch
+    accerl::FcSampleParams fc_sample = {};         // used by a Step::FC_SAMPLE, FC_HEAD or FC_TILE launch
     accerl::FcHeadParams fc_head = {};             // used by a Step::FC_HEAD launch
+    accerl::FcTileParams fc_tile = {};             // used by a Step::FC_TILE launch
+    alignas(64) unsigned char fc_tile_map[128] = {};
+    accerl::ActivationMap fc_tile_a;
     std::vector<int> tensor_s2d;          // space-to-depth factor of tensor t at [t + 1]
     int sm_count = 0;
     std::vector<accerl::DeviceBuf> bufs;  // bufs[0] holds the quantised input
@@ -314,6 +327,11 @@ accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int 
 bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
 accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out);
 cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const float *u, int B, float *logits,
+                           int32_t *actions, float *logp, float *value, float *entropy, const Route &route, int sm_count,
+                           cudaStream_t st);
+bool fc_tile_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
+accerl_status build_fc_tile(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out);
+cudaError_t launch_fc_tile(const void *map_x, const FcTileParams &h, const FcSampleParams &q, const float *u, int B, float *logits,
                            int32_t *actions, float *logp, float *value, float *entropy, const Route &route, int sm_count,
                            cudaStream_t st);
 cudaError_t launch_fc_sample(const FcSampleParams &q, const float *u, int B, float *logits,

@@ -78,7 +78,7 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
         switch (s.kind) {
         case Step::RES_FIRST: resident = true; break;
         case Step::RES_STACK1: case Step::RES_STACK23: case Step::MLP_FUSED: case Step::CONV1_FRAMES: case Step::CONV_ROWS: case Step::ATARI:
-        case Step::FC_SAMPLE: case Step::FC_HEAD: case Step::SAMPLE: break;
+        case Step::FC_SAMPLE: case Step::FC_HEAD: case Step::FC_TILE: case Step::SAMPLE: break;
         case Step::TC_GEMM: {
             const TcGemmParams &g = p->tc_steps[s.tc].prm;  // no padded layouts, no residual or second output
             if (g.out2 || g.skip || g.px_per_row || g.out_row_off) return nullptr;
@@ -157,6 +157,8 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
             move(q->atari.out);
         } else if (s.kind == Step::FC_HEAD) {
             move(q->fc_head.x);
+        } else if (s.kind == Step::FC_TILE) {
+            remap(q->fc_tile_map, q->fc_tile_a);
         } else if (s.kind == Step::FC_SAMPLE) {
             move(q->fc_sample.x);
         } else if (s.kind == Step::RES_FIRST) {

@@ -496,9 +496,10 @@ accerl_status build_tc_mixed_plan(accerl_policy *p, const accerl_layer_desc *lay
             steps.push_back(s);
             continue;
         }
-        if (role[i] == TCFC && fc_head_fits(p, layers, n_layers, i)) {
+        const bool head = role[i] == TCFC && fc_head_fits(p, layers, n_layers, i);
+        if (head || (role[i] == TCFC && fc_tile_fits(p, layers, n_layers, i))) {
             const bool relu_in = (d.flags & ACCERL_RELU_IN) && !(layers[i - 1].flags & ACCERL_RELU_OUT);
-            if ((st = build_fc_head(p, layers, i, relu_in ? fin.p_plain_relu : fin.p_plain, &s)) != ACCERL_OK) return st;
+            if ((st = (head ? build_fc_head : build_fc_tile)(p, layers, i, relu_in ? fin.p_plain_relu : fin.p_plain, &s)) != ACCERL_OK) return st;
             s.layer = -1;
             steps.push_back(s);
             fused_sample = true;

@@ -352,9 +352,10 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
     for (int i = atari_small ? 3 : 0; i < n_layers; ++i) {
         const accerl_layer_desc &d = layers[i];
         const LayerPlan &L = p->layers[i];
-        if (fc_head_fits(p, layers, n_layers, i)) {  // the last two layers and the sampler
+        const bool head = fc_head_fits(p, layers, n_layers, i);
+        if (head || fc_tile_fits(p, layers, n_layers, i)) {  // the last two layers and the sampler
             Step hs;
-            accerl_status hst = build_fc_head(p, layers, i, p->bufs[L.in_buf].ptr, &hs);
+            accerl_status hst = (head ? build_fc_head : build_fc_tile)(p, layers, i, p->bufs[L.in_buf].ptr, &hs);
             if (hst != ACCERL_OK) return hst;
             steps.push_back(hs);
             fused_sample = true;

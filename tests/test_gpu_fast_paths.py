@@ -204,7 +204,7 @@ def test_atari_kernel_with_one_two_and_three_images_per_context(name, b):
     g.close()
 
 
-@pytest.mark.parametrize("hidden,actions,value,b", [(16, 1, False, 1), (80, 8, False, 17), (512, 7, True, 449), (48, 9, False, 31),
+@pytest.mark.parametrize("hidden,actions,value,b", [(16, 1, False, 1), (80, 8, False, 17), (208, 7, True, 449), (48, 9, False, 31),
                                                     (240, 16, False, 100), (64, 24, True, 15), (128, 31, True, 65), (144, 32, False, 16)])
 def test_last_layer_and_sampler_widths(hidden, actions, value, b):
     """The launch of the last layer and the sampler on widths at the edges of its instructions' K and column
@@ -222,4 +222,43 @@ def test_last_layer_and_sampler_widths(hidden, actions, value, b):
     out = {k: v.cpu().numpy() for k, v in g.act_ex(torch.from_numpy(obs).cuda(), torch.from_numpy(u).cuda()).items()}
     g.check()
     compare(ref, out["logits"], out["actions"], out["logp"], value=out.get("value"), entropy=out["entropy"])
+    g.close()
+
+
+@pytest.mark.parametrize("hidden,actions,value,b", [(256, 18, False, 641), (256, 3, True, 2049), (256, 32, False, 4737), (256, 8, True, 9473),
+                                                    (512, 18, True, 449), (512, 31, False, 2176), (512, 6, False, 4737), (512, 5, False, 9500)])
+def test_hidden_layer_last_layer_and_sampler_in_tiles(hidden, actions, value, b):
+    """The launch that ends larger steps at every number of CTAs per tile of states, ragged last tiles, and one
+    state more than it takes (9500 of 512 outputs); device calls, the fixed workspace and routed states."""
+    import paper_2211_15023_b200 as P
+    name, n = "student_cnn_b8192", 300
+    layers = W.nature_cnn(16, 32, 32, hidden, actions=actions)
+    if value:
+        layers = W.with_value_head(layers)
+    pol = oracle.calibrate("u8", (4, 84, 84), layers, W.parameters_for(layers, hidden), W.calibration_batch(name, 16))
+    obs, u = W.observations(name, n, seed=b), W.uniforms(name, n, seed=b)
+    ref = oracle.forward(pol, obs, u, keep=False)
+    at = np.random.default_rng(b).integers(0, n, b)  # the states of the batch, drawn from those
+    ref = {k: v[at] if isinstance(v, np.ndarray) and len(v) == n else v for k, v in ref.items()}
+    g = P.Policy(pol, b)
+    assert ("fc_tile_fc_sample_kernel" in g.info()["plan"]) == (b != 9500)
+    obs, u = torch.from_numpy(obs).cuda()[torch.from_numpy(at).cuda()], torch.from_numpy(u[at]).cuda()
+    res = g.act_ex(obs, u)
+    g.check()
+    out = {k: v.cpu().numpy() for k, v in res.items()}
+    compare(ref, out["logits"], out["actions"], out["logp"], value=out.get("value"), entropy=out["entropy"])
+    if b < 1000:  # (the fixed workspace ends at some 1600 of them)
+        got = [torch.empty_like(res[k]) for k in ("logits", "actions", "logp")]
+        stream = torch.cuda.current_stream().cuda_stream
+        assert g.act_noalloc_raw(obs.data_ptr(), u.data_ptr(), b, *(t.data_ptr() for t in got), stream) == 0
+        for k, t in zip(("logits", "actions", "logp"), got):
+            assert torch.equal(t, res[k]), k
+    if b <= 2176:
+        other = P.Policy(pol, b)
+        mixed = P.act_mixed(g, other, obs, u, torch.rand(b, device="cuda"), 0.4)
+        g.check()
+        other.check()
+        for k in ("logits", "actions", "logp"):
+            assert torch.equal(mixed[k], res[k]), k
+        other.close()
     g.close()
