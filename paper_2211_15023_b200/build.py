@@ -17,7 +17,7 @@ CALLS = os.path.join(HERE, "_calls.so")
 
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-         "-Xcompiler", "-fPIC,-ffp-contract=off,-fno-fast-math", "-cudart", "static",
+         "-Xcompiler", "-fPIC,-ffp-contract=off,-fno-fast-math,-falign-functions=64,-falign-loops=32", "-cudart", "static",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 
 

@@ -241,7 +241,7 @@ void set_routed_steps(accerl_policy *p, const std::vector<Step> &front)
     p->routed_steps = r;
 }
 
-accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev)
+accerl_status upload_room(accerl_policy *p, size_t bytes, void **host, void **dev)
 {
     *dev = nullptr;
     const size_t need = (bytes + 255) / 256 * 256 + 256;
@@ -256,10 +256,18 @@ accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, voi
         p->uploads.push_back(std::move(b));
     }
     UploadBlock &b = p->uploads.back();
-    if (bytes) memcpy(b.host.data() + b.used, host, bytes);
+    *host = b.host.data() + b.used;
     *dev = b.dev + b.used;
     b.used += need;
     return ACCERL_OK;
+}
+
+accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev)
+{
+    void *to = nullptr;
+    const accerl_status st = upload_room(p, bytes, &to, dev);
+    if (st == ACCERL_OK && bytes) memcpy(to, host, bytes);
+    return st;
 }
 
 accerl_status flush_uploads(accerl_policy *p)

@@ -336,14 +336,14 @@ accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, i
     const LayerPlan &L = p->layers[i];
     const int K = L.in_h * L.in_w * L.in_cp, N = d.out_c, pieces = (K + 63) / 64;
     // [piece][column / 8][lane 4 g + t]: bytes 16 t .. 16 t + 15 of the piece, column g
-    std::vector<int8_t> w((size_t)pieces * N * 64, 0);
     const int8_t *rows = reinterpret_cast<const int8_t *>(L.host_words.data());
-    for (int o = 0; o < N; ++o)
-        for (int k = 0; k < K; k += 16)
-            memcpy(&w[(((size_t)(k / 64) * (N / 8) + o / 8) * 32 + 4 * (o % 8) + (k % 64) / 16) * 16], rows + (size_t)o * K + k, 16);
-    void *dev = nullptr;
-    accerl_status st = upload_bytes(p, w.data(), w.size(), &dev);
+    void *dev = nullptr, *host = nullptr;
+    accerl_status st = upload_room(p, (size_t)pieces * N * 64, &host, &dev);
     if (st != ACCERL_OK) return st;
+    int8_t *at = (int8_t *)host;
+    for (int k0 = 0; k0 < K; k0 += 64)
+        for (int o = 0; o < N; ++o, at += 64)
+            for (int k = k0; k < K && k < k0 + 64; k += 16) memcpy(at + (k - k0), rows + (size_t)o * K + k, 16);
     FcHeadParams &h = p->fc_head;
     h.x = x;
     h.w = (const uint4 *)dev;

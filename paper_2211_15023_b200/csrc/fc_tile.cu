@@ -270,14 +270,15 @@ accerl_status build_fc_tile(accerl_policy *p, const accerl_layer_desc *layers, i
     const LayerRequant &rq = p->requant[i];
     const int K = L.in_h * L.in_w * L.in_cp, N = d.out_c, chunks = (K + 127) / 128;
     // [chunk of K][column][128 bytes under the 128-byte swizzle]
-    std::vector<int8_t> w((size_t)chunks * N * 128, 0);
     const int8_t *rows = reinterpret_cast<const int8_t *>(L.host_words.data());
-    for (int o = 0; o < N; ++o)
-        for (int k = 0; k < K; k += 16)
-            memcpy(&w[((size_t)(k / 128) * N + o) * 128 + (((k % 128 / 16) ^ (o & 7)) << 4)], rows + (size_t)o * K + k, 16);
-    void *w_dev = nullptr, *k_dev = nullptr, *b_dev = nullptr;
-    accerl_status st = upload_bytes(p, w.data(), w.size(), &w_dev);
-    if (st == ACCERL_OK) st = upload_bytes(p, rq.k.data(), (size_t)N * 4, &k_dev);
+    void *w_host = nullptr, *w_dev = nullptr, *k_dev = nullptr, *b_dev = nullptr;
+    accerl_status st = upload_room(p, (size_t)chunks * N * 128, &w_host, &w_dev);
+    if (st != ACCERL_OK) return st;
+    int8_t *at = (int8_t *)w_host;
+    for (int k0 = 0; k0 < K; k0 += 128)
+        for (int o = 0; o < N; ++o, at += 128)
+            for (int k = k0; k < K && k < k0 + 128; k += 16) memcpy(at + ((((k - k0) / 16) ^ (o & 7)) << 4), rows + (size_t)o * K + k, 16);
+    st = upload_bytes(p, rq.k.data(), (size_t)N * 4, &k_dev);
     if (st == ACCERL_OK) st = upload_bytes(p, rq.b.data(), (size_t)N * 4, &b_dev);
     if (st != ACCERL_OK) return st;
     p->fc_tile_a = ActivationMap{x, 1, K, K, 128, 128};

@@ -320,6 +320,8 @@ cudaError_t launch_mlp_fused(const accerl_policy *p, const float *obs, const flo
 // fills p->routed_steps from the finished plan: `front`, then the plan's fully connected launches
 void set_routed_steps(accerl_policy *p, const std::vector<Step> &front);
 accerl_status upload_bytes(accerl_policy *p, const void *host, size_t bytes, void **dev);  // there once create is done
+// room for the same, zeroed, to be filled in place before the next call of either
+accerl_status upload_room(accerl_policy *p, size_t bytes, void **host, void **dev);
 accerl_status flush_uploads(accerl_policy *p);
 bool fc_sample_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i);
 accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int layer, const int8_t *x,
