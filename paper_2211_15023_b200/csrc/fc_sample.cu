@@ -329,14 +329,14 @@ bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n
     return d.kind == ACCERL_FC && (d.out_c == 256 || d.out_c == 512) && L.in_cp == L.in_c && (L.in_h * L.in_w * L.in_cp) % 16 == 0;
 }
 
-// x: the hidden layer's input rows; its weights in (y, x, c) order are L.host_words
+// x: the hidden layer's input rows; its weights in (y, x, c) order are L.host_rows
 accerl_status build_fc_head(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out)
 {
     const accerl_layer_desc &d = layers[i];
     const LayerPlan &L = p->layers[i];
     const int K = L.in_h * L.in_w * L.in_cp, N = d.out_c, pieces = (K + 63) / 64;
     // [piece][column / 8][lane 4 g + t]: bytes 16 t .. 16 t + 15 of the piece, column g
-    const int8_t *rows = reinterpret_cast<const int8_t *>(L.host_words.data());
+    const int8_t *rows = L.host_rows;
     void *dev = nullptr, *host = nullptr;
     accerl_status st = upload_room(p, (size_t)pieces * N * 64, &host, &dev);
     if (st != ACCERL_OK) return st;

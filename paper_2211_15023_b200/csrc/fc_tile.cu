@@ -262,7 +262,7 @@ bool fc_tile_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n
            (long long)(p->max_batch + 127) / 128 * (d.out_c / 256) <= p->sm_count;
 }
 
-// x: the hidden layer's input rows; its weights in (y, x, c) order are L.host_words
+// x: the hidden layer's input rows; its weights in (y, x, c) order are L.host_rows
 accerl_status build_fc_tile(accerl_policy *p, const accerl_layer_desc *layers, int i, const int8_t *x, Step *out)
 {
     const accerl_layer_desc &d = layers[i];
@@ -270,7 +270,7 @@ accerl_status build_fc_tile(accerl_policy *p, const accerl_layer_desc *layers, i
     const LayerRequant &rq = p->requant[i];
     const int K = L.in_h * L.in_w * L.in_cp, N = d.out_c, chunks = (K + 127) / 128;
     // [chunk of K][column][128 bytes under the 128-byte swizzle]
-    const int8_t *rows = reinterpret_cast<const int8_t *>(L.host_words.data());
+    const int8_t *rows = L.host_rows;
     void *w_host = nullptr, *w_dev = nullptr, *k_dev = nullptr, *b_dev = nullptr;
     accerl_status st = upload_room(p, (size_t)chunks * N * 128, &w_host, &w_dev);
     if (st != ACCERL_OK) return st;

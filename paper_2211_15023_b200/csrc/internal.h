@@ -22,6 +22,8 @@ void set_error(const char *fmt, ...);
 // device memory (device_memory.cu); device_free only when nothing on the device uses the block any more
 cudaError_t device_alloc(void **out, size_t bytes);
 void device_free(void *ptr);
+// pinned host memory in the same manner; given up only when no copy of it is in flight
+cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes);
 
 // a non-blocking stream of the library's own with two events, on the current device; given back idle
 struct SideStream {
@@ -65,7 +67,7 @@ struct LayerPlan {
     int32_t *skip_mul = nullptr;   // [oc_pad] or null
     int oc_pad = 0;                // out_c rounded up to 16
     std::string how;               // which kernel serves the layer (for accerl_policy_info)
-    std::vector<int32_t> host_words;  // w_generic on the host, while the policy is built
+    const int8_t *host_rows = nullptr;  // w_generic on the host, while the policy is built
 };
 
 // One kernel launch of the plan: which kernel, and which part of the path it covers
@@ -171,8 +173,8 @@ struct LayerRequant {
 // parameters on their way to the device (see upload_bytes)
 struct UploadBlock {
     char *dev = nullptr;
-    std::vector<char> host;
-    size_t used = 0;
+    std::shared_ptr<char[]> host;  // (pinned, zero where it is not used yet)
+    size_t size = 0, used = 0;
 };
 
 struct DeviceBuf {
@@ -245,12 +247,14 @@ struct accerl_policy {
     std::vector<cudaEvent_t> copy_events; // one per chunk, and one for the caller's stream
     // the quantised parameters accerl_policy_create_fp32 computed (empty for other handles)
     struct PtqLayer {
-        std::vector<int8_t> w;
-        std::vector<float> s_w;
-        std::vector<int32_t> skip_mul;
+        const int8_t *w = nullptr;  // these three within ptq_data
+        const float *s_w = nullptr;
+        const int32_t *skip_mul = nullptr;
+        size_t n_w = 0, n_s_w = 0, n_skip_mul = 0;
         float s_in = 1.f, s_out = 1.f;
     };
     std::vector<PtqLayer> ptq;
+    std::shared_ptr<char[]> ptq_data;
     // outputs of this policy inside accerl_policy_act_mixed (allocated on its first call)
     float *mix_logits = nullptr, *mix_logp = nullptr, *mix_value = nullptr, *mix_entropy = nullptr;
     int32_t *mix_actions = nullptr;

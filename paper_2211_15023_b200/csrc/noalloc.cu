@@ -126,6 +126,7 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
     q->copy_stream = nullptr;
     q->mix = SideStream();
     q->ptq.clear();
+    q->ptq_data.reset();
     q->max_batch = (int)cap;
     bool ok = true;
     auto move = [&](auto *&ptr) {

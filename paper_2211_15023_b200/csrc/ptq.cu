@@ -420,23 +420,18 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
         ACCERL_CUDA_TRY(cudaGetLastError());
         s_in = i + 1;
     }
-    std::vector<char> back;
-    struct Quant {
-        std::vector<int8_t> w;
-        std::vector<float> s_w, bias;
-        std::vector<int32_t> skip_mul;
-        float s_in = 1.f, s_out = 1.f;
-    };
-    std::vector<Quant> Q;
+    // one block, kept as it comes back: copies of its parts cost their page faults again
+    std::shared_ptr<char[]> back;
+    std::vector<accerl_policy::PtqLayer> Q;
+    ACCERL_CUDA_TRY(pinned_alloc(&back, results_bytes));
     try {
-        back.resize(results_bytes);
         Q.resize(n_layers);
     } catch (const std::bad_alloc &) {
         set_error("create_fp32: out of host memory");
         return ACCERL_ERR_OOM;
     }
-    ACCERL_CUDA_TRY(cudaMemcpy(back.data(), results, results_bytes, cudaMemcpyDeviceToHost));
-    auto host = [&](const void *dev) { return back.data() + ((const char *)dev - results); };
+    ACCERL_CUDA_TRY(cudaMemcpy(back.get(), results, results_bytes, cudaMemcpyDeviceToHost));
+    auto host = [&](const void *dev) { return back.get() + ((const char *)dev - results); };
     auto scale = [&](int at) {
         const float m = reinterpret_cast<const float *>(host(ymax))[at];
         volatile float s = m > 0.f ? m / 127.0f : 1.0f;
@@ -447,19 +442,18 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
     for (int i = 0; i < n_run; ++i) {
         const accerl_layer_fp32 &d = layers[i];
         const Layer &l = net[i];
-        Quant &q = Q[i];
+        accerl_policy::PtqLayer &q = Q[i];
         q.s_in = s_prev;
         q.s_out = (d.flags & ACCERL_LOGITS) ? 1.0f : scale(l.scale);
         s_prev = q.s_out;
         if (!l.nw) continue;
-        const int8_t *w = (const int8_t *)host(l.wq);
-        const float *s_w = (const float *)host(l.s_w);
-        q.w.assign(w, w + l.nw);
-        q.s_w.assign(s_w, s_w + d.out_c);
-        q.bias.assign(d.bias, d.bias + d.out_c);
+        q.w = (const int8_t *)host(l.wq);
+        q.n_w = l.nw;
+        q.s_w = (const float *)host(l.s_w);
+        q.n_s_w = (size_t)d.out_c;
         if (d.skip_from >= 0) {
-            const int *m = (const int *)host(l.mul);
-            q.skip_mul.assign(m, m + d.out_c);
+            q.skip_mul = (const int32_t *)host(l.mul);
+            q.n_skip_mul = (size_t)d.out_c;
         }
     }
 
@@ -477,10 +471,10 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
         e.s_out = Q[i].s_out;
         e.skip_from = d.skip_from;
         if (d.kind != ACCERL_MAXPOOL) {
-            e.w = Q[i].w.data();
-            e.s_w = Q[i].s_w.data();
-            e.bias = Q[i].bias.data();
-            e.skip_mul = d.skip_from >= 0 ? Q[i].skip_mul.data() : nullptr;
+            e.w = Q[i].w;
+            e.s_w = Q[i].s_w;
+            e.bias = d.bias;
+            e.skip_mul = Q[i].skip_mul;
         }
     }
     accerl_status st = accerl_policy_create(out, in_kind, in_shape, s_input, descs.data(), n_layers, max_batch,
@@ -488,14 +482,8 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
     if (st != ACCERL_OK) return st;
     // keep the quantised parameters for accerl_policy_export
     accerl_policy *p = *out;
-    p->ptq.resize(n_layers);
-    for (int i = 0; i < n_layers; ++i) {
-        p->ptq[i].w = std::move(Q[i].w);
-        p->ptq[i].s_w = std::move(Q[i].s_w);
-        p->ptq[i].skip_mul = std::move(Q[i].skip_mul);
-        p->ptq[i].s_in = Q[i].s_in;
-        p->ptq[i].s_out = Q[i].s_out;
-    }
+    p->ptq = std::move(Q);
+    p->ptq_data = std::move(back);
     return ACCERL_OK;
 }
 
@@ -519,13 +507,13 @@ extern "C" accerl_status accerl_policy_export(const accerl_policy *p, int32_t la
     if (s_in_out) *s_in_out = q.s_in;
     if (s_out_out) *s_out_out = q.s_out;
     if (w_host) {
-        if (w_bytes < q.w.size()) {
-            set_error("export: w_host holds %zu bytes, %zu needed", w_bytes, q.w.size());
+        if (w_bytes < q.n_w) {
+            set_error("export: w_host holds %zu bytes, %zu needed", w_bytes, q.n_w);
             return ACCERL_ERR_INVALID_ARG;
         }
-        if (!q.w.empty()) memcpy(w_host, q.w.data(), q.w.size());
+        if (q.n_w) memcpy(w_host, q.w, q.n_w);
     }
-    if (s_w_host && !q.s_w.empty()) memcpy(s_w_host, q.s_w.data(), q.s_w.size() * sizeof(float));
-    if (skip_mul_host && !q.skip_mul.empty()) memcpy(skip_mul_host, q.skip_mul.data(), q.skip_mul.size() * sizeof(int32_t));
+    if (s_w_host && q.n_s_w) memcpy(s_w_host, q.s_w, q.n_s_w * sizeof(float));
+    if (skip_mul_host && q.n_skip_mul) memcpy(skip_mul_host, q.skip_mul, q.n_skip_mul * sizeof(int32_t));
     return ACCERL_OK;
 }

@@ -427,7 +427,7 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
                 g.col_off[j] = 128 * j;
             }
             for (int oc = 0; oc < d.out_c; ++oc) {  // (rows of K bytes in (y, x, c) order)
-                const int8_t *row = reinterpret_cast<const int8_t *>(L.host_words.data()) + (size_t)oc * K;
+                const int8_t *row = L.host_rows + (size_t)oc * K;
                 for (int j = 0; j < g.n_chunks; ++j)
                     memcpy(&packed[((size_t)j * n_total + oc) * 128], &row[128 * j], std::min(128, K - 128 * j));
             }
