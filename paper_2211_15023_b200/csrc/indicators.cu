@@ -122,11 +122,11 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
 }
 
 // A <= 64: one thread per row.  A block's rows are contiguous in memory; they pass through shared
-// memory so that the loads are whole lines and every thread then walks its own row (odd pitch: no
-// bank conflicts).  A warp per row, as for wide rows below, leaves 14 of 32 lanes idle at 18 actions
-// and spends its time in shuffles; with that and a one-block reduction the two launches for 131072
-// rows of 18 took 119 us, now 22.  STATS (one cluster, at most kKlCluster blocks' rows a pass): the mean
-// and the maximum come out of the same launch.
+// memory, by asynchronous copies that are all in flight at once, so that the loads are whole lines and
+// every thread then walks its own row (odd pitch: no bank conflicts).  A warp per row, as for wide rows
+// below, leaves 14 of 32 lanes idle at 18 actions and spends its time in shuffles; with that and a
+// one-block reduction the two launches for 131072 rows of 18 took 119 us, now 20.5.  STATS (one cluster,
+// at most kKlCluster blocks' rows a pass): the mean and the maximum come out of the same launch.
 template <bool STATS>
 __global__ void __launch_bounds__(kKlRows)
 kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B, int A, int pitch,
@@ -142,9 +142,11 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
         const float *src[2] = {zo + row0 * A, zs + row0 * A};
         int r = (int)threadIdx.x / A, c = (int)threadIdx.x - r * A;
         const int dr = kKlRows / A, dc = kKlRows - dr * A;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_rows);
         for (int i = threadIdx.x; i < n; i += kKlRows) {
-            s_rows[r * pitch + c] = __ldg(src[0] + i);
-            s_rows[(kKlRows + r) * pitch + c] = __ldg(src[1] + i);
+            const uint32_t d = dst + 4 * (r * pitch + c);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src[0] + i) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * kKlRows * pitch), "l"(src[1] + i) : "memory");
             r += dr;
             c += dc;
             if (c >= A) {
@@ -152,6 +154,7 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
                 ++r;
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         if ((int)threadIdx.x < rows) {
             const float v = kl_of_row(s_rows + threadIdx.x * pitch, s_rows + (kKlRows + threadIdx.x) * pitch, A, s_table);
@@ -310,8 +313,9 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     const long long blocks = narrow ? ((long long)batch + kKlRows - 1) / kKlRows : ((long long)batch * 32 + 127) / 128;
-    if (narrow && kl_mean_max_dev && blocks <= 2 * kKlCluster) {
-        // few rows: one cluster does it all, two passes at most (a second launch costs more)
+    if (narrow && kl_mean_max_dev && blocks <= (n_actions <= 6 ? 2 : 1) * kKlCluster) {
+        // Few rows: one cluster does it all, in a second pass only where rows are short (a second launch costs 2 us,
+        // a pass over 1024 rows 2 us at 6 actions, 4 at 18, 14 at 64)
         const unsigned n = (unsigned)(blocks < kKlCluster ? blocks : kKlCluster);
         cfg.gridDim = dim3(n);
         cfg.blockDim = dim3(kKlRows);

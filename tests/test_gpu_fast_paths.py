@@ -38,7 +38,7 @@ def test_mlp_widths_and_depths(dims):
         g.close()
 
 
-@pytest.mark.parametrize("b,a", [(127, 18), (128, 18), (129, 3), (1024, 18), (1025, 2), (2048, 9), (2049, 18), (300, 64),
+@pytest.mark.parametrize("b,a", [(127, 18), (128, 18), (129, 3), (1024, 18), (1025, 2), (2048, 9), (2049, 18), (2048, 6), (2049, 6), (1025, 7), (300, 64),
                                  (300, 65), (70001, 5)])
 def test_kl_at_the_edges_of_blocks_and_clusters(b, a):
     import paper_2211_15023_b200 as P
