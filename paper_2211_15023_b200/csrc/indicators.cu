@@ -82,6 +82,9 @@ __device__ __forceinline__ float kl_of_row(const float *zo, const float *zs, int
 constexpr int kKlRows = 128;   // rows (and threads) of a block
 constexpr int kKlCluster = 8;  // CTAs that share the reduction to mean and maximum
 
+// The first thing of a kernel that ends in cluster_stats: this CTA's shared memory may be written from now on.
+__device__ __forceinline__ void cluster_started() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+
 // Mean and maximum over all threads of a cluster (every CTA calls with its own partial sum and
 // maximum); always the same order of additions.
 __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float *stats)
@@ -101,11 +104,14 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
     if (warp == 0) {
         sum = warp_sum(lane < warps ? s_sum[lane] : 0.0);
         mx = warp_maxf(lane < warps ? s_max[lane] : -INFINITY);
-        if (lane == 0) {
-            const unsigned rank = cooperative_groups::this_cluster().block_rank();
-            *cooperative_groups::this_cluster().map_shared_rank(&c_sum[rank], 0) = sum;
-            *cooperative_groups::this_cluster().map_shared_rank(&c_max[rank], 0) = mx;
-        }
+    }
+    // The first CTA's shared memory exists only once that CTA has started (the arrivals of cluster_started lie a
+    // whole pass over the rows back: nothing waits here)
+    asm volatile("barrier.cluster.wait;" ::: "memory");
+    if (threadIdx.x == 0) {
+        const unsigned rank = cooperative_groups::this_cluster().block_rank();
+        *cooperative_groups::this_cluster().map_shared_rank(&c_sum[rank], 0) = sum;
+        *cooperative_groups::this_cluster().map_shared_rank(&c_max[rank], 0) = mx;
     }
     cooperative_groups::this_cluster().sync();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -134,6 +140,7 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
 {
     extern __shared__ float s_rows[];  // [2][kKlRows][pitch]
     __shared__ double s_table[64];
+    if (STATS) cluster_started();
     if (threadIdx.x < 64) s_table[threadIdx.x] = exp2((double)threadIdx.x * (1.0 / 64.0));
     double sum = 0.0;
     float mx = -INFINITY;
@@ -200,6 +207,7 @@ kl_wide_kernel(const float *__restrict__ zo_all, const float *__restrict__ zs_al
 // stats[0] = mean, stats[1] = max of kl[0..B): one cluster, each CTA a contiguous part
 __global__ void __launch_bounds__(1024) kl_stats_kernel(const float *__restrict__ kl, int B, float *stats)
 {
+    cluster_started();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     double sum = 0.0;
     float mx = -INFINITY;
