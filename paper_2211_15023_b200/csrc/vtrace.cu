@@ -10,6 +10,8 @@
 // definition up to the final rounding to float.
 #include <math.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace accerl {
@@ -19,14 +21,58 @@ namespace {
 constexpr int kCols = 32;   // rollouts of a block, one per lane
 constexpr int kSteps = 16;  // time steps of a chunk, one warp each
 
-// The recursion is sequential in t, but only two multiply-adds a step of it: the ratios (an exp),
+// Many rollouts: one thread each, from the last step to the first.  The recursion is sequential in t but
+// its inputs are not: the loads of kAhead steps are issued together (a rollout is one thread, so nothing
+// else hides the memory latency).  Bound by HBM for a million rollouts of one step (12 us for 28 MB) and by
+// the chain of exps, some 0.17 us a step, where every SM has a few warps only.
+constexpr int kAhead = 8;
+__global__ void __launch_bounds__(128)
+vtrace_rollout_kernel(const float *__restrict__ logp_smaller, const float *__restrict__ logp_original,
+                      const float *__restrict__ rewards, const float *__restrict__ values,
+                      const float *__restrict__ bootstrap, const float *__restrict__ discounts, int n, int B,
+                      float gamma, float rho_hat, float c_hat, float *__restrict__ vs, float *__restrict__ adv)
+{
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= B) return;
+    double v_next = (double)bootstrap[b];  // V(x_{t+1})
+    double vs_next = v_next;               // v_{t+1}
+    double carry = 0.0;                    // v_{t+1} - V(x_{t+1})
+    for (int t1 = n - 1; t1 >= 0; t1 -= kAhead) {
+        float lo[kAhead], ls[kAhead], rw[kAhead], vv[kAhead], dc[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const long long i = (long long)max(t1 - j, 0) * B + b;
+            lo[j] = logp_original[i];
+            ls[j] = logp_smaller[i];
+            rw[j] = rewards[i];
+            vv[j] = values[i];
+            dc[j] = discounts ? discounts[i] : gamma;
+        }
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int t = t1 - j;
+            if (t < 0) break;
+            const long long i = (long long)t * B + b;
+            const double ratio = exp((double)lo[j] - (double)ls[j]);
+            const double rho = fmin(ratio, (double)rho_hat), c = fmin(ratio, (double)c_hat);
+            const double g = (double)dc[j], v = (double)vv[j], r = (double)rw[j];
+            const double delta = rho * (r + g * v_next - v);
+            carry = delta + g * c * carry;
+            if (adv) adv[i] = (float)(rho * (r + g * vs_next - v));
+            vs_next = v + carry;
+            vs[i] = (float)vs_next;
+            v_next = v;
+        }
+    }
+}
+
+// Few rollouts.  The recursion is sequential in t, but only two multiply-adds a step of it: the ratios (an exp),
 // the temporal differences and the advantages of all steps are independent.  So a block takes 32
 // rollouts and, from the last step backwards, 16 steps at a time: warp w loads step w of the chunk
 // (whole lines: arrays are time-major) and computes rho, g c and delta, the first warp runs the
 // recursion over the chunk out of shared memory, and every warp writes its step's results.  The next
-// chunk's loads are issued before the recursion of the current one.  With one thread per rollout and
-// loads eight steps ahead the kernel was a chain of exps and memory latencies (6.1 us a call for 16 x 8192,
-// now about 4).
+// chunk's loads are issued before the recursion of the current one.  A chunk costs about 1 us while
+// every SM has a block, whether its steps are used or not.
 __global__ void __launch_bounds__(32 * kSteps)
 vtrace_kernel(const float *__restrict__ logp_smaller, const float *__restrict__ logp_original,
               const float *__restrict__ rewards, const float *__restrict__ values,
@@ -87,6 +133,20 @@ vtrace_kernel(const float *__restrict__ logp_smaller, const float *__restrict__ 
     }
 }
 
+// Which of the two: the time of one thread per rollout grows with the steps (0.17 us each, 0.21 with an
+// array of discounts to load, half as much again where the inputs do not fit L2), that of one warp per step
+// with the chunks of 16 and with the blocks an SM has to run (0.72 us a chunk at the least, 0.25 and 0.55 for
+// every block).  us per call, a thread per rollout / a warp per step: 2.0 / 2.4 for 2 x 32, 4.4 / 2.6 for 16 x 1024,
+// 4.3 / 3.0 for 16 x 8192, 4.7 / 4.6 for 16 x 16384, 5.3 / 6.7 for 16 x 32768, 5.1 / 6.6 for 17 x 16384, 24.4 / 9.6 for
+// 128 x 4096, 49 / 68 for 128 x 65536, 11.8 / 142 for 1 x 1048576.
+bool thread_per_rollout(int n, int batch, bool discounts, int sm_count)
+{
+    const long long chunks = (n + kSteps - 1) / kSteps;
+    const bool beyond_l2 = 4LL * n * batch * (discounts ? 5 : 4) > (64LL << 20);
+    const long long step = (discounts ? 21 : 17) * (beyond_l2 ? 3 : 2) / 2;
+    return step * n < chunks * std::max<long long>(72, 25 + 55LL * batch / (kCols * sm_count));
+}
+
 }  // namespace
 
 }  // namespace accerl
@@ -118,9 +178,20 @@ extern "C" accerl_status accerl_vtrace(const float *logp_smaller_dev, const floa
         set_error("vtrace: misaligned pointer (4 bytes needed)");
         return ACCERL_ERR_INVALID_ARG;
     }
-    vtrace_kernel<<<(unsigned)((batch + kCols - 1) / kCols), 32 * kSteps, 0, (cudaStream_t)cuda_stream>>>(
-        logp_smaller_dev, logp_original_dev, rewards_dev, values_dev, bootstrap_dev, discounts_dev, n_steps,
-        batch, gamma, rho_hat, c_hat, vs_dev, adv_dev);
+    int device = 0, sm_count = 0;
+    ACCERL_CUDA_TRY(cudaGetDevice(&device));
+    ACCERL_CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device));
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    if (thread_per_rollout(n_steps, batch, discounts_dev != nullptr, sm_count)) {
+        const int threads = batch >= sm_count * 128 * 4 ? 128 : 32;  // few rollouts: spread them over the SMs
+        vtrace_rollout_kernel<<<(unsigned)((batch + threads - 1) / threads), threads, 0, st>>>(
+            logp_smaller_dev, logp_original_dev, rewards_dev, values_dev, bootstrap_dev, discounts_dev, n_steps,
+            batch, gamma, rho_hat, c_hat, vs_dev, adv_dev);
+    } else {
+        vtrace_kernel<<<(unsigned)((batch + kCols - 1) / kCols), 32 * kSteps, 0, st>>>(
+            logp_smaller_dev, logp_original_dev, rewards_dev, values_dev, bootstrap_dev, discounts_dev, n_steps,
+            batch, gamma, rho_hat, c_hat, vs_dev, adv_dev);
+    }
     ACCERL_CUDA_TRY(cudaGetLastError());
     return ACCERL_OK;
 }
