@@ -1,9 +1,9 @@
 // The Monitor's indicators and the per-state choice between two policies (Section 2.4).
 //
 // kl_rows_kernel / kl_wide_kernel: KL(pi_original || pi_smaller) per state from two logit matrices
-// (Eq. KL); kl_stats_kernel reduces the per-state values to their mean and maximum (the "KL mean" and
-// "KL max" indicators) in one cluster of CTAs, in a fixed order, so that the result does not depend on
-// scheduling.  mix_select_kernel overwrites the original
+// (Eq. KL), a thread or a warp per state; kl_stats_kernel reduces the per-state values to their mean and
+// maximum (the "KL mean" and "KL max" indicators) in one CTA or one cluster of CTAs, in a fixed order, so
+// that the result does not depend on scheduling.  mix_select_kernel overwrites the original
 // policy's outputs with the smaller policy's for the states whose selector draw falls below alpha
 // (the linear-alpha strategy of Section 3.2: the Actor follows the small network with
 // probability alpha).
@@ -86,7 +86,8 @@ constexpr int kKlCluster = 8;  // CTAs that share the reduction to mean and maxi
 __device__ __forceinline__ void cluster_started() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 
 // Mean and maximum over all threads of a cluster (every CTA calls with its own partial sum and
-// maximum); always the same order of additions.
+// maximum), or of one CTA; always the same order of additions.
+template <bool CLUSTER>
 __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float *stats)
 {
     __shared__ double s_sum[32];
@@ -104,6 +105,13 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
     if (warp == 0) {
         sum = warp_sum(lane < warps ? s_sum[lane] : 0.0);
         mx = warp_maxf(lane < warps ? s_max[lane] : -INFINITY);
+    }
+    if (!CLUSTER) {
+        if (threadIdx.x == 0) {
+            stats[0] = (float)(sum / (double)B);
+            stats[1] = mx;
+        }
+        return;
     }
     // The first CTA's shared memory exists only once that CTA has started (the arrivals of cluster_started lie a
     // whole pass over the rows back: nothing waits here)
@@ -127,10 +135,10 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
     }
 }
 
-// A <= 64: one thread per row.  A block's rows are contiguous in memory; they pass through shared
-// memory, by asynchronous copies that are all in flight at once, so that the loads are whole lines and
-// every thread then walks its own row (odd pitch: no bank conflicts).  A warp per row, as for wide rows
-// below, leaves 14 of 32 lanes idle at 18 actions and spends its time in shuffles; with that and a
+// Many rows of at most 64 actions, or few of at most 12 (see the choice in accerl_policy_kl): one thread per
+// row.  A block's rows are contiguous in memory; they pass through shared memory, by asynchronous copies that
+// are all in flight at once, so that the loads are whole lines and every thread then walks its own row (odd
+// pitch: no bank conflicts), a chain of two exponentials an action.  A warp per row, as below, leaves 14 of 32 lanes idle at 18 actions and spends its time in shuffles; with that and a
 // one-block reduction the two launches for 131072 rows of 18 took 119 us, now 20.5.  STATS (one cluster,
 // at most kKlCluster blocks' rows a pass): the mean and the maximum come out of the same launch.
 template <bool STATS>
@@ -172,10 +180,10 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
         __syncthreads();
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (STATS) cluster_stats(sum, mx, B, stats);
+    if (STATS) cluster_stats<true>(sum, mx, B, stats);
 }
 
-// any A: one warp per row, lanes striding over the actions
+// any A: one warp per row, lanes striding over the actions (a row's chain is short: what few rows need)
 __global__ void __launch_bounds__(128)
 kl_wide_kernel(const float *__restrict__ zo_all, const float *__restrict__ zs_all, int B, int A,
                float *__restrict__ kl)
@@ -204,10 +212,14 @@ kl_wide_kernel(const float *__restrict__ zo_all, const float *__restrict__ zs_al
     if (lane == 0) kl[row] = (float)(acc / so - ((mo + log(so)) - (ms + log(ss))));
 }
 
-// stats[0] = mean, stats[1] = max of kl[0..B): one cluster, each CTA a contiguous part
+// stats[0] = mean, stats[1] = max of kl[0..B): one cluster, or for kOneCta rows at most one CTA, whose threads then
+// have all their loads in flight at once (us per call, rows kernel included, one CTA / cluster of eight: 160 x 18
+// 4.3 / 5.0, 1024 x 18 5.3 / 6.0, 4096 x 64 7.4 / 7.9, 8192 x 64 10.6 / 10.6, 12000 x 64 14.3 / 13.3)
+constexpr int kOneCta = 8192;
+template <bool CLUSTER>
 __global__ void __launch_bounds__(1024) kl_stats_kernel(const float *__restrict__ kl, int B, float *stats)
 {
-    cluster_started();
+    if (CLUSTER) cluster_started();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     double sum = 0.0;
     float mx = -INFINITY;
@@ -223,7 +235,7 @@ __global__ void __launch_bounds__(1024) kl_stats_kernel(const float *__restrict_
             mx = fmaxf(mx, v[j]);
         }
     }
-    cluster_stats(sum, mx, B, stats);
+    cluster_stats<CLUSTER>(sum, mx, B, stats);
 }
 
 struct MixOut {
@@ -311,7 +323,14 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
         return ACCERL_ERR_INVALID_ARG;
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const bool narrow = n_actions <= 64;  // two blocks' worth of rows fit 48 KB up to 47 actions, 66 KB at 64
+    // A thread per row pays from some 256 rows an action on, where a warp per row no longer fits the chip at once
+    // (us per call, thread / warp: 18 actions 8.2 / 5.6 for 2048 rows, 8.2 / 8.4 for 6144, 9.7 / 22.7 for 32768; 64
+    // actions 15.1 / 6.0, 15.3 / 9.1, 18.3 / 27).  Few short rows go to one cluster that does it all, in a second
+    // pass only where they are shorter still: a second launch costs some 2 us, what a pass over 1024 rows takes at 9
+    // actions (9 actions: 4.4 for 1024 rows, 6.6 for 2048, the two launches 5.2 and 5.6).
+    const long long rows_blocks = ((long long)batch + kKlRows - 1) / kKlRows;
+    const bool one_launch = kl_mean_max_dev && n_actions <= 12 && rows_blocks <= (n_actions <= 6 ? 2 : 1) * kKlCluster;
+    const bool narrow = n_actions <= 64 && (one_launch || batch >= 256 * n_actions);  // (66 KB of shared memory at 64)
     const int pitch = n_actions | 1;
     const size_t smem = 2 * sizeof(float) * (size_t)kKlRows * pitch;
     cudaLaunchConfig_t cfg = {};
@@ -320,10 +339,8 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
     cfg.attrs = attr;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    const long long blocks = narrow ? ((long long)batch + kKlRows - 1) / kKlRows : ((long long)batch * 32 + 127) / 128;
-    if (narrow && kl_mean_max_dev && blocks <= (n_actions <= 6 ? 2 : 1) * kKlCluster) {
-        // Few rows: one cluster does it all, in a second pass only where rows are short (a second launch costs 2 us,
-        // a pass over 1024 rows 2 us at 6 actions, 4 at 18, 14 at 64)
+    const long long blocks = narrow ? rows_blocks : ((long long)batch * 32 + 127) / 128;
+    if (one_launch) {
         const unsigned n = (unsigned)(blocks < kKlCluster ? blocks : kKlCluster);
         cfg.gridDim = dim3(n);
         cfg.blockDim = dim3(kKlRows);
@@ -344,13 +361,17 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
     }
     ACCERL_CUDA_TRY(cudaGetLastError());
     if (kl_mean_max_dev) {
-        cfg.gridDim = dim3(kKlCluster);
+        const bool one = batch <= kOneCta;
+        cfg.gridDim = dim3(one ? 1 : kKlCluster);
         cfg.blockDim = dim3(1024);
-        attr[0].val.clusterDim.x = kKlCluster;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.numAttrs = 2;
-        ACCERL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kl_stats_kernel, (const float *)kl_dev, batch, kl_mean_max_dev));
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = kKlCluster;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = one ? 1 : 2;
+        ACCERL_CUDA_TRY(cudaLaunchKernelEx(&cfg, one ? kl_stats_kernel<false> : kl_stats_kernel<true>, (const float *)kl_dev, batch,
+                                           kl_mean_max_dev));
     }
     return ACCERL_OK;
 }

@@ -73,3 +73,55 @@ def test_vtrace_of_short_rollouts_is_bound_by_memory():
         b.synchronize()
         best = min(best, a.elapsed_time(b) * 50.0)
     assert best < 50.0, "%.1f us" % best
+
+
+@pytest.mark.parametrize("a", [1, 5, 6, 7, 9, 12, 13, 18, 33, 63, 64, 65])
+def test_kl_of_few_rows_and_of_many(a):
+    """Row counts on both sides of every choice between one launch, a thread per row and a warp per row:
+    against the oracle over spreads from nothing to far below the least exponential, and each row the same
+    to the last float bit but one whichever kernel takes it (both compute in double)."""
+    import paper_2211_15023_b200 as P
+    rng = np.random.default_rng(a)
+    b = max(256 * min(a, 64) + 130, 8193)
+    zo = (rng.random((b, a)) * rng.choice([1e-6, 1.0, 100.0, 3000.0], size=(b, 1))).astype(np.float32)
+    zs = (zo + rng.standard_normal((b, a)) * rng.choice([1e-3, 0.5, 50.0], size=(b, 1))).astype(np.float32)
+    zs[::7] = zo[::7]
+    if a > 1:  # masked actions
+        zo[1::11, 0] = zs[1::11, 0] = -np.inf
+        zo[2::11, 0] = zs[2::11, 0] = np.finfo(np.float32).min
+    want = oracle.kl(zo, zs)
+    do, ds = torch.from_numpy(zo).cuda(), torch.from_numpy(zs).cuda()
+    whole = None
+    for n in (b, 8193, 8192, 256 * min(a, 64), 256 * min(a, 64) - 1, 2049, 2048, 1025, 1024, 300, 1):
+        n = min(n, b)
+        kl, stats = (t.cpu().numpy() for t in P.kl(do[:n].contiguous(), ds[:n].contiguous()))
+        np.testing.assert_allclose(kl, want[:n], rtol=1e-5, atol=1e-6)
+        assert (kl[::7] == 0.0).all()
+        np.testing.assert_allclose(stats, [want[:n].mean(), want[:n].max()], rtol=1e-5, atol=1e-6)
+        whole = kl if whole is None else whole
+        np.testing.assert_array_max_ulp(kl[kl > 1e-3], whole[:n][kl > 1e-3], maxulp=1)
+
+
+def test_kl_of_few_wide_rows_does_not_wait_for_one_thread():
+    """160 rows of 64 actions: a thread that walks a row of 128 exponentials takes 13 us, a warp and a second
+    launch for the statistics 5.  The bound lies between them."""
+    import paper_2211_15023_b200 as P
+    zo = torch.randn((160, 64), device="cuda")
+    zs = zo + 0.1
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        P.kl(zo, zs)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(20):
+            P.kl(zo, zs)
+    best = 1e9
+    for _ in range(6):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        graph.replay()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 50.0)
+    assert best < 10.0, "%.1f us" % best
