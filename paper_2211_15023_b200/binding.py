@@ -141,6 +141,15 @@ def _stream_of(t, stream):
     return torch.cuda.current_stream(t.device).cuda_stream if stream is None else stream
 
 
+def _check_batch(frames, obs, *per_state):
+    """What a kernel reads as a batch of observations and floats per state must be that, on the device."""
+    import torch
+    assert obs.is_cuda and obs.is_contiguous() and \
+        (obs.element_size() == 1 if frames else obs.dtype == torch.float32)
+    for t in per_state:
+        assert t.device == obs.device and t.is_contiguous() and t.dtype == torch.float32 and t.numel() >= obs.shape[0]
+
+
 def kl(logits_original, logits_smaller, stream=None):
     """accerl_policy_kl on two CUDA fp32 [B, A] tensors; returns (kl [B], mean_max [2]) tensors."""
     r = (_CALLS or _calls()).kl(logits_original, logits_smaller, stream)
@@ -148,7 +157,8 @@ def kl(logits_original, logits_smaller, stream=None):
         return _done(r)
     import torch
     assert logits_original.shape == logits_smaller.shape and logits_original.is_contiguous() and \
-        logits_smaller.is_contiguous() and logits_original.dtype == logits_smaller.dtype == torch.float32
+        logits_smaller.is_contiguous() and logits_original.dtype == logits_smaller.dtype == torch.float32 and \
+        logits_original.is_cuda and logits_smaller.is_cuda
     b, a = logits_original.shape
     out = torch.empty(b, dtype=torch.float32, device=logits_original.device)
     stats = torch.empty(2, dtype=torch.float32, device=logits_original.device)
@@ -170,8 +180,10 @@ def vtrace(logp_smaller, logp_original, rewards, values, bootstrap, gamma, rho_h
     if checked:
         for t in (logp_smaller, logp_original, rewards, values):
             assert t.shape == (n, b) and t.is_contiguous() and t.dtype == torch.float32 and t.is_cuda
-        assert bootstrap.shape == (b,) and bootstrap.is_contiguous() and bootstrap.dtype == torch.float32
-        assert discounts is None or (discounts.shape == (n, b) and discounts.is_contiguous())
+        assert bootstrap.shape == (b,) and bootstrap.is_contiguous() and bootstrap.dtype == torch.float32 and \
+            bootstrap.is_cuda
+        assert discounts is None or (discounts.shape == (n, b) and discounts.is_contiguous() and
+                                     discounts.dtype == torch.float32 and discounts.is_cuda)
     vs, adv = (torch.empty_like(values), torch.empty_like(values)) if out is None else out
     _check(library().accerl_vtrace(logp_smaller.data_ptr(), logp_original.data_ptr(), rewards.data_ptr(),
                                    values.data_ptr(), bootstrap.data_ptr(),
@@ -189,6 +201,7 @@ def act_mixed(smaller, original, obs, uniforms, select_uniforms, alpha, stream=N
     if r is not None:
         return _done(r)
     import torch
+    _check_batch(smaller.in_kind == "u8", obs, uniforms, select_uniforms)
     b, dev = int(obs.shape[0]), obs.device
     out = dict(logits=torch.empty((b, smaller.n_actions), dtype=torch.float32, device=dev),
                actions=torch.empty(b, dtype=torch.int32, device=dev),
@@ -332,6 +345,7 @@ class Policy:
         if r is not None:
             return _done(r)
         import torch
+        _check_batch(self.in_kind == "u8", obs, uniforms)
         b, dev = int(obs.shape[0]), obs.device
         out = dict(logits=torch.empty((b, self.n_actions), dtype=torch.float32, device=dev),
                    actions=torch.empty(b, dtype=torch.int32, device=dev),

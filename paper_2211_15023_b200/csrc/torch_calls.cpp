@@ -4,8 +4,8 @@
 // 160 took 15.0 us through ctypes and torch's Python functions, of which the GPU needed five.
 //
 // Every function returns the results, the status code (an int) of a call that failed, or None when
-// the arguments are not what the fast path takes (binding.py then checks them one by one and raises
-// what it always raised).
+// the arguments are not what the fast path takes (binding.py then checks them one by one, raises for what a
+// kernel could not read, and goes through ctypes with the rest).
 #include <Python.h>
 
 #include <ATen/cuda/EmptyTensor.h>

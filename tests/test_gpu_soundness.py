@@ -125,3 +125,40 @@ def test_kl_of_few_wide_rows_does_not_wait_for_one_thread():
         b.synchronize()
         best = min(best, a.elapsed_time(b) * 50.0)
     assert best < 10.0, "%.1f us" % best
+
+
+def test_act_ex_and_act_mixed_refuse_what_their_kernels_would_misread():
+    """Uniforms or selectors that are too few, of another type, on another device or strided raise on the
+    host, as in act; more of them than states, which the kernels never look at, go through as before."""
+    import paper_2211_15023_b200 as P
+    import workloads as W
+    pol, b = W.drawn_int8_policy("student_cnn_b8192"), 6
+    g, o = P.Policy(pol, b), P.Policy(pol, b)
+    obs = torch.from_numpy(W.observations("student_cnn_b8192", b)).cuda()
+    u, long = torch.rand(b, device="cuda"), torch.rand(2 * b, device="cuda")
+    bad_u = (u[:b - 1], u.double(), u.cpu(), long[::2])
+    bad_obs = (obs.float(), obs.cpu(), obs.transpose(2, 3))
+    for v in bad_u:
+        with pytest.raises(AssertionError):
+            g.act_ex(obs, v)
+        with pytest.raises(AssertionError):
+            P.act_mixed(g, o, obs, v, u, 0.5)
+        with pytest.raises(AssertionError):
+            P.act_mixed(g, o, obs, u, v, 0.5)
+    for v in bad_obs:
+        with pytest.raises(AssertionError):
+            g.act_ex(v, u)
+        with pytest.raises(AssertionError):
+            P.act_mixed(g, o, v, u, u, 0.5)
+    want, got = g.act_ex(obs, long[:b].contiguous()), g.act_ex(obs, long)
+    for k in want:
+        assert torch.equal(want[k], got[k]), k
+    x, boot = torch.zeros((3, b), device="cuda"), torch.zeros(b, device="cuda")
+    for call in (lambda: P.kl(x.cpu(), x.cpu()), lambda: P.kl(x, x.cpu()), lambda: P.vtrace(x, x, x, x, boot.cpu(), 0.99),
+                 lambda: P.vtrace(x, x, x, x, boot, 0.99, discounts=x.double()),
+                 lambda: P.vtrace(x, x, x, x, boot, 0.99, discounts=x.cpu())):
+        with pytest.raises(AssertionError):
+            call()
+    g.check()
+    g.close()
+    o.close()
