@@ -376,8 +376,12 @@ class Policy:
     def act_noalloc_raw(self, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr,
                         stream=0) -> int:
         """accerl_policy_act_noalloc with raw device addresses; returns the status code."""
-        return (_CALLS or _calls()).act_noalloc(self._raw, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr,
-                                                stream)
+        r = (_CALLS or _calls()).act_noalloc(self._raw, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr,
+                                             stream)
+        if r is not None:
+            return r
+        return library().accerl_policy_act_noalloc(self._h, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr,
+                                                   stream)
 
     def act_raw(self, obs_ptr, u_ptr, batch, logits_ptr, actions_ptr, logp_ptr, stream=0) -> int:
         """Unchecked pass-through returning the status code (for ABI tests)."""

@@ -25,6 +25,14 @@ const at::Tensor *cuda_tensor(PyObject *o, at::ScalarType type)
     return t.is_cuda() && t.scalar_type() == type && t.is_contiguous() ? &t : nullptr;
 }
 
+// did a conversion fail?  (binding.py's own then takes what it always took, or raises)
+bool not_for_us()
+{
+    if (!PyErr_Occurred()) return false;
+    PyErr_Clear();
+    return true;
+}
+
 // the stream argument: an integer, or None for torch's current stream of `device`
 bool stream_of(PyObject *o, c10::DeviceIndex device, void **stream)
 {
@@ -33,9 +41,7 @@ bool stream_of(PyObject *o, c10::DeviceIndex device, void **stream)
         return true;
     }
     *stream = PyLong_AsVoidPtr(o);
-    if (*stream || !PyErr_Occurred()) return true;
-    PyErr_Clear();
-    return false;
+    return *stream || !not_for_us();
 }
 
 at::Tensor empty(at::IntArrayRef size, at::ScalarType type, const at::Tensor &like)
@@ -85,7 +91,7 @@ PyObject *py_act(PyObject *, PyObject *const *a, Py_ssize_t n)
     const at::Tensor *obs, *u;
     int64_t b;
     void *stream;
-    if (PyErr_Occurred()) return nullptr;
+    if (not_for_us()) Py_RETURN_NONE;
     if (!act_inputs(a[2], a[3], a[4], &obs, &u, &b) || !stream_of(a[6], obs->device().index(), &stream)) Py_RETURN_NONE;
     void *dst[3];
     at::Tensor t[3];
@@ -128,7 +134,7 @@ PyObject *py_act_ex(PyObject *, PyObject *const *a, Py_ssize_t n)
     const at::Tensor *obs, *u;
     int64_t b;
     void *stream;
-    if (PyErr_Occurred()) return nullptr;
+    if (not_for_us()) Py_RETURN_NONE;
     if (!act_inputs(a[2], a[4], a[5], &obs, &u, &b) || !stream_of(a[6], obs->device().index(), &stream)) Py_RETURN_NONE;
     at::Tensor logits = empty({b, A}, at::kFloat, *obs), actions = empty({b}, at::kInt, *obs),
                logp = empty({b}, at::kFloat, *obs), entropy = empty({b}, at::kFloat, *obs), value;
@@ -162,7 +168,7 @@ PyObject *py_act_mixed(PyObject *, PyObject *const *a, Py_ssize_t n)
     const at::Tensor *obs, *u;
     int64_t b;
     void *stream;
-    if (PyErr_Occurred()) return nullptr;
+    if (not_for_us()) Py_RETURN_NONE;
     const at::Tensor *select = cuda_tensor(a[7], at::kFloat);
     if (!act_inputs(a[3], a[5], a[6], &obs, &u, &b) || !select || select->numel() != b ||
         !stream_of(a[9], obs->device().index(), &stream))
@@ -229,7 +235,7 @@ PyObject *py_vtrace(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (in[0]->size(0) > INT32_MAX || in[0]->size(1) > INT32_MAX || !stream_of(a[9], in[0]->device().index(), &stream))
         Py_RETURN_NONE;
     const double gamma = PyFloat_AsDouble(a[6]), rho = PyFloat_AsDouble(a[7]), c = PyFloat_AsDouble(a[8]);
-    if (PyErr_Occurred()) return nullptr;
+    if (not_for_us()) Py_RETURN_NONE;
     at::Tensor vs = empty(in[0]->sizes(), at::kFloat, *in[0]), adv = empty(in[0]->sizes(), at::kFloat, *in[0]);
     const float *p[6];
     for (int i = 0; i < 6; ++i) p[i] = in[i] ? (const float *)in[i]->data_ptr() : nullptr;
@@ -242,16 +248,21 @@ PyObject *py_vtrace(PyObject *, PyObject *const *a, Py_ssize_t n)
     return Py_BuildValue("(NN)", wrapped(std::move(vs)), wrapped(std::move(adv)));
 }
 
-// act_noalloc(handle, obs, uniforms, batch, logits, actions, logp, stream): raw addresses -> status
+// act_noalloc(handle, obs, uniforms, batch, logits, actions, logp, stream): raw addresses -> status, or None for
+// arguments that are no plain integers (ctypes pointers, numpy integers: binding.py passes those through ctypes)
 PyObject *py_act_noalloc(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     if (n != 8) return Py_BuildValue("");
-    void *p[8];
+    void *p[8] = {};
     for (int i = 0; i < 8; ++i) {
-        p[i] = a[i] == Py_None ? nullptr : PyLong_AsVoidPtr(a[i]);
-        if (!p[i] && PyErr_Occurred()) return nullptr;
+        if (i == 3 || a[i] == Py_None) continue;
+        if (!PyLong_Check(a[i])) Py_RETURN_NONE;
+        p[i] = PyLong_AsVoidPtr(a[i]);
+        if (!p[i] && not_for_us()) Py_RETURN_NONE;
     }
+    if (!PyLong_Check(a[3])) Py_RETURN_NONE;
     const long batch = PyLong_AsLong(a[3]);
+    if (batch == -1 && not_for_us()) Py_RETURN_NONE;
     const accerl_status st = without_gil([&] {
         return accerl_policy_act_noalloc((accerl_policy *)p[0], p[1], (const float *)p[2], (int32_t)batch, (float *)p[4],
                                          (int32_t *)p[5], (float *)p[6], p[7]);

@@ -32,3 +32,16 @@ def test_tensors_the_device_cannot_read_raise_before_the_launch(P):
                  lambda: P.vtrace(x, x, x, x, boot, 0.99)):
         with pytest.raises(AssertionError):
             call()
+
+
+def test_act_noalloc_raw_takes_every_kind_of_address_and_number_ctypes_takes(P):
+    """Integers, None, ctypes pointers, numpy integers for the batch; what is none of these raises."""
+    g, INVALID = _policy(P), 1
+    buf = (C.c_float * 4)()
+    for args in ((0, 0, 5, 0, 0, 0), (None, None, 5, None, None, None, None), (0, 0, np.int64(5), 0, 0, 0),
+                 (C.c_void_p(0), None, 5, buf, C.byref(buf), 0, C.c_void_p(0)), (0, 0, np.int32(5), 0, 0, 0),
+                 (0, 0, True, 0, 0, 0), (0, 0, 1 << 70, 0, 0, 0), (0, 0, -1, 0, 0, 0)):
+        assert g.act_noalloc_raw(*args) == INVALID, args
+    for args in ((0, 0, 5.0, 0, 0, 0), (0, 0, None, 0, 0, 0), (0, 0, "5", 0, 0, 0), (2.0, 0, 5, 0, 0, 0)):
+        with pytest.raises(C.ArgumentError):
+            g.act_noalloc_raw(*args)
