@@ -317,21 +317,6 @@ using namespace accerl;
 // results up to this size are written to pinned host memory by the kernels themselves
 static constexpr size_t kDirectBytes = 64 << 10;
 
-// Can kernels on the current device use this host range at its own address (pinned and mapped, 4-byte aligned)?
-static bool device_reaches(const void *host, size_t bytes)
-{
-    if ((uintptr_t)host & 3) return false;
-    for (const char *at : {(const char *)host, (const char *)host + bytes - 1}) {
-        cudaPointerAttributes attr;
-        if (cudaPointerGetAttributes(&attr, at) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        if (attr.type != cudaMemoryTypeHost || attr.devicePointer != (void *)at) return false;
-    }
-    return true;
-}
-
 // argument checks shared by the act entry points (nothing is launched when they fail)
 static accerl_status check_act_args(accerl_policy *p, const void *obs_dev,
                                     const float *uniforms_dev, int32_t batch, float *logits_dev,

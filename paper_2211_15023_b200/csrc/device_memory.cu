@@ -10,6 +10,8 @@
 // Pinned host memory for parameters on their way to the device and quantised ones on their way back is
 // kept in the same manner (at most kKeptHost bytes): pageable blocks of that size are fresh pages for
 // every policy, 0.4 ms of faults each, and copies from and to them are staged by the driver.
+#include <cuda.h>
+
 #include <algorithm>
 #include <chrono>
 #include <list>
@@ -197,6 +199,32 @@ cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes)
     const cudaError_t e = memory().take(&ptr, bytes, kHost);
     if (e == cudaSuccess) *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at); });
     return e;
+}
+
+// Pinned and mapped, 4-byte aligned, and all of it inside one allocation or registration: with its two ends in
+// different ones there may be pageable memory between them.
+bool device_reaches(const void *host, size_t bytes)
+{
+    if ((uintptr_t)host & 3) return false;
+    typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Query query = [] {
+        void *sym = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttributes", &sym, cudaEnableDefault, &found) == cudaSuccess &&
+                        found == cudaDriverEntryPointSuccess;
+        return ok ? (Query)sym : (Query) nullptr;
+    }();
+    if (!query) return false;
+    unsigned type = 0, managed = 0;  // (stays 0 for memory the driver does not know)
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &managed, &device, &start, &size};
+    if (query(5, what, to, (CUdeviceptr)host) != CUDA_SUCCESS) return false;
+    const CUdeviceptr at = (CUdeviceptr)host;
+    return type == CU_MEMORYTYPE_HOST && !managed && device == at && start && start <= at && at - start <= size &&
+           bytes <= size - (at - start);
 }
 
 }  // namespace accerl

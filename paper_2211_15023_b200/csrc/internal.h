@@ -24,6 +24,8 @@ cudaError_t device_alloc(void **out, size_t bytes);
 void device_free(void *ptr);
 // pinned host memory in the same manner; given up only when no copy of it is in flight
 cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes);
+// can kernels on the current device use this host range at its own address?
+bool device_reaches(const void *host, size_t bytes);
 
 // a non-blocking stream of the library's own with two events, on the current device; given back idle
 struct SideStream {

@@ -1,0 +1,97 @@
+// csrc/device_memory.cu on the host, against a fake of the CUDA calls it makes.  One check per run, named on
+// the command line; exits 0 when it holds, else says what does not.
+#include <cuda.h>
+#include <cuda_runtime.h>
+#include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <map>
+#include <mutex>
+#include <string>
+
+namespace fake {
+struct Range {  // host memory the driver knows
+    size_t bytes;
+    unsigned type;
+    bool mapped;
+};
+std::map<uintptr_t, Range> ranges;
+
+CUresult pointer_attributes(unsigned n, CUpointer_attribute *what, void **to, CUdeviceptr at)
+{
+    auto it = ranges.upper_bound((uintptr_t)at);
+    const bool known = it != ranges.begin() && (uintptr_t)at < (--it)->first + it->second.bytes;
+    for (unsigned i = 0; i < n; ++i) {
+        switch (what[i]) {
+        case CU_POINTER_ATTRIBUTE_MEMORY_TYPE: *(unsigned *)to[i] = known ? it->second.type : 0; break;
+        case CU_POINTER_ATTRIBUTE_IS_MANAGED: *(unsigned *)to[i] = 0; break;
+        case CU_POINTER_ATTRIBUTE_DEVICE_POINTER: *(CUdeviceptr *)to[i] = known && it->second.mapped ? at : 0; break;
+        case CU_POINTER_ATTRIBUTE_RANGE_START_ADDR: *(CUdeviceptr *)to[i] = known ? (CUdeviceptr)it->first : 0; break;
+        case CU_POINTER_ATTRIBUTE_RANGE_SIZE: *(size_t *)to[i] = known ? it->second.bytes : 0; break;
+        default: return CUDA_ERROR_INVALID_VALUE;
+        }
+    }
+    return CUDA_SUCCESS;
+}
+}  // namespace fake
+
+extern "C" {
+cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaMalloc(void **out, size_t bytes) { return *out = malloc(bytes), cudaSuccess; }
+cudaError_t cudaFree(void *p) { return free(p), cudaSuccess; }
+cudaError_t cudaHostAlloc(void **out, size_t bytes, unsigned) { return *out = malloc(bytes), cudaSuccess; }
+cudaError_t cudaFreeHost(void *p) { return free(p), cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)malloc(1), cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { return free(e), cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = (cudaStream_t)malloc(1), cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t s) { return free(s), cudaSuccess; }
+cudaError_t cudaGetDriverEntryPoint(const char *name, void **out, unsigned long long, cudaDriverEntryPointQueryResult *found)
+{
+    const bool known = !strcmp(name, "cuPointerGetAttributes");
+    *out = known ? (void *)fake::pointer_attributes : nullptr;
+    *found = known ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+    return cudaSuccess;
+}
+}
+
+#include "device_memory.cu"
+
+#define CHECK(x)                                              \
+    do {                                                      \
+        if (!(x)) {                                           \
+            printf("line %d: %s does not hold\n", __LINE__, #x); \
+            return 1;                                         \
+        }                                                     \
+    } while (0)
+
+using namespace accerl;
+
+// a range counts as the device's only when all of it lies in one known, mapped piece of host memory
+static int reach()
+{
+    alignas(4096) static char memory[16384];
+    const uintptr_t m = (uintptr_t)memory;
+    CHECK(!device_reaches(memory, 64));
+    fake::ranges[m] = {4096, CU_MEMORYTYPE_HOST, true};
+    fake::ranges[m + 8192] = {4096, CU_MEMORYTYPE_HOST, true};
+    CHECK(device_reaches(memory, 4096) && device_reaches(memory + 4092, 4) && device_reaches(memory + 8192, 64));
+    CHECK(!device_reaches(memory + 4092, 8));
+    CHECK(!device_reaches(memory, 8192 + 64));  // both ends known, pageable memory between them
+    CHECK(!device_reaches(memory + 64, 8192));
+    CHECK(!device_reaches(memory + 2, 4));
+    fake::ranges[m + 8192].mapped = false;
+    CHECK(!device_reaches(memory + 8192, 64));
+    fake::ranges[m].type = CU_MEMORYTYPE_DEVICE;
+    CHECK(!device_reaches(memory, 64));
+    return 0;
+}
+
+int main(int argc, char **argv)
+{
+    const std::string name = argc > 1 ? argv[1] : "";
+    if (name == "reach") return reach();
+    printf("no check %s\n", name.c_str());
+    return 2;
+}
