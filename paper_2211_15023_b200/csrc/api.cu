@@ -924,7 +924,12 @@ accerl_status accerl_policy_act_host(accerl_policy *p, const void *obs_host,
         const size_t bytes[3] = {4 * B * (size_t)p->n_actions, 4 * B, 4 * B};
         const bool direct = bytes[0] <= kDirectBytes && device_reaches(logits_host, bytes[0]) &&
                             device_reaches(actions_host, bytes[1]) && device_reaches(logp_host, bytes[2]);
-        const bool direct_u = direct && device_reaches(uniforms_host, 4 * B);
+        // (not where a result lies over them: a state's draw may be read after another state's results are written)
+        auto apart = [&](const void *result, size_t n) {
+            return (const char *)result + n <= (const char *)uniforms_host || (const char *)(uniforms_host + B) <= (const char *)result;
+        };
+        const bool direct_u = direct && apart(logits_host, bytes[0]) && apart(actions_host, bytes[1]) && apart(logp_host, bytes[2]) &&
+                              device_reaches(uniforms_host, 4 * B);
         if (!direct_u) ACCERL_CUDA_TRY(cudaMemcpyAsync(p->st_u, uniforms_host, 4 * B, cudaMemcpyHostToDevice, st));
         accerl_status s = run_steps(p, p->st_obs, direct_u ? uniforms_host : p->st_u, batch, direct ? logits_host : p->st_logits,
                                     direct ? actions_host : p->st_actions, direct ? logp_host : p->st_logp, nullptr, nullptr,

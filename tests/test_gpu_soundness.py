@@ -162,3 +162,29 @@ def test_act_ex_and_act_mixed_refuse_what_their_kernels_would_misread():
     g.check()
     g.close()
     o.close()
+
+
+@pytest.mark.parametrize("b", [33, 200])
+@pytest.mark.parametrize("over", ["logits", "actions", "logp"])
+def test_act_host_with_the_uniforms_in_the_place_of_a_result(over, b):
+    """A caller that reuses the pinned buffer of the draws for a result: the draws are all read before any
+    result is written, whatever the order of the states."""
+    import paper_2211_15023_b200 as P
+    import workloads as W
+    name = "student_cnn_b8192"
+    g = P.Policy(W.drawn_int8_policy(name, seed=8), b)
+    obs, u = torch.from_numpy(W.observations(name, b, seed=b)), torch.from_numpy(W.uniforms(name, b, seed=b))
+    want = [t.cpu() for t in g.act(obs.cuda(), u.cuda())]
+    out = dict(logits=torch.zeros((b, g.n_actions)).pin_memory(), actions=torch.zeros(b, dtype=torch.int32).pin_memory(),
+               logp=torch.zeros(b).pin_memory())
+    draws = out[over].view(torch.float32).reshape(-1)[:b]
+    if over == "logits":
+        draws = out[over].reshape(-1)[g.n_actions * b - b:]  # the last states' logits
+    pinned_obs = obs.pin_memory()
+    for _ in range(20):
+        draws.copy_(u)
+        g.act_host(pinned_obs, draws, tuple(out.values()))
+        for x, y in zip(out.values(), want):
+            assert torch.equal(x, y)
+    g.check()
+    g.close()
