@@ -18,6 +18,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "epilogue.cuh"
@@ -250,7 +251,7 @@ accerl_status build_mlp_plan(accerl_policy *p, const accerl_layer_desc *layers, 
     if (round_up(p->in_c, 4) > kMaxWidth) return ACCERL_OK;
     for (int i = 0; i < n_layers; ++i)
         if (layers[i].kind != ACCERL_FC || layers[i].out_c > kMaxWidth ||
-            (layers[i].flags & ACCERL_RELU_IN))
+            (layers[i].flags & ACCERL_RELU_IN) || !std::isfinite(1.0f / layers[i].s_out))  // (the kernel multiplies by it)
             return ACCERL_OK;
     auto prm = std::make_shared<MlpFusedParams>();
     memset(prm.get(), 0, sizeof(MlpFusedParams));

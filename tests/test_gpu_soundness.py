@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
+from parity_util import compare
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -187,4 +188,36 @@ def test_act_host_with_the_uniforms_in_the_place_of_a_result(over, b):
         for x, y in zip(out.values(), want):
             assert torch.equal(x, y)
     g.check()
+    g.close()
+
+
+def _with_tiny_scale(pol, layer):
+    """The policy with one layer's output on a grid so fine that the reciprocal of its scale is infinite,
+    weights and the next layer's weights scaled to match."""
+    tiny, ls = np.float32(1e-39), pol["layers"]
+    a, b = ls[layer], ls[layer + 1]
+    back = float(a["s_out"])
+    a["s_w"] = (a["s_w"].astype(np.float64) * (float(tiny) / back)).astype(np.float32)  # (subnormal, a few bits each)
+    a["bias"] = (a["bias"].astype(np.float64) * (float(tiny) / back)).astype(np.float32)
+    a["s_out"] = b["s_in"] = tiny
+    b["s_w"] = (b["s_w"].astype(np.float64) * (back / float(tiny))).astype(np.float32)
+    return pol
+
+
+def test_mlp_layer_whose_scale_has_no_finite_reciprocal():
+    import paper_2211_15023_b200 as P
+    import workloads as W
+    rng = np.random.default_rng(0)
+    layers = W.mlp([12, 96, 64, 5])
+    params = W.parameters_for(layers, 0)
+    calib = rng.standard_normal((64, 12)).astype(np.float32)
+    pol = _with_tiny_scale(oracle.calibrate("f32", (12, 1, 1), layers, params, calib), 0)
+    obs, u = rng.standard_normal((200, 12)).astype(np.float32), rng.random(200, dtype=np.float32)
+    ref = oracle.forward(pol, obs, u)
+    codes = ref["activations"][0]
+    assert len(np.unique(codes)) > 20 and (codes == 127).mean() < 0.5  # (a grid that is used)
+    g = P.Policy(pol, 200)
+    logits, actions, logp = g.act(torch.from_numpy(obs).cuda(), torch.from_numpy(u).cuda())
+    g.check()
+    compare(ref, logits.cpu().numpy(), actions.cpu().numpy(), logp.cpu().numpy())
     g.close()
