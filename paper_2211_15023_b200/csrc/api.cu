@@ -506,12 +506,14 @@ void accerl_policy_destroy(accerl_policy *p)
 {
     if (!p) return;
     DeviceGuard g(p->device);
-    cudaDeviceSynchronize();
-    for (void *d : p->owned) device_free(d);
+    // (refused while the process captures a graph, for one: kernels of this handle may still run then)
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    if (!idle) cudaGetLastError();
+    for (void *d : p->owned) device_free(d, idle);
     for (cudaEvent_t ev : p->events) cudaEventDestroy(ev);
     for (cudaEvent_t ev : p->copy_events) cudaEventDestroy(ev);
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
-    give_side_stream(p->mix);
+    give_side_stream(p->mix, idle);
     delete p->noalloc_twin;  // owns nothing on the device
     delete p;
 }

@@ -57,15 +57,14 @@ struct Memory {
     }
     static void release(void *ptr, int device)
     {
-        if (device == kHost) cudaFreeHost(ptr);
-        else cudaFree(ptr);
+        if ((device == kHost ? cudaFreeHost(ptr) : cudaFree(ptr)) != cudaSuccess) cudaGetLastError();
     }
     static cudaError_t fresh(void **out, size_t bytes, int device)
     {
         return device == kHost ? cudaHostAlloc(out, bytes, cudaHostAllocPortable) : cudaMalloc(out, bytes);
     }
     cudaError_t take(void **out, size_t bytes, int device);
-    void give(void *ptr);
+    void give(void *ptr, bool idle);
 };
 
 Memory &memory()
@@ -114,10 +113,10 @@ cudaError_t take_side_stream(SideStream *out)
     return e;
 }
 
-void give_side_stream(SideStream &s)
+void give_side_stream(SideStream &s, bool idle)
 {
     if (!s.stream) return;
-    {
+    if (idle) {
         std::lock_guard<std::mutex> lock(g_stream_mu);
         if (kept_streams().size() < kKeptStreams) {
             kept_streams().push_back(s);
@@ -160,7 +159,7 @@ cudaError_t Memory::take(void **out, size_t bytes, int device)
     return e;
 }
 
-void Memory::give(void *ptr)
+void Memory::give(void *ptr, bool idle)
 {
     if (!ptr) return;
     std::lock_guard<std::mutex> lock(mu);
@@ -170,7 +169,7 @@ void Memory::give(void *ptr)
     const auto [bytes, device] = it->second;
     live.erase(it);
     const size_t limit = device == kHost ? kKeptHost : kKept;
-    if (bytes > limit) {
+    if (!idle || bytes > limit) {
         release(ptr, device);
         return;
     }
@@ -191,13 +190,13 @@ cudaError_t device_alloc(void **out, size_t bytes)
     return e == cudaSuccess ? memory().take(out, bytes, device) : e;
 }
 
-void device_free(void *ptr) { memory().give(ptr); }
+void device_free(void *ptr, bool idle) { memory().give(ptr, idle); }
 
 cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes)
 {
     void *ptr = nullptr;
     const cudaError_t e = memory().take(&ptr, bytes, kHost);
-    if (e == cudaSuccess) *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at); });
+    if (e == cudaSuccess) *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at, true); });
     return e;
 }
 

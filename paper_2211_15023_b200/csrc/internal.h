@@ -19,22 +19,23 @@ namespace accerl {
 
 void set_error(const char *fmt, ...);
 
-// device memory (device_memory.cu); device_free only when nothing on the device uses the block any more
+// device memory (device_memory.cu).  `idle`: nothing on the device uses the block any more, the next policy may
+// have it; where that could not be established (a synchronisation failed) it goes back to the driver.
 cudaError_t device_alloc(void **out, size_t bytes);
-void device_free(void *ptr);
+void device_free(void *ptr, bool idle);
 // pinned host memory in the same manner; given up only when no copy of it is in flight
 cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes);
 // can kernels on the current device use this host range at its own address?
 bool device_reaches(const void *host, size_t bytes);
 
-// a non-blocking stream of the library's own with two events, on the current device; given back idle
+// a non-blocking stream of the library's own with two events, on the current device
 struct SideStream {
     cudaStream_t stream = nullptr;
     cudaEvent_t events[2] = {nullptr, nullptr};
     int device = 0;
 };
 cudaError_t take_side_stream(SideStream *out);
-void give_side_stream(SideStream &s);
+void give_side_stream(SideStream &s, bool idle);
 
 // let a kernel use `bytes` of dynamic shared memory on the current device (api.cu)
 cudaError_t allow_smem(const void *kernel, size_t bytes);

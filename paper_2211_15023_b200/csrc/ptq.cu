@@ -174,8 +174,8 @@ struct DeviceArena {
     size_t at = 0;
     ~DeviceArena()
     {
-        if (base) cudaStreamSynchronize(0);  // (where a call failed, its kernels may still run)
-        device_free(base);
+        // (where a call failed, its kernels may still run)
+        if (base) device_free(base, cudaStreamSynchronize(0) == cudaSuccess);
     }
     template <typename T>
     T *take(size_t count)

@@ -201,8 +201,8 @@ accerl_status fit_requants(accerl_policy *p, const accerl_layer_desc *layers, in
         char *ptr = nullptr;
         ~Device()
         {
-            if (ptr) cudaStreamSynchronize(0);  // (where a call failed, its kernels may still run)
-            device_free(ptr);
+            // (where a call failed, its kernels may still run)
+            if (ptr) device_free(ptr, cudaStreamSynchronize(0) == cudaSuccess);
         }
     } dev;
     const size_t job_bytes = (jobs.size() * sizeof(FitJob) + 255) / 256 * 256, res_bytes = (jobs.size() * sizeof(FitResult) + 255) / 256 * 256;

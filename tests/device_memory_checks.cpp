@@ -36,17 +36,22 @@ CUresult pointer_attributes(unsigned n, CUpointer_attribute *what, void **to, CU
 }
 }  // namespace fake
 
+namespace fake {
+int allocations = 0, frees = 0;  // of device memory
+int streams = 0;                 // alive
+}  // namespace fake
+
 extern "C" {
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
-cudaError_t cudaMalloc(void **out, size_t bytes) { return *out = malloc(bytes), cudaSuccess; }
-cudaError_t cudaFree(void *p) { return free(p), cudaSuccess; }
+cudaError_t cudaMalloc(void **out, size_t bytes) { return ++fake::allocations, *out = malloc(bytes), cudaSuccess; }
+cudaError_t cudaFree(void *p) { return ++fake::frees, free(p), cudaSuccess; }
 cudaError_t cudaHostAlloc(void **out, size_t bytes, unsigned) { return *out = malloc(bytes), cudaSuccess; }
 cudaError_t cudaFreeHost(void *p) { return free(p), cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)malloc(1), cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return free(e), cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = (cudaStream_t)malloc(1), cudaSuccess; }
-cudaError_t cudaStreamDestroy(cudaStream_t s) { return free(s), cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return ++fake::streams, *s = (cudaStream_t)malloc(1), cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t s) { return --fake::streams, free(s), cudaSuccess; }
 cudaError_t cudaGetDriverEntryPoint(const char *name, void **out, unsigned long long, cudaDriverEntryPointQueryResult *found)
 {
     const bool known = !strcmp(name, "cuPointerGetAttributes");
@@ -88,10 +93,34 @@ static int reach()
     return 0;
 }
 
+// what is given back idle serves the next allocation; what may still be in use goes back to the driver
+static int busy()
+{
+    void *a = nullptr, *b = nullptr;
+    CHECK(device_alloc(&a, 100000) == cudaSuccess && fake::allocations == 1);
+    device_free(a, true);
+    CHECK(fake::frees == 0);
+    CHECK(device_alloc(&b, 100000) == cudaSuccess && b == a && fake::allocations == 1);
+    device_free(b, false);
+    CHECK(fake::frees == 1);
+    CHECK(device_alloc(&a, 100000) == cudaSuccess && fake::allocations == 2);
+    device_free(a, true);
+    device_free(nullptr, false);
+    SideStream s;
+    CHECK(take_side_stream(&s) == cudaSuccess && fake::streams == 1);
+    give_side_stream(s, false);
+    CHECK(fake::streams == 0 && !s.stream);
+    CHECK(take_side_stream(&s) == cudaSuccess);
+    give_side_stream(s, true);
+    CHECK(fake::streams == 1 && take_side_stream(&s) == cudaSuccess && fake::streams == 1);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const std::string name = argc > 1 ? argv[1] : "";
     if (name == "reach") return reach();
+    if (name == "busy") return busy();
     printf("no check %s\n", name.c_str());
     return 2;
 }
