@@ -16,6 +16,7 @@
 #include <chrono>
 #include <list>
 #include <mutex>
+#include <new>
 #include <unordered_map>
 #include <vector>
 
@@ -196,8 +197,16 @@ cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes)
 {
     void *ptr = nullptr;
     const cudaError_t e = memory().take(&ptr, bytes, kHost);
-    if (e == cudaSuccess) *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at, true); });
-    return e;
+    if (e == cudaSuccess) {
+        *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at, true); });
+        return e;
+    }
+    // pageable memory serves as well: the driver stages its copies
+    cudaGetLastError();
+    char *pageable = new (std::nothrow) char[std::max<size_t>(bytes, 1)];
+    if (!pageable) return e;
+    *out = std::shared_ptr<char[]>(pageable);
+    return cudaSuccess;
 }
 
 // Pinned and mapped, 4-byte aligned, and all of it inside one allocation or registration: with its two ends in

@@ -39,6 +39,7 @@ CUresult pointer_attributes(unsigned n, CUpointer_attribute *what, void **to, CU
 namespace fake {
 int allocations = 0, frees = 0;  // of device memory
 int streams = 0;                 // alive
+bool refuse_pinned = false;
 }  // namespace fake
 
 extern "C" {
@@ -46,7 +47,10 @@ cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMalloc(void **out, size_t bytes) { return ++fake::allocations, *out = malloc(bytes), cudaSuccess; }
 cudaError_t cudaFree(void *p) { return ++fake::frees, free(p), cudaSuccess; }
-cudaError_t cudaHostAlloc(void **out, size_t bytes, unsigned) { return *out = malloc(bytes), cudaSuccess; }
+cudaError_t cudaHostAlloc(void **out, size_t bytes, unsigned)
+{
+    return fake::refuse_pinned ? cudaErrorMemoryAllocation : (*out = malloc(bytes), cudaSuccess);
+}
 cudaError_t cudaFreeHost(void *p) { return free(p), cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)malloc(1), cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return free(e), cudaSuccess; }
@@ -116,11 +120,26 @@ static int busy()
     return 0;
 }
 
+// where the driver grants no pinned memory, parameters travel in ordinary memory
+static int pageable()
+{
+    std::shared_ptr<char[]> a, b;
+    fake::refuse_pinned = true;
+    CHECK(pinned_alloc(&a, 5000) == cudaSuccess && a);
+    memset(a.get(), 1, 5000);
+    CHECK(pinned_alloc(&b, 0) == cudaSuccess && b);
+    a.reset();
+    fake::refuse_pinned = false;
+    CHECK(pinned_alloc(&a, 5000) == cudaSuccess && a);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const std::string name = argc > 1 ? argv[1] : "";
     if (name == "reach") return reach();
     if (name == "busy") return busy();
+    if (name == "pageable") return pageable();
     printf("no check %s\n", name.c_str());
     return 2;
 }
