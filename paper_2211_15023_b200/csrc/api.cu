@@ -518,7 +518,7 @@ void accerl_policy_destroy(accerl_policy *p)
     delete p;
 }
 
-accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const int32_t in_shape[3],
+static accerl_status create_policy(accerl_policy **out, int32_t in_kind, const int32_t in_shape[3],
                                    float s_input, const accerl_layer_desc *layers,
                                    int32_t n_layers, int32_t max_batch, uint32_t flags,
                                    int32_t device)
@@ -607,11 +607,11 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
     p->n_out = cur.c;
     p->n_actions = cur.c - (value_head ? 1 : 0);
 
+    struct Unfinished {  // the handle goes with a failure
+        accerl_policy *p;
+        ~Unfinished() { accerl_policy_destroy(p); }
+    } unfinished{p};
     accerl_status st = ACCERL_OK;
-    auto fail = [&](accerl_status s) {
-        accerl_policy_destroy(p);
-        return s;
-    };
 
     // ---- layer plans and parameters
     Shape in{p->in_c, p->in_h, p->in_w};
@@ -630,7 +630,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         L.oc_pad = round_up(L.out_c, 16);
         if (d.kind != ACCERL_MAXPOOL) {
             void *words = nullptr, *words_dev = nullptr;  // (packed in place: for large layers a copy costs as much)
-            if ((st = upload_room(p, generic_bytes(d, L), &words, &words_dev)) != ACCERL_OK) return fail(st);
+            if ((st = upload_room(p, generic_bytes(d, L), &words, &words_dev)) != ACCERL_OK) return st;
             pack_generic(d, L, (int8_t *)words);
             L.w_generic = (int32_t *)words_dev;
             L.host_rows = (const int8_t *)words;
@@ -640,12 +640,12 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
                 ks[c] = k;
                 bs[c] = d.bias[c];
             }
-            if ((st = upload(p, ks, &L.kscale)) != ACCERL_OK) return fail(st);
-            if ((st = upload(p, bs, &L.bias)) != ACCERL_OK) return fail(st);
+            if ((st = upload(p, ks, &L.kscale)) != ACCERL_OK) return st;
+            if ((st = upload(p, bs, &L.bias)) != ACCERL_OK) return st;
             if (d.skip_from >= 0) {
                 std::vector<int32_t> sm(L.oc_pad, 0);
                 for (int c = 0; c < d.out_c; ++c) sm[c] = d.skip_mul[c];
-                if ((st = upload(p, sm, &L.skip_mul)) != ACCERL_OK) return fail(st);
+                if ((st = upload(p, sm, &L.skip_mul)) != ACCERL_OK) return st;
             }
             L.how = d.kind == ACCERL_CONV2D ? "conv_dp4a_kernel" : "fc_dp4a_kernel";
         } else {
@@ -699,7 +699,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         if (e != cudaSuccess) {
             set_error("create: cudaMalloc of %zu workspace bytes failed: %s", total, cudaGetErrorString(e));
             cudaGetLastError();
-            return fail(e == cudaErrorMemoryAllocation ? ACCERL_ERR_OOM : ACCERL_ERR_CUDA);
+            return e == cudaErrorMemoryAllocation ? ACCERL_ERR_OOM : ACCERL_ERR_CUDA;
         }
         p->owned.push_back(d);
         p->workspace_bytes += total;
@@ -719,7 +719,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
             r = r < -128.f ? -128.f : (r > 127.f ? 127.f : r);
             lut[u] = (int8_t)r;
         }
-        if ((st = upload(p, lut, &p->lut)) != ACCERL_OK) return fail(st);
+        if ((st = upload(p, lut, &p->lut)) != ACCERL_OK) return st;
         p->ingest_arith = fit_ingest_line(lut.data(), &p->ingest_mul, &p->ingest_add) ? 1 : 0;
         p->ingest_shift1 = true;
         for (int u = 0; u < 256; ++u)
@@ -736,7 +736,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         if (e != cudaSuccess) {
             set_error("create: cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
             cudaGetLastError();
-            return fail(e == cudaErrorMemoryAllocation ? ACCERL_ERR_OOM : ACCERL_ERR_CUDA);
+            return e == cudaErrorMemoryAllocation ? ACCERL_ERR_OOM : ACCERL_ERR_CUDA;
         }
         p->owned.push_back(d);
         p->z_scratch = (float *)d;
@@ -744,7 +744,7 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
     }
     {
         std::vector<int> zero(256, 0);  // word 0 is the status; the rest is trace space
-        if ((st = upload(p, zero, &p->status_word)) != ACCERL_OK) return fail(st);
+        if ((st = upload(p, zero, &p->status_word)) != ACCERL_OK) return st;
     }
     // ---- launch plan
     {
@@ -779,31 +779,45 @@ accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const i
         if (pe == cudaSuccess) pe = cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
         if (pe != cudaSuccess) {
             set_error("create: cudaDeviceGetAttribute: %s", cudaGetErrorString(pe));
-            return fail(ACCERL_ERR_CUDA);
+            return ACCERL_ERR_CUDA;
         }
         if (major != 10) {
             set_error("create: this library is built for sm_100a only (device is sm_%d%d)", major, minor);
-            return fail(ACCERL_ERR_UNSUPPORTED);
+            return ACCERL_ERR_UNSUPPORTED;
         }
     }
     if (!(flags & ACCERL_FLAG_FORCE_GENERIC)) {
         bool used = false;
-        if ((st = build_tc_plan(p, layers, n_layers, &used)) != ACCERL_OK) return fail(st);
+        if ((st = build_tc_plan(p, layers, n_layers, &used)) != ACCERL_OK) return st;
         if (!used && (st = build_tc_mixed_plan(p, layers, n_layers, &used)) != ACCERL_OK)
-            return fail(st);
+            return st;
         if (!used && !unfuse_for_taps(p) &&
             (st = build_mlp_plan(p, layers, n_layers, &used)) != ACCERL_OK)
-            return fail(st);
+            return st;
     }
-    if ((st = flush_uploads(p)) != ACCERL_OK) return fail(st);
+    if ((st = flush_uploads(p)) != ACCERL_OK) return st;
     for (LayerPlan &L : p->layers) L.host_rows = nullptr;
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         set_error("create: %s", cudaGetErrorString(e));
-        return fail(ACCERL_ERR_CUDA);
+        return ACCERL_ERR_CUDA;
     }
+    unfinished.p = nullptr;
     *out = p;
     return ACCERL_OK;
+}
+
+accerl_status accerl_policy_create(accerl_policy **out, int32_t in_kind, const int32_t in_shape[3],
+                                   float s_input, const accerl_layer_desc *layers,
+                                   int32_t n_layers, int32_t max_batch, uint32_t flags,
+                                   int32_t device)
+{
+    try {
+        return create_policy(out, in_kind, in_shape, s_input, layers, n_layers, max_batch, flags, device);
+    } catch (const std::bad_alloc &) {
+        set_error("create: out of host memory");
+        return ACCERL_ERR_OOM;
+    }
 }
 
 accerl_status accerl_policy_act(accerl_policy *p, const void *obs_dev, const float *uniforms_dev,

@@ -7,6 +7,9 @@
 // driver when an allocation fails.  Blocks are handed back only when nothing on the device uses them any
 // more, so any thread and any stream may have them next.
 //
+// Running out of host memory for the bookkeeping is an allocation that fails, or a block that is not kept:
+// nothing here throws.
+//
 // Pinned host memory for parameters on their way to the device and quantised ones on their way back is
 // kept in the same manner (at most kKeptHost bytes): pageable blocks of that size are fresh pages for
 // every policy, 0.4 ms of faults each, and copies from and to them are staged by the driver.
@@ -18,7 +21,6 @@
 #include <mutex>
 #include <new>
 #include <unordered_map>
-#include <vector>
 
 #include "internal.h"
 
@@ -70,18 +72,16 @@ struct Memory {
 
 Memory &memory()
 {
-    static Memory *m = new Memory;  // (never destroyed: the driver may be gone before static objects are)
+    alignas(Memory) static char room[sizeof(Memory)];
+    static Memory *m = new (room) Memory;  // (never destroyed: the driver may be gone before static objects are)
     return *m;
 }
 
 // side streams not in use (creating one, with its events, takes a tenth of a millisecond)
 constexpr size_t kKeptStreams = 8;
 std::mutex g_stream_mu;
-std::vector<SideStream> &kept_streams()
-{
-    static std::vector<SideStream> *v = new std::vector<SideStream>;  // (as above)
-    return *v;
-}
+SideStream g_streams[kKeptStreams];
+size_t g_n_streams = 0;
 
 }  // namespace
 
@@ -92,11 +92,10 @@ cudaError_t take_side_stream(SideStream *out)
     if (e != cudaSuccess) return e;
     {
         std::lock_guard<std::mutex> lock(g_stream_mu);
-        std::vector<SideStream> &kept = kept_streams();
-        for (size_t i = 0; i < kept.size(); ++i)
-            if (kept[i].device == device) {
-                *out = kept[i];
-                kept.erase(kept.begin() + (long)i);
+        for (size_t i = 0; i < g_n_streams; ++i)
+            if (g_streams[i].device == device) {
+                *out = g_streams[i];
+                g_streams[i] = g_streams[--g_n_streams];
                 return cudaSuccess;
             }
     }
@@ -119,8 +118,8 @@ void give_side_stream(SideStream &s, bool idle)
     if (!s.stream) return;
     if (idle) {
         std::lock_guard<std::mutex> lock(g_stream_mu);
-        if (kept_streams().size() < kKeptStreams) {
-            kept_streams().push_back(s);
+        if (g_n_streams < kKeptStreams) {
+            g_streams[g_n_streams++] = s;
             s = SideStream();
             return;
         }
@@ -143,9 +142,17 @@ cudaError_t Memory::take(void **out, size_t bytes, int device)
         if (it->device == device && it->bytes >= want && it->bytes <= want + want / 2 + grain &&
             (best == kept.end() || it->bytes < best->bytes))
             best = it;
+    auto handed_out = [&](void *ptr, size_t size) {
+        try {
+            live[ptr] = {size, device};
+            return true;
+        } catch (const std::bad_alloc &) {
+            return false;
+        }
+    };
     if (best != kept.end()) {
+        if (!handed_out(best->ptr, best->bytes)) return cudaErrorMemoryAllocation;
         *out = best->ptr;
-        live[best->ptr] = {best->bytes, device};
         bytes_of(device) -= best->bytes;
         kept.erase(best);
         return cudaSuccess;
@@ -156,7 +163,11 @@ cudaError_t Memory::take(void **out, size_t bytes, int device)
         while (!kept.empty()) drop(kept.begin());
         e = fresh(out, want, device);
     }
-    if (e == cudaSuccess) live[*out] = {want, device};
+    if (e == cudaSuccess && !handed_out(*out, want)) {
+        release(*out, device);
+        *out = nullptr;
+        e = cudaErrorMemoryAllocation;
+    }
     return e;
 }
 
@@ -174,7 +185,12 @@ void Memory::give(void *ptr, bool idle)
         release(ptr, device);
         return;
     }
-    kept.push_back(Block{ptr, bytes, device, std::chrono::steady_clock::now()});
+    try {
+        kept.push_back(Block{ptr, bytes, device, std::chrono::steady_clock::now()});
+    } catch (const std::bad_alloc &) {
+        release(ptr, device);
+        return;
+    }
     bytes_of(device) += bytes;
     for (auto at = kept.begin(); bytes_of(device) > limit; ) {  // the oldest of its kind
         const auto next = std::next(at);
@@ -197,16 +213,18 @@ cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes)
 {
     void *ptr = nullptr;
     const cudaError_t e = memory().take(&ptr, bytes, kHost);
-    if (e == cudaSuccess) {
-        *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at, true); });
-        return e;
+    try {
+        if (e == cudaSuccess) {  // (where the shared pointer cannot be made, it gives the block back itself)
+            *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at, true); });
+            return e;
+        }
+        // pageable memory serves as well: the driver stages its copies
+        cudaGetLastError();
+        *out = std::shared_ptr<char[]>(new char[std::max<size_t>(bytes, 1)]);
+        return cudaSuccess;
+    } catch (const std::bad_alloc &) {
+        return cudaErrorMemoryAllocation;
     }
-    // pageable memory serves as well: the driver stages its copies
-    cudaGetLastError();
-    char *pageable = new (std::nothrow) char[std::max<size_t>(bytes, 1)];
-    if (!pageable) return e;
-    *out = std::shared_ptr<char[]>(pageable);
-    return cudaSuccess;
 }
 
 // Pinned and mapped, 4-byte aligned, and all of it inside one allocation or registration: with its two ends in

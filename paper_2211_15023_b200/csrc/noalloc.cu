@@ -3,6 +3,7 @@
 // The activation workspace of this variant is a fixed array inside the library image instead of
 // buffers obtained from cudaMalloc.  See the declaration in accerl.h for who needs it and why.
 #include <algorithm>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <type_traits>
@@ -67,11 +68,8 @@ using namespace accerl;
 // lead there.  Weights, scales and the status word are the handle's; nothing is allocated on the device.
 // (Stepping through the CUDA-core kernels instead took 182 us for 160 states of the Nature-CNN.)
 // Null when the plan keeps tensors whose borders must stay zero, or taps.
-accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
+std::unique_ptr<accerl_policy> make_twin(accerl_policy *p, unsigned char *base)
 {
-    std::lock_guard<std::mutex> lock(g_mu);
-    if (p->noalloc_tried) return p->noalloc_twin;
-    p->noalloc_tried = true;
     if (p->flags & (ACCERL_FLAG_KEEP_ACTIVATIONS | ACCERL_FLAG_FORCE_GENERIC)) return nullptr;
     bool resident = false;
     for (const Step &s : p->steps) {
@@ -117,8 +115,7 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
         r.new_base = (char *)base + at;
         at += (r.per_state * cap + 1023) / 1024 * 1024;
     }
-    accerl_policy *q = new (std::nothrow) accerl_policy(*p);
-    if (!q) return nullptr;
+    std::unique_ptr<accerl_policy> q(new accerl_policy(*p));
     q->noalloc_twin = nullptr;
     q->owned.clear();
     q->events.clear();
@@ -171,12 +168,22 @@ accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
         }
     }
     move(q->z_scratch);
-    if (!ok) {
-        delete q;
-        return nullptr;
-    }
-    p->noalloc_twin = q;
+    if (!ok) q.reset();
     return q;
+}
+
+// made once per handle; null for good where there is none, or no host memory for it
+accerl_policy *twin_of(accerl_policy *p, unsigned char *base)
+{
+    std::lock_guard<std::mutex> lock(g_mu);
+    if (!p->noalloc_tried) {
+        p->noalloc_tried = true;
+        try {
+            p->noalloc_twin = make_twin(p, base).release();
+        } catch (const std::bad_alloc &) {
+        }
+    }
+    return p->noalloc_twin;
 }
 
 }  // namespace

@@ -194,7 +194,7 @@ unsigned blocks_for(long long n) { return (unsigned)((n + 255) / 256); }
 
 using namespace accerl;
 
-extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t in_kind,
+static accerl_status quantise_and_create(accerl_policy **out, int32_t in_kind,
                                                    const int32_t in_shape[3],
                                                    const accerl_layer_fp32 *layers, int32_t n_layers,
                                                    const void *calib_obs_host, int32_t calib_rows,
@@ -287,13 +287,7 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
         size_t nw, packed_bytes;
         int scale;        // index of the maximum its output scale comes from (a pool passes its input's on)
     };
-    std::vector<Layer> net;
-    try {
-        net.resize(n_layers);
-    } catch (const std::bad_alloc &) {
-        set_error("create_fp32: out of host memory");
-        return ACCERL_ERR_OOM;
-    }
+    std::vector<Layer> net(n_layers);
     int n_run = n_layers;  // layers up to the one with the logits
     DeviceArena mem;
     void *obs_dev = nullptr;
@@ -422,14 +416,8 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
     }
     // one block, kept as it comes back: copies of its parts cost their page faults again
     std::shared_ptr<char[]> back;
-    std::vector<accerl_policy::PtqLayer> Q;
+    std::vector<accerl_policy::PtqLayer> Q(n_layers);
     ACCERL_CUDA_TRY(pinned_alloc(&back, results_bytes));
-    try {
-        Q.resize(n_layers);
-    } catch (const std::bad_alloc &) {
-        set_error("create_fp32: out of host memory");
-        return ACCERL_ERR_OOM;
-    }
     ACCERL_CUDA_TRY(cudaMemcpy(back.get(), results, results_bytes, cudaMemcpyDeviceToHost));
     auto host = [&](const void *dev) { return back.get() + ((const char *)dev - results); };
     auto scale = [&](int at) {
@@ -485,6 +473,22 @@ extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t 
     p->ptq = std::move(Q);
     p->ptq_data = std::move(back);
     return ACCERL_OK;
+}
+
+extern "C" accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t in_kind,
+                                                   const int32_t in_shape[3],
+                                                   const accerl_layer_fp32 *layers, int32_t n_layers,
+                                                   const void *calib_obs_host, int32_t calib_rows,
+                                                   int32_t prune_2_4, int32_t max_batch, uint32_t flags,
+                                                   int32_t device)
+{
+    try {
+        return quantise_and_create(out, in_kind, in_shape, layers, n_layers, calib_obs_host, calib_rows, prune_2_4, max_batch, flags,
+                                   device);
+    } catch (const std::bad_alloc &) {
+        set_error("create_fp32: out of host memory");
+        return ACCERL_ERR_OOM;
+    }
 }
 
 extern "C" accerl_status accerl_policy_export(const accerl_policy *p, int32_t layer, int8_t *w_host,

@@ -8,7 +8,19 @@
 
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
+
+// the allocations that are still granted
+static long grants = 1L << 40;
+void *operator new(size_t bytes)
+{
+    void *p = grants-- > 0 ? malloc(bytes ? bytes : 1) : nullptr;
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void *p) noexcept { free(p); }
+void operator delete(void *p, size_t) noexcept { free(p); }
 
 namespace fake {
 struct Range {  // host memory the driver knows
@@ -134,12 +146,36 @@ static int pageable()
     return 0;
 }
 
+// host memory that runs out anywhere on the way fails the call or drops the block, and throws nothing
+static int hungry()
+{
+    void *first = nullptr;
+    for (long n = 0; n < 12; ++n) {
+        void *a = nullptr, *b = nullptr;
+        std::shared_ptr<char[]> h;
+        SideStream s;
+        grants = n;
+        const cudaError_t ea = device_alloc(&a, 1000), eb = device_alloc(&b, 5 << 20), eh = pinned_alloc(&h, 1000);
+        CHECK((ea == cudaSuccess) == (a != nullptr) && (eb == cudaSuccess) == (b != nullptr) && (eh == cudaSuccess) == !!h);
+        CHECK(ea == cudaSuccess || ea == cudaErrorMemoryAllocation);
+        CHECK(take_side_stream(&s) == cudaSuccess);
+        device_free(a, true);
+        device_free(b, true);
+        h.reset();
+        give_side_stream(s, true);
+        grants = 1L << 40;
+    }
+    CHECK(device_alloc(&first, 1000) == cudaSuccess);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const std::string name = argc > 1 ? argv[1] : "";
     if (name == "reach") return reach();
     if (name == "busy") return busy();
     if (name == "pageable") return pageable();
+    if (name == "hungry") return hungry();
     printf("no check %s\n", name.c_str());
     return 2;
 }

@@ -18,7 +18,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("check", ["reach", "busy", "pageable"])
+@pytest.mark.parametrize("check", ["reach", "busy", "pageable", "hungry"])
 def test_device_memory(program, check):
     r = subprocess.run([program, check], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
