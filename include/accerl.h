@@ -437,11 +437,20 @@ accerl_status accerl_tc_probe_i8(int32_t device, int32_t n, int32_t issuing_warp
 
 /*
  * Free the handle and its device memory.  Synchronises the device.  NULL is allowed.  Up to 512 MB of such
- * memory per process stays with the library for the next policy (building one is then free of cudaMalloc
- * and cudaFree): no block for more than 30 s without use once another policy is built or destroyed, none
- * when an allocation fails.
+ * memory per process, and 64 MB of pinned host memory, stay with the library for the next policy (building one
+ * is then free of cudaMalloc and cudaFree), the transient memory of accerl_policy_create_fp32 among them: no
+ * block for more than 30 s without use (a thread of the library's own returns it then, and ends when nothing
+ * is kept), none when an allocation of the library fails, none after accerl_trim.  Returning memory can hold up
+ * launches of the process for as long as cudaFree does: who cannot have that later calls accerl_trim when it suits.
  */
 void accerl_policy_destroy(accerl_policy *p);
+
+/*
+ * Give back to the driver what the library keeps for the next policy, now: for a process that shares the
+ * device's memory with others, after its policies are built or when another part of it needs the room.  Frees
+ * memory (cudaFree may wait for the device): not while a stream is being captured.  Any thread.
+ */
+void accerl_trim(void);
 
 /* Message for the calling thread's most recent failing call; never NULL. */
 const char *accerl_last_error(void);

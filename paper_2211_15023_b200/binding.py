@@ -87,6 +87,7 @@ def library() -> C.CDLL:
         lib.accerl_tc_probe_i8.restype = C.c_int
         lib.accerl_policy_destroy.argtypes = [vp]
         lib.accerl_policy_destroy.restype = None
+        lib.accerl_trim.argtypes, lib.accerl_trim.restype = [], None
         lib.accerl_last_error.restype = C.c_char_p
         lib.accerl_version.restype = C.c_char_p
         for f in ("create", "act", "act_timed", "act_noalloc", "act_host", "read_activation", "check", "info"):
@@ -134,6 +135,11 @@ def tc_probe_i8(n: int, issuing_warps: int = 1, mmas_per_warp: int = 4096, ctas:
     ops = ctas * issuing_warps * mmas_per_warp * 2.0 * 128 * n * 32
     return dict(n=n, issuing_warps=issuing_warps, mmas_per_warp=mmas_per_warp, ctas=ctas, layout=layout, a_shift_rows=a_shift_rows, commit_every=commit_every,
                 ms=ms.value, cycles_per_mma=cyc.value, tops=ops / (ms.value * 1e-3) / 1e12)
+
+
+def trim():
+    """accerl_trim: give back the memory kept for the next policy."""
+    library().accerl_trim()
 
 
 def _stream_of(t, stream):

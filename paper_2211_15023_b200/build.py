@@ -68,8 +68,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         list(pool.map(subprocess.check_call, cmds))
     if force or _stale(SO, objs):
         tmp = SO + ".%d.tmp" % os.getpid()
-        subprocess.check_call([NVCC, "-shared", "-cudart", "static", "-gencode",
-                               "arch=compute_100a,code=sm_100a", "-o", tmp, *objs])
+        # (nodelete: a thread of the library may be asleep in it when a program closes it)
+        subprocess.check_call([NVCC, "-shared", "-cudart", "static", "-gencode", "arch=compute_100a,code=sm_100a",
+                               "-Xlinker", "-z", "-Xlinker", "nodelete", "-o", tmp, *objs])
         os.replace(tmp, SO)
     _build_calls(force)
     return SO

@@ -502,6 +502,8 @@ extern "C" {
 const char *accerl_last_error(void) { return g_err; }
 const char *accerl_version(void) { return "accerl-b200 0.1 (sm_100a)"; }
 
+void accerl_trim(void) { release_kept(); }
+
 void accerl_policy_destroy(accerl_policy *p)
 {
     if (!p) return;

@@ -3,9 +3,10 @@
 // do the same, and a Compressor that hands over a new policy every few seconds pays for a dozen of them
 // each time (building and calibrating the residual network: 9 ms at best, 20 to 300 on a busy host).
 // So blocks that policies give back are kept for the next one: at most kKept bytes per process, none for
-// longer than kIdle without use once the library is called again, and all of them are returned to the
-// driver when an allocation fails.  Blocks are handed back only when nothing on the device uses them any
-// more, so any thread and any stream may have them next.
+// longer than kIdle without use, and all of them are returned to the driver when an allocation fails or the
+// caller asks (accerl_trim).  A thread that exists only while something is kept returns what has lain idle:
+// a process that builds a policy and then only steps it makes no call that could.  Blocks are handed back
+// only when nothing on the device uses them any more, so any thread and any stream may have them next.
 //
 // Running out of host memory for the bookkeeping is an allocation that fails, or a block that is not kept:
 // nothing here throws.
@@ -20,6 +21,7 @@
 #include <list>
 #include <mutex>
 #include <new>
+#include <thread>
 #include <unordered_map>
 
 #include "internal.h"
@@ -30,13 +32,19 @@ namespace {
 
 constexpr size_t kKept = (size_t)512 << 20;
 constexpr size_t kKeptHost = (size_t)64 << 20;
-constexpr std::chrono::seconds kIdle(30);
+#ifndef ACCERL_KEEP_IDLE_MS
+#define ACCERL_KEEP_IDLE_MS 30000
+#endif
+constexpr std::chrono::milliseconds kIdle(ACCERL_KEEP_IDLE_MS);
 constexpr int kHost = -1;  // in place of a device
 
-struct Block {
-    void *ptr;
+struct Piece {
     size_t bytes;
-    int device;
+    int device;  // or kHost
+    int current; // the device that was current when it was allocated
+};
+struct Block : Piece {
+    void *ptr;
     std::chrono::steady_clock::time_point since;
 };
 
@@ -44,19 +52,16 @@ struct Memory {
     std::mutex mu;
     std::list<Block> kept;  // oldest first
     size_t kept_bytes = 0, kept_host_bytes = 0;
-    std::unordered_map<void *, std::pair<size_t, int>> live;  // size and device of every block handed out
+    std::unordered_map<void *, Piece> live;  // every block handed out
+    bool watched = false;                    // the thread that ends what is idle runs
 
     size_t &bytes_of(int device) { return device == kHost ? kept_host_bytes : kept_bytes; }
-    void drop(std::list<Block>::iterator it)
+    Block pop(std::list<Block>::iterator it)
     {
-        bytes_of(it->device) -= it->bytes;
-        release(it->ptr, it->device);
+        const Block b = *it;
+        bytes_of(b.device) -= b.bytes;
         kept.erase(it);
-    }
-    void drop_idle()
-    {
-        const auto now = std::chrono::steady_clock::now();
-        while (!kept.empty() && now - kept.front().since > kIdle) drop(kept.begin());
+        return b;
     }
     static void release(void *ptr, int device)
     {
@@ -66,8 +71,11 @@ struct Memory {
     {
         return device == kHost ? cudaHostAlloc(out, bytes, cudaHostAllocPortable) : cudaMalloc(out, bytes);
     }
-    cudaError_t take(void **out, size_t bytes, int device);
+    cudaError_t take(void **out, size_t bytes, int device, int current);
     void give(void *ptr, bool idle);
+    void release_all();
+    bool watch();
+    void end_idle();
 };
 
 Memory &memory()
@@ -82,6 +90,12 @@ constexpr size_t kKeptStreams = 8;
 std::mutex g_stream_mu;
 SideStream g_streams[kKeptStreams];
 size_t g_n_streams = 0;
+void destroy(SideStream &s)
+{
+    for (cudaEvent_t ev : s.events) cudaEventDestroy(ev);
+    cudaStreamDestroy(s.stream);
+    s = SideStream();
+}
 
 }  // namespace
 
@@ -124,46 +138,41 @@ void give_side_stream(SideStream &s, bool idle)
             return;
         }
     }
-    for (cudaEvent_t ev : s.events) cudaEventDestroy(ev);
-    cudaStreamDestroy(s.stream);
-    s = SideStream();
+    destroy(s);
 }
 
-cudaError_t Memory::take(void **out, size_t bytes, int device)
+cudaError_t Memory::take(void **out, size_t bytes, int device, int current)
 {
     *out = nullptr;
     bytes = std::max<size_t>(bytes, 1);
     const size_t grain = bytes < ((size_t)1 << 20) ? (size_t)64 << 10 : (size_t)2 << 20;
     const size_t want = (bytes + grain - 1) / grain * grain;
     std::lock_guard<std::mutex> lock(mu);
-    drop_idle();
     auto best = kept.end();  // the smallest kept block that is not much too large
     for (auto it = kept.begin(); it != kept.end(); ++it)
         if (it->device == device && it->bytes >= want && it->bytes <= want + want / 2 + grain &&
             (best == kept.end() || it->bytes < best->bytes))
             best = it;
-    auto handed_out = [&](void *ptr, size_t size) {
+    auto handed_out = [&](void *ptr, const Piece &piece) {
         try {
-            live[ptr] = {size, device};
+            live[ptr] = piece;
             return true;
         } catch (const std::bad_alloc &) {
             return false;
         }
     };
     if (best != kept.end()) {
-        if (!handed_out(best->ptr, best->bytes)) return cudaErrorMemoryAllocation;
-        *out = best->ptr;
-        bytes_of(device) -= best->bytes;
-        kept.erase(best);
+        if (!handed_out(best->ptr, *best)) return cudaErrorMemoryAllocation;
+        *out = pop(best).ptr;
         return cudaSuccess;
     }
     cudaError_t e = fresh(out, want, device);
     if (e == cudaErrorMemoryAllocation && !kept.empty()) {
         cudaGetLastError();
-        while (!kept.empty()) drop(kept.begin());
+        release_all();
         e = fresh(out, want, device);
     }
-    if (e == cudaSuccess && !handed_out(*out, want)) {
+    if (e == cudaSuccess && !handed_out(*out, Piece{want, device, current})) {
         release(*out, device);
         *out = nullptr;
         e = cudaErrorMemoryAllocation;
@@ -175,28 +184,75 @@ void Memory::give(void *ptr, bool idle)
 {
     if (!ptr) return;
     std::lock_guard<std::mutex> lock(mu);
-    drop_idle();
     const auto it = live.find(ptr);
     if (it == live.end()) return;
-    const auto [bytes, device] = it->second;
+    const Piece piece = it->second;
     live.erase(it);
-    const size_t limit = device == kHost ? kKeptHost : kKept;
-    if (!idle || bytes > limit) {
-        release(ptr, device);
+    const size_t limit = piece.device == kHost ? kKeptHost : kKept;
+    if (!idle || piece.bytes > limit || !watch()) {
+        release(ptr, piece.device);
         return;
     }
     try {
-        kept.push_back(Block{ptr, bytes, device, std::chrono::steady_clock::now()});
+        kept.push_back(Block{piece, ptr, std::chrono::steady_clock::now()});
     } catch (const std::bad_alloc &) {
-        release(ptr, device);
+        release(ptr, piece.device);
         return;
     }
-    bytes_of(device) += bytes;
-    for (auto at = kept.begin(); bytes_of(device) > limit; ) {  // the oldest of its kind
+    bytes_of(piece.device) += piece.bytes;
+    for (auto at = kept.begin(); bytes_of(piece.device) > limit; ) {  // the oldest of its kind
         const auto next = std::next(at);
-        if ((at->device == kHost) == (device == kHost)) drop(at);
+        if ((at->device == kHost) == (piece.device == kHost)) {
+            const Block b = pop(at);
+            release(b.ptr, b.device);
+        }
         at = next;
     }
+}
+
+void Memory::release_all()
+{
+    int before = 0;
+    const bool back = cudaGetDevice(&before) == cudaSuccess;
+    while (!kept.empty()) {
+        const Block b = pop(kept.begin());
+        if (cudaSetDevice(b.current) == cudaSuccess) release(b.ptr, b.device);
+    }
+    if (back) cudaSetDevice(before);
+}
+
+// the thread for end_idle, if it is not there; false: there can be none
+bool Memory::watch()
+{
+    if (watched) return true;
+    try {
+        std::thread([this] { end_idle(); }).detach();
+        watched = true;
+    } catch (const std::exception &) {
+    }
+    return watched;
+}
+
+void Memory::end_idle()
+{
+    // (a free on this thread is none of a capture's business: nothing that is kept is used by any)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    std::unique_lock<std::mutex> lock(mu);
+    while (!kept.empty()) {
+        const auto due = kept.front().since + kIdle;
+        if (std::chrono::steady_clock::now() < due) {
+            lock.unlock();
+            std::this_thread::sleep_until(due);
+            lock.lock();
+            continue;
+        }
+        const Block b = pop(kept.begin());
+        lock.unlock();
+        if (cudaSetDevice(b.current) == cudaSuccess) release(b.ptr, b.device);  // (else the process ends)
+        lock.lock();
+    }
+    watched = false;
 }
 
 cudaError_t device_alloc(void **out, size_t bytes)
@@ -204,7 +260,17 @@ cudaError_t device_alloc(void **out, size_t bytes)
     *out = nullptr;
     int device = 0;
     const cudaError_t e = cudaGetDevice(&device);
-    return e == cudaSuccess ? memory().take(out, bytes, device) : e;
+    return e == cudaSuccess ? memory().take(out, bytes, device, device) : e;
+}
+
+void release_kept()
+{
+    {
+        std::lock_guard<std::mutex> lock(memory().mu);
+        memory().release_all();
+    }
+    std::lock_guard<std::mutex> lock(g_stream_mu);
+    while (g_n_streams) destroy(g_streams[--g_n_streams]);
 }
 
 void device_free(void *ptr, bool idle) { memory().give(ptr, idle); }
@@ -212,7 +278,9 @@ void device_free(void *ptr, bool idle) { memory().give(ptr, idle); }
 cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes)
 {
     void *ptr = nullptr;
-    const cudaError_t e = memory().take(&ptr, bytes, kHost);
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = memory().take(&ptr, bytes, kHost, device);
     try {
         if (e == cudaSuccess) {  // (where the shared pointer cannot be made, it gives the block back itself)
             *out = std::shared_ptr<char[]>((char *)ptr, [](char *at) { memory().give(at, true); });

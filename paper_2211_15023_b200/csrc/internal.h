@@ -23,6 +23,7 @@ void set_error(const char *fmt, ...);
 // have it; where that could not be established (a synchronisation failed) it goes back to the driver.
 cudaError_t device_alloc(void **out, size_t bytes);
 void device_free(void *ptr, bool idle);
+void release_kept();  // all that is kept for the next policy, side streams included
 // host memory in the same manner, pinned where the driver grants that; given up only when no copy of it is in flight
 cudaError_t pinned_alloc(std::shared_ptr<char[]> *out, size_t bytes);
 // can kernels on the current device use this host range at its own address?

@@ -6,13 +6,16 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
+#include <chrono>
 #include <map>
 #include <mutex>
 #include <new>
 #include <string>
+#include <thread>
 
 // the allocations that are still granted
-static long grants = 1L << 40;
+static std::atomic<long> grants{1L << 40};
 void *operator new(size_t bytes)
 {
     void *p = grants-- > 0 ? malloc(bytes ? bytes : 1) : nullptr;
@@ -49,21 +52,36 @@ CUresult pointer_attributes(unsigned n, CUpointer_attribute *what, void **to, CU
 }  // namespace fake
 
 namespace fake {
-int allocations = 0, frees = 0;  // of device memory
+std::atomic<int> allocations{0}, frees{0}, host_frees{0};  // frees: of device memory
 int streams = 0;                 // alive
 bool refuse_pinned = false;
+thread_local int device = 0;
+thread_local bool relaxed = false;
+std::atomic<int> freed_on{-1};
+std::atomic<bool> freed_relaxed{false};
 }  // namespace fake
 
 extern "C" {
-cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { return *d = fake::device, cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { return fake::device = d, cudaSuccess; }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *mode)
+{
+    fake::relaxed = *mode == cudaStreamCaptureModeRelaxed;
+    return cudaSuccess;
+}
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMalloc(void **out, size_t bytes) { return ++fake::allocations, *out = malloc(bytes), cudaSuccess; }
-cudaError_t cudaFree(void *p) { return ++fake::frees, free(p), cudaSuccess; }
+cudaError_t cudaFree(void *p)
+{
+    fake::freed_on = fake::device;
+    fake::freed_relaxed = fake::relaxed;
+    return ++fake::frees, free(p), cudaSuccess;
+}
 cudaError_t cudaHostAlloc(void **out, size_t bytes, unsigned)
 {
     return fake::refuse_pinned ? cudaErrorMemoryAllocation : (*out = malloc(bytes), cudaSuccess);
 }
-cudaError_t cudaFreeHost(void *p) { return free(p), cudaSuccess; }
+cudaError_t cudaFreeHost(void *p) { return ++fake::host_frees, free(p), cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)malloc(1), cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return free(e), cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return ++fake::streams, *s = (cudaStream_t)malloc(1), cudaSuccess; }
@@ -169,6 +187,70 @@ static int hungry()
     return 0;
 }
 
+static bool soon(const std::atomic<int> &count, int value)
+{
+    for (int i = 0; i < 100 && count != value; ++i) std::this_thread::sleep_for(std::chrono::milliseconds(20));
+    return count == value;
+}
+
+// what lies idle goes back without another call of the library, on its own device and outside any capture's
+// rules; twice, since the thread that does it ends in between
+static int idle()
+{
+    using std::chrono::milliseconds;
+    for (int round = 1; round <= 2; ++round) {
+        void *a = nullptr, *b = nullptr;
+        std::shared_ptr<char[]> h;
+        fake::device = 3;
+        CHECK(device_alloc(&a, 100000) == cudaSuccess && device_alloc(&b, 9 << 20) == cudaSuccess && pinned_alloc(&h, 1000) == cudaSuccess);
+        device_free(a, true);
+        h.reset();
+        fake::device = 0;
+        CHECK(fake::frees == 2 * (round - 1) && fake::host_frees == round - 1);
+        CHECK(soon(fake::frees, 2 * round - 1) && soon(fake::host_frees, round));
+        CHECK(fake::freed_on == 3 && fake::freed_relaxed && fake::device == 0);
+        std::this_thread::sleep_for(milliseconds(3 * ACCERL_KEEP_IDLE_MS));
+        CHECK(fake::frees == 2 * round - 1);  // (b is in use)
+        device_free(b, false);
+    }
+    return 0;
+}
+
+// used blocks do not age: what is given back again and again stays
+static int in_use()
+{
+    for (int i = 0; i < 30; ++i) {
+        void *a = nullptr;
+        CHECK(device_alloc(&a, 100000) == cudaSuccess);
+        std::this_thread::sleep_for(std::chrono::milliseconds(ACCERL_KEEP_IDLE_MS / 10));
+        device_free(a, true);
+    }
+    CHECK(fake::allocations == 1 && fake::frees == 0);
+    return 0;
+}
+
+// accerl_trim
+static int trim()
+{
+    void *a = nullptr, *b = nullptr, *c = nullptr;
+    std::shared_ptr<char[]> h;
+    SideStream s;
+    CHECK(device_alloc(&a, 100000) == cudaSuccess && device_alloc(&b, 9 << 20) == cudaSuccess && pinned_alloc(&h, 1000) == cudaSuccess);
+    CHECK(take_side_stream(&s) == cudaSuccess && device_alloc(&c, 5000) == cudaSuccess);
+    device_free(a, true);
+    device_free(b, true);
+    h.reset();
+    give_side_stream(s, true);
+    CHECK(fake::frees == 0 && fake::streams == 1);
+    release_kept();
+    CHECK(fake::frees == 2 && fake::host_frees == 1 && fake::streams == 0);
+    release_kept();
+    CHECK(fake::frees == 2);
+    device_free(c, true);
+    CHECK(device_alloc(&a, 5000) == cudaSuccess && a == c);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const std::string name = argc > 1 ? argv[1] : "";
@@ -176,6 +258,9 @@ int main(int argc, char **argv)
     if (name == "busy") return busy();
     if (name == "pageable") return pageable();
     if (name == "hungry") return hungry();
+    if (name == "idle") return idle();
+    if (name == "in_use") return in_use();
+    if (name == "trim") return trim();
     printf("no check %s\n", name.c_str());
     return 2;
 }

@@ -12,13 +12,13 @@ ROOT = os.path.dirname(HERE)
 @pytest.fixture(scope="module")
 def program(tmp_path_factory):
     out = str(tmp_path_factory.mktemp("device_memory") / "checks")
-    subprocess.check_call(["g++", "-std=c++17", "-O1", "-pthread", "-x", "c++", os.path.join(HERE, "device_memory_checks.cpp"), "-o", out,
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-pthread", "-DACCERL_KEEP_IDLE_MS=250", "-x", "c++", os.path.join(HERE, "device_memory_checks.cpp"), "-o", out,
                            "-I/usr/local/cuda/include", "-I" + os.path.join(ROOT, "include"),
                            "-I" + os.path.join(ROOT, "paper_2211_15023_b200", "csrc")])
     return out
 
 
-@pytest.mark.parametrize("check", ["reach", "busy", "pageable", "hungry"])
+@pytest.mark.parametrize("check", ["reach", "busy", "pageable", "hungry", "idle", "in_use", "trim"])
 def test_device_memory(program, check):
     r = subprocess.run([program, check], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr

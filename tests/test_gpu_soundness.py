@@ -221,3 +221,30 @@ def test_mlp_layer_whose_scale_has_no_finite_reciprocal():
     g.check()
     compare(ref, logits.cpu().numpy(), actions.cpu().numpy(), logp.cpu().numpy())
     g.close()
+
+
+def test_trim_gives_back_what_is_kept_for_the_next_policy():
+    """The memory of a destroyed policy stays with the library, serves the next one, and is the device's again
+    after trim; a policy that is alive goes on stepping."""
+    import paper_2211_15023_b200 as P
+    import workloads as W
+    name = "student_cnn_b8192"
+    pol = W.drawn_int8_policy(name)
+    obs, u = torch.from_numpy(W.observations(name, 8)).cuda(), torch.from_numpy(W.uniforms(name, 8)).cuda()
+    alive = P.Policy(pol, 8)
+    want = alive.act(obs, u)
+    P.trim()
+    free = lambda: torch.cuda.mem_get_info()[0]  # noqa: E731
+    before = free()
+    P.Policy(pol, 4096).close()
+    kept = before - free()
+    assert kept > 30 << 20
+    P.Policy(pol, 4096).close()
+    assert before - free() == kept
+    P.trim()
+    assert free() >= before
+    P.trim()
+    for x, y in zip(alive.act(obs, u), want):
+        assert torch.equal(x, y)
+    alive.check()
+    alive.close()
