@@ -451,8 +451,8 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
         // The two networks share nothing but the lists: side by side on two streams their small launches
         // fill each other's gaps (one after the other: 88 us for the case above).
         if (!smaller->mix.stream) ACCERL_CUDA_TRY(take_side_stream(&smaller->mix));
-        ACCERL_CUDA_TRY(cudaEventRecord(smaller->mix.events[0], st));
-        ACCERL_CUDA_TRY(cudaStreamWaitEvent(smaller->mix.stream, smaller->mix.events[0], 0));
+        SideWork side(st, smaller->mix);
+        ACCERL_CUDA_TRY(side.begin());
         accerl_status result = ACCERL_OK;
         for (int i = 1; i >= 0; --i) {
             Route r;
@@ -464,9 +464,8 @@ extern "C" accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_
             if (result == ACCERL_OK) result = s;
         }
         smaller->last_stream = st;  // (which waits for the other)
-        ACCERL_CUDA_TRY(cudaEventRecord(smaller->mix.events[1], smaller->mix.stream));
-        ACCERL_CUDA_TRY(cudaStreamWaitEvent(st, smaller->mix.events[1], 0));
         if (result != ACCERL_OK) return result;
+        ACCERL_CUDA_TRY(side.join());
         return ACCERL_OK;
     }
     // the original policy writes the caller's buffers, the smaller one the handle's own

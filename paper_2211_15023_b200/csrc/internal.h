@@ -38,6 +38,37 @@ struct SideStream {
 cudaError_t take_side_stream(SideStream *out);
 void give_side_stream(SideStream &s, bool idle);
 
+// Work on a side stream beside the caller's.  However the scope ends, the caller's stream is ordered behind what
+// was launched there: by an event, or, where that fails, by waiting for it.
+class SideWork {
+public:
+    SideWork(cudaStream_t caller, const SideStream &side) : caller_(caller), side_(side) {}
+    cudaError_t begin()
+    {
+        cudaError_t e = cudaEventRecord(side_.events[0], caller_);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(side_.stream, side_.events[0], 0);
+        open_ = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t join()
+    {
+        cudaError_t e = cudaEventRecord(side_.events[1], side_.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(caller_, side_.events[1], 0);
+        if (e != cudaSuccess) cudaStreamSynchronize(side_.stream);
+        open_ = false;
+        return e;
+    }
+    ~SideWork()
+    {
+        if (open_) join();
+    }
+
+private:
+    cudaStream_t caller_;
+    const SideStream &side_;
+    bool open_ = false;
+};
+
 // let a kernel use `bytes` of dynamic shared memory on the current device (api.cu)
 cudaError_t allow_smem(const void *kernel, size_t bytes);
 

@@ -1,4 +1,4 @@
-// csrc/device_memory.cu on the host, against a fake of the CUDA calls it makes.  One check per run, named on
+// csrc/device_memory.cu and the side streams of csrc/internal.h on the host, against a fake of the CUDA calls they make.  One check per run, named on
 // the command line; exits 0 when it holds, else says what does not.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -52,6 +52,13 @@ CUresult pointer_attributes(unsigned n, CUpointer_attribute *what, void **to, CU
 }  // namespace fake
 
 namespace fake {
+std::string steps;  // calls that order streams
+int failing = -1;   // which of them fails
+cudaError_t step(const char *name)
+{
+    steps += std::string(steps.empty() ? "" : " ") + name;
+    return failing-- == 0 ? cudaErrorUnknown : cudaSuccess;
+}
 std::atomic<int> allocations{0}, frees{0}, host_frees{0};  // frees: of device memory
 int streams = 0;                 // alive
 bool refuse_pinned = false;
@@ -86,6 +93,9 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cu
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return free(e), cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return ++fake::streams, *s = (cudaStream_t)malloc(1), cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { return --fake::streams, free(s), cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return fake::step("record"); }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return fake::step("wait"); }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return fake::step("synchronize"); }
 cudaError_t cudaGetDriverEntryPoint(const char *name, void **out, unsigned long long, cudaDriverEntryPointQueryResult *found)
 {
     const bool known = !strcmp(name, "cuPointerGetAttributes");
@@ -251,6 +261,28 @@ static int trim()
     return 0;
 }
 
+// a side stream that work was launched on is always waited for, whichever call fails
+static int side()
+{
+    SideStream s;
+    CHECK(take_side_stream(&s) == cudaSuccess);
+    const char *want[5] = {"record", "record wait", "record wait record synchronize", "record wait record wait synchronize",
+                           "record wait record wait"};
+    for (int returns_early = 0; returns_early < 2; ++returns_early)
+        for (int i = 0; i < 5; ++i) {
+            fake::steps.clear();
+            fake::failing = i;
+            {
+                SideWork work(nullptr, s);
+                const cudaError_t e = work.begin();
+                CHECK((e == cudaSuccess) == (i >= 2));
+                if (e == cudaSuccess && !returns_early) CHECK((work.join() == cudaSuccess) == (i >= 4));
+            }
+            CHECK(fake::steps == want[i]);
+        }
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const std::string name = argc > 1 ? argv[1] : "";
@@ -261,6 +293,7 @@ int main(int argc, char **argv)
     if (name == "idle") return idle();
     if (name == "in_use") return in_use();
     if (name == "trim") return trim();
+    if (name == "side") return side();
     printf("no check %s\n", name.c_str());
     return 2;
 }

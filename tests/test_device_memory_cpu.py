@@ -1,5 +1,5 @@
-"""The memory the library keeps and what it takes host memory for (csrc/device_memory.cu), compiled for
-the host against a fake of the CUDA calls: failing calls and odd address ranges without a device."""
+"""The memory the library keeps, what it takes host memory for and its side streams (csrc/device_memory.cu,
+csrc/internal.h), compiled for the host against a fake of the CUDA calls: failing calls and odd address ranges without a device."""
 import os
 import subprocess
 
@@ -18,7 +18,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("check", ["reach", "busy", "pageable", "hungry", "idle", "in_use", "trim"])
+@pytest.mark.parametrize("check", ["reach", "busy", "pageable", "hungry", "idle", "in_use", "trim", "side"])
 def test_device_memory(program, check):
     r = subprocess.run([program, check], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
