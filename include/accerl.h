@@ -174,9 +174,9 @@ typedef struct {
  *   calib_obs_host  host, calib_rows observations in the layout `act` takes (uint8 [rows, C, H, W]
  *                   or fp32 [rows, D])
  *   the other arguments are those of accerl_policy_create; ACCERL_FLAG_VALUE_HEAD as there
- * Create-time work with plain kernels (tens of milliseconds for a thousand frames); transient
- * device memory: the calibration batch's int8 activations plus one int32 tensor of the largest
- * layer output.  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA; *out is NULL then.
+ * Create-time work on CUDA-core kernels (3.4 ms for the IMPALA network and 256 frames).  Device memory for
+ * the time of the call: weights, the calibration batch, its int8 activations and one int32 tensor of the
+ * largest layer output; kept for the next policy like that of a destroyed one (accerl_policy_destroy).  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA; *out is NULL then.
  */
 accerl_status accerl_policy_create_fp32(accerl_policy **out, int32_t in_kind, const int32_t in_shape[3],
                                         const accerl_layer_fp32 *layers, int32_t n_layers,
@@ -258,10 +258,13 @@ accerl_status accerl_policy_kl(const float *logits_original_dev, const float *lo
  *   alpha                in [0, 1]
  *   use_smaller_dev      device, uint8 [batch], written: 1 where `smaller` was used; NULL to skip
  *   value_dev            needs ACCERL_FLAG_VALUE_HEAD on both handles; NULL to skip
- * Both networks run on the whole batch and a last kernel selects per state, so the cost is the sum
- * of the two steps; results do not depend on which other states share the batch.  The first call
- * allocates, in `smaller`, result buffers for max_batch states (freed with the handle).  Uses both
- * handles' workspaces: no other call on either may overlap with it on the GPU.
+ * For the image-resident plans (the Atari and IMPALA networks of accerl_policy_info's plans) the states are
+ * listed per network on the device and every state runs through its own network only, the smaller network's
+ * launches on a stream of the library's own that `cuda_stream` waits for.  With other plans both networks
+ * run on the whole batch and a last kernel selects per state.  Results do not depend on which other states
+ * share the batch.  The first call allocates, in `smaller`, the lists or result buffers for max_batch states
+ * (freed with the handle).  Uses both handles' workspaces: no other call on either may overlap with it on
+ * the GPU.
  * Errors: INVALID_ARG, BATCH_TOO_LARGE, OOM, CUDA.
  */
 accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_policy *original,
@@ -285,8 +288,8 @@ accerl_status accerl_policy_act_mixed(accerl_policy *smaller, accerl_policy *ori
  *   all arrays      device, fp32, time-major [n_steps, batch]; bootstrap_dev [batch]
  *   discounts_dev   NULL, or [n_steps, batch]
  *   vs_dev          written; adv_dev written, NULL to skip
- * One thread per rollout runs the backward recursion the sums telescope into, in double, and
- * rounds the results to float.  Enqueues on `cuda_stream`, returns without synchronising,
+ * The backward recursion the sums telescope into runs in double, and the results are rounded to
+ * float once; they do not depend on how many rollouts share the call.  Enqueues on `cuda_stream`, returns without synchronising,
  * allocates nothing.  Errors: INVALID_ARG, CUDA.
  */
 accerl_status accerl_vtrace(const float *logp_smaller_dev, const float *logp_original_dev,
@@ -331,7 +334,8 @@ accerl_status accerl_policy_act_timed(accerl_policy *p, const void *obs_dev,
  * no cudaMalloc / cudaFree or any other allocating routine.
  *
  * First call on a device: the library asks the CUDA runtime for the array's address on that
- * device (once per device, remembered afterwards).  Make this first call during start-up, before
+ * device (once per device, remembered afterwards).  First call on a handle: a copy of its plan that works
+ * in the array is made, in host memory (where there is none for it, the CUDA-core kernels step).  Make this first call during start-up, before
  * any stream capture is begun.  The CUDA runtime loads a library's device code lazily, so the
  * array's memory may only be reserved when this first call (or any earlier kernel of the library
  * on that device, accerl_policy_create included) triggers the load; on a device without 64 MiB to

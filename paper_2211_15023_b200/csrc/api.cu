@@ -167,7 +167,6 @@ accerl_status validate_layer(const accerl_layer_desc &d, int i, int n_layers, Sh
     return ACCERL_OK;
 }
 
-// Repack OIHW int8 weights into the word layouts of the generic kernels.
 // dst[i * pitch + c] = src[c * n + i] for c < rows, i < n; in 8 x 8 pieces (halves, quarters, eighths of the
 // words trade places): a byte at a time the 3136 x 512 weights of the Nature-CNN took 0.7 ms, so 0.2
 void transpose_bytes(const int8_t *src, int rows, int n, int8_t *dst, int pitch)
@@ -201,7 +200,7 @@ size_t generic_bytes(const accerl_layer_desc &d, const LayerPlan &L)
     return d.kind == ACCERL_CONV2D ? (size_t)d.kh * d.kw * L.in_cp * L.oc_pad : (size_t)L.oc_pad * L.in_h * L.in_w * L.in_cp;
 }
 
-// `bytes` are zero before
+// Repack OIHW int8 weights into the word layouts of the generic kernels; `bytes` are zero before
 void pack_generic(const accerl_layer_desc &d, const LayerPlan &L, int8_t *bytes)
 {
     const int C4 = L.in_cp / 4;
@@ -251,9 +250,6 @@ cudaError_t allow_smem(const void *kernel, size_t bytes)
     return e;
 }
 
-// Parameters go to the device in a few large blocks, collected on the host and copied when the plan is
-// complete: an allocation and a blocking copy for each of some fifty small arrays took longer than
-// everything else accerl_policy_create does.
 void set_routed_steps(accerl_policy *p, const std::vector<Step> &front)
 {
     if (p->flags & ACCERL_FLAG_KEEP_ACTIVATIONS) return;
@@ -267,6 +263,9 @@ void set_routed_steps(accerl_policy *p, const std::vector<Step> &front)
     p->routed_steps = r;
 }
 
+// Parameters go to the device in a few large blocks, collected on the host and copied when the plan is
+// complete: an allocation and a blocking copy for each of some fifty small arrays took longer than
+// everything else accerl_policy_create does.
 accerl_status upload_room(accerl_policy *p, size_t bytes, void **host, void **dev)
 {
     *dev = nullptr;

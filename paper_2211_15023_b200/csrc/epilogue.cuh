@@ -90,9 +90,10 @@ __device__ __forceinline__ uint32_t relu_bytes(uint32_t w)
 
 // One requantised code by the three-step division: t = y * r, e = y - s * t (exact in one fma),
 // d = t + e * r.  With r = fl(1 / s) this is the classical correctly rounded quotient except for
-// rare operand patterns, so it is only used for scales for which fastdiv_code() has been compared
-// with exact_code() over every fp32 value y can take (see verify_fastdiv in tc_plan.cu).  ReLU
-// is applied to the code, which has the sign of y; the saturating pack does the clamp.
+// rare operand patterns, so it is only used for scales for which it has been compared with the IEEE
+// divide (verify_fastdiv_kernel in requant_fit.cu): every positive y from 0.4 s to 130 s.  The others need
+// no comparison: every operation of both is odd in y, below both quotients round to 0, above both
+// saturate.  ReLU is applied to the code, which has the sign of y; the saturating pack does the clamp.
 __device__ __forceinline__ int fastdiv_rint(float y, float s, float r)
 {
     const float t = __fmul_rn(y, r);
@@ -107,16 +108,9 @@ __device__ __forceinline__ int exact_code(float y, float s, bool relu)
     return (int)requant(y, s);
 }
 
-template <bool RELU>
-__device__ __forceinline__ int fastdiv_code(float y, float s, float r)
-{
-    const int q = min(max(fastdiv_rint(y, s, r), -128), 127);  // what the saturating pack does
-    return RELU ? max(q, 0) : q;                               // and relu_bytes()
-}
-
 // Sixteen codes by the three-step division, two elements per instruction: the packed fp32
 // operations of sm_100 round each half exactly as their scalar forms do, so the codes are those
-// of fastdiv_code(); they only take half the issue slots.
+// of fastdiv_rint(), clamped by the pack; they only take half the issue slots.
 template <bool RELU>
 __device__ __forceinline__ void requant16_fastdiv(const int (&acc)[16], const float (&ks)[16],
                                                   const float (&bs)[16], float s_out,
@@ -145,7 +139,7 @@ __device__ __forceinline__ void requant16_fastdiv(const int (&acc)[16], const fl
 // requantiser is a non-decreasing step function of the INTEGER accumulator, and so is this one
 // (k2 > 0); for every output channel the pair (k2, b2) near (k / s_out, b / s_out) is searched at
 // create until the two functions agree on every accumulator between the two points where both
-// saturate, which makes them equal on all of int32 (fit_affine_requant in requant_fit.cu).
+// saturate, which makes them equal on all of int32 (fit_affine_kernel in requant_fit.cu).
 template <bool RELU>
 __device__ __forceinline__ int affine_code(int acc, float k2, float b2)
 {

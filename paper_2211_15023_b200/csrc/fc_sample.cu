@@ -315,18 +315,22 @@ accerl_status build_fc_sample(accerl_policy *p, const accerl_layer_desc &d, int 
     return ACCERL_OK;
 }
 
+// Clusters of eight that find their SMs at once: 15 on 148 SMs; one less, should another chip's SMs lie less well
+static int head_clusters(int sm_count) { return sm_count / 10; }
+
 // Do the hidden layer `i` and the last one behind it run as that launch?  Handles for more states end in
 // tiles of 128 (fc_tile.cu), which read the weights less often, or in two launches.  The line lies where this
-// launch's clusters no longer fit the chip at once, with 16 states each for 512 outputs, 32 for 256 (us per
-// step, this launch / tiles: 512 outputs of 3136 inputs 15.4 / 19.3 at 160 states, 22.1 / 20.3 at 256; 256 of 1568
-// 11.0 / 13.6, 15.9 / 17.4 at 448, 22.3 / 18.7 at 640).
+// launch's clusters no longer fit the chip at once, with 16 states each for 512 outputs, 32 for 256: 224 and 448
+// states on 148 SMs (us per step, this launch / tiles: 512 outputs of 3136 inputs 15.4 / 19.3 at 160 states, 22.1 /
+// 20.3 at 256; 256 of 1568 11.0 / 13.6, 15.9 / 17.4 at 448, 22.3 / 18.7 at 640).  A handle made for one state, as
+// accerl_policy_act_noalloc asks for, has this launch at every batch of its fixed workspace.
 bool fc_head_fits(const accerl_policy *p, const accerl_layer_desc *layers, int n_layers, int i)
 {
-    if (i != n_layers - 2 || i < 1 || unfuse_for_taps(p) || p->max_batch > (layers[i].out_c == 512 ? kFcHeadMaxWide : kFcHeadMaxNarrow) || !fc_sample_fits(p, layers, n_layers, i + 1))
-        return false;
+    if (i != n_layers - 2 || i < 1 || unfuse_for_taps(p) || !fc_sample_fits(p, layers, n_layers, i + 1)) return false;
     const accerl_layer_desc &d = layers[i];
     const LayerPlan &L = p->layers[i];
-    return d.kind == ACCERL_FC && (d.out_c == 256 || d.out_c == 512) && L.in_cp == L.in_c && (L.in_h * L.in_w * L.in_cp) % 16 == 0;
+    return d.kind == ACCERL_FC && (d.out_c == 256 || d.out_c == 512) && p->max_batch <= head_clusters(p->sm_count) * (d.out_c == 512 ? 16 : 32) &&
+           L.in_cp == L.in_c && (L.in_h * L.in_w * L.in_cp) % 16 == 0;
 }
 
 // x: the hidden layer's input rows; its weights in (y, x, c) order are L.host_rows
@@ -386,9 +390,9 @@ cudaError_t launch_fc_head(const FcHeadParams &h, const FcSampleParams &q, const
         cfg.numAttrs = 2;
         return cudaLaunchKernelEx(&cfg, kernel, h, q, u, B, route, logits, actions, logp, value, entropy);
     };
-    // 16 states per cluster while their clusters fit the chip once: 15 clusters of eight find their SMs (one less
-    // here, see launch_fc_tile); with 16, at 256 states, a step of the narrow network took 15.4 us, with half as many 12.9
-    const bool two = ((route.count ? route.expect : B) + 15) / 16 > sm_count / 10;
+    // 16 states per cluster while their clusters fit the chip at once: with 16 clusters, at 256 states, a step of the
+    // narrow network took 15.4 us, with half as many 12.9
+    const bool two = ((route.count ? route.expect : B) + 15) / 16 > head_clusters(sm_count);
     if (h.N == 512) return two ? go(fc_hidden_fc_sample_kernel<2, 8>, 32) : go(fc_hidden_fc_sample_kernel<1, 8>, 16);
     return two ? go(fc_hidden_fc_sample_kernel<2, 4>, 32) : go(fc_hidden_fc_sample_kernel<1, 4>, 16);
 }

@@ -329,8 +329,9 @@ cudaError_t launch_fc_tile(const void *map_x, const FcTileParams &h, const FcSam
         memcpy(&map, map_x, sizeof(map));
         return cudaLaunchKernelEx(&cfg, kernel, map, h, q, u, B, route, logits, actions, logp, value, entropy);
     };
-    // As many CTAs per tile of states as the chip holds at once: 15 clusters of eight (16 in two waves cost 4 us of
-    // 60 at 2048 states), 33 of four, 74 of two; one less than that, should another chip's SMs lie less well.
+    // As many CTAs per tile of states as the chip holds at once: 148 SMs take 15 clusters of eight (16 in two waves cost
+    // 4 us of 60 at 2048 states), 33 of four, 74 of two.  One less of the larger ones, should another chip's SMs lie
+    // less well; pairs lie wherever two SMs do.
     const int tiles = ((route.count ? route.expect : B) + 127) / 128;
     const int c = tiles <= sm_count / 10 ? 8 : tiles <= sm_count * 2 / 9 ? 4 : tiles <= sm_count / 2 || h.N == 512 ? 2 : 1;
     if (h.N == 512) return c == 8 ? go(OpIndex<64>(), OpIndex<8>()) : c == 4 ? go(OpIndex<128>(), OpIndex<4>()) : go(OpIndex<256>(), OpIndex<2>());

@@ -3,10 +3,10 @@
 // kl_rows_kernel / kl_wide_kernel: KL(pi_original || pi_smaller) per state from two logit matrices
 // (Eq. KL), a thread or a warp per state; kl_stats_kernel reduces the per-state values to their mean and
 // maximum (the "KL mean" and "KL max" indicators) in one CTA or one cluster of CTAs, in a fixed order, so
-// that the result does not depend on scheduling.  mix_select_kernel overwrites the original
-// policy's outputs with the smaller policy's for the states whose selector draw falls below alpha
-// (the linear-alpha strategy of Section 3.2: the Actor follows the small network with
-// probability alpha).
+// that the result does not depend on scheduling.  route_kernel lists the states of each network for
+// the linear-alpha strategy of Section 3.2 (the Actor follows the small network where the selector draw falls
+// below alpha), so that each runs on its own states only; where a plan cannot do that, both run on all of them and
+// mix_select_kernel overwrites the original policy's outputs with the smaller policy's.
 #include <cooperative_groups.h>
 #include <math.h>
 

@@ -161,7 +161,6 @@ struct FcHeadParams {
     float s_out;
     int8_t *tap;      // parity tap of its output, or null
 };
-constexpr int kFcHeadMaxWide = 224, kFcHeadMaxNarrow = 448;  // states, for 512 and 256 outputs
 
 // the same for more states (fc_tile.cu)
 struct FcTileParams {

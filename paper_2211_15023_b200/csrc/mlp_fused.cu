@@ -346,8 +346,8 @@ cudaError_t launch_mlp_fused(const accerl_policy *p, const float *obs, const flo
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, prm, obs, u, B, logits, actions, logp, value, entropy);
     };
-    // 32 states per CTA once 16 would give every SM more than one CTA: the weights are then read half
-    // as often
+    // 32 states per CTA once 16 would give every SM more than the two CTAs it holds at once: the weights are
+    // then read half as often
     return B > 32 * p->sm_count ? go(mlp_fused_kernel<2>, 32) : go(mlp_fused_kernel<1>, 16);
 }
 
