@@ -22,11 +22,16 @@
 // nine K steps).  N = 32 instructions cost 40 cycles, bound by reading their 4 KB operand: wider rows
 // (N = 64, four pixels) would save a tenth of the tensor time and quadruple the weights' shared memory.
 //
-// What bounds it: instruction issue of the epilogues (about half of the 37 000 warp instructions an image
-// takes in res_stack1 convert and pack its 164 000 codes), then the tensor pipe by instruction count
-// (10 080 cycles an image in res_stack1, 8 640 in res_stack23, of 14 700 and 13 800).  Batch 16384, us per
-// launch: two contexts with constants from the constant bank 608 / 1079 / 1103, as it is
-// 483 / 827 / 775.
+// A layer's operand is handed over tile by tile: a tile of the next layer is contracted as soon as the
+// operand rows its taps reach are there (its own tile and the neighbours), so no layer ends in a wait for all
+// of its warps; the issuing warp also lets the next image land as soon as its last MMA has read this one.
+//
+// What bounds it: the tensor pipe by instruction count (10 080 cycles an image in res_stack1, 8 640 in
+// res_stack23, of 14 300 and 11 900; an MMA of N = 32 reads its operands at the full rate of shared memory)
+// and instruction issue of the epilogues (about half of the 37 000 warp instructions an image takes in
+// res_stack1 convert and pack its 164 000 codes).  Batch 16384, us per launch: whole layers handed over, both
+// requantisers in the code 489 / 841 / 769, as it is 478 / 810 / 674; 100 images, one context with two or four
+// warpgroups: step 53.6 / 47.7.  A third warpgroup in res_first: 513 (spills).
 //
 // Every wait is bounded.  A role whose wait gives up sets the status word and goes on (all further
 // waits return at once), so that the barriers inside a context always see all their warps.
@@ -46,13 +51,14 @@ namespace accerl {
 namespace {
 
 constexpr int kMaxCtx = 3;  // images in flight per CTA
-constexpr int kMaxSlots = 5;
+constexpr int kMaxSlots = 7;
+constexpr int kMaxTiles = 7;  // 128-row tiles of a layer whose operand is waited for tile by tile
 
 
 struct __align__(8) ResBars {
     uint64_t w_ready;
     uint64_t land[kMaxCtx];                // an image has arrived
-    uint64_t ready[kMaxCtx];               // the operand of the next layer is complete
+    uint64_t ready[kMaxCtx][kMaxTiles];    // a tile of the next layer's operand (or all of it) is complete
     uint64_t acc_full[kMaxCtx][kMaxSlots], acc_empty[kMaxCtx][kMaxSlots];
     uint32_t tmem_base;
     int abort_flag;
@@ -110,6 +116,7 @@ struct ByteMax {
 // wavefronts of the port the MMAs read their operands through (res_stack1: 12 000 of 20 000 cycles an
 // image); and held in registers over a layer they push the kernels into spills, which are deadly
 // beside 220 KB of shared memory, with hardly any L1 left (2.4 ms instead of 1.1).
+template <bool AFFINE, bool RELU>
 __device__ __forceinline__ uint4 requant_res(const int (&acc)[16], const ResLayer &L, int c0)
 {
     float ks[16], bs[16];
@@ -121,10 +128,9 @@ __device__ __forceinline__ uint4 requant_res(const int (&acc)[16], const ResLaye
         bs[4 * g] = bv.x; bs[4 * g + 1] = bv.y; bs[4 * g + 2] = bv.z; bs[4 * g + 3] = bv.w;
     }
     uint32_t w[4];
-    if (L.affine) requant16_affine<false>(acc, ks, bs, w);
-    else requant16_fastdiv<false>(acc, ks, bs, L.s_out, L.inv_s_out, w);
-    const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-    return L.relu ? relu16(v) : v;
+    if (AFFINE || L.affine) requant16_affine<RELU>(acc, ks, bs, w);
+    else requant16_fastdiv<RELU>(acc, ks, bs, L.s_out, L.inv_s_out, w);
+    return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // acc[i] += skip_mul[c0 + i] * x[i], one dp2a each
@@ -141,6 +147,13 @@ __device__ __forceinline__ void add_skip(int (&acc)[16], uint4 x, const ResLayer
     }
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, int *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
 __device__ __forceinline__ uint4 tmem_ld4(uint32_t taddr)
 {
     uint4 v;
@@ -159,7 +172,8 @@ constexpr uint32_t kDescFlatLo = (16u >> 4) << 16;                        // the
 // what every kernel of this file does first: barriers, tensor memory, weights; returns the tensor-memory base
 template <int EPI_WARPS>
 __device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, int buffer_bytes, uint8_t *w_smem,
-                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals, int wide_slot)
+                                              const uint8_t *w, uint32_t w_bytes, int warp, int epi_arrivals, int wide_slot,
+                                              int tile_arrivals, int wide_ready)
 {
     // borders and padding stay zero for the life of the CTA
     for (int i = threadIdx.x; i < buffer_bytes / 16; i += blockDim.x)
@@ -168,7 +182,7 @@ __device__ __forceinline__ uint32_t res_setup(ResBars &bars, uint8_t *buffers, i
         mbar_init(smem_u32(&bars.w_ready), 1);
         for (int c = 0; c < kMaxCtx; ++c) {
             mbar_init(smem_u32(&bars.land[c]), 1);
-            mbar_init(smem_u32(&bars.ready[c]), epi_arrivals);
+            for (int t = 0; t < kMaxTiles; ++t) mbar_init(smem_u32(&bars.ready[c][t]), t == wide_ready ? epi_arrivals : tile_arrivals);
             for (int s = 0; s < kMaxSlots; ++s) {
                 mbar_init(smem_u32(&bars.acc_full[c][s]), 1);
                 mbar_init(smem_u32(&bars.acc_empty[c][s]), s == wide_slot ? epi_arrivals : 4);
@@ -228,7 +242,7 @@ constexpr int kFirstSmem = 1024 + 8192 + kFirstCtx * (kFrameBytes + kHpBytes);
 static_assert((kFirstTiles * 128 + 45) * 16 <= kFrameBytes && 83 * 21 * 32 <= kHpBytes, "buffers");
 }  // namespace
 
-template <bool SHIFT, bool TAP>
+template <bool SHIFT, bool TAP, bool AFFINE>
 __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_kernel(const __grid_constant__ ResFirstParams p)
 {
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
@@ -237,14 +251,14 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + 8192;
     const uint32_t tmem = res_setup<kFirstEpi>(bars, bufs, kFirstCtx * (kFrameBytes + kHpBytes), smem, p.w, kResFirstWeights,
-                                               warp, kFirstWg * 4, -1);
+                                               warp, kFirstWg * 4, -1, kFirstWg * 4, -1);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kFirstCtx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kFirstEpi) {
         // ------------------------------------------------------------------ MMA issuers
         const int ctx = warp - kFirstEpi;
-        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t a0 = ((smem_u32(bufs) + (uint32_t)ctx * (kFrameBytes + kHpBytes)) >> 4) | kDescFlatLo;
         const uint32_t b0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
         const int ctx = warp / (kFirstWg * 4), wg = (warp >> 2) % kFirstWg, q = warp & 3;
         const int tid = (int)threadIdx.x - ctx * kFirstT;
         const uint32_t frame = smem_u32(bufs) + (uint32_t)ctx * (kFrameBytes + kHpBytes), hp = frame + kFrameBytes;
-        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * 256;
         auto convert = [&](int n) {
@@ -323,20 +337,23 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
                 const bool valid = X < 21 && y < 83;
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    int a[16], b[16], c[16];
+                    int a[16], b[16];  // eight columns of the three pixels at a time
                     const uint32_t ta = tlane + slot * 80 + (uint32_t)(32 * j);
-                    tmem_ld16(ta, a);
-                    tmem_ld16(ta + 16, b);
-                    tmem_ld16(ta + 32, c);
-                    tmem_wait_ld();
+#pragma unroll
+                    for (int h = 0; h < 16; h += 8) {
+                        tmem_ld8(ta + h, a + h);
+                        tmem_ld8(ta + h + 16, b);
+                        tmem_ld8(ta + h + 32, b + 8);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) a[h + i] = __vimax3_s32(a[h + i], b[i], b[8 + i]);
+                    }
                     if (j == 1) {
                         fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(empty0 + 8 * slot);
                     }
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) a[i] = __vimax3_s32(a[i], b[i], c[i]);
-                    const uint4 v = requant_res(a, p.layer, 0);
+                    const uint4 v = requant_res<AFFINE, false>(a, p.layer, 0);
                     if (valid) sts16(hp + row_off(R, j), v);
                 }
             }
@@ -371,45 +388,70 @@ __global__ void __launch_bounds__(32 * (kFirstEpi + kFirstCtx), 1) res_first_ker
 // memory: the thread that adds it is the thread that wrote it.  The 16 -> 32 conv runs as two halves of
 // sixteen output channels, so that the un-pooled half fits the buffer between the convs.
 namespace {
-constexpr int kS1Ctx = 3, kS1Wg = 2;                        // images in flight, warpgroups of each
-constexpr int kS1T = kS1Wg * 128, kS1Epi = kS1Ctx * kS1Wg * 4;
-constexpr int kS1Tiles = 7, kS1Slots = 3, kS1Ops = 6;       // 41 * 21 GEMM rows; accumulators; layers and half layers
+constexpr int kS1Tiles = 7, kS1Ops = 6;                     // 41 * 21 GEMM rows; layers and half layers
 constexpr int kS1Buf = 30 * 1024;                           // an image's rows and what the last tile reads past them
-constexpr int kS1XCol = kS1Slots * 32, kS1Cols = 168;       // tensor memory of a context: accumulators, then 8 columns of x per tile
-constexpr int kS1Smem = 1024 + kRes1Weights + kS1Ctx * 2 * kS1Buf;
-static_assert((kS1Tiles * 128 + 2 * 21 + 1) * 32 <= kS1Buf && kS1XCol + 8 * kS1Tiles <= kS1Cols && kS1Ctx * kS1Cols <= 512, "buffers");
+// CTX images in flight, WG warpgroups of each
+template <int CTX, int WG>
+struct S1Shape {
+    static constexpr int T = WG * 128, Epi = CTX * WG * 4, Threads = 32 * (Epi + CTX);
+    static constexpr int Slots = CTX == 1 ? kS1Tiles : 3;       // accumulators of a context
+    static constexpr int XCol = Slots * 32, Cols = XCol + 8 * kS1Tiles;  // tensor memory: accumulators, then 8 columns of x per tile
+    static constexpr int Smem = 1024 + kRes1Weights + CTX * 2 * kS1Buf;
+    // Two warpgroups take the tiles of all layers in turn, so the odd seventh falls to one and the other
+    // alternately; x's tiles (written in layers 1, read in 1 and 3) stay with one of them.  A warpgroup that
+    // waits for an accumulator has seen one of the last `Slots` uses complete, so the wait's parity is
+    // unambiguous; more warpgroups have an accumulator per tile and always the same tiles.
+    __host__ __device__ static constexpr int shift(int op) { return WG == 2 && Slots < kS1Tiles ? op & 1 : 0; }
+    static_assert((WG <= 2 || Slots == kS1Tiles) && Slots <= kMaxSlots && Cols * CTX <= 512, "tiles of a warpgroup");
+};
+static_assert((kS1Tiles * 128 + 2 * 21 + 1) * 32 <= kS1Buf && kS1Tiles <= kMaxTiles, "buffers");
 }  // namespace
 
-template <bool TAP>
-__global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(const __grid_constant__ ResStack1Params p)
+template <bool TAP, bool AFFINE, int CTX, int WG>
+__global__ void __launch_bounds__(S1Shape<CTX, WG>::Threads, 1) res_stack1_kernel(const __grid_constant__ ResStack1Params p)
 {
+    using S = S1Shape<CTX, WG>;
+    constexpr int kS1Ctx = CTX, kS1Wg = WG, kS1T = S::T, kS1Epi = S::Epi, kS1Slots = S::Slots, kS1XCol = S::XCol, kS1Cols = S::Cols;
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes1Weights;
-    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kS1Ctx * 2 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, -1);
+    const uint32_t tmem = res_setup<kS1Epi>(bars, bufs, kS1Ctx * 2 * kS1Buf, smem, p.w, kRes1Weights, warp, kS1Wg * 4, -1, 4, -1);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kS1Ctx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kS1Epi) {
         // ------------------------------------------------------------------ MMA issuers
         const int ctx = warp - kS1Epi;
-        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)(ctx * 2) * kS1Buf) >> 4) | kDescSw32Lo, h0 = r0 + (kS1Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo;
+        const uint32_t land_bar = smem_u32(&bars.land[ctx]);
+        auto fetch = [&](int n) {
+            if (elect_one()) {
+                mbar_expect_tx(land_bar, kRes1Bytes);
+                bulk_load((r0 & 0x3fff) << 4, p.x1 + (size_t)n * kRes1Bytes, kRes1Bytes, land_bar);
+                if (n + step < batch)  // the image after this one on its way into L2
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.x1 + (size_t)(n + step) * kRes1Bytes), "r"(kRes1Bytes)
+                                 : "memory");
+            }
+            __syncwarp();
+        };
+        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
+        if (n < batch) fetch(n);
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t slot = 0, phase = 0, rdy = 0;
-        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step) {
+        for (; n < batch; n += step) {
             for (int op = 0; op < kS1Ops; ++op) {
-                if (op < 5) {  // (the second half of the last conv reads what the first half read)
-                    image_wait(ready, rdy, abort_flag, p.status, 8);
-                    rdy ^= 1;
-                    fence_after();
-                }
                 const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0, b_op = w0 + (uint32_t)op * (6 * 1024 >> 4);
+                uint32_t last_full = 0, last_phase = 0;
+                if (op < 5) image_wait(ready, rdy, abort_flag, p.status, 8);
                 for (int t = 0; t < kS1Tiles; ++t) {
+                    // a tile's taps reach 43 rows past it: it needs the operand tile after it too, not the whole layer
+                    // (the second half of the last conv reads what the first half read)
+                    if (op < 5 && t + 1 < kS1Tiles) image_wait(ready + 8 * (t + 1), rdy, abort_flag, p.status, 8);
                     image_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
@@ -421,7 +463,14 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                         mma_commit(full0 + 8 * slot);
                     }
                     __syncwarp();
+                    last_full = full0 + 8 * slot;
+                    last_phase = phase;
                     if (++slot == kS1Slots) slot = 0, phase ^= 1;
+                }
+                if (op < 5) rdy ^= 1;
+                else if (n + step < batch) {  // the MMAs have read the image: the next one may land
+                    image_wait(last_full, last_phase, abort_flag, p.status, 16);
+                    fetch(n + step);
                 }
             }
         }
@@ -430,30 +479,25 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
         const int ctx = warp / (kS1Wg * 4), wg = (warp >> 2) % kS1Wg, q = warp & 3;
         const int tid = (int)threadIdx.x - ctx * kS1T;
         const uint32_t rbuf = smem_u32(bufs) + (uint32_t)(ctx * 2) * kS1Buf, hbuf = rbuf + kS1Buf;
-        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
         const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ctx * kS1Cols;
-        auto fetch = [&](int n) {  // one thread
-            mbar_expect_tx(land_bar, kRes1Bytes);
-            bulk_load(rbuf, p.x1 + (size_t)n * kRes1Bytes, kRes1Bytes, land_bar);
-        };
-        auto operand_done = [&]() {
+        auto operand_done = [&](int t) {
             fence_async();
             __syncwarp();
-            if (lane == 0) mbar_arrive(ready);
+            if (lane == 0) mbar_arrive(ready + 8 * t);
         };
+        auto first_tile = [&](int shift) { return (wg + shift) % kS1Wg; };
         // GEMM row m = 128 t + row of this thread: is its second pixel part of the image (bit t)?
         const int row = q * 32 + lane;
         uint32_t second = 0;
         for (int t = 0; t < kS1Tiles; ++t)
             if ((t * 128 + row) % 21 < 20 && t * 128 + row < 861) second |= 1u << t;
-        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (tid == 0 && n < batch) fetch(n);
         uint32_t seq0 = 0, it = 0;  // tiles handed over before this layer, images
-        for (; n < batch; n += step, ++it) {
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step, ++it) {
             // the image: x to tensor memory, ReLU(x) in place for the first conv
             image_wait(land_bar, it & 1, abort_flag, p.status, 1);
-            for (int t = wg; t < kS1Tiles; t += kS1Wg) {
+            for (int t = first_tile(S::shift(1)); t < kS1Tiles; t += kS1Wg) {
                 const int m = t * 128 + row, r = m + 21;
                 const bool v[2] = {m < 861, ((second >> t) & 1) != 0};
 #pragma unroll
@@ -466,15 +510,15 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                     }
                     tmem_st4(tlane + kS1XCol + 8 * t + 4 * h, x);
                 }
+                operand_done(t);
             }
             tmem_wait_st();
-            operand_done();
             auto layer = [&](auto op_c) {
                 constexpr int op = decltype(op_c)::value, c0 = op == 5 ? 16 : 0;
                 constexpr bool skip = op == 1 || op == 3;      // second conv of a block
                 const ResLayer &L = p.layer[op < 4 ? op : 4];
                 const uint32_t dst = skip ? rbuf : hbuf;
-                for (int t = wg; t < kS1Tiles; t += kS1Wg) {
+                for (int t = first_tile(S::shift(op)); t < kS1Tiles; t += kS1Wg) {
                     const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS1Slots;
                     const int m = t * 128 + row, r = m + 21;
                     const bool v[2] = {m < 861, ((second >> t) & 1) != 0};
@@ -493,7 +537,7 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                             if (lane == 0) mbar_arrive(empty0 + 8 * slot);
                         }
                         if (skip) add_skip(a, x, L, 0);
-                        uint4 c = requant_res(a, L, c0);
+                        uint4 c = requant_res<AFFINE, op == 0 || op == 2>(a, L, c0);
                         if (TAP && op < 4 && v[h]) {
                             const int Y = m / 21, X = m - Y * 21;
                             *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 41 + Y) * 41 + 2 * X + h) * 16) = c;
@@ -504,19 +548,13 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
                         }
                         if (v[h]) sts16(dst + row_off(r + h, h ^ 1), c);
                     }
+                    if (op < 4) operand_done(t);
                 }
                 seq0 += kS1Tiles;
                 if (op == 1) tmem_wait_st();
-                if (op < 4) {
-                    operand_done();
-                    return;
-                }
+                if (op < 4) return;
                 // a half of the 16 -> 32 conv is complete: 3 x 3 stride-2 max over it
                 ctx_sync<kS1T>(ctx);
-                if (op == 5 && tid == 0 && n + step < batch) {  // the MMAs have read the image: the next one may land
-                    fence_async();
-                    fetch(n + step);
-                }
                 int8_t *out = p.x2 + (size_t)n * kRes2Bytes;
                 if (tid < 62) {  // the zero pixels: lines 0 and 21, the first one of the lines between
                     const int s = tid < 21 ? tid : tid < 42 ? 21 * 21 + tid - 21 : (tid - 41) * 21;
@@ -558,48 +596,68 @@ __global__ void __launch_bounds__(32 * (kS1Epi + kS1Ctx), 1) res_stack1_kernel(c
 // As above with one pixel per GEMM row.  At 9 x 9, where a layer is one tile, the two warpgroups of a
 // context take half of the channels each and a thread keeps its part of x in registers.
 namespace {
-constexpr int kS2Ctx = 3, kS2Wg = 2;                        // images in flight, warpgroups of each
-constexpr int kS2T = kS2Wg * 128, kS2Epi = kS2Ctx * kS2Wg * 4;
 constexpr int kS2Tiles = 4, kS2Ops = 9;                     // 20 * 21 GEMM rows; layers
 constexpr int kS2Buf = 18 * 1024, kS3Buf = 5 * 1024, kS2CtxBytes = 2 * kS2Buf + 2 * kS3Buf;
-constexpr int kS2Slots = 3, kS2Slot3 = 3;                   // accumulators 0 .. 2: the tiles at 20 x 20, 3: the layers at 9 x 9
-constexpr int kS2XCol = 128, kS2Cols = 160;                 // x: 8 columns a tile behind them
-constexpr int kS2Smem = 1024 + kRes2Weights + kS2Ctx * kS2CtxBytes;
-static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kS2Ctx * kS2Cols <= 512, "buffers");
+template <int CTX, int WG>
+struct S2Shape {
+    static constexpr int T = WG * 128, Epi = CTX * WG * 4, Threads = 32 * (Epi + CTX);
+    static constexpr int Slots = CTX == 1 ? kS2Tiles : 3, Slot3 = Slots;     // accumulators of the tiles at 20 x 20, then one for the layers at 9 x 9
+    static constexpr int XCol = (Slots + 1) * 32, Cols = XCol + 8 * kS2Tiles;  // x: 8 columns a tile behind them
+    static constexpr int Smem = 1024 + kRes2Weights + CTX * kS2CtxBytes;
+    static_assert((WG == 2 || (WG == kS2Tiles && Slots == kS2Tiles)) && Slots < kMaxSlots && Cols * CTX <= 512, "tiles of a warpgroup");
+};
+static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kS2Tiles < kMaxTiles, "buffers");
 }  // namespace
 
-template <bool TAP>
-__global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
+template <bool TAP, bool AFFINE, int CTX, int WG>
+__global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
 {
+    using S = S2Shape<CTX, WG>;
+    constexpr int kS2Ctx = CTX, kS2Wg = WG, kS2T = S::T, kS2Epi = S::Epi, kS2Slots = S::Slots, kS2Slot3 = S::Slot3, kS2XCol = S::XCol,
+                  kS2Cols = S::Cols;
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes2Weights;
-    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kS2Ctx * kS2CtxBytes, smem, p.w, kRes2Weights, warp, kS2Wg * 4,
-                                            kS2Slot3);
+    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kS2Ctx * kS2CtxBytes, smem, p.w, kRes2Weights, warp, 8, kS2Slot3, 4,
+                                            kS2Tiles);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kS2Ctx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kS2Epi) {
         // ------------------------------------------------------------------ MMA issuers
         const int ctx = warp - kS2Epi;
-        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
                        r3 = h0 + (kS2Buf >> 4), h3 = r3 + (kS3Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo, d0 = tmem + (uint32_t)ctx * kS2Cols;
+        const uint32_t land_bar = smem_u32(&bars.land[ctx]);
+        auto fetch = [&](int n) {
+            if (elect_one()) {
+                mbar_expect_tx(land_bar, kRes2Bytes);
+                bulk_load((r0 & 0x3fff) << 4, p.x2 + (size_t)n * kRes2Bytes, kRes2Bytes, land_bar);
+                if (n + step < batch)  // the image after this one on its way into L2
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.x2 + (size_t)(n + step) * kRes2Bytes), "r"(kRes2Bytes)
+                                 : "memory");
+            }
+            __syncwarp();
+        };
+        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
+        if (n < batch) fetch(n);
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t rdy = 0, slot = 0, phase = 0, k3 = 0;  // k3: layers done at 9 x 9
-        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step) {
+        for (; n < batch; n += step) {
             for (int op = 0; op < kS2Ops; ++op) {
-                image_wait(ready, rdy, abort_flag, p.status, 8);
-                rdy ^= 1;
-                fence_after();
                 const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
                 if (op < 5) {
                     const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
+                    uint32_t last_full = 0, last_phase = 0;
+                    image_wait(ready, rdy, abort_flag, p.status, 8);
                     for (int t = 0; t < kS2Tiles; ++t) {
+                        // a tile's taps reach 44 rows past it: it needs the operand tile after it too, not the whole layer
+                        if (t + 1 < kS2Tiles) image_wait(ready + 8 * (t + 1), rdy, abort_flag, p.status, 8);
                         image_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                         fence_after();
                         if (elect_one()) {
@@ -611,10 +669,18 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                             mma_commit(full0 + 8 * slot);
                         }
                         __syncwarp();
+                        last_full = full0 + 8 * slot;
+                        last_phase = phase;
                         if (++slot == kS2Slots) slot = 0, phase ^= 1;
+                    }
+                    rdy ^= 1;
+                    if (op == 4 && n + step < batch) {  // the MMAs have read the image: the next one may land
+                        image_wait(last_full, last_phase, abort_flag, p.status, 16);
+                        fetch(n + step);
                     }
                 } else {
                     const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3;
+                    image_wait(ready + 8 * kS2Tiles, k3 & 1, abort_flag, p.status, 8);
                     image_wait(empty0 + 8 * kS2Slot3, (k3 & 1) ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
@@ -632,20 +698,15 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
     } else {
         // ------------------------------------------------------------------ epilogue
         const int ctx = warp / (kS2Wg * 4), wg = (warp >> 2) % kS2Wg, q = warp & 3;
-        const int tid = (int)threadIdx.x - ctx * kS2T;
         const uint32_t rbuf = smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes, hbuf = rbuf + kS2Buf, r3buf = hbuf + kS2Buf,
                        h3buf = r3buf + kS3Buf;
-        const uint32_t ready = smem_u32(&bars.ready[ctx]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
                        empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
         const uint32_t tctx = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ctx * kS2Cols);
-        auto fetch = [&](int n) {  // one thread
-            mbar_expect_tx(land_bar, kRes2Bytes);
-            bulk_load(rbuf, p.x2 + (size_t)n * kRes2Bytes, kRes2Bytes, land_bar);
-        };
-        auto operand_done = [&]() {
+        auto operand_done = [&](int t) {  // tile t at 20 x 20, or (kS2Tiles) a warp's part at 9 x 9
             fence_async();
             __syncwarp();
-            if (lane == 0) mbar_arrive(ready);
+            if (lane == 0) mbar_arrive(ready + 8 * t);
         };
         const int row = q * 32 + lane;
         uint32_t inside = 0;  // bit t: row 128 t + row is a pixel of the 20 x 20 image
@@ -655,12 +716,10 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
         const int Y3 = row / 10, X3 = row - Y3 * 10;
         const bool v3 = Y3 < 9 && X3 < 9;
         const uint32_t off3 = row_off(row + 11, wg);
-        int n = (int)blockIdx.x + ctx * (int)gridDim.x;
-        if (tid == 0 && n < batch) fetch(n);
         uint32_t seq0 = 0, k3 = 0, it = 0;
-        for (; n < batch; n += step, ++it) {
+        for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step, ++it) {
             image_wait(land_bar, it & 1, abort_flag, p.status, 1);
-            for (int t = wg; t < kS2Tiles; t += kS2Wg)
+            for (int t = wg; t < kS2Tiles; t += kS2Wg) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t at = rbuf + (off2 ^ (16 * h)) + t * 4096;
@@ -671,8 +730,9 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                     }
                     tmem_st4(tctx + kS2XCol + 8 * t + 4 * h, x);
                 }
+                operand_done(t);
+            }
             tmem_wait_st();
-            operand_done();
             auto layer20 = [&](auto op_c) {
                 constexpr int op = decltype(op_c)::value;
                 constexpr bool skip = op == 1 || op == 3;
@@ -696,7 +756,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                             if (lane == 0) mbar_arrive(empty0 + 8 * slot);
                         }
                         if (skip) add_skip(a, x, L, 16 * h);
-                        uint4 c = requant_res(a, L, 16 * h);
+                        uint4 c = requant_res<AFFINE, op == 0 || op == 2>(a, L, 16 * h);
                         if (TAP && v) {
                             const int m = t * 128 + row, Y = m / 21, X = m - Y * 21;
                             *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 20 + Y) * 20 + X) * 32 + 16 * h) = c;
@@ -707,10 +767,10 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                         }
                         if (v) sts16(dst + (off2 ^ (16 * h)) + t * 4096, c);
                     }
+                    if (op < 4) operand_done(t);
                 }
                 seq0 += kS2Tiles;
                 if (op == 1) tmem_wait_st();
-                if (op < 4) operand_done();
             };
             layer20(OpIndex<0>());
             layer20(OpIndex<1>());
@@ -719,10 +779,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
             layer20(OpIndex<4>());
             // 3 x 3 stride-2 max over the last one: every thread its pixel and channels of the 9 x 9 tensor
             ctx_sync<kS2T>(ctx);
-            if (tid == 0 && n + step < batch) {  // the MMAs have read the image's buffer: the next one may land
-                fence_async();
-                fetch(n + step);
-            }
+            if (wg >= 2) continue;  // (two warpgroups do the layers at 9 x 9)
             uint4 x = make_uint4(0, 0, 0, 0);
             if (v3) {
                 const int R = (2 * Y3 + 1) * 21 + 2 * X3 + 1;
@@ -734,7 +791,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                 sts16(r3buf + off3, relu16(x));
                 if (TAP) *reinterpret_cast<uint4 *>(p.tap_x3 + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = x;
             }
-            operand_done();
+            operand_done(kS2Tiles);
             auto layer9 = [&](auto op_c, auto half_c) {
                 constexpr int op = decltype(op_c)::value, half = decltype(half_c)::value;
                 constexpr bool skip = op == 6 || op == 8;
@@ -748,7 +805,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty0 + 8 * kS2Slot3);
                 if (skip) add_skip(a, x, L, 16 * half);
-                uint4 c = requant_res(a, L, 16 * half);
+                uint4 c = requant_res<AFFINE, op == 5 || op == 7>(a, L, 16 * half);
                 if (TAP && v3 && op < 8) *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * half) = c;
                 if (skip) {
                     x = c;
@@ -758,7 +815,7 @@ __global__ void __launch_bounds__(32 * (kS2Epi + kS2Ctx), 1) res_stack23_kernel(
                     if (v3) *reinterpret_cast<uint4 *>(p.x3 + (size_t)n * kRes3Bytes + (Y3 * 9 + X3) * 32 + 16 * half) = c;
                 } else {
                     if (v3) sts16((skip ? r3buf : h3buf) + off3, c);
-                    operand_done();
+                    operand_done(kS2Tiles);
                 }
                 ++k3;
             };
@@ -801,23 +858,43 @@ cudaError_t res_launch(K kernel, const P &p, int threads, size_t smem, int sm_co
 
 }  // namespace
 
-cudaError_t res_first_launch(const ResFirstParams &p, int sm_count, cudaStream_t st)
+// Calls `go(TAP, AFFINE)` with both as compile-time values.  Kernels whose layers all have the single-fma pair do
+// without the division's code (half of the requantiser's instructions, and the unrolled layers exceed the
+// instruction cache); the parity taps take the general form.
+template <typename P, typename F>
+cudaError_t res_dispatch(const P &p, const ResLayer *layer, int layers, bool tap, F go)
 {
-    auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kFirstEpi + kFirstCtx), kFirstSmem, sm_count, st); };
-    if (p.tap_in) return p.ingest_mode == 2 ? go(res_first_kernel<true, true>) : go(res_first_kernel<false, true>);
-    return p.ingest_mode == 2 ? go(res_first_kernel<true, false>) : go(res_first_kernel<false, false>);
+    bool affine = true;
+    for (int i = 0; i < layers; ++i) affine &= layer[i].affine != 0;
+    if (tap) return go(std::true_type(), std::false_type());
+    return affine ? go(std::false_type(), std::true_type()) : go(std::false_type(), std::false_type());
 }
 
+cudaError_t res_first_launch(const ResFirstParams &p, int sm_count, cudaStream_t st)
+{
+    return res_dispatch(p, &p.layer, 1, p.tap_in != nullptr, [&](auto tap, auto affine) {
+        auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kFirstEpi + kFirstCtx), kFirstSmem, sm_count, st); };
+        return p.ingest_mode == 2 ? go(res_first_kernel<true, tap(), affine()>) : go(res_first_kernel<false, tap(), affine()>);
+    });
+}
+
+// Up to an image per SM only one context would work: then it has all the warps (four warpgroups).
 cudaError_t res_stack1_launch(const ResStack1Params &p, int sm_count, cudaStream_t st)
 {
-    auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kS1Epi + kS1Ctx), kS1Smem, sm_count, st); };
-    return p.tap_x2 ? go(res_stack1_kernel<true>) : go(res_stack1_kernel<false>);
+    return res_dispatch(p, p.layer, 5, p.tap_x2 != nullptr, [&](auto tap, auto affine) {
+        if (p.batch <= sm_count)
+            return res_launch(res_stack1_kernel<tap(), affine(), 1, 4>, p, S1Shape<1, 4>::Threads, S1Shape<1, 4>::Smem, sm_count, st);
+        return res_launch(res_stack1_kernel<tap(), affine(), 3, 2>, p, S1Shape<3, 2>::Threads, S1Shape<3, 2>::Smem, sm_count, st);
+    });
 }
 
 cudaError_t res_stack23_launch(const ResStack23Params &p, int sm_count, cudaStream_t st)
 {
-    auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kS2Epi + kS2Ctx), kS2Smem, sm_count, st); };
-    return p.tap_x3 ? go(res_stack23_kernel<true>) : go(res_stack23_kernel<false>);
+    return res_dispatch(p, p.layer, 9, p.tap_x3 != nullptr, [&](auto tap, auto affine) {
+        if (p.batch <= sm_count)
+            return res_launch(res_stack23_kernel<tap(), affine(), 1, 4>, p, S2Shape<1, 4>::Threads, S2Shape<1, 4>::Smem, sm_count, st);
+        return res_launch(res_stack23_kernel<tap(), affine(), 3, 2>, p, S2Shape<3, 2>::Threads, S2Shape<3, 2>::Smem, sm_count, st);
+    });
 }
 
 }  // namespace accerl

@@ -262,3 +262,23 @@ def test_hidden_layer_last_layer_and_sampler_in_tiles(hidden, actions, value, b)
             assert torch.equal(mixed[k], res[k]), k
         other.close()
     g.close()
+
+
+@pytest.mark.parametrize("b", [1, 148, 149, 445, 900])
+@pytest.mark.parametrize("flag", ["", "FLAG_TEST_NO_AFFINE"], ids=["single_fma", "division"])
+def test_residual_network_kernels_by_images_per_sm(b, flag):
+    """One image per SM, two or three at once, several in turn; single-fma and dividing code: the logits of the
+    dp4a kernels, bit for bit."""
+    import paper_2211_15023_b200 as P
+    pol = W.drawn_int8_policy("impala_resnet_b16384", seed=21)
+    obs = torch.from_numpy(W.observations("impala_resnet_b16384", b, seed=b)).cuda()
+    u = torch.from_numpy(W.uniforms("impala_resnet_b16384", b, seed=b)).cuda()
+    got = []
+    for flags in (getattr(P, flag) if flag else 0, P.FLAG_FORCE_GENERIC):
+        g = P.Policy(pol, b, flags=flags)
+        assert ("res_stack1_kernel" in g.info()["plan"]) == (flags != P.FLAG_FORCE_GENERIC)
+        got.append([t.clone() for t in g.act(obs, u)])
+        g.check()
+        g.close()
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
