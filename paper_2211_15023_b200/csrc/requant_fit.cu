@@ -4,8 +4,11 @@
 // non-decreasing step function of the int32 accumulator (k = s_in * s_w[c] > 0; every rounding
 // in it is monotone).  So is a(acc) = relu?(clamp(rint(fmaf((float)acc, k2, b2)))) for k2 > 0.
 // Two non-decreasing functions that agree on every integer of [lo, hi], with both already at the
-// lowest code at lo and at 127 at hi, agree on all of int32.  The band [lo, hi] has a few hundred
-// thousand integers, so the comparison is exhaustive and cheap.  (k2, b2) = (fl(k / s_out),
+// lowest code at lo and at 127 at hi, agree on all of int32.  And they agree on [lo, hi] if they agree at
+// its ends and rise to each code at the same integer.  So a thread finds the first accumulator of one
+// code by bisection, and a candidate pair is compared there and one below: two evaluations a thread
+// instead of the whole band of a few hundred thousand integers, with the same outcome for every
+// candidate.  (k2, b2) = (fl(k / s_out),
 // fl(b / s_out)) is right for most channels; where a handful of accumulators near a rounding tie
 // come out differently, neighbours of the pair are tried -- b2 in steps of 2^-21, k2 in ulps --
 // until one agrees everywhere.  A layer all of whose channels have such a pair runs its epilogue
@@ -27,8 +30,7 @@ namespace {
 constexpr int kKOffsets = 25;   // k2: 0, +1, -1, ... +12, -12 ulps
 constexpr int kBOffsets = 49;   // b2: 0, +1, -1, ... +24, -24 steps of 2^-21
 constexpr int kFitThreads = 256;
-constexpr int kPerThread = 16;  // accumulators a thread compares between two votes
-constexpr int kMaxBad = 16;
+constexpr int kFitGroup = 8;    // candidates compared between two votes
 
 struct FitJob {
     float s_out;
@@ -46,56 +48,62 @@ struct FitResult {
 
 __device__ __forceinline__ int alternate(int i) { return (i & 1) ? (i + 1) / 2 : -(i / 2); }  // 0, 1, -1, 2, -2, ...
 
+// A block per channel, a thread per code above the band's lowest (at most 255).  Bound by the chain of
+// votes over the candidates of a channel that has no pair at all (a few per wide fully connected layer).
 __global__ void __launch_bounds__(kFitThreads) fit_affine_kernel(const FitJob *jobs, FitResult *results)
 {
-    __shared__ long long bad[kMaxBad];  // accumulators on which an earlier candidate failed: tried first
-    __shared__ int n_bad;
+    __shared__ unsigned failed[3];  // candidates of a group that some thread refutes, three groups in turn
     const FitJob job = jobs[blockIdx.x];
     const bool relu = job.relu != 0;
-    const float s_out = job.s_out;
-    auto affine = [&](int acc, float k2, float b2) { return relu ? affine_code<true>(acc, k2, b2) : affine_code<false>(acc, k2, b2); };
-    if (threadIdx.x == 0) n_bad = 0;
-    __syncthreads();
-    auto agree = [&](long long a, float k2, float b2) {
-        return affine((int)a, k2, b2) == exact_code(epilogue_float((int)a, job.k, job.b, false), s_out, relu);
+    auto code = [&](long long a) { return exact_code(epilogue_float((int)a, job.k, job.b, false), job.s_out, relu); };
+    const int code_lo = code(job.lo), code_hi = code(job.hi), mine = code_lo + 1 + (int)threadIdx.x;
+    if (threadIdx.x < 3) failed[threadIdx.x] = 0;
+    // The first accumulator with this thread's code or a higher one; the thread behind the last code takes the
+    // band's ends instead.
+    const bool rises = mine <= code_hi, ends = mine == code_hi + 1;
+    long long below = job.lo, first = job.hi;
+    if (rises) {
+        while (first - below > 1) {
+            const long long mid = below + (first - below) / 2;
+            if (code(mid) >= mine) first = mid;
+            else below = mid;
+        }
+    }
+    const float x0 = __int2float_rn((int)below), x1 = __int2float_rn((int)first);
+    // saturated at an end that is no int32 limit
+    const bool ends_ok = (!job.check_lo || code_lo == (relu ? 0 : -128)) && (!job.check_hi || code_hi == 127);
+    auto refuted = [&](float k2, float b2) {
+        auto affine = [&](float x) {
+            const int q = min(max(__float2int_rn(__fmaf_rn(x, k2, b2)), -128), 127);
+            return relu ? max(q, 0) : q;
+        };
+        const int a0 = affine(x0), a1 = affine(x1);
+        return rises ? a0 >= mine || a1 < mine : ends && (!ends_ok || a0 != code_lo || a1 != code_hi);
     };
-    for (int cand = 0; cand < kKOffsets * kBOffsets; ++cand) {
-        const float k2 = __uint_as_float(__float_as_uint(job.k0) + (unsigned)alternate(cand % kKOffsets));
-        const float b2 = __fadd_rn(job.b0, __int2float_rn(alternate(cand / kKOffsets)) * 4.76837158203125e-7f);
-        if (!(k2 > 0.f)) continue;  // uniform over the block
-        // the accumulators that refuted earlier candidates, and the two ends of the band
-        bool fail = false;
-        const int known = min(n_bad, kMaxBad);
-        if ((int)threadIdx.x < known) fail = !agree(bad[threadIdx.x], k2, b2);
-        if (threadIdx.x == kFitThreads - 1) {
-            if (job.check_lo && affine((int)job.lo, k2, b2) != (relu ? 0 : -128)) fail = true;
-            if (job.check_hi && affine((int)job.hi, k2, b2) != 127) fail = true;
+    auto candidate_k = [&](int cand) { return __uint_as_float(__float_as_uint(job.k0) + (unsigned)alternate(cand % kKOffsets)); };
+    auto candidate_b = [&](int cand) { return __fadd_rn(job.b0, __int2float_rn(alternate(cand / kKOffsets)) * 4.76837158203125e-7f); };
+    __syncthreads();
+    constexpr int kCands = kKOffsets * kBOffsets;
+    for (int cand0 = 0, group = 0; cand0 < kCands; cand0 += kFitGroup, group = group == 2 ? 0 : group + 1) {
+        unsigned mask = 0;
+#pragma unroll
+        for (int j = 0; j < kFitGroup; ++j) {
+            const float k2 = candidate_k(cand0 + j);
+            if (cand0 + j >= kCands || !(k2 > 0.f) || refuted(k2, candidate_b(cand0 + j))) mask |= 1u << j;
         }
-        if (__syncthreads_or(fail)) continue;
-        // the whole band, a slice at a time
-        bool refuted = false;
-        for (long long base = job.lo; base <= job.hi && !refuted; base += (long long)kFitThreads * kPerThread) {
-            long long first_bad = 0;
-            bool any_bad = false;
-            for (int j = 0; j < kPerThread; ++j) {
-                const long long a = base + (long long)j * kFitThreads + threadIdx.x;
-                if (a <= job.hi && !any_bad && !agree(a, k2, b2)) {
-                    first_bad = a;
-                    any_bad = true;
-                }
-            }
-            if (any_bad) {
-                const int slot = atomicAdd(&n_bad, 1);
-                if (slot < kMaxBad) bad[slot] = first_bad;
-            }
-            refuted = __syncthreads_or(any_bad) != 0;
-        }
-        if (!refuted) {
-            if (threadIdx.x == 0) results[blockIdx.x] = FitResult{k2, b2, 1, cand + 1};
+        mask = __reduce_or_sync(0xffffffffu, mask);
+        if ((threadIdx.x & 31) == 0 && mask) atomicOr(&failed[group], mask);
+        __syncthreads();
+        const unsigned left = ~failed[group] & ((1u << kFitGroup) - 1);
+        // (the group before was read before this vote and its word is written again after the next one)
+        if (threadIdx.x == 0) failed[group == 0 ? 2 : group - 1] = 0;
+        if (left) {
+            const int cand = cand0 + __ffs(left) - 1;
+            if (threadIdx.x == 0) results[blockIdx.x] = FitResult{candidate_k(cand), candidate_b(cand), 1, cand + 1};
             return;
         }
     }
-    if (threadIdx.x == 0) results[blockIdx.x] = FitResult{job.k0, job.b0, 0, kKOffsets * kBOffsets};
+    if (threadIdx.x == 0) results[blockIdx.x] = FitResult{job.k0, job.b0, 0, kCands};
 }
 
 // band of accumulators outside which both requantisers are saturated (or which int32 ends)
