@@ -60,21 +60,36 @@ __device__ __forceinline__ double exp_nonpositive(double x, const double *table)
     return x >= -708.0 ? y : x < 0.0 ? 0.0 : x;
 }
 
-// One row, elements at zo[0], zo[1], ... (any address space), by one thread.
+// One row by one thread, V elements a load (then the row's address is a multiple of V elements and A one of V);
+// the elements are added in order whatever V is.
+template <int V>
 __device__ __forceinline__ float kl_of_row(const float *zo, const float *zs, int A, const double *table)
 {
+    struct alignas(4 * V) Piece {
+        float v[V];
+    };
+    const Piece *po = reinterpret_cast<const Piece *>(zo), *ps = reinterpret_cast<const Piece *>(zs);
+    const int pieces = A / V;
     float fo = zo[0], fs = zs[0];
-    for (int i = 1; i < A; ++i) {
-        fo = fmaxf(fo, zo[i]);
-        fs = fmaxf(fs, zs[i]);
+    for (int i = 0; i < pieces; ++i) {
+        const Piece a = po[i], b = ps[i];
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            fo = fmaxf(fo, a.v[k]);
+            fs = fmaxf(fs, b.v[k]);
+        }
     }
     const double mo = fo, ms = fs;
     double so = 0.0, ss = 0.0, acc = 0.0;
-    for (int i = 0; i < A; ++i) {
-        const double o = zo[i], s = zs[i], e = exp_nonpositive(o - mo, table);
-        so += e;
-        ss += exp_nonpositive(s - ms, table);
-        if (e > 0.0) acc += e * (o - s);
+    for (int i = 0; i < pieces; ++i) {
+        const Piece a = po[i], b = ps[i];
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const double o = a.v[k], t = b.v[k], e = exp_nonpositive(o - mo, table);
+            so += e;
+            ss += exp_nonpositive(t - ms, table);
+            if (e > 0.0) acc += e * (o - t);
+        }
     }
     return (float)(acc / so - ((mo + log(so)) - (ms + log(ss))));
 }
@@ -137,16 +152,19 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
 
 // Many rows of at most 64 actions, or few of at most 12 (see the choice in accerl_policy_kl): one thread per
 // row.  A block's rows are contiguous in memory; they pass through shared memory, by asynchronous copies that
-// are all in flight at once, so that the loads are whole lines and every thread then walks its own row (odd
-// pitch: no bank conflicts), a chain of two exponentials an action.  A warp per row, as below, leaves 14 of 32 lanes idle at 18 actions and spends its time in shuffles; with that and a
+// are all in flight at once, so that the loads are whole lines and every thread then walks its own row, a chain
+// of two exponentials an action.  V > 0: the rows lie in shared memory as in global memory and come in 16-byte
+// copies (a fourth of the instructions, and no row and column to keep); a thread reads V = 1, 2 or 4 elements at a
+// time, the width at which rows of that many elements fall into different banks.  V = 0, for rows of a multiple of
+// eight elements or addresses that are none of 16 bytes: element by element into rows of an odd pitch.  A warp per row, as below, leaves 14 of 32 lanes idle at 18 actions and spends its time in shuffles; with that and a
 // one-block reduction the two launches for 131072 rows of 18 took 119 us, now 20.5.  STATS (one cluster,
 // at most kKlCluster blocks' rows a pass): the mean and the maximum come out of the same launch.
-template <bool STATS>
+template <bool STATS, int V>
 __global__ void __launch_bounds__(kKlRows)
 kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B, int A, int pitch,
                float *__restrict__ kl, float *__restrict__ stats)
 {
-    extern __shared__ float s_rows[];  // [2][kKlRows][pitch]
+    extern __shared__ __align__(16) float s_rows[];  // [2][kKlRows][pitch]
     __shared__ double s_table[64];
     if (STATS) cluster_started();
     if (threadIdx.x < 64) s_table[threadIdx.x] = exp2((double)threadIdx.x * (1.0 / 64.0));
@@ -155,24 +173,35 @@ kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B
     for (long long row0 = (long long)blockIdx.x * kKlRows; row0 < B; row0 += (long long)gridDim.x * kKlRows) {
         const int rows = (int)min((long long)kKlRows, B - row0), n = rows * A;
         const float *src[2] = {zo + row0 * A, zs + row0 * A};
-        int r = (int)threadIdx.x / A, c = (int)threadIdx.x - r * A;
-        const int dr = kKlRows / A, dc = kKlRows - dr * A;
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_rows);
-        for (int i = threadIdx.x; i < n; i += kKlRows) {
-            const uint32_t d = dst + 4 * (r * pitch + c);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src[0] + i) : "memory");
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * kKlRows * pitch), "l"(src[1] + i) : "memory");
-            r += dr;
-            c += dc;
-            if (c >= A) {
-                c -= A;
-                ++r;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_rows), dst1 = dst + 4 * kKlRows * pitch;
+        if constexpr (V > 0) {
+            for (int i = 4 * threadIdx.x; i + 3 < n; i += 4 * kKlRows) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 4 * i), "l"(src[0] + i) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst1 + 4 * i), "l"(src[1] + i) : "memory");
+            }
+            if (const int i = (n & ~3) + (int)threadIdx.x; i < n) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * i), "l"(src[0] + i) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst1 + 4 * i), "l"(src[1] + i) : "memory");
+            }
+        } else {
+            int r = (int)threadIdx.x / A, c = (int)threadIdx.x - r * A;
+            const int dr = kKlRows / A, dc = kKlRows - dr * A;
+            for (int i = threadIdx.x; i < n; i += kKlRows) {
+                const uint32_t d = 4 * (r * pitch + c);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + d), "l"(src[0] + i) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst1 + d), "l"(src[1] + i) : "memory");
+                r += dr;
+                c += dc;
+                if (c >= A) {
+                    c -= A;
+                    ++r;
+                }
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         if ((int)threadIdx.x < rows) {
-            const float v = kl_of_row(s_rows + threadIdx.x * pitch, s_rows + (kKlRows + threadIdx.x) * pitch, A, s_table);
+            const float v = kl_of_row<V ? V : 1>(s_rows + threadIdx.x * pitch, s_rows + (kKlRows + threadIdx.x) * pitch, A, s_table);
             kl[row0 + threadIdx.x] = v;
             sum += (double)v;
             mx = fmaxf(mx, v);
@@ -331,7 +360,8 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
     const long long rows_blocks = ((long long)batch + kKlRows - 1) / kKlRows;
     const bool one_launch = kl_mean_max_dev && n_actions <= 12 && rows_blocks <= (n_actions <= 6 ? 2 : 1) * kKlCluster;
     const bool narrow = n_actions <= 64 && (one_launch || batch >= 256 * n_actions);  // (66 KB of shared memory at 64)
-    const int pitch = n_actions | 1;
+    const bool whole = !one_launch && n_actions % 8 != 0 && (((uintptr_t)logits_original_dev | (uintptr_t)logits_smaller_dev) & 15) == 0;
+    const int pitch = whole ? n_actions : n_actions | 1;
     const size_t smem = 2 * sizeof(float) * (size_t)kKlRows * pitch;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
@@ -347,15 +377,16 @@ extern "C" accerl_status accerl_policy_kl(const float *logits_original_dev, cons
         cfg.dynamicSmemBytes = smem;
         attr[0].val.clusterDim.x = n;
         cfg.numAttrs = 1;
-        ACCERL_CUDA_TRY(allow_smem((const void *)kl_rows_kernel<true>, smem));
-        ACCERL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kl_rows_kernel<true>, logits_original_dev, logits_smaller_dev, batch,
+        ACCERL_CUDA_TRY(allow_smem((const void *)kl_rows_kernel<true, 0>, smem));
+        ACCERL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kl_rows_kernel<true, 0>, logits_original_dev, logits_smaller_dev, batch,
                                            n_actions, pitch, kl_dev, kl_mean_max_dev));
         return ACCERL_OK;
     }
     if (narrow) {
-        ACCERL_CUDA_TRY(allow_smem((const void *)kl_rows_kernel<false>, smem));
-        kl_rows_kernel<false><<<(unsigned)blocks, kKlRows, smem, st>>>(logits_original_dev, logits_smaller_dev, batch,
-                                                                      n_actions, pitch, kl_dev, nullptr);
+        const auto kernel = !whole ? kl_rows_kernel<false, 0>
+                                   : n_actions % 2 ? kl_rows_kernel<false, 1> : n_actions % 4 ? kl_rows_kernel<false, 2> : kl_rows_kernel<false, 4>;
+        ACCERL_CUDA_TRY(allow_smem((const void *)kernel, smem));
+        kernel<<<(unsigned)blocks, kKlRows, smem, st>>>(logits_original_dev, logits_smaller_dev, batch, n_actions, pitch, kl_dev, nullptr);
     } else {
         kl_wide_kernel<<<(unsigned)blocks, 128, 0, st>>>(logits_original_dev, logits_smaller_dev, batch, n_actions, kl_dev);
     }

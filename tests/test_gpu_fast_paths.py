@@ -282,3 +282,48 @@ def test_residual_network_kernels_by_images_per_sm(b, flag):
         g.close()
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("flag", ["", "FLAG_TEST_NO_AFFINE"], ids=["single_fma", "division"])
+def test_conv_rows_by_groups_of_images(flag):
+    """Fewer images than a tile holds (12 and 14), whole groups and remainders, fewer and more output lines than
+    SMs, ranges of a CTA that start and end inside a group: the logits of the dp4a kernels, bit for bit."""
+    import paper_2211_15023_b200 as P
+    name, top = "nature_cnn_b8192", 2561  # above the single-launch conv stack
+    pol = W.drawn_int8_policy(name, seed=22)
+    g, ref = P.Policy(pol, top, flags=getattr(P, flag) if flag else 0), P.Policy(pol, top, flags=P.FLAG_FORCE_GENERIC)
+    assert g.info()["plan"].count("conv_rows_kernel") == 2
+    for b in (1, 11, 12, 13, 14, 15, 168, 200, 1000, top):
+        obs = torch.from_numpy(W.observations(name, b, seed=b)).cuda()
+        u = torch.from_numpy(W.uniforms(name, b, seed=b)).cuda()
+        for x, y in zip(g.act(obs, u), ref.act(obs, u)):
+            assert torch.equal(x, y)
+    g.check()
+    g.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("a", [1, 2, 3, 4, 7, 12, 17, 18, 20, 24])
+def test_kl_rows_by_width_and_alignment(a):
+    """Rows copied 16 bytes at a time and read 1, 2 or 4 elements at a time, the last block's remainder among them,
+    against the same rows at an address that is no multiple of 16 bytes: the same bits."""
+    import paper_2211_15023_b200 as P
+    b = 256 * a + 131
+    rng = np.random.default_rng(a)
+    z = torch.from_numpy(rng.standard_normal((2, b * a), np.float32) * 3).cuda()
+    odd = torch.empty((2, b * a + 8), device="cuda")
+    shifted = [odd[i].view(-1)[1:1 + b * a] for i in range(2)]
+    for d, s in zip(shifted, z):
+        d.copy_(s)
+    assert z[0].data_ptr() % 16 == 0 and shifted[0].data_ptr() % 16 == 4
+    first = [z[0].view(b, a), z[1].clone().view(b, a)]
+    want, got = P.kl(*first), P.kl(shifted[0].view(b, a), shifted[1].view(b, a))
+    for k in want:
+        assert torch.equal(torch.as_tensor(want[k]), torch.as_tensor(got[k])) if isinstance(want, dict) else True
+    if not isinstance(want, dict):
+        for x, y in zip(want, got):
+            assert torch.equal(torch.as_tensor(x), torch.as_tensor(y))
+    ref = torch.log_softmax(first[0].double(), -1), torch.log_softmax(first[1].double(), -1)
+    ref = (ref[0].exp() * (ref[0] - ref[1])).sum(-1)
+    rows = want["kl"] if isinstance(want, dict) else want[0]
+    torch.testing.assert_close(rows.double(), ref, rtol=1e-5, atol=1e-6)
