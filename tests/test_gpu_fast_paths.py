@@ -322,3 +322,24 @@ def test_kl_rows_by_width_and_alignment(a):
         assert torch.equal(x, y)
     po, ps = torch.log_softmax(zo.double(), -1), torch.log_softmax(zs.double(), -1)
     np.testing.assert_allclose(want[0].cpu().numpy(), (po.exp() * (po - ps)).sum(-1).cpu().numpy(), rtol=RTOL, atol=ATOL)
+
+
+@pytest.mark.parametrize("rows", [1, 37])
+@pytest.mark.parametrize("c1,c2,hidden", [(5, 18, 33), (16, 70, 40), (20, 48, 300)])
+def test_calibration_of_odd_shapes(rows, c1, c2, hidden):
+    """Channels that fill no word, no 16 and no 32 columns, padding, strides, a window of more words than a piece of
+    weights, remainders of positions and rows: scales and codes are the oracle's bits."""
+    import paper_2211_15023_b200 as P
+    rng = np.random.default_rng(rows * 100 + c1)
+    shape = (3, 17, 13)
+    layers = [W._conv(3, 17, 13, c1, 5, 2, 2), W._conv(c1, 9, 7, c2, 3, 1, 1), W._conv(c2, 9, 7, 8, 7, 3, 0),
+              W._fc(8, hidden), W._fc(hidden, 5, relu_out=False, logits=True)]
+    params = W.parameters_for(layers, 17)
+    calib = rng.integers(0, 256, (rows,) + shape, dtype=np.uint8)
+    want = oracle.calibrate("u8", shape, layers, params, calib)
+    g = P.Policy.from_fp32("u8", shape, layers, params, calib, 3)
+    for i, l in enumerate(want["layers"]):
+        got = g.export(i)
+        assert got["s_in"] == np.float32(l["s_in"]) and got["s_out"] == np.float32(l["s_out"]), i
+        assert np.array_equal(got["w"], l["w"]) and np.array_equal(got["s_w"], l["s_w"])
+    g.close()
