@@ -121,7 +121,6 @@ struct ActivationMap {
     const void *base = nullptr;
     long long rows_per_state = 0, pitch = 0;
     int row_bytes = 0, box_rows = 0, box_bytes = 0;
-    int grid_w = 0, images = 0;  // with `images`: boxes of one grid line of so many images (tc_make_line_map)
 };
 
 // One launch of the tensor-core contraction: TMA descriptors (built once, for max_batch rows) and

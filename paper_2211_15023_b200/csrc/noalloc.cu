@@ -137,9 +137,7 @@ std::unique_ptr<accerl_policy> make_twin(accerl_policy *p, unsigned char *base)
     };
     auto remap = [&](void *map, ActivationMap &m) {
         move(m.base);
-        if (ok && m.images) {
-            if (tc_make_line_map(map, m.base, (long long)cap, (int)m.rows_per_state / m.grid_w, m.grid_w, m.row_bytes, m.images) != ACCERL_OK) ok = false;
-        } else if (ok && tc_make_map(map, m.base, m.rows_per_state * (long long)cap, m.row_bytes, m.pitch, m.box_rows, m.box_bytes) != ACCERL_OK)
+        if (ok && tc_make_map(map, m.base, m.rows_per_state * (long long)cap, m.row_bytes, m.pitch, m.box_rows, m.box_bytes) != ACCERL_OK)
             ok = false;
     };
     for (const Step &s : q->steps) {

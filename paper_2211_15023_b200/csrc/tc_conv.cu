@@ -1,23 +1,19 @@
 // Strided, unpadded convolutions on int8 activations (the second and third layer of the paper's
-// Atari networks, table "network architecture and inference time"): a conv with stride s and window
-// k = s * t on a tensor stored space-to-depth(s) is a t x t stride-1 conv on its grid.
+// Atari networks, table "network architecture and inference time") in the form the first-conv
+// kernel has: a conv with stride s and window k = s * t on a tensor stored space-to-depth(s) is a
+// t x t stride-1 conv on its grid, one GEMM row per grid position, every tap a fixed row offset of
+// ONE operand block in shared memory.
 //
-// A tile is ONE grid line of G = 128 / grid_w images (12 x 10 or 14 x 9 positions for the Atari layers): its
-// 128 GEMM rows are (image, x).  So the operand tile of input line y has the same rows as the accumulators of
-// the output lines y, y - 1, .. y - t + 1 it contributes to, one per vertical tap, and ONE instruction serves
-// all of them: N = t * 64, the weights of the vertical taps side by side and the accumulators of t consecutive
-// lines in consecutive columns of tensor memory.  An instruction costs max(39, 32 + N / 4, N / 2) cycles, so
-// t of them at N = 64 (48 each) become one at 64 (t = 2) or 96 (t = 3).  Tiles of whole grid rows with a
-// row-shifted operand per tap, as the other kernels have them, took 640 and 555 cycles an image for the
-// second and third layer, these take 430 and 310.  (The first instruction on a new line must overwrite it
-// and not the lines beside it, and lines that wrap around the ring of accumulators are two pieces: a few
-// per cent.)  Horizontal taps are row-shifted views of the tile.
-//
-// - A pipeline stage is one input line: one four-dimensional TMA box (row bytes, x, one y, G images).
-// - The CTAs share the (group of images, output line) pairs evenly; a CTA's range starts and ends anywhere in a
-//   group and costs the t - 1 input lines before its first output line.
-// - Scales and biases are kernel parameters read from the constant bank, because shared-memory loads of the
-//   epilogue queue behind the operand reads of the MMAs.
+// What differs from the general contraction kernel (tc_gemm.cu):
+// - a tile is S whole grid rows (S * Ws <= 128 GEMM rows): a thread of the epilogue owns the same
+//   (row, X) of every tile, its output address costs two multiplies per tile;
+// - a pipeline step is T tiles whose operand block (the T * S grid rows and the t - 1 rows the taps
+//   reach into) arrives by a few TMA boxes issued by one warp; kStages2 blocks are in flight;
+// - four warps issue the MMAs, tiles in turn (descriptors computed in registers; one warp that
+//   shares its scheduler with five others issues an instruction every six to eight cycles, and a
+//   tile takes some two hundred: measured 49 / 41 / 36 us for the layer with one / two / four
+//   issuing warps), sixteen warps drain accumulators; scales and biases are kernel parameters read from the constant bank, because
+//   shared-memory loads of the epilogue queue behind the operand reads of the MMAs.
 //
 // Every wait is bounded; a wait that gives up sets the status word and all roles leave.
 #include <cuda.h>
@@ -33,36 +29,27 @@ namespace accerl {
 
 namespace {
 
-constexpr int kEpiWarps2 = 16;           // warps 0..15 drain accumulators
-constexpr int kMmaWarp2 = kEpiWarps2, kTmaWarp2 = kEpiWarps2 + 1;
-constexpr int kThreads2 = 32 * (kEpiWarps2 + 2);
-constexpr int kMaxStages2 = 12, kMaxSlots2 = 16;
+constexpr int kMmaWarps2 = 4;            // warps 0..3 issue MMAs, the CTA's tiles in turn
+constexpr int kEpiWarps2 = 16;           // warps 4..19 drain accumulators
+constexpr int kWarps2 = 4 + kEpiWarps2 + 1;  // the last warp issues the TMA loads
+constexpr int kThreads2 = 32 * kWarps2;
+constexpr int kStages2 = 4;
+constexpr int kMaxSlots2 = 16;
 
 struct __align__(8) Bars2 {
-    uint64_t full[kMaxStages2], empty[kMaxStages2];
+    uint64_t full[kStages2], empty[kStages2];
     uint64_t acc_full[kMaxSlots2], acc_empty[kMaxSlots2];
     uint64_t b_ready;
     uint32_t tmem_base;
     int abort_flag;
 };
 
-// the single warps that issue and load wait without sleeping first: the whole CTA waits for them
-__device__ __forceinline__ bool line_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status, int code)
-{
-    return mbar_wait_limited(bar, parity, abort_flag, status, code, 2048, kWaitLimitPolls);
-}
-
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
-        : "memory");
-}
-
 }  // namespace
 
-template <int NCOLS, bool AFFINE>
+// TAPS_T / RB_T: taps per side and bytes of an operand row as compile-time constants (0 = taken from
+// the parameters); with them the issue loop of a tile is straight-line code, and the issuing warps'
+// instruction count is what bounds how fast tiles start.
+template <int NCOLS, int TAPS_T, int RB_T, bool AFFINE>
 __global__ void __launch_bounds__(kThreads2, 1)
 conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                  const __grid_constant__ ConvRowsParams p)
@@ -71,18 +58,19 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw2 + 1023) & ~(uintptr_t)1023);
     __shared__ Bars2 bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kAccSlots = 512 / NCOLS < kMaxSlots2 ? 512 / NCOLS : kMaxSlots2;  // ring of accumulators, NCOLS columns each
-    const int RB = p.row_bytes, taps = p.taps;
-    const int b_bytes = taps * taps * NCOLS * RB;
+    constexpr int kSlotCols = NCOLS <= 32 ? 32 : 64;     // tensor-memory columns of one accumulator
+    constexpr int kAccSlots = 512 / kSlotCols;
+    const int RB = RB_T ? RB_T : p.row_bytes, taps = TAPS_T ? TAPS_T : p.taps, n_taps = taps * taps;
+    const int b_bytes = n_taps * NCOLS * RB;
     uint8_t *b_tiles = smem;
     uint8_t *stages = smem + ((b_bytes + 1023) & ~1023);
-    const int n_stages = p.n_stages;
+    const int stage_bytes = p.stage_bytes;
     volatile int *abort_flag = &bars.abort_flag;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < n_stages; ++s) {
+        for (int s = 0; s < kStages2; ++s) {
             mbar_init(smem_u32(&bars.full[s]), 1);
-            mbar_init(smem_u32(&bars.empty[s]), 1);
+            mbar_init(smem_u32(&bars.empty[s]), kMmaWarps2);
         }
         for (int a = 0; a < kAccSlots; ++a) {
             mbar_init(smem_u32(&bars.acc_full[a]), 1);
@@ -93,7 +81,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == kMmaWarp2) {
+    if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(&bars.tmem_base)), "r"(512u)
                      : "memory");
@@ -106,185 +94,176 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     // the next launch may set itself up while this grid drains
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // this CTA's output lines, numbered through all groups of images
-    const int out_h = p.out_h;
-    const int line0 = (int)((long long)blockIdx.x * p.total_lines / gridDim.x);
-    const int n_lines = (int)((long long)(blockIdx.x + 1) * p.total_lines / gridDim.x) - line0;
-    const int group0 = line0 / out_h, y0 = line0 - group0 * out_h;
+    const int T = p.tiles_per_step, S = p.rows_per_tile, Ws = p.grid_w, Hs = p.grid_h;
+    const int my_steps = (int)blockIdx.x < p.total_steps
+                             ? (p.total_steps - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const uint32_t full0 = smem_u32(&bars.full[0]), empty0 = smem_u32(&bars.empty[0]);
     const uint32_t acc_full0 = smem_u32(&bars.acc_full[0]), acc_empty0 = smem_u32(&bars.acc_empty[0]);
 
-    if (warp == kMmaWarp2) {
-        // ------------------------------------------------------------------ MMA issuer
-        const int ksteps = RB >> 5, n_j = taps * ksteps;  // 32-byte K steps of a position, of all horizontal taps
-        if (elect_one()) {  // weights: per K step the vertical taps side by side, the last one first, in rows of 32 bytes
+    if (warp < kMmaWarps2) {
+        // ------------------------------------------------------------------ MMA issuers
+        if (warp == 0 && elect_one()) {
             mbar_expect_tx(smem_u32(&bars.b_ready), (uint32_t)b_bytes);
-            for (int j = 0; j < n_j; ++j)
-                for (int b = 0; b < taps; ++b)
-                    tma_load_2d(smem_u32(b_tiles) + (j * taps + b) * NCOLS * 32, &map_b, 32 * (j % ksteps),
-                                ((taps - 1 - b) * taps + j / ksteps) * NCOLS, smem_u32(&bars.b_ready));
+            for (int j = 0; j < n_taps; ++j)
+                tma_load_2d(smem_u32(b_tiles) + j * NCOLS * RB, &map_b, 0, j * NCOLS, smem_u32(&bars.b_ready));
         }
         __syncwarp();
         bool ok = mbar_wait(smem_u32(&bars.b_ready), 0, abort_flag, p.status, 2);
-        auto idesc = [](int lines) {
-            return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(lines * (NCOLS >> 3)) << 17) | ((uint32_t)(128 >> 4) << 24);
-        };
-        // descriptors: constant upper word | (address >> 4); operand rows of RB bytes, weights of 32, swizzled K-major
-        const uint64_t a_hi = (uint64_t)(((uint32_t)(8 * RB) >> 4) | (1u << 14) | ((RB == 128 ? 2u : (RB == 64 ? 4u : 6u)) << 29)) << 32;
-        const uint64_t b_hi = (uint64_t)((256u >> 4) | (1u << 14) | (6u << 29)) << 32;
+        const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NCOLS >> 3) << 17) |
+                               ((uint32_t)(128 >> 4) << 24);
+        // swizzled K-major rows of RB bytes: descriptor = constant upper word | (address >> 4)
+        const uint64_t desc_hi =
+            (uint64_t)(((uint32_t)(8 * RB) >> 4) | (1u << 14) | ((RB == 128 ? 2u : (RB == 64 ? 4u : 6u)) << 29)) << 32;
         const uint32_t lo_flags = 1u << 16;
-        const uint32_t b_lo = (smem_u32(b_tiles) >> 4) | lo_flags, a_lo = (smem_u32(stages) >> 4) | lo_flags;
-        constexpr uint32_t b_line = NCOLS * 32 / 16;
-        const uint32_t b_step = (uint32_t)taps * b_line, stage16 = (uint32_t)(p.stage_bytes >> 4);
-        int stage = 0;
-        uint32_t phase = 0, a0 = a_lo;
-        int slot = 0;            // accumulator of the lowest line that is still being added to
-        int new_slot = 0;        // and of the next new line
-        uint32_t new_phase = 1;
-        int ya = y0, left = n_lines;
-        while (left > 0 && ok) {  // a segment: output lines ya .. yb - 1 of one group
-            const int yb = min(out_h, ya + left);
-            for (int y = ya; y < yb + taps - 1; ++y) {
-                const int lo = max(ya, y - taps + 1), lines = min(yb - 1, y) - lo + 1;  // output lines lo .. lo + lines - 1
-                const bool fresh = y < yb;                                              // the last of them is new
-                const uint32_t d_new = tmem_base + (uint32_t)(new_slot * NCOLS);
-                if (fresh) {
-                    ok = line_wait(acc_empty0 + 8 * new_slot, new_phase, abort_flag, p.status, 4);
-                    if (!ok) break;
-                    if (++new_slot == kAccSlots) new_slot = 0, new_phase ^= 1;
-                }
-                ok = line_wait(full0 + 8 * stage, phase, abort_flag, p.status, 8);
+        const uint32_t b_lo = (smem_u32(b_tiles) >> 4) | lo_flags;
+        const uint32_t row16 = (uint32_t)(RB >> 4), ksteps = (uint32_t)(RB >> 5);
+        const uint32_t b_tap = (uint32_t)(NCOLS * RB) >> 4;
+        for (int k = 0; k < my_steps && ok; ++k) {
+            const int step = (int)blockIdx.x + k * (int)gridDim.x;
+            const int s = k % kStages2;
+            ok = mbar_wait(full0 + 8 * s, (uint32_t)((k / kStages2) & 1), abort_flag, p.status, 8);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t st_lo = ((smem_u32(stages) + (uint32_t)(s * stage_bytes)) >> 4) | lo_flags;
+            for (int i = 0; i < T && ok; ++i) {
+                if (step * T + i >= p.total_tiles) break;
+                const int seq = k * T + i, slot = seq % kAccSlots;  // the CTA's tiles in order
+                if (seq % kMmaWarps2 != warp) continue;
+                ok = mbar_wait(acc_empty0 + 8 * slot, (uint32_t)(((seq / kAccSlots) & 1) ^ 1), abort_flag, p.status, 4);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const bool complete = y - taps + 1 >= ya;  // the lowest line is complete with this one
                 if (elect_one()) {
-                    // Lines in consecutive columns: n1 of them, and n2 that wrap around the ring.  A short loop and not
-                    // straight-line code: the warp shares its scheduler's instruction buffer with the epilogue's long
-                    // code and executes nothing that is not in a loop from there.
-                    const int n1 = min(lines, kAccSlots - slot), n2 = lines - n1;
-                    const uint32_t d1 = tmem_base + (uint32_t)(slot * NCOLS), i1 = idesc(n1), i2 = idesc(n2);
-                    uint64_t a = a_hi | a0, b1 = b_hi | (b_lo + (uint32_t)(taps - 1 - (y - lo)) * b_line);
-                    const uint64_t b12 = (uint64_t)((uint32_t)n1 * b_line);
-                    int j = 0;
-                    if (fresh) {  // the first instruction on a new line overwrites it
-                        const int old = lines - 1, o1 = min(old, n1), o2 = old - o1;
-                        mma_i8(d_new, a, b1 + (uint32_t)old * b_line, idesc(1), 0);
-                        if (o1) mma_i8(d1, a, b1, idesc(o1), 1);
-                        if (o2) mma_i8(tmem_base, a, b1 + b12, idesc(o2), 1);
-                        j = 1;
-                        a += 2;
-                        b1 += b_step;
+                    const uint32_t d = tmem_base + (uint32_t)(slot * kSlotCols);
+                    const uint32_t a_tile = st_lo + (uint32_t)(i * S * Ws) * row16;
+                    if constexpr (TAPS_T != 0 && RB_T != 0) {
+                        const uint32_t a_row = (uint32_t)Ws * row16;
+#pragma unroll
+                        for (int ty = 0; ty < TAPS_T; ++ty)
+#pragma unroll
+                            for (int tx = 0; tx < TAPS_T; ++tx)
+#pragma unroll
+                                for (int ks = 0; ks < RB_T / 32; ++ks)
+                                    mma_i8(d, desc_hi | (a_tile + ty * a_row + (uint32_t)(tx * (RB_T / 16) + 2 * ks)),
+                                           desc_hi | (b_lo + (uint32_t)((ty * TAPS_T + tx) * (NCOLS * RB_T / 16) + 2 * ks)),
+                                           idesc, (uint32_t)(ty | tx | ks));
+                    } else {
+                        uint32_t b_j = b_lo, first = 0;
+                        for (int ty = 0; ty < taps; ++ty) {
+                            uint32_t a_j = a_tile + (uint32_t)(ty * Ws) * row16;
+                            for (int tx = 0; tx < taps; ++tx) {
+                                for (uint32_t ks = 0; ks < ksteps; ++ks) {
+                                    mma_i8(d, desc_hi | (a_j + 2 * ks), desc_hi | (b_j + 2 * ks), idesc, first);
+                                    first = 1;
+                                }
+                                a_j += row16;
+                                b_j += b_tap;
+                            }
+                        }
                     }
-#pragma unroll 1
-                    for (; j < n_j; ++j) {
-                        mma_i8(d1, a, b1, i1, 1);
-                        if (n2) mma_i8(tmem_base, a, b1 + b12, i2, 1);
-                        a += 2;  // the horizontal taps and their K steps are consecutive 32-byte pieces
-                        b1 += b_step;
-                    }
-                    mma_commit(empty0 + 8 * stage);  // the stage is free when these MMAs retire
-                    if (complete) mma_commit(acc_full0 + 8 * slot);
+                    mma_commit(acc_full0 + 8 * slot);
                 }
                 __syncwarp();
-                if (complete && ++slot == kAccSlots) slot = 0;
-                a0 += stage16;
-                if (++stage == n_stages) stage = 0, phase ^= 1, a0 = a_lo;
             }
-            left -= yb - ya;
-            ya = 0;
+            if (ok && elect_one()) mma_commit(empty0 + 8 * s);  // the block is free when these MMAs retire
+            __syncwarp();
         }
-    } else if (warp == kTmaWarp2) {
+    } else if (warp == kWarps2 - 1) {
         // ------------------------------------------------------------------ TMA producer
         asm volatile("griddepcontrol.wait;" ::: "memory");  // the activations are the previous launch's output
         bool ok = true;
-        int stage = 0, ya = y0, left = n_lines, image = group0 * p.images;
-        uint32_t phase = 0;
-        const uint32_t bytes = (uint32_t)(p.images * p.grid_w * RB);
-        while (left > 0 && ok) {
-            const int yb = min(out_h, ya + left);
-            for (int y = ya; y < yb + taps - 1; ++y) {
-                ok = line_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 1);
-                if (!ok) break;
-                if (elect_one()) {
-                    mbar_expect_tx(full0 + 8 * stage, bytes);
-                    tma_load_4d(smem_u32(stages) + (uint32_t)(stage * p.stage_bytes), &map_a, 0, 0, y, image, full0 + 8 * stage);
-                }
-                __syncwarp();
-                if (++stage == n_stages) stage = 0, phase ^= 1;
+        for (int k = 0; k < my_steps && ok; ++k) {
+            const int step = (int)blockIdx.x + k * (int)gridDim.x;
+            const int s = k % kStages2;
+            ok = mbar_wait(empty0 + 8 * s, (uint32_t)(((k / kStages2) & 1) ^ 1), abort_flag, p.status, 1);
+            if (!ok) break;
+            if (elect_one()) {
+                const uint32_t full = full0 + 8 * s;
+                const uint32_t dst = smem_u32(stages) + (uint32_t)(s * stage_bytes);
+                const int row0 = step * T * S * Ws;  // first grid position of the step
+                mbar_expect_tx(full, (uint32_t)(p.boxes_per_stage * p.box_rows * RB));
+                for (int b = 0; b < p.boxes_per_stage; ++b)
+                    tma_load_2d(dst + (uint32_t)(b * p.box_rows * RB), &map_a, 0, row0 + b * p.box_rows, full);
             }
-            left -= yb - ya;
-            ya = 0;
-            image += p.images;
+            __syncwarp();
         }
     } else {
         // ------------------------------------------------------------------ epilogue
-        const int wg = warp >> 2, q = warp & 3;
+        const int ew = warp - 4, wg = ew >> 2, q = warp & 3;
         constexpr int kGroups = kEpiWarps2 / 4;
-        const int r = q * 32 + lane;  // this thread's row of every tile: position X of image `in_group` of the group
-        const int in_group = r / p.grid_w, X = r - in_group * p.grid_w;
+        const int r = q * 32 + lane;  // this thread's row of every tile
+        const int Rl = (int)__umulhi((unsigned)r, p.ws_magic), X = r - Rl * Ws;
         const int sh = p.out_s2d_log2, smask = (1 << sh) - 1;
-        const bool row_ok = in_group < p.images && X < p.out_w;
+        const bool row_ok = r < S * Ws && X < p.out_w;
         const int x_off = (X >> sh) * p.out_pitch + (X & smask) * p.n_total;
         const float s_out = p.s_out, inv_s_out = p.inv_s_out;
         asm volatile("griddepcontrol.wait;" ::: "memory");  // the output may reuse a buffer an earlier launch reads
         bool ok = true;
-        int Y = y0 + wg, group = group0;
-        for (int seq = wg; seq < n_lines && ok; seq += kGroups, Y += kGroups) {  // every fourth line of the CTA
-            while (Y >= out_h) Y -= out_h, ++group;
-            const int slot = seq % kAccSlots;
-            ok = mbar_wait(acc_full0 + 8 * slot, (uint32_t)((seq / kAccSlots) & 1), abort_flag, p.status, 16);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(slot * NCOLS);
-            const int n = group * p.images + in_group;
-            const bool valid = row_ok && n < p.batch;
-            int8_t *dst = p.out + (size_t)((unsigned)n * (unsigned)p.out_rows_per_image + (unsigned)((Y >> sh) * p.out_grid_w)) *
-                                      (size_t)p.out_pitch +
-                          (((Y & smask) << sh) * p.n_total + x_off);
-            constexpr int kHalves = (NCOLS + 31) / 32;  // 32 columns at a time
+        // warpgroup wg takes the CTA's tiles wg, wg + kGroups, ... (seq: the CTA's tiles in order;
+        // T is 1, 2 or 4)
+        const int t_log2 = T == 4 ? 2 : (T == 2 ? 1 : 0);
+        for (int seq = wg; ok; seq += kGroups) {
+            {
+                const int k = seq >> t_log2, i = seq & (T - 1);
+                if (k >= my_steps) break;
+                const int tile = ((int)blockIdx.x + k * (int)gridDim.x) * T + i;
+                if (tile >= p.total_tiles) break;  // only the last step is short, and later tiles lie behind it
+                const int slot = seq % kAccSlots;
+                ok = mbar_wait(acc_full0 + 8 * slot, (uint32_t)((seq / kAccSlots) & 1), abort_flag, p.status, 16);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(slot * kSlotCols);
+                const unsigned R = (unsigned)(tile * S + Rl);
+                const unsigned n = __umulhi(R, p.hs_magic);
+                const int Y = (int)(R - n * (unsigned)Hs);
+                const bool valid = row_ok && Y < p.out_h && (int)n < p.batch;
+                int8_t *dst = p.out + (size_t)(n * (unsigned)p.out_rows_per_image + (unsigned)((Y >> sh) * p.out_grid_w)) *
+                                          (size_t)p.out_pitch +
+                              (((Y & smask) << sh) * p.n_total + x_off);
+                constexpr int kHalves = (NCOLS + 31) / 32;  // 32 columns at a time
 #pragma unroll
-            for (int hh = 0; hh < kHalves; ++hh) {
-                constexpr int kPieces = NCOLS >= 32 ? 2 : 1;
-                int acc[kPieces][16];
+                for (int hh = 0; hh < kHalves; ++hh) {
+                    constexpr int kPieces = NCOLS >= 32 ? 2 : 1;
+                    int acc[kPieces][16];
 #pragma unroll
-                for (int h = 0; h < kPieces; ++h) tmem_ld16(taddr + 32 * hh + 16 * h, acc[h]);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (hh == kHalves - 1) {  // the last read of the accumulator: hand it back
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(acc_empty0 + 8 * slot);
-                }
-                uint32_t wq[kPieces][4];
-#pragma unroll
-                for (int h = 0; h < kPieces; ++h) {
-                    if (32 * hh + 16 * h >= NCOLS) continue;
-                    float ks[16], bs[16];
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {  // kernel parameters: 16-byte reads from the constant bank
-                        const float4 kv = *reinterpret_cast<const float4 *>(&p.ks[32 * hh + 16 * h + 4 * g]);
-                        const float4 bv = *reinterpret_cast<const float4 *>(&p.bs[32 * hh + 16 * h + 4 * g]);
-                        ks[4 * g] = kv.x; ks[4 * g + 1] = kv.y; ks[4 * g + 2] = kv.z; ks[4 * g + 3] = kv.w;
-                        bs[4 * g] = bv.x; bs[4 * g + 1] = bv.y; bs[4 * g + 2] = bv.z; bs[4 * g + 3] = bv.w;
+                    for (int h = 0; h < kPieces; ++h) tmem_ld16(taddr + 32 * hh + 16 * h, acc[h]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (hh == kHalves - 1) {  // the last read of the accumulator: hand it back
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(acc_empty0 + 8 * slot);
                     }
-                    uint32_t (&wv)[4] = wq[h];
-                    if (AFFINE) {
-                        if (p.relu) requant16_affine<true>(acc[h], ks, bs, wv);
-                        else requant16_affine<false>(acc[h], ks, bs, wv);
-                    } else {
-                        if (p.relu) requant16_fastdiv<true>(acc[h], ks, bs, s_out, inv_s_out, wv);
-                        else requant16_fastdiv<false>(acc[h], ks, bs, s_out, inv_s_out, wv);
-                    }
-                }
-                if (valid) {  // 32 channels in one store where the channel count is a multiple of 32
-                    if constexpr (NCOLS % 32 == 0) {  // positions are then 32-byte aligned
-                        stg32(dst + 32 * hh, wq[0], wq[1]);
-                    } else {
+                    uint32_t wq[kPieces][4];
 #pragma unroll
-                        for (int h = 0; h < kPieces; ++h)
-                            if (32 * hh + 16 * h < NCOLS)
-                                *reinterpret_cast<uint4 *>(dst + 32 * hh + 16 * h) =
-                                    make_uint4(wq[h][0], wq[h][1], wq[h][2], wq[h][3]);
+                    for (int h = 0; h < kPieces; ++h) {
+                        if (32 * hh + 16 * h >= NCOLS) continue;
+                        float ks[16], bs[16];
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {  // kernel parameters: 16-byte reads from the constant bank
+                            const float4 kv = *reinterpret_cast<const float4 *>(&p.ks[32 * hh + 16 * h + 4 * g]);
+                            const float4 bv = *reinterpret_cast<const float4 *>(&p.bs[32 * hh + 16 * h + 4 * g]);
+                            ks[4 * g] = kv.x; ks[4 * g + 1] = kv.y; ks[4 * g + 2] = kv.z; ks[4 * g + 3] = kv.w;
+                            bs[4 * g] = bv.x; bs[4 * g + 1] = bv.y; bs[4 * g + 2] = bv.z; bs[4 * g + 3] = bv.w;
+                        }
+                        uint32_t (&wv)[4] = wq[h];
+                        if (AFFINE) {
+                            if (p.relu) requant16_affine<true>(acc[h], ks, bs, wv);
+                            else requant16_affine<false>(acc[h], ks, bs, wv);
+                        } else {
+                            if (p.relu) requant16_fastdiv<true>(acc[h], ks, bs, s_out, inv_s_out, wv);
+                            else requant16_fastdiv<false>(acc[h], ks, bs, s_out, inv_s_out, wv);
+                        }
+                    }
+                    if (valid) {  // 32 channels in one store where the channel count is a multiple of 32
+                        if constexpr (NCOLS % 32 == 0) {  // positions are then 32-byte aligned
+                            stg32(dst + 32 * hh, wq[0], wq[1]);
+                        } else {
+#pragma unroll
+                            for (int h = 0; h < kPieces; ++h)
+                                if (32 * hh + 16 * h < NCOLS)
+                                    *reinterpret_cast<uint4 *>(dst + 32 * hh + 16 * h) =
+                                        make_uint4(wq[h][0], wq[h][1], wq[h][2], wq[h][3]);
+                        }
                     }
                 }
             }
@@ -297,7 +276,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == kMmaWarp2) {
+    if (warp == 0) {
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u)
                      : "memory");
@@ -308,10 +287,43 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // host side
 // ---------------------------------------------------------------------------------------
 
-size_t conv_rows_smem_bytes(const ConvRowsParams &q)
+static bool magic_exact2(unsigned d, unsigned long long max_x, unsigned *magic)
 {
+    const unsigned long long m = ((1ULL << 32) + d - 1) / d;
+    if (m >= (1ULL << 32)) return false;
+    *magic = (unsigned)m;
+    const unsigned long long e = m * d - (1ULL << 32);  // umulhi(x, m) = x / d while x * e < 2^32
+    return e == 0 || max_x < (1ULL << 32) / e;
+}
+
+static int rows_needed(const ConvRowsParams &q, int T)
+{
+    // grid positions a step's MMAs can touch: the last tile reads 128 rows plus the taps' reach
+    return (T - 1) * q.rows_per_tile * q.grid_w + 128 + (q.taps - 1) * q.grid_w + (q.taps - 1);
+}
+
+static void conv_rows_shape(ConvRowsParams &q, int T)
+{
+    q.tiles_per_step = T;
+    q.boxes_per_stage = (rows_needed(q, T) + q.box_rows - 1) / q.box_rows;
+    q.stage_bytes = (int)(((size_t)q.boxes_per_stage * q.box_rows * q.row_bytes + 1023) & ~(size_t)1023);
+}
+
+// TMA boxes of a step's operand block: as few as the 256-row limit of a box allows, equal in size
+// (a multiple of the eight rows of a swizzle atom), sized for max_tiles_per_step
+static void conv_rows_box(ConvRowsParams &q)
+{
+    const int rows = rows_needed(q, q.max_tiles_per_step);
+    const int boxes = (rows + 255) / 256;
+    q.box_rows = (((rows + boxes - 1) / boxes) + 7) & ~7;
+}
+
+size_t conv_rows_smem_bytes(const ConvRowsParams &q0)
+{
+    ConvRowsParams q = q0;
+    conv_rows_shape(q, q.max_tiles_per_step);
     const size_t b_bytes = (((size_t)q.taps * q.taps * q.n_cols * q.row_bytes) + 1023) & ~(size_t)1023;
-    return 1024 + b_bytes + (size_t)q.n_stages * q.stage_bytes;
+    return 1024 + b_bytes + (size_t)kStages2 * q.stage_bytes;
 }
 
 // Does the kernel serve a conv with `taps` x `taps` stride-1 taps on a grid_h x grid_w grid of
@@ -322,21 +334,25 @@ bool conv_rows_plan(int grid_h, int grid_w, int row_bytes, int taps, int n_total
     if ((row_bytes != 32 && row_bytes != 64 && row_bytes != 128) || taps < 1 || taps > 4 || n_total % 16 ||
         n_total < 16 || n_total > 64 || grid_w < taps || grid_h < taps || grid_w > 64)
         return false;
-    const int images = 128 / grid_w;
-    if (images * grid_w < 108) return false;  // too many idle rows per tile
-    if (max_batch * grid_h * grid_w + 512 >= (1LL << 31)) return false;
+    const int S = 128 / grid_w;
+    if (S * grid_w < 108) return false;  // too many idle rows per tile
+    const long long rows = max_batch * grid_h;
+    if (rows * grid_w + 512 >= (1LL << 31)) return false;
     memset(q, 0, sizeof(*q));
+    if (!magic_exact2((unsigned)grid_w, 256, &q->ws_magic)) return false;
+    if (!magic_exact2((unsigned)grid_h, (unsigned long long)rows + 256, &q->hs_magic)) return false;
     q->grid_h = grid_h;
     q->grid_w = grid_w;
     q->row_bytes = row_bytes;
     q->taps = taps;
-    q->images = images;
+    q->rows_per_tile = S;
     q->n_cols = n_total;
-    // a line's MMAs read 128 rows from each horizontal tap on
-    q->stage_bytes = (((128 + taps - 1) * row_bytes) + 1023) & ~1023;
-    // stages (input lines): a line takes some 0.3 us, the way from memory under load some 2 us
-    for (q->n_stages = kMaxStages2; q->n_stages >= 4; --q->n_stages)
-        if (conv_rows_smem_bytes(*q) <= 216 * 1024) return true;
+    // tiles per step: as many (up to 4) as leave kStages2 operand blocks beside the weights
+    for (int T = 4; T >= 1; T /= 2) {
+        q->max_tiles_per_step = T;
+        conv_rows_box(*q);
+        if (conv_rows_smem_bytes(*q) <= 200 * 1024) return true;
+    }
     return false;
 }
 
@@ -345,9 +361,14 @@ cudaError_t conv_rows_launch(const void *map_a, const void *map_b, const ConvRow
 {
     ConvRowsParams q = q0;
     q.batch = batch;
-    q.total_lines = (batch + q.images - 1) / q.images * q.out_h;
-    const int grid = q.total_lines < sm_count ? q.total_lines : sm_count;
-    const size_t smem = conv_rows_smem_bytes(q);
+    const long long grid_rows = (long long)batch * q.grid_h;
+    q.total_tiles = (int)((grid_rows + q.rows_per_tile - 1) / q.rows_per_tile);
+    int T = q.max_tiles_per_step;
+    while (T > 1 && (q.total_tiles + T - 1) / T < 2 * sm_count) T /= 2;
+    conv_rows_shape(q, T);
+    q.total_steps = (q.total_tiles + T - 1) / T;
+    const int grid = q.total_steps < sm_count ? q.total_steps : sm_count;
+    const size_t smem = conv_rows_smem_bytes(q0);
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = allow_smem((const void *)kernel, smem);
         if (e != cudaSuccess) return e;
@@ -365,12 +386,17 @@ cudaError_t conv_rows_launch(const void *map_a, const void *map_b, const ConvRow
     };
     cudaError_t e;
     // (the requantiser is a template parameter, not a branch: both epilogues in one kernel cost time)
-    switch (q.n_cols) {
-    case 16: e = q.affine ? go(conv_rows_kernel<16, true>) : go(conv_rows_kernel<16, false>); break;
-    case 32: e = q.affine ? go(conv_rows_kernel<32, true>) : go(conv_rows_kernel<32, false>); break;
-    case 48: e = q.affine ? go(conv_rows_kernel<48, true>) : go(conv_rows_kernel<48, false>); break;
-    default: e = q.affine ? go(conv_rows_kernel<64, true>) : go(conv_rows_kernel<64, false>);
-    }
+    if (q.n_cols == 64 && q.taps == 2 && q.row_bytes == 128)
+        e = q.affine ? go(conv_rows_kernel<64, 2, 128, true>) : go(conv_rows_kernel<64, 2, 128, false>);
+    else if (q.n_cols == 64 && q.taps == 3 && q.row_bytes == 64)
+        e = q.affine ? go(conv_rows_kernel<64, 3, 64, true>) : go(conv_rows_kernel<64, 3, 64, false>);
+    else
+        e = q.affine ? (q.n_cols == 16 ? go(conv_rows_kernel<16, 0, 0, true>)
+                        : q.n_cols == 32 ? go(conv_rows_kernel<32, 0, 0, true>)
+                        : q.n_cols == 48 ? go(conv_rows_kernel<48, 0, 0, true>) : go(conv_rows_kernel<64, 0, 0, true>))
+                     : (q.n_cols == 16 ? go(conv_rows_kernel<16, 0, 0, false>)
+                        : q.n_cols == 32 ? go(conv_rows_kernel<32, 0, 0, false>)
+                        : q.n_cols == 48 ? go(conv_rows_kernel<48, 0, 0, false>) : go(conv_rows_kernel<64, 0, 0, false>));
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

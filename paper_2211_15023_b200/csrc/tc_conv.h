@@ -11,9 +11,11 @@ struct ConvRowsParams {
     // input: space-to-depth(s) grid of grid_h x grid_w positions per image, row_bytes bytes each;
     // the conv is taps x taps stride 1 on that grid
     int batch, grid_h, grid_w, row_bytes, taps;
-    // tiling: a tile is one grid line of `images` images, a pipeline stage one such line of the input;
-    // total_lines: output lines of all groups of images
-    int images, n_stages, stage_bytes, total_lines;
+    unsigned ws_magic, hs_magic;     // ceil(2^32 / grid_w), ceil(2^32 / grid_h)
+    // tiling: a tile is rows_per_tile whole grid rows, a pipeline step tiles_per_step tiles whose
+    // operand block arrives as boxes_per_stage TMA boxes of box_rows rows
+    int rows_per_tile, max_tiles_per_step, tiles_per_step, total_tiles, total_steps;
+    int box_rows, boxes_per_stage, stage_bytes;
     int n_cols;                      // output channels: 16, 32, 48 or 64
     // output: position (n, Y, X) is stored at row n * out_rows_per_image + (Y >> s) * out_grid_w + (X >> s),
     // byte (((Y & m) << s) + (X & m)) * n_total + channel, rows out_pitch bytes apart (s = out_s2d_log2)

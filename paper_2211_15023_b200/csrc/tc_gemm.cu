@@ -885,11 +885,6 @@ static EncodeTiledFn encode_fn()
     return fn;
 }
 
-static CUtensorMapSwizzle swizzle_of(int row_bytes)
-{
-    return row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
-}
-
 // 2-D uint8 tensor [rows][row_bytes] with pitch `pitch`; box [box_rows][box_bytes], swizzled.
 accerl_status tc_make_map(void *map_out, const void *base, long long rows, int row_bytes,
                           long long pitch, int box_rows, int box_bytes)
@@ -903,35 +898,15 @@ accerl_status tc_make_map(void *map_out, const void *base, long long rows, int r
     cuuint64_t strides[1] = {(cuuint64_t)pitch};
     cuuint32_t box[2] = {(cuuint32_t)box_bytes, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
+    CUtensorMapSwizzle sw = box_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                            : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                              : CU_TENSOR_MAP_SWIZZLE_32B;
     CUresult r = fn((CUtensorMap *)map_out, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, (void *)base, dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(box_bytes),
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         set_error("cuTensorMapEncodeTiled failed (%d) for rows=%lld row_bytes=%d pitch=%lld box=%dx%d",
                   (int)r, rows, row_bytes, pitch, box_rows, box_bytes);
-        return ACCERL_ERR_CUDA;
-    }
-    return ACCERL_OK;
-}
-
-// 4-D uint8 tensor [n][grid_h][grid_w][row_bytes]; box: one grid line of `images` images, swizzled.
-accerl_status tc_make_line_map(void *map_out, const void *base, long long n, int grid_h, int grid_w, int row_bytes, int images)
-{
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) {
-        set_error("cuTensorMapEncodeTiled is not available from this driver");
-        return ACCERL_ERR_CUDA;
-    }
-    const cuuint64_t line = (cuuint64_t)row_bytes * grid_w;
-    cuuint64_t dims[4] = {(cuuint64_t)row_bytes, (cuuint64_t)grid_w, (cuuint64_t)grid_h, (cuuint64_t)n};
-    cuuint64_t strides[3] = {(cuuint64_t)row_bytes, line, line * grid_h};
-    cuuint32_t box[4] = {(cuuint32_t)row_bytes, (cuuint32_t)grid_w, 1, (cuuint32_t)images};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn((CUtensorMap *)map_out, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, (void *)base, dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(row_bytes),
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled failed (%d) for %lld x %d x %d x %d, %d images a box", (int)r, n, grid_h, grid_w, row_bytes, images);
         return ACCERL_ERR_CUDA;
     }
     return ACCERL_OK;

@@ -98,8 +98,6 @@ struct TcGemmParams {
 
 accerl_status tc_make_map(void *map_out, const void *base, long long rows, int row_bytes,
                           long long pitch, int box_rows, int box_bytes);
-// the same for a tensor [n][grid_h][grid_w][row_bytes]: boxes of one grid line of `images` images
-accerl_status tc_make_line_map(void *map_out, const void *base, long long n, int grid_h, int grid_w, int row_bytes, int images);
 bool tc_choose_pipeline(TcGemmParams &p, bool resident_b);
 size_t tc_smem_bytes(const TcGemmParams &p, bool resident_b);
 cudaError_t tc_launch(const void *map_a, const void *map_b, const TcGemmParams &p, bool resident_b,

@@ -588,10 +588,12 @@ accerl_status build_tc_plan(accerl_policy *p, const accerl_layer_desc *layers, i
                 void *w2_dev = nullptr;
                 accerl_status st2 = upload_bytes(p, packed.data(), packed.size(), &w2_dev);
                 if (st2 != ACCERL_OK) return st2;
-                cs.a_map = ActivationMap{p->bufs[L.in_buf].ptr, rows_in_per_image, row_bytes, row_bytes, 0, 0, c2.grid_w, c2.images};
-                st2 = tc_make_line_map(cs.map_a, p->bufs[L.in_buf].ptr, p->max_batch, c2.grid_h, c2.grid_w, row_bytes, c2.images);
+                cs.a_map = ActivationMap{p->bufs[L.in_buf].ptr, rows_in_per_image, row_bytes, row_bytes, c2.box_rows, row_bytes};
+                st2 = tc_make_map(cs.map_a, p->bufs[L.in_buf].ptr, (long long)p->max_batch * rows_in_per_image,
+                                  row_bytes, row_bytes, c2.box_rows, row_bytes);
                 if (st2 != ACCERL_OK) return st2;
-                st2 = tc_make_map(cs.map_b, w2_dev, (long long)g.n_chunks * n_total, row_bytes, row_bytes, n_total, 32);
+                st2 = tc_make_map(cs.map_b, w2_dev, (long long)g.n_chunks * n_total, row_bytes, row_bytes, n_total,
+                                  row_bytes);
                 if (st2 != ACCERL_OK) return st2;
                 p->conv_rows.push_back(cs);
                 Step s;
