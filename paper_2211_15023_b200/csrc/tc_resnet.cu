@@ -656,74 +656,65 @@ __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kern
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
         uint32_t rdy = 0, k3 = 0;  // parity of the layers at 20 x 20, layers done at 9 x 9
         for (; n < batch; n += step) {
-            // The layers at 20 x 20, unrolled: with everything but two bases known at compile time an instruction costs the
-            // issuing warp about three others; computed at run time (a loop over the pieces) the issue took longer than
-            // the instructions saved (726 against 674 us).
-            auto layer20 = [&](auto op_c) {
-                constexpr int op = decltype(op_c)::value, s = op & 3;
-                const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0, b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
-                // `cnt` lines' accumulators from tile `col` on, operand rows from `a_row` on, weights from vertical tap
-                // 2 - blk on downwards; `fresh`: 1 the last of them, 2 all of them are overwritten by the first instruction
-                auto piece = [&](int a_row, int col, int cnt, int blk, int fresh) {
-                    const uint32_t d = d0 + (uint32_t)col * 32, a = a_op + (uint32_t)a_row * 2, b = b_op + (uint32_t)blk * 64;
-                    const uint32_t id = idesc_for(32 * cnt);
-                    if (fresh == 1) {
-                        if (cnt > 1) mma_i8(d, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b), idesc_for(32 * (cnt - 1)), 1);
-                        mma_i8(d + (uint32_t)(cnt - 1) * 32, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b + (uint32_t)(cnt - 1) * 64), idesc_for(32), 0);
-                    } else mma_i8(d, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b), id, fresh ? 0 : 1);
+            for (int op = 0; op < kS2Ops; ++op) {
+                const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
+                if (op < 5) {
+                    const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
+                    const int s = op & 3;
+                    // `cnt` lines' accumulators from tile `col` on, operand rows from `a_row` on, weights from vertical tap
+                    // 2 - blk on downwards; `fresh`: 1 the last of them, 2 all of them are overwritten by the first instruction
+                    auto piece = [&](int a_row, int col, int cnt, int blk, int fresh) {
+                        const uint32_t d = d0 + (uint32_t)col * 32, a = a_op + (uint32_t)a_row * 2, b = b_op + (uint32_t)blk * 64;
+                        const uint32_t id = idesc_for(0) + ((uint32_t)cnt << 19);
+                        if (fresh == 1) {
+                            if (cnt > 1) mma_i8(d, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b), id - (1u << 19), 1);
+                            mma_i8(d + (uint32_t)(cnt - 1) * 32, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b + (uint32_t)(cnt - 1) * 64), idesc_for(32), 0);
+                        } else mma_i8(d, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b), id, fresh ? 0 : 1);
 #pragma unroll
-                    for (int kx = 1; kx < 3; ++kx)
-                        mma_i8(d, desc(kDescSw32Hi, a + 2 * kx), desc(kDescSw32Hi, b + 3 * 64 * kx), id, 1);
-                };
-                image_wait(ready + 8 * s, rdy, abort_flag, p.status, 8);
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {  // operand tiles s, s + 1, s + 2, s + 3, and s once more
-                    const int t = (s + k) & 3;
-                    if (k < 3) {
-                        image_wait(ready + 8 * ((t + 1) & 3), rdy, abort_flag, p.status, 8);
+                        for (int kx = 1; kx < 3; ++kx)
+                            mma_i8(d, desc(kDescSw32Hi, a + 2 * kx), desc(kDescSw32Hi, b + 3 * 64 * kx), id, 1);
+                    };
+                    image_wait(ready + 8 * s, rdy, abort_flag, p.status, 8);
+#pragma unroll 1
+                    for (int k = 0; k < 5; ++k) {  // operand tiles s, s + 1, s + 2, s + 3, and s once more
+                        const int t = (s + k) & 3;
+                        if (k < 3) image_wait(ready + 8 * ((t + 1) & 3), rdy, abort_flag, p.status, 8);
                         fence_after();
-                    }
-                    if (elect_one()) {
-                        // output lines lo .. hi relative to the interleaving: -1 is tile 3 a line up, 4 tile 0 a line down
-                        const int lo = k == 0 ? t : t - 1, hi = k == 4 ? t - 1 : t + 1, fresh = k == 0 ? 2 : k < 3 ? 1 : 0;
-                        const int u0 = lo < 0 ? 0 : lo, u1 = hi > 3 ? 3 : hi;
-                        if (lo < 0) piece(21, 3, 1, 0, 0);
-                        if (u0 <= u1) piece(res2_line(t), u0, u1 - u0 + 1, u0 - t + 1, hi > 3 && fresh == 1 ? 0 : fresh);
-                        if (hi > 3) piece(336, 0, 1, 2, fresh ? 2 : 0);
-                        // (the last two together: a warpgroup that has seen one of them has seen all four)
-                        if (k == 2 || k == 3) mma_commit(full0 + 8 * ((s + k - 1) & 3));
-                        if (k == 4) {
-                            mma_commit(full0 + 8 * ((s + 3) & 3));
-                            mma_commit(full0 + 8 * s);
+                        if (elect_one()) {
+                            // output lines lo .. hi relative to the interleaving: -1 is tile 3 a line up, 4 tile 0 a line down
+                            const int lo = k == 0 ? t : t - 1, hi = k == 4 ? t - 1 : t + 1, fresh = k == 0 ? 2 : k < 3 ? 1 : 0;
+                            const int u0 = max(lo, 0), u1 = min(hi, 3);
+                            if (lo < 0) piece(21, 3, 1, 0, 0);
+                            if (u0 <= u1) piece(res2_line(t), u0, u1 - u0 + 1, u0 - t + 1, hi > 3 && fresh == 1 ? 0 : fresh);
+                            if (hi > 3) piece(336, 0, 1, 2, fresh ? 2 : 0);
+                            // (the last two together: a warpgroup that has seen one of them has seen all four)
+                            if (k == 2 || k == 3) mma_commit(full0 + 8 * ((s + k - 1) & 3));
+                            if (k == 4) {
+                                mma_commit(full0 + 8 * ((s + 3) & 3));
+                                mma_commit(full0 + 8 * s);
+                            }
                         }
+                        __syncwarp();
+                    }
+                    if (op == 4 && n + step < batch) {  // the MMAs have read the image: the next one may land
+                        image_wait(full0 + 8 * s, rdy, abort_flag, p.status, 16);
+                        fetch(n + step);
+                    }
+                    rdy ^= 1;
+                } else {
+                    const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3;
+                    image_wait(ready + 8 * kS2Tiles, k3 & 1, abort_flag, p.status, 8);
+                    fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int j = 0; j < 9; ++j)
+                            mma_i8(d0, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
+                                   desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
+                        mma_commit(full0 + 8 * kS2Tiles);
                     }
                     __syncwarp();
+                    ++k3;
                 }
-                if (op == 4 && n + step < batch) {  // the MMAs have read the image: the next one may land
-                    image_wait(full0 + 8 * s, rdy, abort_flag, p.status, 16);
-                    fetch(n + step);
-                }
-                rdy ^= 1;
-            };
-            layer20(OpIndex<0>());
-            layer20(OpIndex<1>());
-            layer20(OpIndex<2>());
-            layer20(OpIndex<3>());
-            layer20(OpIndex<4>());
-            for (int op = 5; op < kS2Ops; ++op) {
-                const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
-                const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3;
-                image_wait(ready + 8 * kS2Tiles, k3 & 1, abort_flag, p.status, 8);
-                fence_after();
-                if (elect_one()) {
-#pragma unroll
-                    for (int j = 0; j < 9; ++j)
-                        mma_i8(d0, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
-                               desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
-                    mma_commit(full0 + 8 * kS2Tiles);
-                }
-                __syncwarp();
-                ++k3;
             }
         }
     } else {
