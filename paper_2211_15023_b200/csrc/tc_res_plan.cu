@@ -99,12 +99,10 @@ accerl_status build_res_steps(accerl_policy *p, const accerl_layer_desc *layers,
                             weight(layers[op < 4 ? 2 + op : 6], op == 5 ? 16 + oc : oc, kk % 16, j / 2, 2 * (j % 2) + kk / 16 - px);
     const int of_op[9] = {8, 9, 10, 11, 12, 14, 15, 16, 17};
     for (int op = 0; op < 9; ++op)
-        for (int j = 0; j < 9; ++j) {  // at 20 x 20 per horizontal tap the vertical taps side by side, the last one first
-            const int ky = op < 5 ? 2 - j % 3 : j / 3, kx = op < 5 ? j / 3 : j % 3;
+        for (int j = 0; j < 9; ++j)
             for (int oc = 0; oc < 32; ++oc)
                 for (int kk = 0; kk < 32; ++kk)
-                    w2[(size_t)(op * 9 + j) * 1024 + weight_at(oc, kk)] = weight(layers[of_op[op]], oc, kk, ky, kx);
-        }
+                    w2[(size_t)(op * 9 + j) * 1024 + weight_at(oc, kk)] = weight(layers[of_op[op]], oc, kk, j / 3, j % 3);
     void *d0 = nullptr, *d1 = nullptr, *d2 = nullptr;
     accerl_status st = upload_bytes(p, w0.data(), w0.size(), &d0);
     if (st == ACCERL_OK) st = upload_bytes(p, w1.data(), w1.size(), &d1);

@@ -556,8 +556,8 @@ __global__ void __launch_bounds__(S1Shape<CTX, WG>::Threads, 1) res_stack1_kerne
                 // a half of the 16 -> 32 conv is complete: 3 x 3 stride-2 max over it
                 ctx_sync<kS1T>(ctx);
                 int8_t *out = p.x2 + (size_t)n * kRes2Bytes;
-                if (tid < 63) {  // the zero pixels: in front of every line, the zero lines, behind the last line
-                    const int s = tid < 20 ? res2_line(tid) : tid < 41 ? 105 + tid - 20 : tid < 62 ? 336 + tid - 41 : kRes2Rows - 1;
+                if (tid < 62) {  // the zero pixels: lines 0 and 21, the first one of the lines between
+                    const int s = tid < 21 ? tid : tid < 42 ? 21 * 21 + tid - 21 : (tid - 41) * 21;
                     *reinterpret_cast<uint4 *>(out + row_off(s, op - 4)) = make_uint4(0, 0, 0, 0);
                 }
                 for (int i = tid; i < 400; i += kS1T) {
@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(S1Shape<CTX, WG>::Threads, 1) res_stack1_kerne
                         mx.take(u2);
                     }
                     const uint4 c = mx.result();
-                    *reinterpret_cast<uint4 *>(out + row_off(res2_line(oy) + ox + 1, op - 4)) = c;
+                    *reinterpret_cast<uint4 *>(out + row_off((oy + 1) * 21 + ox + 1, op - 4)) = c;
                     if (TAP) *reinterpret_cast<uint4 *>(p.tap_x2 + ((size_t)n * 400 + i) * 32 + 16 * (op - 4)) = c;
                 }
                 ctx_sync<kS1T>(ctx);
@@ -593,50 +593,43 @@ __global__ void __launch_bounds__(S1Shape<CTX, WG>::Threads, 1) res_stack1_kerne
 // ---------------------------------------------------------------------------------------
 // two residual blocks at 20 x 20 x 32, conv 32 -> 32, max-pool, two blocks at 9 x 9 x 32
 // ---------------------------------------------------------------------------------------
-// As above with one pixel per GEMM row, but at 20 x 20 ONE instruction serves the three vertical taps.  Tile T
-// holds the lines T, T + 4, .. T + 16 (res2_line), so that the operand tile of the lines y has the same rows as
-// the accumulators of the lines y - 1, y and y + 1: N = 3 * 32, the weights of the vertical taps side by side, the
-// four tiles' accumulators in consecutive columns.  56 cycles instead of three times 40, a third of the layer's
-// tensor time with the edges counted.  Lines next to one another at the ends of the interleaving (tile 3 above tile
-// 0) are a view of tile 3 or 0 shifted by a line.
-//
-// A layer takes its operand tiles in the order the layer before delivered them: s, s + 1, s + 2, s + 3 (mod 4),
-// and delivers s + 1, s + 2, s + 3, s.  The tile s goes to the accumulators of s and s + 1 first and to that of
-// s - 1, which is drained last, at the end; thus a tile that is ready is also a drained accumulator.
-//
-// At 9 x 9, where a layer is one tile, the two warpgroups of a context take half of the channels each and a
-// thread keeps its part of x in registers.
+// As above with one pixel per GEMM row.  At 9 x 9, where a layer is one tile, the two warpgroups of a
+// context take half of the channels each and a thread keeps its part of x in registers.
 namespace {
 constexpr int kS2Tiles = 4, kS2Ops = 9;                     // 20 * 21 GEMM rows; layers
 constexpr int kS2Buf = 18 * 1024, kS3Buf = 5 * 1024, kS2CtxBytes = 2 * kS2Buf + 2 * kS3Buf;
 template <int CTX, int WG>
 struct S2Shape {
     static constexpr int T = WG * 128, Epi = CTX * WG * 4, Threads = 32 * (Epi + CTX);
-    static constexpr int XCol = kS2Tiles * 32, Cols = XCol + 8 * kS2Tiles;  // accumulators (the first also at 9 x 9), then 8 columns of x per tile
+    static constexpr int Slots = CTX == 1 ? kS2Tiles : 3, Slot3 = Slots;     // accumulators of the tiles at 20 x 20, then one for the layers at 9 x 9
+    static constexpr int XCol = (Slots + 1) * 32, Cols = XCol + 8 * kS2Tiles;  // x: 8 columns a tile behind them
     static constexpr int Smem = 1024 + kRes2Weights + CTX * kS2CtxBytes;
-    static_assert((WG == 2 || WG == kS2Tiles) && Cols * CTX <= 512, "tiles of a warpgroup");
+    static_assert((WG == 2 || (WG == kS2Tiles && Slots == kS2Tiles)) && Slots < kMaxSlots && Cols * CTX <= 512, "tiles of a warpgroup");
 };
-static_assert((357 + 128 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kS2Tiles < kMaxTiles && kS2Tiles < kMaxSlots, "buffers");
+static_assert((kS2Tiles * 128 + 2 * 21 + 2) * 32 <= kS2Buf && (128 + 22) * 32 <= kS3Buf && kS2Tiles < kMaxTiles, "buffers");
 }  // namespace
 
 template <bool TAP, bool AFFINE, int CTX, int WG>
 __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kernel(const __grid_constant__ ResStack23Params p)
 {
     using S = S2Shape<CTX, WG>;
-    constexpr int kS2Ctx = CTX, kS2Wg = WG, kS2T = S::T, kS2Epi = S::Epi, kS2XCol = S::XCol, kS2Cols = S::Cols;
+    constexpr int kS2Ctx = CTX, kS2Wg = WG, kS2T = S::T, kS2Epi = S::Epi, kS2Slots = S::Slots, kS2Slot3 = S::Slot3, kS2XCol = S::XCol,
+                  kS2Cols = S::Cols;
     extern __shared__ __align__(1024) uint8_t res_smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)res_smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ ResBars bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *bufs = smem + kRes2Weights;
-    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kS2Ctx * kS2CtxBytes, smem, p.w, kRes2Weights, warp, 8, -1, 4, kS2Tiles);
+    const uint32_t tmem = res_setup<kS2Epi>(bars, bufs, kS2Ctx * kS2CtxBytes, smem, p.w, kRes2Weights, warp, 8, kS2Slot3, 4,
+                                            kS2Tiles);
     volatile int *abort_flag = &bars.abort_flag;
     const int step = kS2Ctx * (int)gridDim.x, batch = routed_batch(p.route, p.batch);
 
     if (warp >= kS2Epi) {
         // ------------------------------------------------------------------ MMA issuers
         const int ctx = warp - kS2Epi;
-        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]);
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]);
         const uint32_t r0 = ((smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes) >> 4) | kDescSw32Lo, h0 = r0 + (kS2Buf >> 4),
                        r3 = h0 + (kS2Buf >> 4), h3 = r3 + (kS3Buf >> 4);
         const uint32_t w0 = (smem_u32(smem) >> 4) | kDescSw32Lo, d0 = tmem + (uint32_t)ctx * kS2Cols;
@@ -654,63 +647,48 @@ __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kern
         int n = (int)blockIdx.x + ctx * (int)gridDim.x;
         if (n < batch) fetch(n);
         image_wait(smem_u32(&bars.w_ready), 0, abort_flag, p.status, 2);
-        uint32_t rdy = 0, k3 = 0;  // parity of the layers at 20 x 20, layers done at 9 x 9
+        uint32_t rdy = 0, slot = 0, phase = 0, k3 = 0;  // k3: layers done at 9 x 9
         for (; n < batch; n += step) {
             for (int op = 0; op < kS2Ops; ++op) {
                 const uint32_t b_op = w0 + (uint32_t)op * (9 * 1024 >> 4);
                 if (op < 5) {
                     const uint32_t a_op = (op == 1 || op == 3) ? h0 : r0;
-                    const int s = op & 3;
-                    // `cnt` lines' accumulators from tile `col` on, operand rows from `a_row` on, weights from vertical tap
-                    // 2 - blk on downwards; `fresh`: 1 the last of them, 2 all of them are overwritten by the first instruction
-                    auto piece = [&](int a_row, int col, int cnt, int blk, int fresh) {
-                        const uint32_t d = d0 + (uint32_t)col * 32, a = a_op + (uint32_t)a_row * 2, b = b_op + (uint32_t)blk * 64;
-                        const uint32_t id = idesc_for(0) + ((uint32_t)cnt << 19);
-                        if (fresh == 1) {
-                            if (cnt > 1) mma_i8(d, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b), id - (1u << 19), 1);
-                            mma_i8(d + (uint32_t)(cnt - 1) * 32, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b + (uint32_t)(cnt - 1) * 64), idesc_for(32), 0);
-                        } else mma_i8(d, desc(kDescSw32Hi, a), desc(kDescSw32Hi, b), id, fresh ? 0 : 1);
-#pragma unroll
-                        for (int kx = 1; kx < 3; ++kx)
-                            mma_i8(d, desc(kDescSw32Hi, a + 2 * kx), desc(kDescSw32Hi, b + 3 * 64 * kx), id, 1);
-                    };
-                    image_wait(ready + 8 * s, rdy, abort_flag, p.status, 8);
-#pragma unroll 1
-                    for (int k = 0; k < 5; ++k) {  // operand tiles s, s + 1, s + 2, s + 3, and s once more
-                        const int t = (s + k) & 3;
-                        if (k < 3) image_wait(ready + 8 * ((t + 1) & 3), rdy, abort_flag, p.status, 8);
+                    uint32_t last_full = 0, last_phase = 0;
+                    image_wait(ready, rdy, abort_flag, p.status, 8);
+                    for (int t = 0; t < kS2Tiles; ++t) {
+                        // a tile's taps reach 44 rows past it: it needs the operand tile after it too, not the whole layer
+                        if (t + 1 < kS2Tiles) image_wait(ready + 8 * (t + 1), rdy, abort_flag, p.status, 8);
+                        image_wait(empty0 + 8 * slot, phase ^ 1, abort_flag, p.status, 4);
                         fence_after();
                         if (elect_one()) {
-                            // output lines lo .. hi relative to the interleaving: -1 is tile 3 a line up, 4 tile 0 a line down
-                            const int lo = k == 0 ? t : t - 1, hi = k == 4 ? t - 1 : t + 1, fresh = k == 0 ? 2 : k < 3 ? 1 : 0;
-                            const int u0 = max(lo, 0), u1 = min(hi, 3);
-                            if (lo < 0) piece(21, 3, 1, 0, 0);
-                            if (u0 <= u1) piece(res2_line(t), u0, u1 - u0 + 1, u0 - t + 1, hi > 3 && fresh == 1 ? 0 : fresh);
-                            if (hi > 3) piece(336, 0, 1, 2, fresh ? 2 : 0);
-                            // (the last two together: a warpgroup that has seen one of them has seen all four)
-                            if (k == 2 || k == 3) mma_commit(full0 + 8 * ((s + k - 1) & 3));
-                            if (k == 4) {
-                                mma_commit(full0 + 8 * ((s + 3) & 3));
-                                mma_commit(full0 + 8 * s);
-                            }
+                            const uint32_t a = a_op + (uint32_t)t * (128 * 2);
+#pragma unroll
+                            for (int j = 0; j < 9; ++j)
+                                mma_i8(d0 + slot * 32, desc(kDescSw32Hi, a + (uint32_t)((j / 3) * 21 + j % 3) * 2),
+                                       desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
+                            mma_commit(full0 + 8 * slot);
                         }
                         __syncwarp();
-                    }
-                    if (op == 4 && n + step < batch) {  // the MMAs have read the image: the next one may land
-                        image_wait(full0 + 8 * s, rdy, abort_flag, p.status, 16);
-                        fetch(n + step);
+                        last_full = full0 + 8 * slot;
+                        last_phase = phase;
+                        if (++slot == kS2Slots) slot = 0, phase ^= 1;
                     }
                     rdy ^= 1;
+                    if (op == 4 && n + step < batch) {  // the MMAs have read the image: the next one may land
+                        image_wait(last_full, last_phase, abort_flag, p.status, 16);
+                        fetch(n + step);
+                    }
                 } else {
                     const uint32_t a_op = (op == 6 || op == 8) ? h3 : r3;
                     image_wait(ready + 8 * kS2Tiles, k3 & 1, abort_flag, p.status, 8);
+                    image_wait(empty0 + 8 * kS2Slot3, (k3 & 1) ^ 1, abort_flag, p.status, 4);
                     fence_after();
                     if (elect_one()) {
 #pragma unroll
                         for (int j = 0; j < 9; ++j)
-                            mma_i8(d0, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
+                            mma_i8(d0 + kS2Slot3 * 32, desc(kDescSw32Hi, a_op + (uint32_t)((j / 3) * 10 + j % 3) * 2),
                                    desc(kDescSw32Hi, b_op + (uint32_t)j * 64), idesc_for(32), (uint32_t)j);
-                        mma_commit(full0 + 8 * kS2Tiles);
+                        mma_commit(full0 + 8 * kS2Slot3);
                     }
                     __syncwarp();
                     ++k3;
@@ -722,35 +700,31 @@ __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kern
         const int ctx = warp / (kS2Wg * 4), wg = (warp >> 2) % kS2Wg, q = warp & 3;
         const uint32_t rbuf = smem_u32(bufs) + (uint32_t)ctx * kS2CtxBytes, hbuf = rbuf + kS2Buf, r3buf = hbuf + kS2Buf,
                        h3buf = r3buf + kS3Buf;
-        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
+        const uint32_t ready = smem_u32(&bars.ready[ctx][0]), full0 = smem_u32(&bars.acc_full[ctx][0]),
+                       empty0 = smem_u32(&bars.acc_empty[ctx][0]), land_bar = smem_u32(&bars.land[ctx]);
         const uint32_t tctx = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ctx * kS2Cols);
-        // tile t at 20 x 20, or (kS2Tiles) a warp's part at 9 x 9: written for the next layer, its accumulator drained
-        auto operand_done = [&](int t) {
+        auto operand_done = [&](int t) {  // tile t at 20 x 20, or (kS2Tiles) a warp's part at 9 x 9
             fence_async();
-            fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(ready + 8 * t);
         };
         const int row = q * 32 + lane;
-        const int line5 = row / 21;                        // this thread's row of a tile is in its line 4 * line5 + tile
-        const bool v = row < 105 && row - 21 * line5 < 20;  // and a pixel
-        // a warpgroup's tiles: of two, every other one in the order a layer delivers them (x's tiles stay with it:
-        // the image's and those of the layers 1 and 3); of four, one
-        auto first_tile = [&](int s) { return kS2Wg == 2 ? s + wg : wg; };
+        uint32_t inside = 0;  // bit t: row 128 t + row is a pixel of the 20 x 20 image
+        for (int t = 0; t < kS2Tiles; ++t)
+            if ((t * 128 + row) % 21 < 20 && t * 128 + row < 420) inside |= 1u << t;
+        const uint32_t off2 = row_off(row + 22, 0);  // first half of the row of tile 0; the other half: ^ 16, tile t: + 4096 t
         const int Y3 = row / 10, X3 = row - Y3 * 10;
         const bool v3 = Y3 < 9 && X3 < 9;
         const uint32_t off3 = row_off(row + 11, wg);
-        uint32_t full_phase = 0, k3 = 0, it = 0;
+        uint32_t seq0 = 0, k3 = 0, it = 0;
         for (int n = (int)blockIdx.x + ctx * (int)gridDim.x; n < batch; n += step, ++it) {
             image_wait(land_bar, it & 1, abort_flag, p.status, 1);
-            for (int k = first_tile(0); k < kS2Tiles; k += kS2Wg) {
-                const int t = k & 3;
-                const uint32_t off = row_off(res2_line(t) + row + 1, 0);
+            for (int t = wg; t < kS2Tiles; t += kS2Wg) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const uint32_t at = rbuf + (off ^ (16 * h));
+                    const uint32_t at = rbuf + (off2 ^ (16 * h)) + t * 4096;
                     uint4 x = make_uint4(0, 0, 0, 0);
-                    if (v) {
+                    if ((inside >> t) & 1) {
                         x = lds16(at);
                         sts16(at, relu16(x));
                     }
@@ -764,34 +738,38 @@ __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kern
                 constexpr bool skip = op == 1 || op == 3;
                 const ResLayer &L = p.layer[op];
                 const uint32_t dst = skip ? rbuf : hbuf;
-                constexpr int s = (op + 1) & 3;  // delivered first
-                for (int k = first_tile(s); k < s + kS2Tiles && (kS2Wg == 2 || k < kS2Tiles); k += kS2Wg) {
-                    const int t = k & 3;
-                    const uint32_t off = row_off(res2_line(t) + row + 1, 0);
-                    image_wait(full0 + 8 * t, full_phase, abort_flag, p.status, 16);
+                for (int t = wg; t < kS2Tiles; t += kS2Wg) {
+                    const uint32_t seq = seq0 + (uint32_t)t, slot = seq % kS2Slots;
+                    const bool v = (inside >> t) & 1;
+                    image_wait(full0 + 8 * slot, (seq / kS2Slots) & 1, abort_flag, p.status, 16);
                     fence_after();
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         int a[16];
                         uint4 x = make_uint4(0, 0, 0, 0);
-                        tmem_ld16(tctx + t * 32 + 16 * h, a);
+                        tmem_ld16(tctx + slot * 32 + 16 * h, a);
                         if (skip) x = tmem_ld4(tctx + kS2XCol + 8 * t + 4 * h);
                         tmem_wait_ld();
+                        if (h == 1) {
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                        }
                         if (skip) add_skip(a, x, L, 16 * h);
                         uint4 c = requant_res<AFFINE, op == 0 || op == 2>(a, L, 16 * h);
                         if (TAP && v) {
-                            const int Y = 4 * line5 + t, X = row - 21 * line5;
+                            const int m = t * 128 + row, Y = m / 21, X = m - Y * 21;
                             *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 20 + Y) * 20 + X) * 32 + 16 * h) = c;
                         }
                         if (op == 1) {  // the next block's x; its first conv reads ReLU(x)
                             tmem_st4(tctx + kS2XCol + 8 * t + 4 * h, c);
                             c = relu16(c);
                         }
-                        if (v) sts16(dst + (off ^ (16 * h)), c);
+                        if (v) sts16(dst + (off2 ^ (16 * h)) + t * 4096, c);
                     }
                     if (op < 4) operand_done(t);
                 }
-                full_phase ^= 1;
+                seq0 += kS2Tiles;
                 if (op == 1) tmem_wait_st();
             };
             layer20(OpIndex<0>());
@@ -804,13 +782,11 @@ __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kern
             if (wg >= 2) continue;  // (two warpgroups do the layers at 9 x 9)
             uint4 x = make_uint4(0, 0, 0, 0);
             if (v3) {
+                const int R = (2 * Y3 + 1) * 21 + 2 * X3 + 1;
                 ByteMax mx;
+                mx.first(lds16(hbuf + row_off(R, wg)));
 #pragma unroll
-                for (int j = 0; j < 9; ++j) {
-                    const uint4 u = lds16(hbuf + row_off(res2_line(2 * Y3 + j / 3) + 2 * X3 + 1 + j % 3, wg));
-                    if (j == 0) mx.first(u);
-                    else mx.take(u);
-                }
+                for (int j = 1; j < 9; ++j) mx.take(lds16(hbuf + row_off(R + (j / 3) * 21 + j % 3, wg)));
                 x = mx.result();
                 sts16(r3buf + off3, relu16(x));
                 if (TAP) *reinterpret_cast<uint4 *>(p.tap_x3 + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * wg) = x;
@@ -820,11 +796,14 @@ __global__ void __launch_bounds__(S2Shape<CTX, WG>::Threads, 1) res_stack23_kern
                 constexpr int op = decltype(op_c)::value, half = decltype(half_c)::value;
                 constexpr bool skip = op == 6 || op == 8;
                 const ResLayer &L = p.layer[op];
-                image_wait(full0 + 8 * kS2Tiles, k3 & 1, abort_flag, p.status, 16);
+                image_wait(full0 + 8 * kS2Slot3, k3 & 1, abort_flag, p.status, 16);
                 fence_after();
                 int a[16];
-                tmem_ld16(tctx + 16 * half, a);
+                tmem_ld16(tctx + kS2Slot3 * 32 + 16 * half, a);
                 tmem_wait_ld();
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + 8 * kS2Slot3);
                 if (skip) add_skip(a, x, L, 16 * half);
                 uint4 c = requant_res<AFFINE, op == 5 || op == 7>(a, L, 16 * half);
                 if (TAP && v3 && op < 8) *reinterpret_cast<uint4 *>(p.tap[op] + (((size_t)n * 9 + Y3) * 9 + X3) * 32 + 16 * half) = c;

@@ -17,12 +17,8 @@ struct ResLayer {
 
 // Geometry: 84 x 84 frames, stacks of 41 x 41 x 16, 20 x 20 x 32 and 9 x 9 x 32.  Every tensor is a
 // sequence of 32-byte rows (the operand rows of the MMAs), image lines W + 1 pixels apart: the zero
-// pixel in front of a line is also the one behind the line before it.  Zero lines above and below.
-constexpr int kRes1Rows = 43 * 21, kRes2Rows = 463;            // stored rows of an image
-// The 20 x 20 x 32 tensor is stored interleaved: the lines y = T, T + 4, .. T + 16 behind one another as tile T, a zero
-// line behind tile 0 and in front of tile 3.  Row of the zero pixel in front of line y (or tile y's first row):
-__host__ __device__ constexpr int res2_line(int y) { return (y & 3) * 105 + ((y & 3) > 0 ? 21 : 0) + ((y & 3) > 2 ? 21 : 0) + (y >> 2) * 21; }
-static_assert(res2_line(19) + 22 == kRes2Rows, "the zero pixel behind the last line is the last row");
+// pixel in front of a line is also the one behind the line before it.  One zero line above and below.
+constexpr int kRes1Rows = 43 * 21, kRes2Rows = 22 * 21;        // stored rows of an image
 constexpr int kRes1Bytes = kRes1Rows * 32, kRes2Bytes = kRes2Rows * 32;
 constexpr int kRes3Bytes = 81 * 32;                            // plain, the fc layer's input row
 constexpr int kResFirstWeights = 3 * 80 * 32;                  // first conv: 3 K steps of 80 columns
