@@ -90,8 +90,19 @@ struct ConvArgs {
     int H, W, C4, OH, OW, KH, KW, stride, pad, oc_pad, out_cp;
     float s_out;
     int relu_in, relu_out;
+    int *acc;             // ACC: [px][out_cp] accumulators instead of codes,
+    float *ymax;          // and the largest |y| of the layer
 };
 
+// largest value of a block into *out (values >= 0: their bit patterns order like the values)
+__device__ __forceinline__ void block_max_to(float v, float *out)
+{
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(reinterpret_cast<unsigned *>(out), m);
+}
+
+// ACC: for calibration, which needs the largest epilogue value before it can requantise
+template <bool ACC>
 __global__ void __launch_bounds__(128) conv_dp4a_kernel(ConvArgs a)
 {
     extern __shared__ int32_t s_w[];  // [tap][C4][16] for this block's channel group
@@ -103,7 +114,10 @@ __global__ void __launch_bounds__(128) conv_dp4a_kernel(ConvArgs a)
     }
     __syncthreads();
     long long px = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (px >= a.total_px) return;
+    if (!ACC && px >= a.total_px) return;
+    const bool live = px < a.total_px;  // (with ACC the whole warp takes part in the maximum)
+    if (!live) px = 0;
+    float ymax = 0.f;
     int ox = (int)(px % a.OW);
     long long t = px / a.OW;
     int oy = (int)(t % a.OH);
@@ -146,6 +160,15 @@ __global__ void __launch_bounds__(128) conv_dp4a_kernel(ConvArgs a)
                 for (int b = 0; b < 4; ++b)
                     acc[4 * j + b] += a.skip_mul[oc + b] * (int)(int8_t)(sv >> (8 * b));
             }
+            if (ACC) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    ymax = fmaxf(ymax, fabsf(epilogue_float(acc[4 * j + b], a.kscale[oc + b], a.bias[oc + b], a.relu_out)));
+                if (live)
+                    *reinterpret_cast<int4 *>(a.acc + px * a.out_cp + oc) =
+                        make_int4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+                continue;
+            }
             uint32_t word = 0;
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
@@ -156,10 +179,11 @@ __global__ void __launch_bounds__(128) conv_dp4a_kernel(ConvArgs a)
             reinterpret_cast<uint32_t *>(a.out)[px * out_c4 + oc / 4] = word;
         }
     }
+    if (ACC) block_max_to(live ? ymax : 0.f, a.ymax);
 }
 
-cudaError_t launch_conv_generic(const LayerPlan &L, const int8_t *in, const int8_t *skip,
-                                int8_t *out, int B, cudaStream_t st)
+static cudaError_t launch_conv(const LayerPlan &L, const int8_t *in, const int8_t *skip, int8_t *out, int *acc,
+                               float *ymax, int B, cudaStream_t st)
 {
     ConvArgs a;
     a.in = (const int32_t *)in;
@@ -176,14 +200,31 @@ cudaError_t launch_conv_generic(const LayerPlan &L, const int8_t *in, const int8
     a.s_out = L.s_out;
     a.relu_in = (L.flags & ACCERL_RELU_IN) != 0;
     a.relu_out = (L.flags & ACCERL_RELU_OUT) != 0;
+    a.acc = acc;
+    a.ymax = ymax;
     const size_t smem = (size_t)L.kh * L.kw * a.C4 * 16 * sizeof(int32_t);
-    if (smem > 48 * 1024) {
-        cudaError_t e = allow_smem((const void *)conv_dp4a_kernel, smem);
-        if (e != cudaSuccess) return e;
-    }
-    dim3 grid((unsigned)((a.total_px + 127) / 128), L.oc_pad / 16);
-    conv_dp4a_kernel<<<grid, 128, smem, st>>>(a);
-    return cudaGetLastError();
+    auto go = [&](auto kernel) -> cudaError_t {
+        if (smem > 48 * 1024) {
+            cudaError_t e = allow_smem((const void *)kernel, smem);
+            if (e != cudaSuccess) return e;
+        }
+        dim3 grid((unsigned)((a.total_px + 127) / 128), L.oc_pad / 16);
+        kernel<<<grid, 128, smem, st>>>(a);
+        return cudaGetLastError();
+    };
+    return acc ? go(conv_dp4a_kernel<true>) : go(conv_dp4a_kernel<false>);
+}
+
+cudaError_t launch_conv_generic(const LayerPlan &L, const int8_t *in, const int8_t *skip,
+                                int8_t *out, int B, cudaStream_t st)
+{
+    return launch_conv(L, in, skip, out, nullptr, nullptr, B, st);
+}
+
+cudaError_t launch_conv_acc(const LayerPlan &L, const int8_t *in, const int8_t *skip, int *acc, float *ymax, int B,
+                            cudaStream_t st)
+{
+    return launch_conv(L, in, skip, nullptr, acc, ymax, B, st);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -199,8 +240,11 @@ struct FcArgs {
     int B, K4, oc_pad, out_cp, out_c;
     float s_out;
     int relu_in, relu_out;
+    int *acc;           // ACC: [B][out_cp] accumulators and the largest |y|
+    float *ymax;
 };
 
+template <bool ACC>
 __global__ void __launch_bounds__(256) fc_dp4a_kernel(FcArgs a)
 {
     constexpr int BM = 64, BN = 64, BK = 16;
@@ -240,6 +284,21 @@ __global__ void __launch_bounds__(256) fc_dp4a_kernel(FcArgs a)
         __syncthreads();
     }
     const int oc = col0 + tx * 4;
+    if (ACC) {
+        float ymax = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = row0 + ty * 4 + i;
+            if (row >= a.B || oc >= a.out_cp) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                ymax = fmaxf(ymax, fabsf(epilogue_float(acc[i][j], a.kscale[oc + j], a.bias[oc + j], a.relu_out)));
+            *reinterpret_cast<int4 *>(a.acc + (long long)row * a.out_cp + oc) =
+                make_int4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        }
+        block_max_to(ymax, a.ymax);
+        return;
+    }
     if (oc >= a.oc_pad) return;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -260,8 +319,8 @@ __global__ void __launch_bounds__(256) fc_dp4a_kernel(FcArgs a)
     }
 }
 
-cudaError_t launch_fc_generic(const LayerPlan &L, const int8_t *in, int8_t *out, float *logits,
-                              int B, cudaStream_t st)
+static cudaError_t launch_fc(const LayerPlan &L, const int8_t *in, int8_t *out, float *logits, int *acc, float *ymax,
+                             int B, cudaStream_t st)
 {
     FcArgs a;
     a.in = (const int32_t *)in;
@@ -276,9 +335,23 @@ cudaError_t launch_fc_generic(const LayerPlan &L, const int8_t *in, int8_t *out,
     a.s_out = L.s_out;
     a.relu_in = (L.flags & ACCERL_RELU_IN) != 0;
     a.relu_out = (L.flags & ACCERL_RELU_OUT) != 0;
+    a.acc = acc;
+    a.ymax = ymax;
     dim3 grid((B + 63) / 64, (L.oc_pad + 63) / 64);
-    fc_dp4a_kernel<<<grid, 256, 0, st>>>(a);
+    if (acc) fc_dp4a_kernel<true><<<grid, 256, 0, st>>>(a);
+    else fc_dp4a_kernel<false><<<grid, 256, 0, st>>>(a);
     return cudaGetLastError();
+}
+
+cudaError_t launch_fc_generic(const LayerPlan &L, const int8_t *in, int8_t *out, float *logits,
+                              int B, cudaStream_t st)
+{
+    return launch_fc(L, in, out, logits, nullptr, nullptr, B, st);
+}
+
+cudaError_t launch_fc_acc(const LayerPlan &L, const int8_t *in, int *acc, float *ymax, int B, cudaStream_t st)
+{
+    return launch_fc(L, in, nullptr, nullptr, acc, ymax, B, st);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -320,8 +320,11 @@ cudaError_t launch_conv_generic(const LayerPlan &L, const int8_t *in, const int8
                                 int8_t *out, int B, cudaStream_t st);
 cudaError_t launch_fc_generic(const LayerPlan &L, const int8_t *in, int8_t *out, float *logits,
                               int B, cudaStream_t st);
-// calibration of a layer (calib.cu): the largest |y| into *ymax, which must hold 0, then its codes at that scale
-cudaError_t launch_calib_layer(const LayerPlan &L, const int8_t *in, const int8_t *skip, int8_t *out, float *ymax, int B, cudaStream_t st);
+// the same contractions for calibration: int32 accumulators [positions][out_cp] (residual added) and the
+// largest |y| of the layer, atomically into *ymax
+cudaError_t launch_conv_acc(const LayerPlan &L, const int8_t *in, const int8_t *skip, int *acc, float *ymax, int B,
+                            cudaStream_t st);
+cudaError_t launch_fc_acc(const LayerPlan &L, const int8_t *in, int *acc, float *ymax, int B, cudaStream_t st);
 cudaError_t launch_maxpool_generic(const LayerPlan &L, const int8_t *in, int8_t *out, int B,
                                    cudaStream_t st);
 cudaError_t launch_sample(const float *z, int pitch, const float *u, int B, int A, float *logits_out,

@@ -7,8 +7,8 @@
 // multipliers of the residual adds -- and then builds the handle with accerl_policy_create.
 //
 // The Compressor runs this for every policy it hands over, so it is a path of its own: one block of
-// device memory, every layer run twice on warp-level int8 instructions (calib.cu: the maximum of the epilogue
-// value, then the codes), and no host round trip between the layers -- scales, epilogue constants and
+// device memory, the contractions on the dp4a kernels (NHWC words) with the maximum of the epilogue
+// value taken as they go, and no host round trip between the layers -- scales, epilogue constants and
 // residual multipliers are computed where the maxima lie.  Every result is order-independent (integer
 // sums, maxima), so the scales and codes are the same bits whatever the launch shape.  (One thread per
 // output walking NCHW bytes, an atomic maximum per element and ten blocking copies a layer took 44 ms
@@ -153,6 +153,21 @@ __global__ void layer_scales_kernel(const float *s_w, int oc, const float *ymax_
     if (ymax_skip) mul[c] = (int)fminf(fmaxf(rintf(__fdiv_rn(scale_of(*ymax_skip), kc)), 0.f), 32767.f);
 }
 
+// accumulators -> codes, four channels per thread
+__global__ void calib_requant_kernel(const int4 *acc, const float *k, const float *b, int relu, int c4s, long long words,
+                                     const float *ymax, uint32_t *q)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= words) return;
+    const int c = (int)(i % c4s) * 4;
+    const int4 a = acc[i];
+    const float s = scale_of(*ymax);
+    q[i] = (uint32_t)(uint8_t)requant(epilogue_float(a.x, k[c], b[c], relu), s) |
+           (uint32_t)(uint8_t)requant(epilogue_float(a.y, k[c + 1], b[c + 1], relu), s) << 8 |
+           (uint32_t)(uint8_t)requant(epilogue_float(a.z, k[c + 2], b[c + 2], relu), s) << 16 |
+           (uint32_t)(uint8_t)requant(epilogue_float(a.w, k[c + 3], b[c + 3], relu), s) << 24;
+}
+
 // one block of device memory, handed out piece by piece: sized in a first pass, filled in a second
 struct DeviceArena {
     char *base = nullptr;
@@ -263,7 +278,7 @@ static accerl_status quantise_and_create(accerl_policy **out, int32_t in_kind,
     const long long in_elems = (long long)in_shape[0] * in_shape[1] * in_shape[2] * B;
     const bool u8 = in_kind == ACCERL_IN_U8_NCHW;
     struct Layer {
-        LayerPlan L;      // the NHWC-word kernels' view of the layer
+        LayerPlan L;      // the dp4a kernels' view of the layer
         int8_t *act;      // its int8 output, NHWC
         float *w;
         int8_t *wq, *packed;
@@ -278,6 +293,7 @@ static accerl_status quantise_and_create(accerl_policy **out, int32_t in_kind,
     void *obs_dev = nullptr;
     int8_t *lut = nullptr, *act0 = nullptr;
     float *ymax = nullptr;
+    int *acc = nullptr;
     char *results = nullptr;  // what goes back to the host, in one piece: wq, s_w and mul of every layer, ymax
     size_t results_bytes = 0;
     for (int pass = 0; pass < 2; ++pass) {
@@ -322,10 +338,14 @@ static accerl_status quantise_and_create(accerl_policy **out, int32_t in_kind,
         obs_dev = mem.take<uint8_t>((size_t)in_elems * (u8 ? 1 : 4));
         lut = mem.take<int8_t>(256);
         act0 = mem.take<int8_t>((size_t)B * in_shape[1] * in_shape[2] * round_up(in_shape[0], 4));
+        size_t acc_elems = 0;
         for (int i = 0; i < n_layers; ++i) {
             const LayerPlan &L = net[i].L;
-            net[i].act = mem.take<int8_t>((size_t)B * L.out_h * L.out_w * L.out_cp);
+            const size_t elems = (size_t)B * L.out_h * L.out_w * L.out_cp;
+            net[i].act = mem.take<int8_t>(elems);
+            if (net[i].nw) acc_elems = std::max(acc_elems, elems);
         }
+        acc = mem.take<int>(acc_elems);
         if (pass == 0) {
             ACCERL_CUDA_TRY(device_alloc((void **)&mem.base, mem.at + 256));
             continue;
@@ -385,7 +405,13 @@ static accerl_status quantise_and_create(accerl_policy **out, int32_t in_kind,
                                                                         d.skip_from >= 0 ? ymax + net[d.skip_from].scale : nullptr, l.k, l.mul);
         ACCERL_CUDA_TRY(cudaGetLastError());
         if (d.flags & ACCERL_LOGITS) break;  // its output is not quantised
-        ACCERL_CUDA_TRY(launch_calib_layer(l.L, x, d.skip_from >= 0 ? net[d.skip_from].act : nullptr, l.act, ymax + i + 1, (int)B, 0));
+        if (d.kind == ACCERL_FC) ACCERL_CUDA_TRY(launch_fc_acc(l.L, x, acc, ymax + i + 1, (int)B, 0));
+        else
+            ACCERL_CUDA_TRY(launch_conv_acc(l.L, x, d.skip_from >= 0 ? net[d.skip_from].act : nullptr, acc, ymax + i + 1, (int)B, 0));
+        const long long words = B * l.L.out_h * l.L.out_w * (l.L.out_cp / 4);
+        calib_requant_kernel<<<blocks_for(words), 256>>>((const int4 *)acc, l.k, l.b, (d.flags & ACCERL_RELU_OUT) ? 1 : 0,
+                                                         l.L.out_cp / 4, words, ymax + i + 1, (uint32_t *)l.act);
+        ACCERL_CUDA_TRY(cudaGetLastError());
         s_in = i + 1;
     }
     // one block, kept as it comes back: copies of its parts cost their page faults again
