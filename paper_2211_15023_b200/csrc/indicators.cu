@@ -153,13 +153,16 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
 // Many rows of at most 64 actions, or few of at most 12 (see the choice in accerl_policy_kl): one thread per
 // row.  A block's rows are contiguous in memory; they pass through shared memory, by asynchronous copies that
 // are all in flight at once, so that the loads are whole lines and every thread then walks its own row, a chain
-// of two exponentials an action.  V > 0: the rows lie in shared memory as in global memory and come in 16-byte
-// copies (a fourth of the instructions, and no row and column to keep); a thread reads V = 1, 2 or 4 elements at a
-// time, the width at which rows of that many elements fall into different banks.  V = 0, for rows of a multiple of
-// eight elements or addresses that are none of 16 bytes: element by element into rows of an odd pitch.  (V-trace
-// and KL of 16 x 8192 states of 18 actions in turn: 24.6 us element by element, 22.5 us.)  A warp per row, as below, leaves 14 of 32 lanes idle at 18 actions and spends its time in shuffles; with that and a
-// one-block reduction the two launches for 131072 rows of 18 took 119 us, now 20.5.  STATS (one cluster,
-// at most kKlCluster blocks' rows a pass): the mean and the maximum come out of the same launch.
+// of two exponentials an action.  A warp per row, as below, leaves 14 of 32 lanes idle at 18 actions and spends
+// its time in shuffles; with that and a one-block reduction the two launches for 131072 rows of 18 took 119 us,
+// with this kernel 20.5 element by element and some 18 in 16-byte copies (with V-trace 24.6 and 22.5).
+//
+// V > 0: the rows lie in shared memory as in global memory and come in 16-byte copies (a fourth of the
+// instructions, and no row and column to keep); a thread reads V = 1, 2 or 4 elements at a time, the width at which
+// rows of that many elements fall into different banks.  V = 0, for rows of a multiple of eight elements or
+// addresses that are none of 16 bytes: element by element into rows of an odd pitch.
+//
+// STATS (one cluster, at most kKlCluster blocks' rows a pass): the mean and the maximum come out of the same launch.
 template <bool STATS, int V>
 __global__ void __launch_bounds__(kKlRows)
 kl_rows_kernel(const float *__restrict__ zo, const float *__restrict__ zs, int B, int A, int pitch,
