@@ -860,19 +860,19 @@ cudaError_t res_launch(K kernel, const P &p, int threads, size_t smem, int sm_co
 
 // Calls `go(TAP, AFFINE)` with both as compile-time values.  Kernels whose layers all have the single-fma pair do
 // without the division's code (half of the requantiser's instructions, and the unrolled layers exceed the
-// instruction cache); the parity taps take the general form.
-template <typename P, typename F>
-cudaError_t res_dispatch(const P &p, const ResLayer *layer, int layers, bool tap, F go)
+// instruction cache), with and without parity taps.
+template <typename F>
+cudaError_t res_dispatch(const ResLayer *layer, int layers, bool tap, F go)
 {
     bool affine = true;
     for (int i = 0; i < layers; ++i) affine &= layer[i].affine != 0;
-    if (tap) return go(std::true_type(), std::false_type());
+    if (tap) return affine ? go(std::true_type(), std::true_type()) : go(std::true_type(), std::false_type());
     return affine ? go(std::false_type(), std::true_type()) : go(std::false_type(), std::false_type());
 }
 
 cudaError_t res_first_launch(const ResFirstParams &p, int sm_count, cudaStream_t st)
 {
-    return res_dispatch(p, &p.layer, 1, p.tap_in != nullptr, [&](auto tap, auto affine) {
+    return res_dispatch(&p.layer, 1, p.tap_in != nullptr, [&](auto tap, auto affine) {
         auto go = [&](auto kernel) { return res_launch(kernel, p, 32 * (kFirstEpi + kFirstCtx), kFirstSmem, sm_count, st); };
         return p.ingest_mode == 2 ? go(res_first_kernel<true, tap(), affine()>) : go(res_first_kernel<false, tap(), affine()>);
     });
@@ -881,7 +881,7 @@ cudaError_t res_first_launch(const ResFirstParams &p, int sm_count, cudaStream_t
 // Up to an image per SM only one context would work: then it has all the warps (four warpgroups).
 cudaError_t res_stack1_launch(const ResStack1Params &p, int sm_count, cudaStream_t st)
 {
-    return res_dispatch(p, p.layer, 5, p.tap_x2 != nullptr, [&](auto tap, auto affine) {
+    return res_dispatch(p.layer, 5, p.tap_x2 != nullptr, [&](auto tap, auto affine) {
         if (p.batch <= sm_count)
             return res_launch(res_stack1_kernel<tap(), affine(), 1, 4>, p, S1Shape<1, 4>::Threads, S1Shape<1, 4>::Smem, sm_count, st);
         return res_launch(res_stack1_kernel<tap(), affine(), 3, 2>, p, S1Shape<3, 2>::Threads, S1Shape<3, 2>::Smem, sm_count, st);
@@ -890,7 +890,7 @@ cudaError_t res_stack1_launch(const ResStack1Params &p, int sm_count, cudaStream
 
 cudaError_t res_stack23_launch(const ResStack23Params &p, int sm_count, cudaStream_t st)
 {
-    return res_dispatch(p, p.layer, 9, p.tap_x3 != nullptr, [&](auto tap, auto affine) {
+    return res_dispatch(p.layer, 9, p.tap_x3 != nullptr, [&](auto tap, auto affine) {
         if (p.batch <= sm_count)
             return res_launch(res_stack23_kernel<tap(), affine(), 1, 4>, p, S2Shape<1, 4>::Threads, S2Shape<1, 4>::Smem, sm_count, st);
         return res_launch(res_stack23_kernel<tap(), affine(), 3, 2>, p, S2Shape<3, 2>::Threads, S2Shape<3, 2>::Smem, sm_count, st);

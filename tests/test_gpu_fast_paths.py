@@ -264,24 +264,69 @@ def test_hidden_layer_last_layer_and_sampler_in_tiles(hidden, actions, value, b)
     g.close()
 
 
+def _requantisers(g, kernel):
+    """For each launch of ``kernel`` in the plan: "A" if layers run the single-fma requantiser, "D" if layers run the
+    three-step division, "AD" for some of each."""
+    return [("A" if "single-fma requantiser verified" in l else "") + ("D" if "3-step divide verified" in l else "")
+            for l in g.info()["plan"].splitlines() if kernel in l]
+
+
+# drawn residual networks: every layer with single-fma constants (the kernels without the division's code), layers of
+# both sorts in two launches and none in the first, the search skipped
+RESIDUAL_FORMS = {"single_fma": (1, "", ["A", "A", "A"]), "both": (2, "", ["D", "AD", "AD"]),
+                  "division": (21, "FLAG_TEST_NO_AFFINE", ["D", "D", "D"])}
+
+
 @pytest.mark.parametrize("b", [1, 148, 149, 445, 900])
-@pytest.mark.parametrize("flag", ["", "FLAG_TEST_NO_AFFINE"], ids=["single_fma", "division"])
-def test_residual_network_kernels_by_images_per_sm(b, flag):
-    """One image per SM, two or three at once, several in turn; single-fma and dividing code: the logits of the
-    dp4a kernels, bit for bit."""
+@pytest.mark.parametrize("form", list(RESIDUAL_FORMS))
+def test_residual_network_kernels_by_images_per_sm(b, form):
+    """One image per SM, two or three at once, several in turn; single-fma code, code with both requantisers, division in
+    every layer: the logits of the dp4a kernels, bit for bit."""
     import paper_2211_15023_b200 as P
-    pol = W.drawn_int8_policy("impala_resnet_b16384", seed=21)
+    seed, flag, want = RESIDUAL_FORMS[form]
+    pol = W.drawn_int8_policy("impala_resnet_b16384", seed=seed)
     obs = torch.from_numpy(W.observations("impala_resnet_b16384", b, seed=b)).cuda()
     u = torch.from_numpy(W.uniforms("impala_resnet_b16384", b, seed=b)).cuda()
     got = []
     for flags in (getattr(P, flag) if flag else 0, P.FLAG_FORCE_GENERIC):
         g = P.Policy(pol, b, flags=flags)
-        assert ("res_stack1_kernel" in g.info()["plan"]) == (flags != P.FLAG_FORCE_GENERIC)
+        assert _requantisers(g, "res_") == ([] if flags == P.FLAG_FORCE_GENERIC else want), g.info()["plan"]
         got.append([t.clone() for t in g.act(obs, u)])
         g.check()
         g.close()
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("b", [5, 149, 460])
+@pytest.mark.parametrize("form", list(RESIDUAL_FORMS))
+def test_residual_network_activations_by_images_per_sm(b, form):
+    """The same kernels with the stores of their taps, at one image per SM, at two, and where contexts take several in
+    turn: every tensor that the plan stores is the dp4a kernels', bit for bit."""
+    import paper_2211_15023_b200 as P
+    seed, flag, want = RESIDUAL_FORMS[form]
+    name = "impala_resnet_b16384"
+    pol = W.drawn_int8_policy(name, seed=seed)
+    obs = torch.from_numpy(W.observations(name, b, seed=b)).cuda()
+    u = torch.from_numpy(W.uniforms(name, b, seed=b)).cuda()
+    g = P.Policy(pol, b, flags=P.FLAG_KEEP_ACTIVATIONS | P.FLAG_TAP_FUSED | (getattr(P, flag) if flag else 0))
+    ref = P.Policy(pol, b, flags=P.FLAG_KEEP_ACTIVATIONS | P.FLAG_FORCE_GENERIC)
+    assert _requantisers(g, "res_") == want, g.info()["plan"]
+    for x, y in zip(g.act(obs, u), ref.act(obs, u)):
+        assert torch.equal(x, y)
+    g.check()
+    missing = []
+    for i in range(-1, len(pol["layers"]) - 1):
+        try:
+            got = g.read_activation(i, b)
+        except P.AccerlError as e:
+            assert e.status == 2
+            missing.append(i)
+            continue
+        assert np.array_equal(got, ref.read_activation(i, b)), "layer %d" % i
+    assert missing == [0, 6, 17]  # pooled before they are stored, or kept ReLU'd only
+    g.close()
+    ref.close()
 
 
 @pytest.mark.parametrize("flag", ["", "FLAG_TEST_NO_AFFINE"], ids=["single_fma", "division"])
