@@ -1,6 +1,7 @@
 // Parameters of the image-resident kernel of the Atari conv stacks (tc_atari.cu).
 #pragma once
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace accerl {
@@ -37,6 +38,8 @@ struct AtariParams {
     int *status;
     AtariLayer layer[3];
 };
+
+static_assert(sizeof(AtariLayer) % 16 == 0 && offsetof(AtariParams, layer) % 16 == 0, "constants are read 16 bytes at a time");
 
 constexpr int kAtariWeightsWide = 4 * 32 * 64 + 4 * 64 * 128 + 9 * 64 * 64, kAtariWeightsNarrow = 4 * 16 * 64 + 4 * 32 * 64 + 9 * 32 * 32;
 
