@@ -140,11 +140,10 @@ __device__ __forceinline__ void requant16_fastdiv(const int (&acc)[16], const fl
 // (k2 > 0); for every output channel the pair (k2, b2) near (k / s_out, b / s_out) is searched at
 // create until the two functions agree on every accumulator between the two points where both
 // saturate, which makes them equal on all of int32 (fit_affine_kernel in requant_fit.cu).
-template <bool RELU>
-__device__ __forceinline__ int affine_code(int acc, float k2, float b2)
+__device__ __forceinline__ int affine_code(float acc, float k2, float b2, bool relu)
 {
-    const int q = min(max(__float2int_rn(__fmaf_rn(__int2float_rn(acc), k2, b2)), -128), 127);
-    return RELU ? max(q, 0) : q;
+    const int q = min(max(__float2int_rn(__fmaf_rn(acc, k2, b2)), -128), 127);
+    return relu ? max(q, 0) : q;
 }
 
 // sixteen codes by the single fma, two elements per instruction

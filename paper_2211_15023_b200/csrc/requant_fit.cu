@@ -74,11 +74,7 @@ __global__ void __launch_bounds__(kFitThreads) fit_affine_kernel(const FitJob *j
     // saturated at an end that is no int32 limit
     const bool ends_ok = (!job.check_lo || code_lo == (relu ? 0 : -128)) && (!job.check_hi || code_hi == 127);
     auto refuted = [&](float k2, float b2) {
-        auto affine = [&](float x) {
-            const int q = min(max(__float2int_rn(__fmaf_rn(x, k2, b2)), -128), 127);
-            return relu ? max(q, 0) : q;
-        };
-        const int a0 = affine(x0), a1 = affine(x1);
+        const int a0 = affine_code(x0, k2, b2, relu), a1 = affine_code(x1, k2, b2, relu);
         return rises ? a0 >= mine || a1 < mine : ends && (!ends_ok || a0 != code_lo || a1 != code_hi);
     };
     auto candidate_k = [&](int cand) { return __uint_as_float(__float_as_uint(job.k0) + (unsigned)alternate(cand % kKOffsets)); };
@@ -128,7 +124,8 @@ bool make_job(float k, float b, float s_out, bool relu, FitJob *job)
     job->check_hi = hi <= 2147483647.0;
     job->lo = (long long)std::max(lo, -2147483648.0);
     job->hi = (long long)std::min(hi, 2147483647.0);
-    // (bands of the networks here have 65 k - 350 k accumulators; the limit bounds the search time)
+    // (bands of the networks here have 65 k - 350 k accumulators; the limit is from when the whole band was compared, and
+    // channels with wider ones still divide)
     return job->hi >= job->lo && job->hi - job->lo <= (1LL << 22);
 }
 

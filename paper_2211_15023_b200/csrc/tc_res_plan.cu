@@ -11,7 +11,9 @@ namespace accerl {
 
 namespace {
 
-// layers 0 .. 17 of the IMPALA network on 84 x 84 frames: per stack conv, pool, two blocks of two convs
+// layers 0 .. 17 of the IMPALA network on 84 x 84 frames: per stack conv, pool, two blocks of two convs.  The kernels
+// apply ReLU by a layer's number, to what the first conv of a block writes and to what a block reads; that is right
+// because networks with other flags are refused here.
 bool is_impala(const accerl_layer_desc *layers, int n_layers)
 {
     if (n_layers < kResLayers + 2) return false;
@@ -56,7 +58,6 @@ void res_layer(const accerl_layer_desc &d, const LayerRequant &rq, ResLayer *L)
     L->s_out = d.s_out;
     L->inv_s_out = rq.inv_s_out;
     L->affine = rq.affine;
-    L->relu = (d.flags & ACCERL_RELU_OUT) != 0;
 }
 
 // byte of K position kk of column n inside a K step's [columns][32 bytes] block, 32-byte swizzle

@@ -14,7 +14,7 @@ struct ResLayer {
     float k[32], b[32];  // per channel: the single-fma pair, or (s_in * s_w, bias) for the division
     uint32_t mul[32];    // residual multiplier in the 16-bit lane dp2a reads: skip_mul << (16 * (c & 1))
     float s_out, inv_s_out;
-    int affine, relu;
+    int affine, pad;     // (a multiple of 16 bytes)
 };
 
 // Geometry: 84 x 84 frames, stacks of 41 x 41 x 16, 20 x 20 x 32 and 9 x 9 x 32.  Every tensor is a
