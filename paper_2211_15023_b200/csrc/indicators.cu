@@ -46,7 +46,7 @@ __device__ __forceinline__ float warp_maxf(float v)
 // function", 1989): x = (64 m + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^m 2^(j/64) (1 + r + ... + r^5 / 120);
 // the truncation is below 3e-17, the result within about one ulp.  `table` holds 2^(j/64).  It has half the
 // instructions of exp(), of which the rows kernel needs two per action (16 x 8192 rollouts of 18 actions,
-// V-trace and both launches of the KL: 27 us with exp(), 24.6 us with this).
+// V-trace and both launches of the KL, rows copied element by element as they were then: 27 us with exp(), 24.6 with this).
 __device__ __forceinline__ double exp_nonpositive(double x, const double *table)
 {
     const double shift = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
@@ -155,12 +155,13 @@ __device__ __forceinline__ void cluster_stats(double sum, float mx, int B, float
 // are all in flight at once, so that the loads are whole lines and every thread then walks its own row, a chain
 // of two exponentials an action.  A warp per row, as below, leaves 14 of 32 lanes idle at 18 actions and spends
 // its time in shuffles; with that and a one-block reduction the two launches for 131072 rows of 18 took 119 us,
-// with this kernel 20.5 element by element and some 18 in 16-byte copies (with V-trace 24.6 and 22.5).
+// with this kernel 20.7 element by element and 18.7 in 16-byte copies (with V-trace 24.6 and 22.6; rows of 9 actions 16.5
+// and 14.5, of 31 26.8 and 24.7, of 62 51.1 and 43.2).
 //
 // V > 0: the rows lie in shared memory as in global memory and come in 16-byte copies (a fourth of the
 // instructions, and no row and column to keep); a thread reads V = 1, 2 or 4 elements at a time, the width at which
-// rows of that many elements fall into different banks.  V = 0, for rows of a multiple of eight elements or
-// addresses that are none of 16 bytes: element by element into rows of an odd pitch.
+// rows of that many elements fall into different banks.  V = 0, for rows of a multiple of eight elements,
+// addresses that are none of 16 bytes and always with STATS: element by element into rows of an odd pitch.
 //
 // STATS (one cluster, at most kKlCluster blocks' rows a pass): the mean and the maximum come out of the same launch.
 template <bool STATS, int V>

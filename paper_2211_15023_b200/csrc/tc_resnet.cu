@@ -26,12 +26,20 @@
 // operand rows its taps reach are there (its own tile and the neighbours), so no layer ends in a wait for all
 // of its warps; the issuing warp also lets the next image land as soon as its last MMA has read this one.
 //
-// What bounds it: the tensor pipe by instruction count (10 080 cycles an image in res_stack1, 8 640 in
-// res_stack23, of 14 300 and 11 900; an MMA of N = 32 reads its operands at the full rate of shared memory)
-// and instruction issue of the epilogues (about half of the 37 000 warp instructions an image takes in
-// res_stack1 convert and pack its 164 000 codes).  Batch 16384, us per launch: whole layers handed over, both
-// requantisers in the code 489 / 841 / 769, as it is 478 / 810 / 674; 100 images, one context with two or four
-// warpgroups: step 53.6 / 47.7.  A third warpgroup in res_first: 513 (spills).
+// What bounds it (counters at 4096 states, per image): the tensor pipe by instruction count (10 080 of 15 100 cycles
+// in res_stack1, 8 640 of 12 800 in res_stack23; an MMA of N = 32 reads its operands at the full rate of shared
+// memory) and instruction issue of the epilogues (35 300 and 24 100 warp instructions, 60 and 48 % of the slots; in
+// res_stack1 about half of them convert and pack its 164 000 codes).
+//
+// Batch 16384, us per launch (with events between the launches; a step without them overlaps their ends) and step:
+//   single-fma code in all three                          409 / 808 / 634   1861
+//   the first layer divides, both sorts in the others     478 / 837 / 675   2002
+//   every layer divides                                   476 / 908 / 706   2111
+// One layer without single-fma constants gives its whole launch the code with both requantisers.  Of 60 drawn
+// networks 6 have constants everywhere, of 20 calibrated ones none (first 13, stack 1 eight, stacks 2 and 3 none).
+// Handed over by whole layers, both requantisers in all code: 489 / 841 / 769 for a policy that divides in the first
+// layer and in some of stacks 2 and 3, as it is 478 / 810 / 674; 100 images of it, one context with two or four
+// warpgroups: step 53.6 / 47.7.  A third warpgroup in res_first: 513 (spills) against its 478.
 //
 // Every wait is bounded.  A role whose wait gives up sets the status word and goes on (all further
 // waits return at once), so that the barriers inside a context always see all their warps.
@@ -231,8 +239,10 @@ __device__ __forceinline__ void res_teardown(ResBars &bars, int warp, int alloc_
 // step may overlap the next row's) and holds the eight pixels 4X - 4 .. 4X + 3 of a line: enough for
 // the five outputs 4X - 2 .. 4X + 2 and thus for two pooled ones, whose three-pixel maxima are taken on
 // the accumulators (the requantiser is non-decreasing): N = 5 * 16, one K step per tap row.  The
-// maximum over three lines follows on the codes in shared memory.  The MMAs take 2 340 cycles an image;
-// the epilogue's instructions (33 k codes an image, some 14 k warp instructions) bound the kernel.
+// maximum over three lines follows on the codes in shared memory.  The MMAs take 2 340 of an image's 7 750 cycles
+// (4096 states), the 17 500 warp instructions 57 % of the issue slots; neither is full, as two images an SM take turns
+// at two barriers a context.  55.8 k codes (83 lines of 42 pooled pixels) are requantised and stored before the second
+// pass makes 26.9 k of them.
 namespace {
 constexpr int kFirstCtx = 2, kFirstWg = 2;                   // images in flight, warpgroups of each
 constexpr int kFirstT = kFirstWg * 128, kFirstEpi = kFirstCtx * kFirstWg * 4;
